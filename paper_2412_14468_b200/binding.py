@@ -1,4 +1,5 @@
-"""Thin ctypes binding over libhashattn.so: argument marshalling only.
+"""Thin binding over libhashattn.so: argument marshalling only, done in native code (_hostcall.so) for every call that
+takes tensors, through ctypes for the rest.
 
 Every function has the name and semantics of the C entry point declared in include/hashattn.h;
 tensors are torch tensors used purely as device (or pinned host) memory handles.  There is no
@@ -14,6 +15,7 @@ import torch
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "libhashattn.so")
+HOSTCALL_PATH = os.path.join(HERE, "_hostcall.so")
 
 HA_OK = 0
 HA_ERR_INVALID_ARG, HA_ERR_UNSUPPORTED, HA_ERR_WORKSPACE, HA_ERR_CUDA, HA_ERR_STATIC_LIMIT = 1, 2, 3, 4, 5
@@ -120,6 +122,22 @@ def lib() -> C.CDLL:
     return _lib
 
 
+_hostcall = None
+
+
+def _host():
+    """The native marshalling module: reading some twenty-five pointers, strides and sizes through Python attributes and
+    ctypes costs 11 - 13 us a call, more than the layer-step of a short sequence takes on the GPU."""
+    global _hostcall
+    if _hostcall is None:
+        lib()
+        if not os.path.exists(HOSTCALL_PATH):
+            raise RuntimeError(f"{HOSTCALL_PATH} not found: run `python -m paper_2412_14468_b200.build`")
+        from . import _hostcall as m
+        _hostcall = m
+    return _hostcall
+
+
 def status_string(status: int) -> str:
     return lib().ha_status_string(int(status)).decode()
 
@@ -161,13 +179,7 @@ class MappingWide:
 def ha_encode_wide(mapping: "MappingWide", heads_per_kv: int, x: torch.Tensor, codes: torch.Tensor,
                    slot: Optional[torch.Tensor] = None, stream=None) -> None:
     """x: bf16 [B,H,T,128] (or [B,H,128]); codes: int64 [B,H,>=T,n_bits/64] (the packed 64-bit words, contiguous per token)."""
-    xt = make_tensor(x)
-    B, H = x.shape[0], x.shape[1]
-    T = 1 if x.dim() == 3 else x.shape[2]
-    _dev(codes, torch.int64, "codes")
-    assert codes.dim() == 4 and codes.stride(3) == 1 and codes.stride(2) == codes.shape[3] == mapping.n_bits // 64
-    _check("ha_encode_wide", lib().ha_encode_wide(mapping.ref, heads_per_kv, C.byref(xt), B, H, T, codes.data_ptr(),
-                                                  codes.stride(0), codes.stride(1), _ptr(slot), _stream(stream)))
+    _check("ha_encode_wide", _host().encode_wide(mapping, heads_per_kv, x, codes, mapping.n_bits, slot, stream))
 
 
 def ha_workspace_bytes_wide(shape: ha_shape, max_seq_len: int) -> int:
@@ -184,13 +196,8 @@ def alloc_workspace_wide(shape: ha_shape, max_seq_len: int, device="cuda") -> to
 def ha_score_topk_wide(shape: ha_shape, n_bits: int, q_codes, k_codes, seq_lens, k_per_seq, k_uniform: int, max_seq_len: int,
                        k_max: int, idx, count, workspace, hist_out=None, stream=None) -> None:
     """q_codes int64 [B,Hq,W]; k_codes int64 [B,Hkv,N,W] (W = n_bits/64 words per token); idx int32 [B,Hkv,k_max]."""
-    _dev(q_codes, torch.int64, "q_codes"); _dev(k_codes, torch.int64, "k_codes")
-    assert q_codes.is_contiguous() and k_codes.dim() == 4 and k_codes.stride(3) == 1 and k_codes.stride(2) == k_codes.shape[3]
-    p, n = _ws(workspace)
-    _check("ha_score_topk_wide", lib().ha_score_topk_wide(
-        C.byref(shape), n_bits, q_codes.data_ptr(), k_codes.data_ptr(), k_codes.stride(0), k_codes.stride(1),
-        seq_lens.data_ptr(), _ptr(k_per_seq), k_uniform, max_seq_len, k_max, idx.data_ptr(), idx.stride(0), idx.stride(1),
-        count.data_ptr(), _ptr(hist_out), p, n, _stream(stream)))
+    _check("ha_score_topk_wide", _host().score_topk_wide(shape, n_bits, q_codes, k_codes, seq_lens, k_per_seq, k_uniform,
+                                                         max_seq_len, k_max, idx, count, workspace, hist_out, stream))
 
 
 def ha_inner_products(q: torch.Tensor, K: torch.Tensor, dots: torch.Tensor, stream=None) -> None:
@@ -282,20 +289,10 @@ def alloc_workspace(shape: ha_shape, max_seq_len: int, max_k: int, device="cuda"
     return ws
 
 
-def _ws(ws: torch.Tensor):
-    return ws.data_ptr(), ws.numel() * ws.element_size()
-
-
 def ha_encode(mapping: Mapping, heads_per_kv: int, x: torch.Tensor, codes: torch.Tensor,
               slot: Optional[torch.Tensor] = None, stream=None) -> None:
     """x: bf16 [B,H,T,128] (or [B,H,128]); codes: int32/uint32-as-int32 [B,H,>=T] (last dim contiguous)."""
-    xt = make_tensor(x)
-    B, H = x.shape[0], x.shape[1]
-    T = 1 if x.dim() == 3 else x.shape[2]
-    _dev(codes, torch.int32, "codes")
-    assert codes.dim() == 3 and codes.stride(2) == 1
-    _check("ha_encode", lib().ha_encode(mapping.ref, heads_per_kv, C.byref(xt), B, H, T, codes.data_ptr(),
-                                        codes.stride(0), codes.stride(1), _ptr(slot), _stream(stream)))
+    _check("ha_encode", _host().encode(mapping, heads_per_kv, x, codes, slot, stream))
 
 
 HA_PREFILL_TCGEN05, HA_PREFILL_MMA_SYNC = 0, 1
@@ -304,91 +301,54 @@ HA_PREFILL_TCGEN05, HA_PREFILL_MMA_SYNC = 0, 1
 def ha_encode_prefill(mapping: Mapping, heads_per_kv: int, x: torch.Tensor, codes: torch.Tensor,
                       path: int = HA_PREFILL_TCGEN05, workspace: Optional[torch.Tensor] = None, stream=None) -> None:
     """Tensor-core ENCODE of whole prompts; x: bf16 [B,H,T,128]; codes: int32 [B,H,>=T] (last dim contiguous)."""
-    xt = make_tensor(x)
-    B, H = x.shape[0], x.shape[1]
-    T = 1 if x.dim() == 3 else x.shape[2]
-    _dev(codes, torch.int32, "codes")
-    assert codes.dim() == 3 and codes.stride(2) == 1
-    _check("ha_encode_prefill", lib().ha_encode_prefill(mapping.ref, heads_per_kv, C.byref(xt), B, H, T, codes.data_ptr(),
-                                                        codes.stride(0), codes.stride(1), path, _ptr(workspace),
-                                                        _stream(stream)))
+    _check("ha_encode_prefill", _host().encode_prefill(mapping, heads_per_kv, x, codes, path, workspace, stream))
 
 
 def ha_score_topk(shape: ha_shape, q_codes, k_codes, seq_lens, k_per_seq, k_uniform: int, max_seq_len: int,
                   k_max: int, idx, count, workspace, hist_out=None, stream=None) -> None:
     """q_codes int32 [B,Hq]; k_codes int32 [B,Hkv,N]; idx int32 [B,Hkv,k_max]; count int32 [B,Hkv]."""
-    p, n = _ws(workspace)
-    _check("ha_score_topk", lib().ha_score_topk(
-        C.byref(shape), q_codes.data_ptr(), k_codes.data_ptr(), k_codes.stride(0), k_codes.stride(1),
-        seq_lens.data_ptr(), _ptr(k_per_seq), k_uniform, max_seq_len, k_max, idx.data_ptr(), idx.stride(0),
-        idx.stride(1), count.data_ptr(), _ptr(hist_out), p, n, _stream(stream)))
+    _check("ha_score_topk", _host().score_topk(shape, q_codes, k_codes, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, idx,
+                                               count, workspace, hist_out, stream))
 
 
 def ha_score_topk_sum(shape: ha_shape, q_codes, k_codes, seq_lens, k_per_seq, k_uniform: int, k_max: int, idx, count,
                       hist_out=None, stream=None) -> None:
     """ha_score_topk with the per-head scores of a group added up (0 .. 32 G); hist_out int32 [B,Hkv,32 G + 1]."""
-    _check("ha_score_topk_sum", lib().ha_score_topk_sum(
-        C.byref(shape), q_codes.data_ptr(), k_codes.data_ptr(), k_codes.stride(0), k_codes.stride(1),
-        seq_lens.data_ptr(), _ptr(k_per_seq), k_uniform, k_max, idx.data_ptr(), idx.stride(0), idx.stride(1),
-        count.data_ptr(), _ptr(hist_out), _stream(stream)))
+    _check("ha_score_topk_sum", _host().score_topk_sum(shape, q_codes, k_codes, seq_lens, k_per_seq, k_uniform, k_max, idx, count,
+                                                   hist_out, stream))
 
 
 def ha_score_topk_per_head(shape: ha_shape, q_codes, k_codes, seq_lens, k_per_seq, k_uniform: int, k_max: int, idx, count,
                            hist_out=None, stream=None) -> None:
     """One list per query head (no group reduction): idx int32 [B,Hq,k_max], count int32 [B,Hq], hist_out [B,Hq,33]."""
-    _check("ha_score_topk_per_head", lib().ha_score_topk_per_head(
-        C.byref(shape), q_codes.data_ptr(), k_codes.data_ptr(), k_codes.stride(0), k_codes.stride(1),
-        seq_lens.data_ptr(), _ptr(k_per_seq), k_uniform, k_max, idx.data_ptr(), idx.stride(0), idx.stride(1),
-        count.data_ptr(), _ptr(hist_out), _stream(stream)))
+    _check("ha_score_topk_per_head", _host().score_topk_per_head(shape, q_codes, k_codes, seq_lens, k_per_seq, k_uniform, k_max, idx, count,
+                                                   hist_out, stream))
 
 
 def ha_gather_attn_per_head(shape: ha_shape, q, K, V, seq_lens, idx, count, k_max: int, out, workspace, lse=None,
                             stream=None) -> None:
     """GATHER-ATT through per-query-head lists; workspace sized for the shape with n_kv_heads = n_q_heads."""
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K), make_tensor(V)
-    _check("ha_gather_attn_per_head", lib().ha_gather_attn_per_head(
-        C.byref(shape), q.data_ptr(), C.byref(kt), C.byref(vt), seq_lens.data_ptr(), idx.data_ptr(), idx.stride(0),
-        idx.stride(1), count.data_ptr(), k_max, out.data_ptr(), _ptr(lse), p, n, _stream(stream)))
+    _check("ha_gather_attn_per_head", _host().gather_attn_per_head(shape, q, K, V, seq_lens, idx, count, k_max, out, workspace, lse, stream))
 
 
 def ha_gather_attn(shape: ha_shape, q, K, V, seq_lens, idx, count, k_max: int, out, workspace, lse=None,
                    stream=None) -> None:
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K), make_tensor(V)
-    _check("ha_gather_attn", lib().ha_gather_attn(
-        C.byref(shape), q.data_ptr(), C.byref(kt), C.byref(vt), seq_lens.data_ptr(), idx.data_ptr(), idx.stride(0),
-        idx.stride(1), count.data_ptr(), k_max, out.data_ptr(), _ptr(lse), p, n, _stream(stream)))
+    _check("ha_gather_attn", _host().gather_attn(shape, q, K, V, seq_lens, idx, count, k_max, out, workspace, lse, stream))
 
 
 def ha_gather_attn_paged(shape: ha_shape, q, K_pool, V_pool, block_table, page_size: int, seq_lens, idx, count, k_max: int,
                          out, workspace, lse=None, stream=None) -> None:
     """K_pool, V_pool: bf16 [n_pages, Hkv, page_size, 128]; block_table: int32 [B, pages per sequence]."""
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K_pool), make_tensor(V_pool)
-    _check("ha_gather_attn_paged", lib().ha_gather_attn_paged(
-        C.byref(shape), q.data_ptr(), C.byref(kt), C.byref(vt), block_table.data_ptr(), block_table.stride(0), page_size,
-        seq_lens.data_ptr(), idx.data_ptr(), idx.stride(0), idx.stride(1), count.data_ptr(), k_max, out.data_ptr(),
-        _ptr(lse), p, n, _stream(stream)))
-
-
-def _pool(code_pool: torch.Tensor):
-    """int32 [n_pages, Hkv, page_size] signature pool -> (pointer, page stride, head stride, page size)."""
-    _dev(code_pool, torch.int32, "code_pool")
-    assert code_pool.dim() == 3 and code_pool.stride(2) == 1
-    return code_pool.data_ptr(), code_pool.stride(0), code_pool.stride(1), code_pool.shape[2]
+    _check("ha_gather_attn_paged", _host().gather_attn_paged(shape, q, K_pool, V_pool, block_table, page_size, seq_lens, idx,
+                                                     count, k_max, out, workspace, lse, stream))
 
 
 def ha_score_topk_paged(shape: ha_shape, q_codes, code_pool, block_table, seq_lens, k_per_seq, k_uniform: int, max_seq_len: int,
                         k_max: int, idx, count, workspace, hist_out=None, per_head: bool = False, stream=None) -> None:
     """ha_score_topk (per_head: ha_score_topk_per_head) over a paged signature pool int32 [n_pages, Hkv, page_size]."""
-    p, n = _ws(workspace)
-    cp, sp, sh, ps = _pool(code_pool)
-    fn = lib().ha_score_topk_per_head_paged if per_head else lib().ha_score_topk_paged
-    _check("ha_score_topk_per_head_paged" if per_head else "ha_score_topk_paged", fn(
-        C.byref(shape), q_codes.data_ptr(), cp, sp, sh, block_table.data_ptr(), block_table.stride(0), ps, seq_lens.data_ptr(),
-        _ptr(k_per_seq), k_uniform, max_seq_len, k_max, idx.data_ptr(), idx.stride(0), idx.stride(1), count.data_ptr(),
-        _ptr(hist_out), p, n, _stream(stream)))
+    name = "score_topk_per_head_paged" if per_head else "score_topk_paged"
+    _check("ha_" + name, getattr(_host(), name)(shape, q_codes, code_pool, block_table, seq_lens, k_per_seq, k_uniform, max_seq_len,
+                                                k_max, idx, count, workspace, hist_out, stream))
 
 
 def ha_score_topk_per_head_paged(shape: ha_shape, q_codes, code_pool, block_table, seq_lens, k_per_seq, k_uniform: int,
@@ -400,22 +360,13 @@ def ha_score_topk_per_head_paged(shape: ha_shape, q_codes, code_pool, block_tabl
 
 def ha_gather_attn_per_head_paged(shape: ha_shape, q, K_pool, V_pool, block_table, page_size: int, seq_lens, idx, count,
                                   k_max: int, out, workspace, lse=None, stream=None) -> None:
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K_pool), make_tensor(V_pool)
-    _check("ha_gather_attn_per_head_paged", lib().ha_gather_attn_per_head_paged(
-        C.byref(shape), q.data_ptr(), C.byref(kt), C.byref(vt), block_table.data_ptr(), block_table.stride(0), page_size,
-        seq_lens.data_ptr(), idx.data_ptr(), idx.stride(0), idx.stride(1), count.data_ptr(), k_max, out.data_ptr(),
-        _ptr(lse), p, n, _stream(stream)))
+    _check("ha_gather_attn_per_head_paged", _host().gather_attn_per_head_paged(shape, q, K_pool, V_pool, block_table, page_size, seq_lens, idx,
+                                                     count, k_max, out, workspace, lse, stream))
 
 
 def ha_encode_append_paged(mapping: Mapping, k_new, code_pool, block_table, seq_lens, stream=None) -> None:
     """Signature of k_new bf16 [B, Hkv, 128] written at token seq_lens[b] - 1 of sequence b in the paged pool."""
-    cp, sp, sh, ps = _pool(code_pool)
-    _dev(k_new, torch.bfloat16, "k_new")
-    assert k_new.is_contiguous()
-    _check("ha_encode_append_paged", lib().ha_encode_append_paged(
-        mapping.ref, k_new.data_ptr(), k_new.shape[0], cp, sp, sh, block_table.data_ptr(), block_table.stride(0), ps,
-        seq_lens.data_ptr(), _stream(stream)))
+    _check("ha_encode_append_paged", _host().encode_append_paged(mapping, k_new, code_pool, block_table, seq_lens, stream))
 
 
 def ha_sparse_decode_paged_codes(shape: ha_shape, map_q: Mapping, map_k: Optional[Mapping], q, k_new, K_pool, V_pool, code_pool,
@@ -423,103 +374,65 @@ def ha_sparse_decode_paged_codes(shape: ha_shape, map_q: Mapping, map_k: Optiona
                                  count, out, workspace, lse=None, stream=None) -> None:
     """The whole step with K, V (bf16 [n_pages, Hkv, page_size, 128]) and the signatures (int32 [n_pages, Hkv, page_size])
     all paged through one block table int32 [B, pages]."""
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K_pool), make_tensor(V_pool)
-    cp, sp, sh, ps = _pool(code_pool)
-    _check("ha_sparse_decode_paged_codes", lib().ha_sparse_decode_paged_codes(
-        C.byref(shape), map_q.ref, None if map_k is None else map_k.ref, q.data_ptr(), _ptr(k_new), C.byref(kt), C.byref(vt),
-        cp, sp, sh, block_table.data_ptr(), block_table.stride(0), ps, seq_lens.data_ptr(), _ptr(k_per_seq), k_uniform,
-        max_seq_len, k_max, q_codes.data_ptr(), idx.data_ptr(), idx.stride(0), idx.stride(1), count.data_ptr(), out.data_ptr(),
-        _ptr(lse), p, n, _stream(stream)))
+    _check("ha_sparse_decode_paged_codes", _host().sparse_decode_paged_codes(
+        shape, map_q, map_k, q, k_new, K_pool, V_pool, code_pool, block_table, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max,
+        q_codes, idx, count, out, workspace, lse, stream))
 
 
 def ha_gather_attn_static(shape: ha_shape, q, K, V, seq_lens, idx, count, k_max: int, out, lse=None, stream=None) -> None:
     """ha_gather_attn for callers that cannot allocate a workspace: the scratch is a fixed array inside
     the library (batch * n_kv_heads <= 64).  Make the first call on a device outside stream capture;
     calls that may overlap on the GPU must be ordered by the caller."""
-    kt, vt = make_tensor(K), make_tensor(V)
-    _check("ha_gather_attn_static", lib().ha_gather_attn_static(
-        C.byref(shape), q.data_ptr(), C.byref(kt), C.byref(vt), seq_lens.data_ptr(), idx.data_ptr(), idx.stride(0),
-        idx.stride(1), count.data_ptr(), k_max, out.data_ptr(), _ptr(lse), _stream(stream)))
+    _check("ha_gather_attn_static", _host().gather_attn_static(shape, q, K, V, seq_lens, idx, count, k_max, out, lse, stream))
 
 
 def ha_dense_decode(shape: ha_shape, q, K, V, seq_lens, max_seq_len: int, out, workspace, lse=None,
                     stream=None) -> None:
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K), make_tensor(V)
-    _check("ha_dense_decode", lib().ha_dense_decode(
-        C.byref(shape), q.data_ptr(), C.byref(kt), C.byref(vt), seq_lens.data_ptr(), max_seq_len, out.data_ptr(),
-        _ptr(lse), p, n, _stream(stream)))
+    _check("ha_dense_decode", _host().dense_decode(shape, q, K, V, seq_lens, max_seq_len, out, workspace, lse, stream))
 
 
 def ha_sparse_decode(shape: ha_shape, map_q: Mapping, map_k: Optional[Mapping], q, k_new, K, V, k_codes, seq_lens,
                      k_per_seq, k_uniform: int, max_seq_len: int, k_max: int, q_codes, idx, count, out, workspace,
                      lse=None, stream=None) -> None:
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K), make_tensor(V)
-    _check("ha_sparse_decode", lib().ha_sparse_decode(
-        C.byref(shape), map_q.ref, None if map_k is None else map_k.ref, q.data_ptr(), _ptr(k_new), C.byref(kt),
-        C.byref(vt), k_codes.data_ptr(), k_codes.stride(0), k_codes.stride(1), seq_lens.data_ptr(), _ptr(k_per_seq),
-        k_uniform, max_seq_len, k_max, q_codes.data_ptr(), idx.data_ptr(), idx.stride(0), idx.stride(1),
-        count.data_ptr(), out.data_ptr(), _ptr(lse), p, n, _stream(stream)))
+    _check("ha_sparse_decode", _host().sparse_decode(
+        shape, map_q, map_k, q, k_new, K, V, k_codes, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, q_codes, idx, count, out,
+        workspace, lse, stream))
 
 
 def ha_sparse_decode_pipelined(shape: ha_shape, map_q: Mapping, map_k: Optional[Mapping], q, k_new, K, V, k_codes, seq_lens,
                                k_per_seq, k_uniform: int, max_seq_len: int, k_max: int, q_codes, idx, count, out, workspace,
                                lse=None, stream=None) -> None:
     """ha_sparse_decode on the schedule that runs SCORE + TOPK ahead of GATHER-ATT inside one persistent kernel."""
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K), make_tensor(V)
-    _check("ha_sparse_decode_pipelined", lib().ha_sparse_decode_pipelined(
-        C.byref(shape), map_q.ref, None if map_k is None else map_k.ref, q.data_ptr(), _ptr(k_new), C.byref(kt),
-        C.byref(vt), k_codes.data_ptr(), k_codes.stride(0), k_codes.stride(1), seq_lens.data_ptr(), _ptr(k_per_seq),
-        k_uniform, max_seq_len, k_max, q_codes.data_ptr(), idx.data_ptr(), idx.stride(0), idx.stride(1),
-        count.data_ptr(), out.data_ptr(), _ptr(lse), p, n, _stream(stream)))
+    _check("ha_sparse_decode_pipelined", _host().sparse_decode_pipelined(
+        shape, map_q, map_k, q, k_new, K, V, k_codes, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, q_codes, idx, count, out,
+        workspace, lse, stream))
 
 
 def ha_sparse_decode_paged(shape: ha_shape, map_q: Mapping, map_k: Optional[Mapping], q, k_new, K_pool, V_pool, block_table,
                            page_size: int, k_codes, seq_lens, k_per_seq, k_uniform: int, max_seq_len: int, k_max: int,
                            q_codes, idx, count, out, workspace, lse=None, stream=None) -> None:
     """The whole step over a paged K/V cache: pools bf16 [n_pages, Hkv, page_size, 128], block_table int32 [B, pages]."""
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K_pool), make_tensor(V_pool)
-    _check("ha_sparse_decode_paged", lib().ha_sparse_decode_paged(
-        C.byref(shape), map_q.ref, None if map_k is None else map_k.ref, q.data_ptr(), _ptr(k_new), C.byref(kt),
-        C.byref(vt), block_table.data_ptr(), block_table.stride(0), page_size, k_codes.data_ptr(), k_codes.stride(0),
-        k_codes.stride(1), seq_lens.data_ptr(), _ptr(k_per_seq), k_uniform, max_seq_len, k_max, q_codes.data_ptr(),
-        idx.data_ptr(), idx.stride(0), idx.stride(1), count.data_ptr(), out.data_ptr(), _ptr(lse), p, n, _stream(stream)))
+    _check("ha_sparse_decode_paged", _host().sparse_decode_paged(
+        shape, map_q, map_k, q, k_new, K_pool, V_pool, block_table, page_size, k_codes, seq_lens, k_per_seq, k_uniform, max_seq_len,
+        k_max, q_codes, idx, count, out, workspace, lse, stream))
 
 
 def ha_sparse_decode_host(shape: ha_shape, map_q: Mapping, map_k: Mapping, q_host, k_new_host, v_new_host, K, V,
                           k_codes, seq_lens, k_per_seq, k_uniform: int, max_seq_len: int, k_max: int, idx, count,
                           out_host, workspace, stream=None) -> None:
     """q_host/k_new_host/v_new_host/out_host: pinned CPU bf16 tensors; everything else on the device."""
-    for t in (q_host, k_new_host, v_new_host, out_host):
-        if t.is_cuda or not t.is_contiguous():
-            raise TypeError("host buffers must be contiguous CPU tensors")
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K), make_tensor(V)
-    _check("ha_sparse_decode_host", lib().ha_sparse_decode_host(
-        C.byref(shape), map_q.ref, map_k.ref, q_host.data_ptr(), k_new_host.data_ptr(), v_new_host.data_ptr(),
-        C.byref(kt), C.byref(vt), k_codes.data_ptr(), k_codes.stride(0), k_codes.stride(1), seq_lens.data_ptr(),
-        _ptr(k_per_seq), k_uniform, max_seq_len, k_max, idx.data_ptr(), idx.stride(0), idx.stride(1),
-        count.data_ptr(), out_host.data_ptr(), p, n, _stream(stream)))
+    _check("ha_sparse_decode_host", _host().sparse_decode_host(
+        shape, map_q, map_k, q_host, k_new_host, v_new_host, K, V, k_codes, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, idx,
+        count, out_host, workspace, stream))
 
 
 def ha_sparse_decode_paged_host(shape: ha_shape, map_q: Mapping, map_k: Mapping, q_host, k_new_host, v_new_host, K_pool,
                                 V_pool, block_table, page_size: int, k_codes, seq_lens, k_per_seq, k_uniform: int,
                                 max_seq_len: int, k_max: int, idx, count, out_host, workspace, stream=None) -> None:
     """ha_sparse_decode_host over a paged K/V cache (pools bf16 [n_pages, Hkv, page_size, 128], block_table int32 [B, pages])."""
-    for t in (q_host, k_new_host, v_new_host, out_host):
-        if t.is_cuda or not t.is_contiguous():
-            raise TypeError("host buffers must be contiguous CPU tensors")
-    p, n = _ws(workspace)
-    kt, vt = make_tensor(K_pool), make_tensor(V_pool)
-    _check("ha_sparse_decode_paged_host", lib().ha_sparse_decode_paged_host(
-        C.byref(shape), map_q.ref, map_k.ref, q_host.data_ptr(), k_new_host.data_ptr(), v_new_host.data_ptr(),
-        C.byref(kt), C.byref(vt), block_table.data_ptr(), block_table.stride(0), page_size, k_codes.data_ptr(),
-        k_codes.stride(0), k_codes.stride(1), seq_lens.data_ptr(), _ptr(k_per_seq), k_uniform, max_seq_len, k_max,
-        idx.data_ptr(), idx.stride(0), idx.stride(1), count.data_ptr(), out_host.data_ptr(), p, n, _stream(stream)))
+    _check("ha_sparse_decode_paged_host", _host().sparse_decode_paged_host(
+        shape, map_q, map_k, q_host, k_new_host, v_new_host, K_pool, V_pool, block_table, page_size, k_codes, seq_lens, k_per_seq,
+        k_uniform, max_seq_len, k_max, idx, count, out_host, workspace, stream))
 
 
 class SparseDecodeHostStep:
@@ -531,21 +444,14 @@ class SparseDecodeHostStep:
     def __init__(self, shape: ha_shape, map_q: Mapping, map_k: Mapping, q_host, k_new_host, v_new_host, K, V,
                  k_codes, seq_lens, k_per_seq, k_uniform: int, max_seq_len: int, k_max: int, idx, count, out_host,
                  workspace, stream=None):
-        for t in (q_host, k_new_host, v_new_host, out_host):
-            if t.is_cuda or not t.is_contiguous():
-                raise TypeError("host buffers must be contiguous CPU tensors")
-        p, n = _ws(workspace)
-        self._kt, self._vt = make_tensor(K), make_tensor(V)
         self._keep = (shape, map_q, map_k, q_host, k_new_host, v_new_host, K, V, k_codes, seq_lens, k_per_seq, idx, count,
                       out_host, workspace)
-        self._fn = lib().ha_sparse_decode_host
-        self._args = (C.byref(shape), map_q.ref, map_k.ref, q_host.data_ptr(), k_new_host.data_ptr(), v_new_host.data_ptr(),
-                      C.byref(self._kt), C.byref(self._vt), k_codes.data_ptr(), k_codes.stride(0), k_codes.stride(1),
-                      seq_lens.data_ptr(), _ptr(k_per_seq), k_uniform, max_seq_len, k_max, idx.data_ptr(), idx.stride(0),
-                      idx.stride(1), count.data_ptr(), out_host.data_ptr(), p, n, _stream(stream))
+        self._step = _host().host_step_prepare(shape, map_q, map_k, q_host, k_new_host, v_new_host, K, V, k_codes, seq_lens,
+                                               k_per_seq, k_uniform, max_seq_len, k_max, idx, count, out_host, workspace, stream)
+        self._run = _hostcall.host_step_run
 
     def __call__(self) -> None:
-        status = self._fn(*self._args)
+        status = self._run(self._step)
         if status != HA_OK:
             raise HashAttnError("ha_sparse_decode_host", status)
 

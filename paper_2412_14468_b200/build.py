@@ -1,4 +1,5 @@
-"""Compile the CUDA sources into paper_2412_14468_b200/libhashattn.so for sm_100a (in-tree).
+"""Compile the CUDA sources into paper_2412_14468_b200/libhashattn.so for sm_100a (in-tree), and the native argument
+marshalling of the binding into paper_2412_14468_b200/_hostcall.so, which links against it.
 
 Every .cu file becomes an object under csrc/build/ (compiled in parallel, recompiled only when it or a header
 changed), then the objects are linked into the shared library."""
@@ -8,6 +9,7 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -15,6 +17,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(HERE, "libhashattn.so")
+HOST_SRC = os.path.join(CSRC, "host", "ha_hostcall.cpp")
+HOST_LIB = os.path.join(HERE, "_hostcall.so")
 
 NVCC_FLAGS = [
     "-std=c++17", "-O3", "-lineinfo",
@@ -43,6 +47,21 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _build_hostcall() -> None:
+    """The extension module over torch's own C++ headers; g++ is enough, it has no device code."""
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    inc = [os.path.join(ROOT, "include"), os.path.join(root, "include"),
+           os.path.join(root, "include", "torch", "csrc", "api", "include"), sysconfig.get_paths()["include"],
+           os.path.join(cuda, "include")]
+    cmd = [os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", HOST_SRC, "-o", HOST_LIB]
+    cmd += [x for d in inc for x in ("-I", d)]
+    cmd += ["-L", HERE, "-l:" + os.path.basename(LIB), "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu",
+            "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
+    subprocess.run(cmd, check=True)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     nvcc = os.environ.get("NVCC", "nvcc")
     os.makedirs(OBJ, exist_ok=True)
@@ -61,6 +80,8 @@ def build(force: bool = False, verbose: bool = False) -> str:
         os.remove(stale)
     if todo or force or _stale(LIB, objs):
         subprocess.run([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", LIB] + objs, check=True)
+    if force or _stale(HOST_LIB, [HOST_SRC, os.path.join(ROOT, "include", "hashattn.h")]):
+        _build_hostcall()
     return LIB
 
 
