@@ -106,6 +106,7 @@ int ha_encode(const ha_mapping *map, int32_t heads_per_kv, const ha_tensor *x, i
         a.codes = codes; a.c_sb = c_stride_b; a.c_sh = c_stride_h;
         a.slot = slot; a.slot_minus_one = 0;
         a.n_heads = n_heads; a.heads_per_kv = heads_per_kv; a.n_cta = batch * (n_heads / heads_per_kv);
+        a.n_out = kBits;
         a.map = view(map);
         EncodeJob none{};
         HA_CUDA(launch_encode_vectors(a, none, st));
@@ -336,6 +337,7 @@ static int sparse_decode_impl(const ha_shape *shape, const ha_mapping *map_q, co
     jq.codes = q_codes; jq.c_sb = Hq; jq.c_sh = 1;
     jq.slot = nullptr; jq.slot_minus_one = 0;
     jq.n_heads = Hq; jq.heads_per_kv = Hq / Hkv; jq.n_cta = B * Hkv;
+    jq.n_out = kBits;
     jq.map = view(map_q);
     EncodeJob jk{};
     if (k_new) {
@@ -343,6 +345,7 @@ static int sparse_decode_impl(const ha_shape *shape, const ha_mapping *map_q, co
         jk.codes = k_codes; jk.c_sb = kc_stride_b; jk.c_sh = kc_stride_h;
         jk.slot = seq_lens; jk.slot_minus_one = 1;
         jk.n_heads = Hkv; jk.heads_per_kv = 1; jk.n_cta = B * Hkv;
+        jk.n_out = kBits;
         jk.map = view(map_k);
         jk.pages = code_pages;
     }
@@ -518,6 +521,7 @@ int ha_encode_append_paged(const ha_mapping *map, const uint16_t *k_new, int32_t
     jk.x = k_new; jk.x_sb = (long long)Hkv * kD; jk.x_sh = kD;
     jk.codes = code_pool; jk.slot = seq_lens; jk.slot_minus_one = 1;
     jk.n_heads = Hkv; jk.heads_per_kv = 1; jk.n_cta = batch * Hkv;
+    jk.n_out = kBits;
     jk.map = view(map);
     jk.pages = cp;
     EncodeJob none{};
@@ -668,6 +672,19 @@ int ha_encode_wide(const ha_mapping *map, int32_t heads_per_kv, const ha_tensor 
     if (slot && n_tokens != 1) return HA_ERR_INVALID_ARG;
     if (batch > 65535 || n_heads > 65535) return HA_ERR_UNSUPPORTED;
     if (batch == 0 || n_tokens == 0) return HA_OK;
+    if (n_tokens == 1 && heads_per_kv <= 8) {   // the vectors of a decode step
+        EncodeJob a{};
+        a.x = reinterpret_cast<const uint16_t *>(x->ptr);
+        a.x_sb = x->stride_b; a.x_sh = x->stride_h;
+        a.codes = reinterpret_cast<uint32_t *>(codes); a.c_sb = 2 * c_stride_b; a.c_sh = 2 * c_stride_h;
+        a.slot = slot; a.slot_minus_one = 0;
+        a.n_heads = n_heads; a.heads_per_kv = heads_per_kv; a.n_cta = batch * (n_heads / heads_per_kv);
+        a.n_out = map->n_bits;
+        a.map = view(map);
+        EncodeJob none{};
+        HA_CUDA(launch_encode_vectors(a, none, (cudaStream_t)stream));
+        return HA_OK;
+    }
     HA_CUDA(launch_encode_wide(view(map), map->n_bits, heads_per_kv, view(x), batch, n_heads, n_tokens, codes, c_stride_b,
                                c_stride_h, slot, (cudaStream_t)stream));
     return HA_OK;

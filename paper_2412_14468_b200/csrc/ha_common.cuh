@@ -154,12 +154,13 @@ struct CodePages {
 struct EncodeJob {
     const uint16_t *x;       // bf16, vector (b,h) at x + b*x_sb + h*x_sh
     long long x_sb, x_sh;
-    uint32_t *codes;         // written at codes + b*c_sb + h*c_sh + slot
+    uint32_t *codes;         // n_out / 32 words written at codes + b*c_sb + h*c_sh + slot * (n_out / 32) (strides in 32-bit words)
     long long c_sb, c_sh;
     const int32_t *slot;     // per-sequence slot (device) or NULL = 0
     int slot_minus_one;      // 1: slot[] holds sequence lengths, write at slot[b] - 1
     int n_heads, heads_per_kv, n_cta;   // n_cta = batch * n_heads / heads_per_kv
     int batch, cta_per_net;  // filled in by the launcher: sequences, and CTAs that share one network's items
+    int n_out, out_blocks;   // outputs of the last layer (bits of a signature) and, set by the launcher, the CTAs that share them
     MapView map;
     CodePages pages;         // pages.table != NULL: `codes` is a paged pool and the slot a token of the sequence
 };
@@ -169,7 +170,7 @@ __device__ __forceinline__ uint32_t *encode_slot_ptr(const EncodeJob &J, int b, 
     if (J.pages.table)
         return J.codes + (long long)J.pages.table[(long long)b * J.pages.bt_sb + (slot >> J.pages.shift)] * J.pages.page_stride +
                (long long)h * J.pages.head_stride + (slot & ((1 << J.pages.shift) - 1));
-    return J.codes + (long long)b * J.c_sb + (long long)h * J.c_sh + slot;
+    return J.codes + (long long)b * J.c_sb + (long long)h * J.c_sh + (long long)slot * (J.n_out / 32);
 }
 #endif
 

@@ -24,23 +24,30 @@ namespace ha {
 // shared-memory bandwidth (one 2-byte weight per lane and term), so one warp per scheduler that
 // reuses each weight for all its vectors beats more warps that each re-read the matrix.
 
+//
+// Signatures of 64 to 512 bits take the same kernel with a last layer of kOut = min(bits, 128) outputs per CTA: thread o
+// runs output o, and wider signatures are shared by bits / 128 CTAs that repeat the hidden layers.  (A signature of one
+// token in the 128-token tiles of the prompt kernel took 57 us whatever the batch; 32 keys or 128 queries take 6.)
+
 constexpr int kVecThreads = 128;
 constexpr size_t kVecWeightBytes = (size_t)(kD * kHid + kHid * kHid + kHid * kBits) * 2;
 
-template <int NV>
+template <int NV, int kOut>
 __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, EncodeJob jb) {
     extern __shared__ __align__(128) unsigned char vec_smem[];
     __shared__ __align__(8) unsigned long long s_bar[3];
     uint16_t *sw1 = reinterpret_cast<uint16_t *>(vec_smem);
     uint16_t *sw2 = sw1 + kD * kHid;
     uint16_t *sw3 = sw2 + kHid * kHid;
-    float *actA = reinterpret_cast<float *>(sw3 + kHid * kBits);   // [NV][128]
+    float *actA = reinterpret_cast<float *>(sw3 + kHid * kOut);   // [NV][128]
     float *actB = actA + NV * kD;
 
     int i = blockIdx.x;
     const bool second = i >= ja.n_cta;
     const EncodeJob &J = second ? jb : ja;
     if (second) i -= ja.n_cta;
+    int blk = 0;             // which kOut outputs of the last layer
+    if (kOut != kBits) { blk = i % J.out_blocks; i /= J.out_blocks; }
     const int P = J.cta_per_net, net = i / P, part = i % P;
     const int hpk = J.heads_per_kv;
     const int n_vec = J.batch * hpk;                 // vectors of this network: t -> (b = t / hpk, head net*hpk + t % hpk)
@@ -49,9 +56,10 @@ __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, E
 
     const uint16_t *g1 = J.map.w1 + (size_t)net * kD * kHid;
     const uint16_t *g2 = J.map.w2 + (size_t)net * kHid * kHid;
-    const uint16_t *g3 = J.map.w3 + (size_t)net * kHid * kBits;
+    const int ld3 = kOut == kBits ? kBits : J.n_out;   // row length of W3 in memory
+    const uint16_t *g3 = J.map.w3 + (size_t)net * kHid * ld3 + blk * kOut;
     const uint32_t bar0 = (uint32_t)__cvta_generic_to_shared(&s_bar[0]);
-    // ---- request all weights: three bulk copies, one mbarrier each
+    // ---- request all weights: three bulk copies, one mbarrier each (a block of a wider W3: one copy per row)
     if (tid == 0) {
         mbar_init(bar0, 1);
         mbar_init(bar0 + 8, 1);
@@ -61,12 +69,16 @@ __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, E
         bulk_g2s((uint32_t)__cvta_generic_to_shared(sw1), g1, kD * kHid * 2, bar0);
         mbar_expect_tx(bar0 + 8, kHid * kHid * 2);
         bulk_g2s((uint32_t)__cvta_generic_to_shared(sw2), g2, kHid * kHid * 2, bar0 + 8);
-        mbar_expect_tx(bar0 + 16, kHid * kBits * 2);
-        bulk_g2s((uint32_t)__cvta_generic_to_shared(sw3), g3, kHid * kBits * 2, bar0 + 16);
+        mbar_expect_tx(bar0 + 16, kHid * kOut * 2);
+        if (kOut == kBits) bulk_g2s((uint32_t)__cvta_generic_to_shared(sw3), g3, kHid * kOut * 2, bar0 + 16);
+    }
+    if (kOut != kBits) {
+        __syncthreads();     // the barrier is initialised and knows how much it will receive
+        bulk_g2s((uint32_t)__cvta_generic_to_shared(sw3 + tid * kOut), g3 + (size_t)tid * ld3, kOut * 2, bar0 + 16);
     }
     const float bias1 = J.map.b1 ? __ldg(J.map.b1 + net * kHid + o) : 0.0f;
     const float bias2 = J.map.b2 ? __ldg(J.map.b2 + net * kHid + o) : 0.0f;
-    const float bias3 = J.map.b3 ? __ldg(J.map.b3 + net * kBits + (tid & (kBits - 1))) : 0.0f;
+    const float bias3 = J.map.b3 ? __ldg(J.map.b3 + net * ld3 + blk * kOut + (tid & (kOut - 1))) : 0.0f;
     // The weights do not depend on earlier kernels of the stream; the vectors to encode may.  The
     // kernels behind this one are released only after the wait: whatever they read before their own
     // wait (sequence lengths, budgets, signatures) is then final, whoever wrote it earlier in the stream.
@@ -75,11 +87,12 @@ __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, E
 
     // wait for one weight matrix; if the bulk copy never reports completion, load it the ordinary way
     // (the decision is taken by the whole CTA together, so that the barrier below is never divergent)
-    auto weights_ready = [&](int which, uint16_t *dst, const uint16_t *src, int n_elems) {
+    auto weights_ready = [&](int which, uint16_t *dst, const uint16_t *src, int width, int ld) {
         const bool ok = mbar_wait_bounded(bar0 + 8 * which);
         if (__syncthreads_or(!ok)) {
-            for (int c = tid; c < n_elems / 8; c += kVecThreads)
-                reinterpret_cast<uint4 *>(dst)[c] = __ldg(reinterpret_cast<const uint4 *>(src) + c);
+            const int per_row = width / 8;
+            for (int c = tid; c < kHid * per_row; c += kVecThreads)
+                reinterpret_cast<uint4 *>(dst)[c] = __ldg(reinterpret_cast<const uint4 *>(src + (size_t)(c / per_row) * ld) + c % per_row);
             __syncthreads();
         }
     };
@@ -101,7 +114,7 @@ __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, E
 
         float z[NV];
         // ---- layer 1
-        if (first) weights_ready(0, sw1, g1, kD * kHid);
+        if (first) weights_ready(0, sw1, g1, kHid, kHid);
 #pragma unroll
         for (int v = 0; v < NV; ++v) z[v] = bias1;
         vec_layer<NV>(actA, sw1, kHid, o, z);
@@ -109,7 +122,7 @@ __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, E
         for (int v = 0; v < NV; ++v) actB[v * kD + o] = (z[v] > 0.0f) ? z[v] : 0.0f;
         __syncthreads();
         // ---- layer 2
-        if (first) weights_ready(1, sw2, g2, kHid * kHid);
+        if (first) weights_ready(1, sw2, g2, kHid, kHid);
 #pragma unroll
         for (int v = 0; v < NV; ++v) z[v] = bias2;
         vec_layer<NV>(actB, sw2, kHid, o, z);
@@ -118,9 +131,25 @@ __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, E
         for (int v = 0; v < NV; ++v) actA[v * kD + o] = (z[v] > 0.0f) ? z[v] : 0.0f;
         __syncthreads();
         // ---- layer 3: one output bit per lane; warp w takes vectors w, w + 4 (their chains interleaved)
-        if (first) weights_ready(2, sw3, g3, kHid * kBits);
+        if (first) weights_ready(2, sw3, g3, kOut, ld3);
         first = false;
-        {
+        if constexpr (kOut != kBits) {   // one output bit per thread, every vector of the item
+            if (tid < kOut) {            // warp-uniform
+#pragma unroll
+                for (int v = 0; v < NV; ++v) z[v] = bias3;
+                vec_layer<NV>(actA, sw3, kOut, o, z);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    const uint32_t word = __ballot_sync(0xffffffffu, z[v] > 0.0f);
+                    if (v < nv && (tid & 31) == 0) {
+                        const int t = t0 + v, b = t / hpk;
+                        int slot = 0;
+                        if (J.slot) slot = J.slot[b] - J.slot_minus_one;   // a negative slot skips the sequence
+                        if (slot >= 0) encode_slot_ptr(J, b, net * hpk + t % hpk, slot)[(blk * kOut + tid) >> 5] = word;
+                    }
+                }
+            }
+        } else {
             constexpr int kWarps = kVecThreads / 32, VT3 = (NV + kWarps - 1) / kWarps;
             const int warp = tid >> 5, lane = tid & 31;
             if (warp < nv) {   // warp-uniform; chains of slots >= nv read rows of the activation buffers and are dropped
@@ -146,18 +175,18 @@ __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, E
     }
 }
 
-template <int NV>
+template <int NV, int kOut>
 static cudaError_t launch_vec_t(const EncodeJob &a, const EncodeJob &b, cudaStream_t st) {
-    constexpr size_t smem = kVecWeightBytes + (size_t)2 * NV * kD * 4;
+    constexpr size_t smem = (size_t)(kD * kHid + kHid * kHid + kHid * kOut) * 2 + (size_t)2 * NV * kD * 4;
     static bool done[64] = {};   // opt in to > 48 KB of shared memory once per device
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(encode_vec_kernel<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(encode_vec_kernel<NV, kOut>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         done[dev] = true;
     }
-    cudaError_t e = launch_pdl(encode_vec_kernel<NV>, dim3(a.n_cta + b.n_cta), dim3(kVecThreads), smem, st, a, b);
+    cudaError_t e = launch_pdl(encode_vec_kernel<NV, kOut>, dim3(a.n_cta + b.n_cta), dim3(kVecThreads), smem, st, a, b);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
@@ -370,7 +399,9 @@ cudaError_t launch_encode_vectors(const EncodeJob &a_in, const EncodeJob &b_in, 
         vec_per_net[j] = J.batch * J.heads_per_kv;
     }
     const long long room = 2LL * sm_count();
-    if (vec_per_net[0] + vec_per_net[1] >= kTileMinVectors) {
+    const int n_out = a_in.n_cta > 0 ? a_in.n_out : b_in.n_out;   // both jobs have signatures of one width
+    const int n_blocks = n_out > kVecThreads ? n_out / kVecThreads : 1;
+    if (n_out == kBits && vec_per_net[0] + vec_per_net[1] >= kTileMinVectors) {
         // large batch: tiles of 4, 8 or 16 vectors per CTA, the smallest for which all CTAs are resident at once
         int tv = 4;
         auto tiles = [&](int t) {
@@ -390,7 +421,7 @@ cudaError_t launch_encode_vectors(const EncodeJob &a_in, const EncodeJob &b_in, 
     }
     auto ctas = [&](int m) {
         long long n = 0;
-        for (int j = 0; j < 2; ++j) n += (long long)nets[j] * ((vec_per_net[j] + m - 1) / m);
+        for (int j = 0; j < 2; ++j) n += (long long)nets[j] * ((vec_per_net[j] + m - 1) / m) * n_blocks;
         return n;
     };
     const int m_max = vec_per_net[0] > vec_per_net[1] ? vec_per_net[0] : vec_per_net[1];   // one CTA per network
@@ -400,18 +431,24 @@ cudaError_t launch_encode_vectors(const EncodeJob &a_in, const EncodeJob &b_in, 
     for (int j = 0; j < 2; ++j) {
         EncodeJob &J = job[j];
         J.cta_per_net = (vec_per_net[j] + m - 1) / m;
-        J.n_cta = nets[j] * J.cta_per_net;
+        J.out_blocks = n_blocks;
+        J.n_cta = nets[j] * J.cta_per_net * n_blocks;
     }
-    switch (nv) {
-        case 1: return launch_vec_t<1>(job[0], job[1], st);
-        case 2: return launch_vec_t<2>(job[0], job[1], st);
-        case 3: return launch_vec_t<3>(job[0], job[1], st);
-        case 4: return launch_vec_t<4>(job[0], job[1], st);
-        case 5: return launch_vec_t<5>(job[0], job[1], st);
-        case 6: return launch_vec_t<6>(job[0], job[1], st);
-        case 7: return launch_vec_t<7>(job[0], job[1], st);
-        default: return launch_vec_t<8>(job[0], job[1], st);
+#define HA_VEC(OUT)                                                \
+    switch (nv) {                                                  \
+        case 1: return launch_vec_t<1, OUT>(job[0], job[1], st);   \
+        case 2: return launch_vec_t<2, OUT>(job[0], job[1], st);   \
+        case 3: return launch_vec_t<3, OUT>(job[0], job[1], st);   \
+        case 4: return launch_vec_t<4, OUT>(job[0], job[1], st);   \
+        case 5: return launch_vec_t<5, OUT>(job[0], job[1], st);   \
+        case 6: return launch_vec_t<6, OUT>(job[0], job[1], st);   \
+        case 7: return launch_vec_t<7, OUT>(job[0], job[1], st);   \
+        default: return launch_vec_t<8, OUT>(job[0], job[1], st);  \
     }
+    if (n_out == kBits) HA_VEC(kBits)
+    if (n_out == 64) HA_VEC(64)
+    HA_VEC(kVecThreads)
+#undef HA_VEC
 }
 
 // ------------------------------------------------------------------ token-tiled bulk kernel

@@ -4,7 +4,9 @@
 // layer-step, then the standard top-k of Section 4 with ties towards the lowest token index.  Scores take b + 1
 // values, so the selection is again a histogram threshold plus an index-ordered compaction, never a sort.
 //
-// Three kernels over chunks of every (sequence, KV head) unit, each at full parallelism, nothing waits:
+// Sequences of up to 131072 tokens: ONE kernel, a thread-block cluster per (sequence, KV head) unit
+// (wide_select_cluster_kernel, second half of this file).  Longer ones: three kernels over chunks of every unit, each at
+// full parallelism, nothing waits:
 //   1. wide_scan_kernel      streams the signatures, leaves one 16-bit score per token in the workspace and adds the
 //                            chunk's level counts to the unit's (b + 1)-level histogram;
 //   2. wide_count_kernel     every chunk derives the threshold T (largest level with #{S >= T} >= k) from the unit's
@@ -13,6 +15,8 @@
 //                            their final positions (ascending token index; the first r = k - #{S > T} tokens at T).
 // Tokens that are always in context (the first n_sink, the most recent n_local) carry the score 0xFFFF, which is
 // above every threshold, and are left out of the histogram.
+#include <atomic>
+
 #include "ha_score_dev.cuh"
 
 namespace ha {
@@ -260,6 +264,282 @@ __global__ void __launch_bounds__(kWideThreads) wide_write_kernel(const WideArgs
     }
 }
 
+// ------------------------------------------------------------------ one kernel, a cluster per unit
+//
+// A cluster of up to eight CTAs owns a unit: every CTA leaves the scores of its slice in shared memory (16 bits per
+// token), the CTAs exchange their level counts through distributed shared memory between two cluster barriers, and each
+// compacts its own slice.  Against the three kernels for long sequences there is no memset, no histogram and no score
+// pass through global memory, and the signatures are requested before the programmatic-launch wait.
+// Bound: the population-count unit (16 lanes per clock and SM; a token costs G popcounts per counted word), then HBM.
+// Carry-save adders on the logic unit fold the xor words of a token before they are counted: 3, 4 and 5 counted words
+// instead of 4, 8 and 16 for 128, 256 and 512 bits.
+// Counting: counters [level][column], a lane bumps column lane % kCols (32 columns up to 128 bits, then 16 and 8: the
+// table stays at 17 KB and the scores spread over more levels).
+// Measured, 4 sequences of 32768 tokens with 8 KV heads and groups of 4 at 128 bits, whole decode step through the entry
+// points (ENCODE of keys and of queries, this kernel, GATHER-ATT): 33.6 us, against 155 us with the three kernels above
+// (19 + 5 + 6 us and a memset) and ENCODE in 128-token tiles (57 + 57 us).
+constexpr int kWideSlice = kWideThreads * 8;         // tokens of one row of a CTA: eight per thread
+constexpr int kWideMaxRows = 8;                      // a thread's flags fit one 64-bit word
+constexpr int kWideClusterMaxSeq = 8 * kWideMaxRows * kWideSlice;
+
+template <int W> struct WideShape;                   // tokens per thread and pass (64 to 128 bytes in flight twice), columns
+template <> struct WideShape<1> { static constexpr int kTok = 8, kCols = 32; };
+template <> struct WideShape<2> { static constexpr int kTok = 4, kCols = 32; };
+template <> struct WideShape<4> { static constexpr int kTok = 4, kCols = 16; };
+template <> struct WideShape<8> { static constexpr int kTok = 2, kCols = 8; };
+
+// full adder on bit columns: s + 2 c = x + y + z
+__device__ __forceinline__ void csa(uint32_t x, uint32_t y, uint32_t z, uint32_t &s, uint32_t &c) {
+    s = x ^ y ^ z;
+    c = (x & y) | (x & z) | (y & z);
+}
+// bits set in 2 W words
+template <int W>
+__device__ __forceinline__ int count_words(const uint32_t (&x)[2 * W]) {
+    if constexpr (W == 1) {
+        return __popc(x[0]) + __popc(x[1]);
+    } else if constexpr (W == 2) {
+        uint32_t s, c;
+        csa(x[0], x[1], x[2], s, c);
+        return __popc(s) + __popc(x[3]) + 2 * __popc(c);
+    } else if constexpr (W == 4) {
+        uint32_t s0, s1, s2, c0, c1, c2, t, f;
+        csa(x[0], x[1], x[2], s0, c0);
+        csa(x[3], x[4], x[5], s1, c1);
+        csa(s0, s1, x[6], s2, c2);
+        csa(c0, c1, c2, t, f);
+        return __popc(s2) + __popc(x[7]) + 2 * __popc(t) + 4 * __popc(f);
+    } else {
+        uint32_t s[5], c[7], u0, u1, t0, t1, t2, f0, f1, f2, e, f;
+#pragma unroll
+        for (int i = 0; i < 5; ++i) csa(x[3 * i], x[3 * i + 1], x[3 * i + 2], s[i], c[i]);
+        csa(s[0], s[1], s[2], u0, c[5]);
+        csa(s[3], s[4], x[15], u1, c[6]);          // ones left: u0, u1
+        csa(c[0], c[1], c[2], t0, f0);
+        csa(c[3], c[4], c[5], t1, f1);
+        csa(t0, t1, c[6], t2, f2);                 // twos left: t2
+        csa(f0, f1, f2, f, e);                     // fours: f, eights: e
+        return __popc(u0) + __popc(u1) + 2 * __popc(t2) + 4 * __popc(f) + 8 * __popc(e);
+    }
+}
+
+// flags of eight consecutive 16-bit scores + 1: bit i = score > T / == T, with t2 = (T + 1) in both halves
+__device__ __forceinline__ void wide_flags8(const uint4 &v, uint32_t t2, uint32_t &gt, uint32_t &eq) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    gt = 0u; eq = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t g = __vcmpgtu2(w[i], t2), q = __vcmpeq2(w[i], t2);
+        gt |= ((g & 1u) | ((g >> 15) & 2u)) << (2 * i);
+        eq |= ((q & 1u) | ((q >> 15) & 2u)) << (2 * i);
+    }
+}
+
+template <int W>
+__global__ void __launch_bounds__(kWideThreads) wide_select_cluster_kernel(const WideArgs a, int rows_max) {
+    constexpr int kTok = WideShape<W>::kTok, kCols = WideShape<W>::kCols;
+    extern __shared__ __align__(16) unsigned char wsm[];
+    uint16_t *s_sc = reinterpret_cast<uint16_t *>(wsm);                                   // [rows_max * kWideSlice] score + 1, 0 = none
+    uint32_t *c_hist = reinterpret_cast<uint32_t *>(s_sc + (size_t)rows_max * kWideSlice);    // [levels][kCols]
+    const int levels = a.n_bits + 1;
+    __shared__ int s_hist[kWideMaxLevels + 7], s_tot[kWideMaxLevels + 7], s_bef[kWideMaxLevels + 7];
+    __shared__ __align__(16) unsigned long long s_q[kMaxGroup][W];
+    __shared__ int sh_T, sh_gt, sh_gt_before, sh_eq_before, s_wcnt[kWideThreads / 32];
+    const int rank = (int)cluster_rank(), cs = (int)gridDim.x;                            // the cluster spans the grid's x
+    const int g = blockIdx.y, b = blockIdx.z;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const WideUnit wu = wide_unit(a, b);
+    const int n = wu.n;
+    const int Rb = (n + cs * kWideSlice - 1) / (cs * kWideSlice);                         // the sequence's own length is shared out
+    const int slice = Rb * kWideSlice, base = rank * slice, unit = b * a.Hkv + g;
+    const uint64_t *row = a.k_codes + (long long)b * a.kc_sb + (long long)g * a.kc_sh;
+
+    // a pass: token base + (p kTok + i) 256 + tid for i < kTok, so that a warp reads consecutive signatures
+    auto load_token = [&](unsigned long long (&kw)[W], int t, bool early) {
+        if (W == 1) {
+            kw[0] = early ? __ldg(reinterpret_cast<const unsigned long long *>(row + t)) : __ldcg(reinterpret_cast<const unsigned long long *>(row + t));
+        } else {
+#pragma unroll
+            for (int w = 0; w < W; w += 2) {
+                const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(row + (long long)t * W + w);
+                const ulonglong2 v = early ? __ldg(src) : __ldcg(src);
+                kw[w] = v.x; kw[w + 1] = v.y;
+            }
+        }
+    };
+    auto load_pass = [&](unsigned long long (&kw)[kTok][W], int p, bool early) {
+#pragma unroll
+        for (int i = 0; i < kTok; ++i) {
+            const int l = (p * kTok + i) * kWideThreads + tid;
+            if (l < slice && base + l < n) load_token(kw[i], base + l, early);
+            else
+#pragma unroll
+                for (int w = 0; w < W; ++w) kw[i][w] = 0ull;
+        }
+    };
+    unsigned long long cur[kTok][W], nxt[kTok][W];
+    load_pass(cur, 0, true);
+    for (int i = tid; i < levels * kCols; i += kWideThreads) c_hist[i] = 0u;
+    pdl_launch_dependents();
+    pdl_wait();
+    // the signatures that a library kernel directly in front may just have written (slots n-1 and n-2): read again
+#pragma unroll
+    for (int i = 0; i < kTok; ++i) {
+        const int l = i * kWideThreads + tid, t = base + l;
+        if (l < slice && t < n && t >= n - 2) load_token(cur[i], t, false);
+    }
+    if (tid < a.G * W)
+        s_q[tid / W][tid % W] = __ldcg(reinterpret_cast<const unsigned long long *>(a.q_codes) +
+                                       ((long long)b * a.Hq + (long long)g * a.G + tid / W) * W + tid % W);
+    __syncthreads();
+
+    const int n_pass = Rb * 8 / kTok;
+    for (int p = 0; p < n_pass; ++p) {
+        if (p + 1 < n_pass) load_pass(nxt, p + 1, false);
+        int best[kTok];
+#pragma unroll
+        for (int i = 0; i < kTok; ++i) best[i] = a.n_bits;
+        for (int j = 0; j < a.G; ++j) {
+            unsigned long long qv[W];
+#pragma unroll
+            for (int w = 0; w < W; ++w) qv[w] = s_q[j][w];
+#pragma unroll
+            for (int i = 0; i < kTok; ++i) {
+                uint32_t x[2 * W];
+#pragma unroll
+                for (int w = 0; w < W; ++w) {
+                    const unsigned long long v = cur[i][w] ^ qv[w];
+                    x[2 * w] = (uint32_t)v;
+                    x[2 * w + 1] = (uint32_t)(v >> 32);
+                }
+                best[i] = min(best[i], count_words<W>(x));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kTok; ++i) {
+            const int l = (p * kTok + i) * kWideThreads + tid, t = base + l;
+            if (l < slice) {
+                uint32_t v = 0u;
+                if (t < n) {
+                    const int score = a.n_bits - best[i];
+                    if (t < wu.wbd.sink_end || t >= wu.wbd.local_begin) v = kWideForced;
+                    else { v = (uint32_t)score + 1u; atomicAdd(&c_hist[score * kCols + (lane & (kCols - 1))], 1u); }
+                }
+                s_sc[l] = (uint16_t)v;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kTok; ++i)
+#pragma unroll
+            for (int w = 0; w < W; ++w) cur[i][w] = nxt[i][w];
+    }
+    __syncthreads();
+    for (int l = tid; l < levels; l += kWideThreads) {
+        uint32_t c = 0u;
+#pragma unroll
+        for (int k = 0; k < kCols; ++k) c += c_hist[l * kCols + ((k + l) & (kCols - 1))];
+        s_hist[l] = (int)c;
+    }
+    cluster_sync_all();   // every CTA's level counts are complete and visible cluster-wide
+    for (int l = tid; l < levels; l += kWideThreads) {
+        int tot = 0, bef = 0;
+        for (int r = 0; r < cs; ++r) {
+            const int v = ld_dsmem(&s_hist[l], (uint32_t)r);
+            tot += v;
+            if (r < rank) bef += v;
+        }
+        s_tot[l] = tot;
+        s_bef[l] = bef;
+    }
+    cluster_arrive();     // done with the peers' memory; the matching wait is at the end
+    __syncthreads();
+    if (warp == 0) {
+        int T, gt;
+        wide_threshold(s_tot, levels, wu.keep_rest, lane, T, gt);
+        int gb = 0;
+        for (int l = T + 1 + lane; l < levels; l += 32) gb += s_bef[l];
+#pragma unroll
+        for (int dd = 16; dd > 0; dd >>= 1) gb += __shfl_xor_sync(0xffffffffu, gb, dd);
+        if (lane == 0) { sh_T = T; sh_gt = gt; sh_gt_before = gb; sh_eq_before = T < levels ? s_bef[T] : 0; }
+    }
+    if (rank == 0 && a.hist_out)
+        for (int l = tid; l < levels; l += kWideThreads) a.hist_out[(long long)unit * levels + l] = s_tot[l];
+    __syncthreads();
+    const int T = sh_T, r = wu.keep_rest - sh_gt;   // tokens of score exactly T that are still wanted
+    int32_t *list = a.idx + (long long)b * a.idx_sb + (long long)g * a.idx_sh;
+    if (rank == 0) {
+        if (tid == 0) a.count[unit] = wu.keep;
+        for (int i = wu.keep + tid; i < a.k_max; i += kWideThreads) list[i] = -1;
+    }
+    if (wu.keep == 0) { cluster_wait(); return; }
+
+    // thread = the 8 Rb consecutive tokens from first_l on
+    const uint32_t t2 = (uint32_t)(T + 1) * 0x00010001u;
+    const int first_l = 8 * Rb * tid;
+    uint32_t gt_lo = 0u, gt_hi = 0u, eq_lo = 0u, eq_hi = 0u;
+#pragma unroll
+    for (int j = 0; j < kWideMaxRows; ++j) {
+        if (j < Rb) {
+            uint32_t gf, ef;
+            wide_flags8(*reinterpret_cast<const uint4 *>(s_sc + first_l + 8 * j), t2, gf, ef);
+            if (j < 4) { gt_lo |= gf << (8 * j); eq_lo |= ef << (8 * j); }
+            else { gt_hi |= gf << (8 * (j - 4)); eq_hi |= ef << (8 * (j - 4)); }
+        }
+    }
+    const int packed = (__popc(gt_lo) + __popc(gt_hi)) | ((__popc(eq_lo) + __popc(eq_hi)) << 16);
+    int inc = packed;
+#pragma unroll
+    for (int dd = 1; dd < 32; dd <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, dd);
+        if (lane >= dd) inc += v;
+    }
+    if (lane == 31) s_wcnt[warp] = inc;
+    __syncthreads();
+    int g_run = sh_gt_before + forced_before(wu.wbd, min(base, n)), q_run = sh_eq_before;
+#pragma unroll
+    for (int w = 0; w < kWideThreads / 32; ++w)
+        if (w < warp) { g_run += s_wcnt[w] & 0xffff; q_run += (int)((unsigned)s_wcnt[w] >> 16); }
+    if (packed != 0) {
+        const int excl = inc - packed;
+        g_run += excl & 0xffff;
+        q_run += (int)((unsigned)excl >> 16);
+        write_selected32(list, base + first_l, gt_lo, eq_lo, g_run, q_run, r);
+        write_selected32(list, base + first_l + 32, gt_hi, eq_hi, g_run, q_run, r);
+    }
+    cluster_wait();
+}
+
+template <int W>
+static cudaError_t launch_wide_cluster(const WideArgs &a, int B, int cs, int rows, cudaStream_t st) {
+    const size_t smem = (size_t)rows * kWideSlice * 2 + (size_t)(a.n_bits + 1) * WideShape<W>::kCols * 4;
+    static std::atomic<bool> opted[64];   // opt in to more than 48 KB of shared memory once per device
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64 || !opted[dev].load(std::memory_order_acquire)) {
+        cudaError_t e = cudaFuncSetAttribute(wide_select_cluster_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) opted[dev].store(true, std::memory_order_release);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cs, a.Hkv, B);
+    cfg.blockDim = dim3(kWideThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cs;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, wide_select_cluster_kernel<W>, a, rows);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    return cudaGetLastError();
+}
+
 // Workspace of the wide selection: header | unit histograms | chunk counts | 16-bit scores.
 struct WideLayout {
     size_t off_hist, off_counts, off_scores, score_row, total;
@@ -291,6 +571,21 @@ cudaError_t launch_score_topk_wide(int B, int Hq, int Hkv, int n_bits, const uin
     a.chunk_counts = reinterpret_cast<int32_t *>(ws + L.off_counts);
     a.scores = reinterpret_cast<uint16_t *>(ws + L.off_scores);
     a.score_row = (long long)L.score_row;
+    if (max_seq_len <= kWideClusterMaxSeq) {
+        // One cluster per unit: the largest of 8, 4, 2 CTAs whose grid is resident at once (three CTAs per SM), so that few
+        // units get the most CTAs each; at least as many as the rows of a CTA hold.
+        int cs = 8;
+        while (cs > 2 && (long long)B * Hkv * cs > 3LL * sm_count()) cs >>= 1;
+        while (max_seq_len > cs * kWideMaxRows * kWideSlice) cs <<= 1;
+        const int rows = max(1, (max_seq_len + cs * kWideSlice - 1) / (cs * kWideSlice));
+        switch (n_bits / 64) {
+            case 1: return launch_wide_cluster<1>(a, B, cs, rows, st);
+            case 2: return launch_wide_cluster<2>(a, B, cs, rows, st);
+            case 4: return launch_wide_cluster<4>(a, B, cs, rows, st);
+            case 8: return launch_wide_cluster<8>(a, B, cs, rows, st);
+            default: return cudaErrorInvalidValue;
+        }
+    }
     // chunks of whole passes, about eight CTAs per SM when there is that much work, at most kWideMaxChunks per unit
     const long long units = (long long)B * Hkv, n = max_seq_len > 0 ? max_seq_len : 1;
     long long per_unit = 8LL * sm_count() / (units > 0 ? units : 1);

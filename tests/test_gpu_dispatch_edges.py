@@ -1,0 +1,50 @@
+"""Sizes at which a kernel or a rule of a dispatch can go wrong (edges of tiles, remainders, the smallest and largest of a
+range), against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2412_14468_b200 import binding as ha
+from paper_2412_14468_b200 import workloads as wl
+from tests._util import u16
+from tests.test_gpu_parity import _check_score_topk_wide, _wide_codes, _wide_mapping
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+@pytest.mark.parametrize("n_bits", [64, 128, 256, 512])
+@pytest.mark.parametrize("B,G", [(1, 1), (3, 8), (40, 8)])
+def test_encode_wide_of_single_vectors_at_every_item_width(n_bits, B, G):
+    """One token per head takes the vector kernel: few vectors (one per CTA), more than CTA slots (items of several
+    vectors, several items per CTA), signatures shared by n_bits / 128 CTAs; strided inputs, no biases for the first."""
+    Hkv, W = 2, n_bits // 64
+    m = _wide_mapping(Hkv, n_bits, 60 + n_bits)
+    if B == 1:
+        m = {k: v for k, v in m.items() if k.startswith("w")}
+    mn = wl.mapping_numpy(m)
+    bias = lambda name, g: mn[name][g] if name in mn else None  # noqa: E731
+    x = torch.randn(B, Hkv * G, 3, 128, device=DEV, generator=torch.Generator(DEV).manual_seed(B)).to(torch.bfloat16)[:, :, 1]
+    codes = torch.full((B, Hkv * G, 2, W), -1, dtype=torch.int64, device=DEV)
+    ha.ha_encode_wide(ha.MappingWide(m), G, x, codes)
+    got = codes.cpu().numpy().view(np.uint64)
+    xu = u16(x.contiguous()).reshape(B, Hkv, G, 128)
+    for g in range(Hkv):
+        ref = oracle.encode_wide(np.ascontiguousarray(xu[:, g].reshape(B * G, 128)), mn["w1"][g], mn["w2"][g], mn["w3"][g],
+                                 bias("b1", g), bias("b2", g), bias("b3", g))
+        assert np.array_equal(got[:, g * G:(g + 1) * G, 0].reshape(B * G, W), ref)
+    assert (codes[:, :, 1] == -1).all()
+
+
+@pytest.mark.parametrize("n_bits", [64, 512])
+@pytest.mark.parametrize("lens", [(2047, 2048, 2049), (16383, 16385), (131071, 131072), (131073,), tuple(range(1, 1601, 23))])
+def test_score_topk_wide_at_row_and_cluster_edges(n_bits, lens):
+    """Rows of 2048 tokens, the longest sequence of the one-kernel path and the first beyond it, and a batch that takes
+    smaller clusters."""
+    rng = np.random.default_rng(len(lens))
+    W, Hkv, G = n_bits // 64, 2, 2
+    n_cap = max(lens)
+    kc = _wide_codes(rng, len(lens) * Hkv * n_cap, W).reshape(len(lens), Hkv, n_cap, W)
+    qc = _wide_codes(rng, len(lens) * Hkv * G, W).reshape(len(lens), Hkv * G, W)
+    _check_score_topk_wide(n_bits, qc, kc, list(lens), [max(1, n // 5) for n in lens], Hkv * G, Hkv, 3, 5)
