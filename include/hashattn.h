@@ -331,8 +331,8 @@ int ha_sparse_decode_paged_host(const ha_shape *shape, const ha_mapping *map_q, 
  *   ha_gather_attn_per_head_paged  ha_gather_attn_per_head over paged K/V pools (as ha_gather_attn_paged)
  *   ha_encode_append_paged         the append of Section 4.1 into the pool: signature of k_new [batch][n_kv_heads][128]
  *                                  (phi_kv) written at token seq_lens[b] - 1 of sequence b (skipped if that is < 0)
- *   ha_sparse_decode_paged_codes   the whole layer-step with K, V and the signatures all paged (ENCODE with the append
- *                                  into the pool, SCORE + TOPK, GATHER-ATT as separate kernels) */
+ *   ha_sparse_decode_paged_codes   the whole layer-step with K, V and the signatures all paged (one launch for few units,
+ *                                  else ENCODE with the append into the pool, SCORE + TOPK, GATHER-ATT) */
 int ha_score_topk_paged(const ha_shape *shape, const uint32_t *q_codes, const uint32_t *code_pool, int64_t cp_stride_page,
                         int64_t cp_stride_head, const int32_t *block_table, int64_t bt_stride_b, int32_t page_size,
                         const int32_t *seq_lens, const int32_t *k_per_seq, int32_t k_uniform, int32_t max_seq_len,

@@ -310,7 +310,7 @@ static int sparse_decode_impl(const ha_shape *shape, const ha_mapping *map_q, co
                             max_seq_len, k_max, idx, count));
     HA_TRY(check_mapping(map_q, shape->n_kv_heads));
     if (k_new) HA_TRY(check_mapping(map_k, shape->n_kv_heads));
-    const bool codes_paged = code_pages.table != nullptr;   // then only the kernel-by-kernel path knows the layout
+    const bool codes_paged = code_pages.table != nullptr;
     if (codes_paged && (pipelined || v_new_host)) return HA_ERR_UNSUPPORTED;
     HA_TRY(check_tensor(K));
     HA_TRY(check_tensor(V));
@@ -322,12 +322,12 @@ static int sparse_decode_impl(const ha_shape *shape, const ha_mapping *map_q, co
     const int B = shape->batch, Hq = shape->n_q_heads, Hkv = shape->n_kv_heads;
 
     if (pipelined && !pipe_step_eligible(B, Hq, Hkv)) return HA_ERR_UNSUPPORTED;
-    if (!pipelined && !codes_paged && fused_step_eligible(B, Hq, Hkv, max_seq_len, k_max)) {
+    if (!pipelined && fused_step_eligible(B, Hq, Hkv, max_seq_len, k_max)) {
         // small batch: the whole step is one cluster kernel
         HA_CUDA(launch_fused_step(B, Hq, Hkv, shape->sm_scale, view(map_q), k_new ? view(map_k) : MapView{}, q, k_new,
                                   view(K), view(V), k_codes, kc_stride_b, kc_stride_h, seq_lens, k_per_seq, k_uniform,
                                   max_seq_len, k_max, q_codes, idx, idx_stride_b, idx_stride_h, count, out, lse, st,
-                                  Windows{shape->n_sink, shape->n_local}, block_table, bt_stride_b, page_shift, v_new_host));
+                                  Windows{shape->n_sink, shape->n_local}, block_table, bt_stride_b, page_shift, v_new_host, code_pages));
         return HA_OK;
     }
     if (v_new_host) return HA_ERR_INVALID_ARG;   // only the fused kernel appends by itself

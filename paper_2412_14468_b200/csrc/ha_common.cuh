@@ -203,7 +203,7 @@ cudaError_t launch_score_topk(int B, int Hq, int Hkv, const uint32_t *q_codes, c
                               int32_t *idx, long long idx_sb, long long idx_sh, int32_t *count,
                               int32_t *hist_out, int32_t *ws_hist, unsigned char *ws_scores, cudaStream_t st, Windows win = Windows{0, 0},
                               CodePages pages = CodePages{nullptr, 0, 0, 0, 0}, int row_shift = -1);
-// pages.table != NULL: k_codes is a paged pool (always the two-kernel path); row_shift >= 0: one unit per QUERY head
+// pages.table != NULL: k_codes is a paged pool; row_shift >= 0: one unit per QUERY head
 // (Hq units per sequence, groups of one head), whose signature row is that of KV head h >> row_shift.
 
 // SCORE + TOPK with the group's per-head scores added instead of maximised (one cluster per unit, no scratch);
@@ -232,7 +232,8 @@ cudaError_t launch_fused_step(int B, int Hq, int Hkv, float sm_scale, const MapV
                               int k_uniform, int max_seq_len, int k_max, uint32_t *q_codes, int32_t *idx,
                               long long idx_sb, long long idx_sh, int32_t *count, uint16_t *out, float *lse,
                               cudaStream_t st, Windows win = Windows{0, 0}, const int32_t *block_table = nullptr,
-                              long long bt_sb = 0, int page_shift = 0, const uint16_t *v_new_host = nullptr);
+                              long long bt_sb = 0, int page_shift = 0, const uint16_t *v_new_host = nullptr,
+                              CodePages code_pages = CodePages{nullptr, 0, 0, 0, 0});
 
 // SCORE + TOPK and GATHER-ATT of a step in one persistent kernel whose SCORE warps run ahead of its GATHER warps
 // (steps of more units than the single-cluster kernel holds; the query signatures come from ENCODE in front).

@@ -58,6 +58,7 @@ struct FusedArgs {
     const uint16_t *q, *k_new;
     TensorView K, V;
     uint32_t *k_codes;
+    CodePages code_pages;    // table != NULL: k_codes is a paged pool
     long long kc_sb, kc_sh;
     const int32_t *seq_lens, *k_per_seq;
     int k_uniform, max_seq_len, k_max, Hq, Hkv;
@@ -277,8 +278,14 @@ __device__ __forceinline__ void fused_attention(const FusedArgs &a, uint32_t ran
     }
 }
 
-template <int G, int S, int CS, bool kHost>
+// Where the step's inputs lie, a compile-time variant because the one-stage kernel sits at its 128 registers (the test for
+// paged signatures at run time cost the cluster-of-4 kernel 0.9 us): everything in contiguous device memory; q, k_new and
+// v_new in mapped host memory; the signatures in pages.
+constexpr int kModeDevice = 0, kModeHost = 1, kModePagedCodes = 2;
+
+template <int G, int S, int CS, int kMode>
 __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kernel(const FusedArgs a) {
+    constexpr bool kHost = kMode == kModeHost, codes_paged = kMode == kModePagedCodes;
     constexpr int kFusedUnionBytes = fused_union_bytes(S);
     constexpr int kFusedActBytes = fused_act_bytes(G, CS);
     constexpr int kL = kFusedMaxSeq / (CS * 4096) * 4;   // uint4 of signatures per thread: 4, 8 or 16
@@ -317,7 +324,14 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     const int keep_rest = max(0, min(min(k, a.k_max - n_forced), n - n_forced));   // heavy tokens among the others
     const int keep = n_forced + keep_rest;
     const long long head0 = (long long)b * Hq + (long long)kvh * G;
-    uint32_t *row = a.k_codes + (long long)b * a.kc_sb + (long long)kvh * a.kc_sh;
+    // contiguous signatures: the unit's row; paged: the pool from this head's offset on
+    uint32_t *row = codes_paged ? a.k_codes + (long long)kvh * a.code_pages.head_stride
+                                : a.k_codes + (long long)b * a.kc_sb + (long long)kvh * a.kc_sh;
+    const int32_t *code_table = a.code_pages.table + (codes_paged ? (long long)b * a.code_pages.bt_sb : 0);
+    auto code_slot = [&](int t) -> uint32_t * {
+        if (!codes_paged) return row + t;
+        return row + (long long)__ldg(code_table + (t >> a.code_pages.shift)) * a.code_pages.page_stride + (t & ((1 << a.code_pages.shift) - 1));
+    };
     const bool has_new_key = (a.k_new != nullptr) && n > 0;
 
     // ---------------- P0: requests that do not depend on earlier kernels
@@ -328,7 +342,8 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
 #pragma unroll
         for (int p = 0; p < kL; ++p) {
             const int base = wbase + p * 4;
-            c[p] = (p < Lb && base < n) ? load_codes4(row, base, n) : make_uint4(0, 0, 0, 0);
+            c[p] = make_uint4(0, 0, 0, 0);
+            if (p < Lb && base < n) c[p] = codes_paged ? load_codes4_paged(a.code_pages, row, code_table, base, n) : load_codes4(row, base, n);
         }
     };
     if (kPreload) load_signatures();
@@ -394,7 +409,7 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     // the signatures also go to global memory (outputs of the step; nobody in this kernel reads them there):
     // stored after the barrier, so that its release had nothing but shared-memory stores to wait for
     if (enc_q && tid < kQPer) a.q_codes[head0 + kQPer * (int)rank + tid] = s_codes[kQPer * (int)rank + tid];
-    if (enc_k && tid == 0) row[n - 1] = s_codes[G];
+    if (enc_k && tid == 0) *code_slot(n - 1) = s_codes[G];
     if (kHost && tid < G * 16) reinterpret_cast<uint4 *>(actA)[tid] = q_stage;   // the activations are dead
     uint32_t qc[G];
 #pragma unroll
@@ -416,8 +431,8 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     if (has_new_key) replace_slot(n - 1, s_codes[G]);
     if (kPreload) {
         const int lo = wbase, hi = wbase + 4 * Lb;   // this lane's tokens (contiguous)
-        if (!has_new_key && n - 1 >= lo && n - 1 < hi) replace_slot(n - 1, __ldcg(row + n - 1));
-        if (n - 2 >= lo && n - 2 < hi) replace_slot(n - 2, __ldcg(row + n - 2));
+        if (!has_new_key && n - 1 >= lo && n - 1 < hi) replace_slot(n - 1, __ldcg(code_slot(n - 1)));
+        if (n - 2 >= lo && n - 2 < hi) replace_slot(n - 2, __ldcg(code_slot(n - 2)));
     }
 
     // ---------------- P2: SCORE, histogram, threshold, compaction
@@ -731,14 +746,14 @@ static void fused_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2]
 
 // Opt in to the shared-memory carve-out (once per device) and return how many clusters of this variant the
 // device holds at once (0 on error).
-template <int G, int S, int CS, bool kHost = false>
+template <int G, int S, int CS, int kMode = kModeDevice>
 static int fused_prepare() {
     static int clusters[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
     if (!clusters[dev]) {
-        if (cudaFuncSetAttribute(fused_step_kernel<G, S, CS, kHost>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(fused_step_kernel<G, S, CS, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  fused_smem_bytes(G, S, CS)) != cudaSuccess)
             return 0;
         cudaLaunchConfig_t cfg;
@@ -746,19 +761,19 @@ static int fused_prepare() {
         fused_config<G, S, CS>(cfg, attr, 1, 64, nullptr);
         cfg.numAttrs = 1;   // the cluster shape is all the occupancy query looks at
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, fused_step_kernel<G, S, CS, kHost>, &cfg) != cudaSuccess || n <= 0) return 0;
+        if (cudaOccupancyMaxActiveClusters(&n, fused_step_kernel<G, S, CS, kMode>, &cfg) != cudaSuccess || n <= 0) return 0;
         clusters[dev] = n;
     }
     return clusters[dev];
 }
 
-template <int G, int S, int CS, bool kHost = false>
+template <int G, int S, int CS, int kMode = kModeDevice>
 static cudaError_t launch_fused_gsc(const FusedArgs &args, int B, cudaStream_t st) {
-    if (fused_prepare<G, S, CS, kHost>() <= 0) return cudaErrorInvalidConfiguration;
+    if (fused_prepare<G, S, CS, kMode>() <= 0) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     fused_config<G, S, CS>(cfg, attr, args.Hkv, B, st);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, fused_step_kernel<G, S, CS, kHost>, args);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fused_step_kernel<G, S, CS, kMode>, args);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
@@ -820,8 +835,14 @@ static cudaError_t launch_fused_g(const FusedArgs &args, int B, cudaStream_t st)
     int stages = 0;
     const int cs = fused_variant<G>((long long)B * args.Hkv, args.k_max, &stages);
     if (args.v_new) {   // host-buffer entry: only the one-stage variants read their inputs across the bus
-        if (stages == 1 && cs == 8) return launch_fused_gsc<G, 1, 8, true>(args, B, st);
-        if (stages == 1 && cs == 4) return launch_fused_gsc<G, 1, 4, true>(args, B, st);
+        if (stages == 1 && cs == 8) return launch_fused_gsc<G, 1, 8, kModeHost>(args, B, st);
+        if (stages == 1 && cs == 4) return launch_fused_gsc<G, 1, 4, kModeHost>(args, B, st);
+        return cudaErrorInvalidConfiguration;
+    }
+    if (args.code_pages.table) {
+        if (stages == 2 && cs == 8) return launch_fused_gsc<G, 2, 8, kModePagedCodes>(args, B, st);
+        if (cs == 8) return launch_fused_gsc<G, 1, 8, kModePagedCodes>(args, B, st);
+        if (cs == 4) return launch_fused_gsc<G, 1, 4, kModePagedCodes>(args, B, st);
         return cudaErrorInvalidConfiguration;
     }
     if (stages == 2 && cs == 8) return launch_fused_gsc<G, 2, 8>(args, B, st);
@@ -836,8 +857,9 @@ cudaError_t launch_fused_step(int B, int Hq, int Hkv, float sm_scale, const MapV
                               int k_uniform, int max_seq_len, int k_max, uint32_t *q_codes, int32_t *idx,
                               long long idx_sb, long long idx_sh, int32_t *count, uint16_t *out, float *lse,
                               cudaStream_t st, Windows win, const int32_t *block_table, long long bt_sb, int page_shift,
-                              const uint16_t *v_new_host) {
+                              const uint16_t *v_new_host, CodePages code_pages) {
     FusedArgs a{};
+    a.code_pages = code_pages;
     a.v_new = v_new_host;
     a.win = win;
     a.block_table = block_table; a.bt_sb = bt_sb; a.page_shift = page_shift;

@@ -6,7 +6,8 @@
 //
 // Two implementations share the arithmetic:
 //  * sequences of up to 131072 tokens: ONE kernel, a thread-block cluster per (sequence, KV head)
-//    (score_select_cluster_kernel, second half of this file);
+//    (score_select_cluster_kernel, second half of this file), over contiguous or paged signatures (24 sequences of 2000 -
+//    65536 tokens in pages of 16, whole step: 61.4 us against 84.1 us with the two kernels below);
 //  * longer sequences: two kernels over chunks of the sequence, with the per-chunk histograms and
 //    one score byte per token passed through the workspace (scan_score_kernel, select_kernel).
 // No CTA ever spins on another: hand-offs are hardware cluster barriers or kernel boundaries.
@@ -291,12 +292,15 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
 
 constexpr int kClusterMaxRows = 8;   // rows of 8 tokens per lane: a lane's flags fit one 64-bit word each
 
-template <int G, int CS>
-__global__ void __launch_bounds__(kScanThreads, 6) score_select_cluster_kernel(
+// kPaged: the signatures lie in a pool behind a block table.  Pages of 8 tokens or more hold a lane's 8 tokens in one piece, so
+// a row costs one table entry per lane (neighbouring lanes share it) and the same two 16-byte loads.  The table entries of the
+// next two rows are fetched while the current ones are scored; five CTAs per SM instead of six pay for the registers.
+template <int G, int CS, bool kPaged>
+__global__ void __launch_bounds__(kScanThreads, kPaged ? 5 : 6) score_select_cluster_kernel(
     const uint32_t *__restrict__ q_codes, const uint32_t *__restrict__ k_codes, long long kc_sb, long long kc_sh,
     const int32_t *__restrict__ seq_lens, int max_seq_len, const int32_t *__restrict__ k_per_seq, int k_uniform,
     int k_max, int Hq, int Hkv, int32_t *__restrict__ idx, long long idx_sb, long long idx_sh,
-    int32_t *__restrict__ count, int32_t *__restrict__ hist_out, Windows win) {
+    int32_t *__restrict__ count, int32_t *__restrict__ hist_out, Windows win, const CodePages cp, int kv_shift) {
     extern __shared__ __align__(16) unsigned char s_sc[];      // score + 1 of this CTA's tokens (0 = no token)
     __shared__ __align__(16) uint32_t c_hist[kBins][32];       // counters [level][lane]
     __shared__ int s_hist[kBins + 3];          // this CTA's histogram, read by the whole cluster
@@ -312,7 +316,10 @@ __global__ void __launch_bounds__(kScanThreads, 6) score_select_cluster_kernel(
     const int n_forced = forced_before(wbd, n);
     const int keep_rest = max(0, min(min(k, k_max - n_forced), n - n_forced));   // heavy tokens among the others
     const int keep = n_forced + keep_rest;
-    const uint32_t *row = k_codes + (long long)b * kc_sb + (long long)g * kc_sh;
+    const int kvh = g >> kv_shift;   // the KV head whose signatures this unit scans
+    // contiguous cache: the unit's row; paged cache: the pool from this head's offset on
+    const uint32_t *row = kPaged ? k_codes + (long long)kvh * cp.head_stride : k_codes + (long long)b * kc_sb + (long long)kvh * kc_sh;
+    const int32_t *table_b = kPaged ? cp.table + (long long)b * cp.bt_sb : nullptr;
     // The sequence's own length is divided over the CS CTAs (ragged batches stay balanced): Rb rows per
     // lane, a warp owns the 256*Rb tokens from wb on, a CTA 2048*Rb; row p of a lane is
     // wb + 256 p + 8 lane .. + 7.
@@ -320,26 +327,40 @@ __global__ void __launch_bounds__(kScanThreads, 6) score_select_cluster_kernel(
     const int wl = warp * 256 * Rb;                    // the warp's first token inside the CTA's slice
     const int wb = (int)rank * 2048 * Rb + wl;
 
-    auto load_row = [&](int p, uint4 &lo, uint4 &hi, bool early) {
+    // paged: the pool words from which the lane's 8 tokens of row p are addressed by token number (pages of >= 8 tokens)
+    auto row_ptr = [&](int p) -> const uint32_t * {
+        if (!kPaged) return row;
         const int t = wb + p * 256 + lane * 8;
-        if (p < Rb && t + 8 <= n) {
-            const uint4 *src = reinterpret_cast<const uint4 *>(row + t);
+        if (cp.shift < 3 || p >= Rb || t >= n) return row;
+        return row + (long long)__ldg(table_b + (t >> cp.shift)) * cp.page_stride - (t & ~((1 << cp.shift) - 1));
+    };
+    auto load_row = [&](int p, const uint32_t *src_row, uint4 &lo, uint4 &hi, bool early) {
+        const int t = wb + p * 256 + lane * 8;
+        if (kPaged && cp.shift < 3) {   // small pages: four tokens (or one) at a time
+            lo = (p < Rb && t < n) ? load_codes4_paged(cp, row, table_b, t, n) : make_uint4(0, 0, 0, 0);
+            hi = (p < Rb && t + 4 < n) ? load_codes4_paged(cp, row, table_b, t + 4, n) : make_uint4(0, 0, 0, 0);
+        } else if (p < Rb && t + 8 <= n) {
+            const uint4 *src = reinterpret_cast<const uint4 *>(src_row + t);
             if (early) { lo = __ldg(src); hi = __ldg(src + 1); }
             else { lo = __ldcg(src); hi = __ldcg(src + 1); }
         } else {
-            lo = (p < Rb && t < n) ? load_codes4(row, t, n) : make_uint4(0, 0, 0, 0);
-            hi = (p < Rb && t + 4 < n) ? load_codes4(row, t + 4, n) : make_uint4(0, 0, 0, 0);
+            lo = (p < Rb && t < n) ? load_codes4(src_row, t, n) : make_uint4(0, 0, 0, 0);
+            hi = (p < Rb && t + 4 < n) ? load_codes4(src_row, t + 4, n) : make_uint4(0, 0, 0, 0);
         }
     };
     uint4 c[4];   // two rows
-    load_row(0, c[0], c[1], true);
-    load_row(1, c[2], c[3], true);
+    const uint32_t *r0 = row_ptr(0), *r1 = row_ptr(1);
+    load_row(0, r0, c[0], c[1], true);
+    load_row(1, r1, c[2], c[3], true);
     // the other rows of this warp start their way from HBM to L2 now (one request per 128-byte line, no registers): the
     // loads that follow turn by turn then wait for L2 only, which is what counts when few CTAs share the SM
     for (int p = 2; p < Rb; ++p) {
         const int t = wb + p * 256 + lane * 8;
-        if ((lane & 3) == 0 && t < n) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + t));
+        // a page of one head is a run of 4 << shift bytes: one request per 32 tokens, or per page if those are smaller
+        const int every = (kPaged && cp.shift < 5) ? (1 << (max(cp.shift, 3) - 3)) - 1 : 3;
+        if ((lane & every) == 0 && t < n && !(kPaged && cp.shift < 3)) asm volatile("prefetch.global.L2 [%0];" ::"l"(row_ptr(p) + t));
     }
+    if (kPaged) { r0 = row_ptr(2); r1 = row_ptr(3); }
     for (int i = tid; i < kBins * 32 / 4; i += kScanThreads)
         reinterpret_cast<uint4 *>(&c_hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < kBins + 3) s_hist[tid] = 0;
@@ -353,8 +374,14 @@ __global__ void __launch_bounds__(kScanThreads, 6) score_select_cluster_kernel(
         if (e_last >= 0 && e_last < 512 && e_last < 256 * Rb && ((e_last & 255) >> 3) == lane) {
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
-                patch_token(c[2 * j], wb + j * 256 + lane * 8, n - back, row);
-                patch_token(c[2 * j + 1], wb + j * 256 + lane * 8 + 4, n - back, row);
+                const int t = wb + j * 256 + lane * 8;
+                if (kPaged) {
+                    patch_token_paged(c[2 * j], t, n - back, cp, row, table_b);
+                    patch_token_paged(c[2 * j + 1], t + 4, n - back, cp, row, table_b);
+                } else {
+                    patch_token(c[2 * j], t, n - back, row);
+                    patch_token(c[2 * j + 1], t + 4, n - back, row);
+                }
             }
         }
     }
@@ -394,8 +421,9 @@ __global__ void __launch_bounds__(kScanThreads, 6) score_select_cluster_kernel(
     };
     for (int p0 = 0; p0 < Rb; p0 += 2) {   // CTA-uniform
         if (p0 > 0) {
-            load_row(p0, c[0], c[1], false);
-            load_row(p0 + 1, c[2], c[3], false);
+            load_row(p0, r0, c[0], c[1], false);
+            load_row(p0 + 1, r1, c[2], c[3], false);
+            if (kPaged) { r0 = row_ptr(p0 + 2); r1 = row_ptr(p0 + 3); }
         }
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -497,18 +525,18 @@ __global__ void __launch_bounds__(kScanThreads, 6) score_select_cluster_kernel(
     cluster_wait();
 }
 
-template <int G, int CS>
+template <int G, int CS, bool kPaged>
 static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint32_t *q_codes, const uint32_t *k_codes,
                                     long long kc_sb, long long kc_sh, const int32_t *seq_lens,
                                     const int32_t *k_per_seq, int k_uniform, int max_seq_len, int k_max, int32_t *idx,
                                     long long idx_sb, long long idx_sh, int32_t *count, int32_t *hist_out,
-                                    cudaStream_t st, Windows win) {
+                                    cudaStream_t st, Windows win, CodePages cp, int kv_shift) {
     static bool opted[64] = {};   // opt in to the padded shared-memory sizes once per device
     {
         int dev = 0;
         cudaGetDevice(&dev);
         if (dev >= 0 && dev < 64 && !opted[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(score_select_cluster_kernel<G, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+            cudaError_t e = cudaFuncSetAttribute(score_select_cluster_kernel<G, CS, kPaged>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
             if (e != cudaSuccess) return e;
             opted[dev] = true;
         }
@@ -526,7 +554,7 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
         const int n_ctas = CS * Hkv * B, n_sm = sm_count();
         const int cap = (n_ctas + n_sm - 1) / n_sm;   // CTAs per SM
         const bool slack = CS == 2 || 2 * (cap * n_sm - n_ctas) >= n_sm;
-        if (n_ctas > n_sm && cap < 6 && slack) {
+        if (n_ctas > n_sm && cap < (kPaged ? 5 : 6) && slack) {
             static size_t pad[64][6] = {};   // per device and cap: the least dynamic shared memory with which only `cap` CTAs fit
             int dev = 0;
             cudaGetDevice(&dev);
@@ -535,7 +563,7 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
                 size_t found = 0;
                 for (size_t kb = 8; kb <= 100 && !found; ++kb) {
                     int occ = 0;
-                    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, score_select_cluster_kernel<G, CS>, kScanThreads, kb * 1024) != cudaSuccess) break;
+                    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, score_select_cluster_kernel<G, CS, kPaged>, kScanThreads, kb * 1024) != cudaSuccess) break;
                     if (occ <= cap) found = kb * 1024;
                 }
                 pad[dev][cap] = found ? found : 1;
@@ -553,9 +581,9 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, score_select_cluster_kernel<G, CS>, q_codes, k_codes, kc_sb, kc_sh,
+    cudaError_t e = cudaLaunchKernelEx(&cfg, score_select_cluster_kernel<G, CS, kPaged>, q_codes, k_codes, kc_sb, kc_sh,
                                        seq_lens, max_seq_len, k_per_seq, k_uniform, k_max, Hq, Hkv, idx, idx_sb, idx_sh,
-                                       count, hist_out, win);
+                                       count, hist_out, win, cp, kv_shift);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
@@ -567,23 +595,25 @@ static cudaError_t launch_g(int B, int Hq, int Hkv, const uint32_t *q_codes, con
                             int k_uniform, int max_seq_len, int k_max, int32_t *idx, long long idx_sb,
                             long long idx_sh, int32_t *count, int32_t *hist_out, int32_t *ws_hist,
                             unsigned char *ws_scores, cudaStream_t st, Windows win, CodePages cp, int row_shift) {
-    if (max_seq_len <= kClusterMaxSeq && !cp.table && row_shift < 0) {
+    if (max_seq_len <= kClusterMaxSeq) {
         // Fused path: one cluster per unit.  Cluster size: the largest of 8, 4, 2 whose grid still fits
         // the GPU in one wave (about six 256-thread CTAs per SM), so that small batches get the most
         // parallelism per sequence and large batches the most work per cluster barrier; a lane then
         // holds R = ceil(n / (CS * 2048)) rows of 8 tokens (R <= 8).
-        const int units = B * Hkv, one_wave = 6 * sm_count();
+        const int units = B * Hkv, one_wave = (cp.table ? 5 : 6) * sm_count();
         int cs = 8;
         while (cs > 2 && units * cs > one_wave) cs >>= 1;
         while ((max_seq_len + cs * 2048 - 1) / (cs * 2048) > kClusterMaxRows) cs <<= 1;
         const int rows = max(1, (max_seq_len + cs * 2048 - 1) / (cs * 2048));
-#define HA_CL(CSZ)                                                                                                    \
-    return launch_cluster_t<G, CSZ>(rows, B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq, k_uniform, \
-                                    max_seq_len, k_max, idx, idx_sb, idx_sh, count, hist_out, st, win)
+        const int kv_shift = row_shift < 0 ? 0 : row_shift;
+#define HA_CL_ARGS rows, B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, idx, \
+                   idx_sb, idx_sh, count, hist_out, st, win, cp, kv_shift
+#define HA_CL(CSZ) return cp.table ? launch_cluster_t<G, CSZ, true>(HA_CL_ARGS) : launch_cluster_t<G, CSZ, false>(HA_CL_ARGS)
         if (cs == 8) HA_CL(8);
         if (cs == 4) HA_CL(4);
         HA_CL(2);
 #undef HA_CL
+#undef HA_CL_ARGS
     }
     const int chunk_tokens = chunk_tokens_for(B * Hkv, max_seq_len, sm_count());
     const int n_chunks = max(1, (max_seq_len + chunk_tokens - 1) / chunk_tokens);

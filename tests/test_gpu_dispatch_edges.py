@@ -8,7 +8,8 @@ import oracle
 from paper_2412_14468_b200 import binding as ha
 from paper_2412_14468_b200 import workloads as wl
 from tests._util import u16
-from tests.test_gpu_parity import _check_score_topk_wide, _wide_codes, _wide_mapping
+from tests.test_gpu_parity import _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
+    test_whole_step_with_keys_values_and_signatures_all_paged as _whole_paged_step
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -48,3 +49,36 @@ def test_score_topk_wide_at_row_and_cluster_edges(n_bits, lens):
     kc = _wide_codes(rng, len(lens) * Hkv * n_cap, W).reshape(len(lens), Hkv, n_cap, W)
     qc = _wide_codes(rng, len(lens) * Hkv * G, W).reshape(len(lens), Hkv * G, W)
     _check_score_topk_wide(n_bits, qc, kc, list(lens), [max(1, n // 5) for n in lens], Hkv * G, Hkv, 3, 5)
+
+
+@pytest.mark.parametrize("page_size", [2, 4, 8, 32])
+@pytest.mark.parametrize("lens", [(255, 256, 257), (2049, 16383, 16385), (131072, 131071), (131073,), tuple(range(1, 2200, 29))])
+def test_score_topk_paged_at_row_page_and_cluster_edges(page_size, lens):
+    """Pages below and above a lane's eight tokens; rows of 256 tokens, slices of 2048, the longest sequence of the cluster
+    kernel and the first beyond it, and a batch that takes smaller clusters."""
+    rng = np.random.default_rng(page_size + len(lens))
+    B, Hq, Hkv, G = len(lens), 8, 2, 4
+    n_cap, ks = max(lens), [max(1, n // 7) for n in lens]
+    n_sink, n_local = 2, 9
+    codes = rng.integers(0, 2**32, size=(B, Hkv, n_cap), dtype=np.uint64).astype(np.uint32)
+    qc = rng.integers(0, 2**32, size=(B, Hq), dtype=np.uint64).astype(np.uint32)
+    pool, table = _page_codes(codes, lens, page_size, rng)
+    k_max = max(ks) + n_sink + n_local
+    shape = ha.make_shape(B, Hq, Hkv, 1.0, n_sink=n_sink, n_local=n_local)
+    ws = ha.alloc_workspace(shape, n_cap, k_max)
+    idx = torch.full((B, Hkv, k_max), 5, dtype=torch.int32, device=DEV)
+    cnt = torch.full((B, Hkv), 5, dtype=torch.int32, device=DEV)
+    to = lambda a: torch.from_numpy(a.view(np.int32)).to(DEV)  # noqa: E731
+    ha.ha_score_topk_paged(shape, to(qc), to(pool), to(table), torch.tensor(lens, dtype=torch.int32, device=DEV),
+                           torch.tensor(ks, dtype=torch.int32, device=DEV), 0, n_cap, k_max, idx, cnt, ws)
+    got, n_got = idx.cpu().numpy(), cnt.cpu().numpy()
+    for b, n in enumerate(lens):
+        for g in range(Hkv):
+            ref = oracle.topk_windows(oracle.score(qc[b, g * G:(g + 1) * G], codes[b, g, :n]), ks[b], n_sink, n_local)
+            assert n_got[b, g] == len(ref) and np.array_equal(got[b, g, :len(ref)], ref) and (got[b, g, len(ref):] == -1).all()
+
+
+@pytest.mark.parametrize("page_size,B", [(4, 2), (16, 45), (2, 45)])
+def test_whole_paged_step_in_one_launch_and_in_three(page_size, B):
+    """Few units take the one-kernel step over the pools, 90 units ENCODE, SCORE + TOPK and GATHER-ATT one by one."""
+    _whole_paged_step(page_size, B)
