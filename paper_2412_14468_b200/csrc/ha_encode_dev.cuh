@@ -17,17 +17,30 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void *src, uint32_t
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
-// Bounded wait for phase 0 of an mbarrier.  Returns false if the copy has not completed after the
-// limit (never seen; the caller then fetches the data with ordinary loads instead).
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar) {
-    for (int it = 0; it < (1 << 20); ++it) {
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    return done != 0u;
+}
+// Bounded wait for one phase of an mbarrier; false if it has not completed after the limit (never seen).  test_wait first:
+// try_wait takes some 300 cycles even when the phase is complete (measured; test_wait 40), so it only parks a warp whose
+// barrier is far from ready.
+__device__ __forceinline__ bool mbar_wait_parity(uint32_t bar, uint32_t parity) {
+#pragma unroll 1
+    for (int it = 0; it < 32; ++it)
+        if (mbar_test(bar, parity)) return true;
+#pragma unroll 1
+    for (int it = 0; it < (1 << 18); ++it) {
         uint32_t done;
         asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                     : "=r"(done) : "r"(bar), "r"(0u) : "memory");
+                     : "=r"(done) : "r"(bar), "r"(parity) : "memory");
         if (done) return true;
     }
     return false;
 }
+// Phase 0: the arrival of a bulk copy.  A caller that gets false fetches the data with ordinary loads instead.
+__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar) { return mbar_wait_parity(bar, 0u); }
 
 // z[v] += sum_k hin[v][k] * w[k][o], ascending k, one fmaf per term; the VT chains are independent
 // (vector v starts at hin + v * vstride).
