@@ -238,6 +238,12 @@ int ha_gather_attn_per_head(const ha_shape *shape, const uint16_t *q, const ha_t
     if (shape->batch == 0) return HA_OK;
     int shift = 0;
     while ((shape->n_kv_heads << shift) < shape->n_q_heads) ++shift;
+    if (gather_cluster_eligible(shape->batch, shape->n_q_heads, shape->n_q_heads, k_max)) {
+        HA_CUDA(launch_gather_cluster(shape->batch, shape->n_q_heads, shape->n_q_heads, shape->sm_scale, q, view(K), view(V), seq_lens,
+                                      idx, idx_stride_b, idx_stride_h, count, k_max, out, lse, ws_ptr<uint32_t>(workspace, 0),
+                                      (cudaStream_t)stream, nullptr, 0, 0, shift));
+        return HA_OK;
+    }
     HA_CUDA(launch_attention(true, shape->batch, shape->n_q_heads, shape->n_q_heads, shape->sm_scale, q, view(K), view(V),
                              seq_lens, idx, idx_stride_b, idx_stride_h, count, k_max, out, lse,
                              ws_ptr<float>(workspace, L.off_part_ml), ws_ptr<float>(workspace, L.off_part_acc),
@@ -500,6 +506,12 @@ int ha_gather_attn_per_head_paged(const ha_shape *shape, const uint16_t *q, cons
     int kv_shift = 0, page_shift = 0;
     while ((shape->n_kv_heads << kv_shift) < shape->n_q_heads) ++kv_shift;
     while ((1 << page_shift) < page_size) ++page_shift;
+    if (gather_cluster_eligible(shape->batch, shape->n_q_heads, shape->n_q_heads, k_max)) {
+        HA_CUDA(launch_gather_cluster(shape->batch, shape->n_q_heads, shape->n_q_heads, shape->sm_scale, q, view(K_pool), view(V_pool),
+                                      seq_lens, idx, idx_stride_b, idx_stride_h, count, k_max, out, lse, ws_ptr<uint32_t>(workspace, 0),
+                                      (cudaStream_t)stream, block_table, bt_stride_b, page_shift, kv_shift));
+        return HA_OK;
+    }
     HA_CUDA(launch_attention(true, shape->batch, shape->n_q_heads, shape->n_q_heads, shape->sm_scale, q, view(K_pool), view(V_pool),
                              seq_lens, idx, idx_stride_b, idx_stride_h, count, k_max, out, lse,
                              ws_ptr<float>(workspace, L.off_part_ml), ws_ptr<float>(workspace, L.off_part_acc),

@@ -252,7 +252,7 @@ cudaError_t launch_gather_cluster(int B, int Hq, int Hkv, float sm_scale, const 
                                   const int32_t *seq_lens, const int32_t *idx, long long idx_sb, long long idx_sh,
                                   const int32_t *count, int k_max, uint16_t *out, float *lse, uint32_t *status,
                                   cudaStream_t st, const int32_t *block_table = nullptr, long long bt_sb = 0,
-                                  int page_shift = 0);
+                                  int page_shift = 0, int kv_shift = 0);   // kv_shift as in launch_attention
 
 // Signatures of 64 .. 512 bits through ENCODE and SCORE + TOPK (packed 64-bit words; strides in words).
 cudaError_t launch_encode_wide(const MapView &map, int n_bits, int heads_per_kv, TensorView x, int B, int H, int T,

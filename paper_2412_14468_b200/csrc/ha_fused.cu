@@ -58,7 +58,6 @@ struct FusedArgs {
     const uint16_t *q, *k_new;
     TensorView K, V;
     uint32_t *k_codes;
-    CodePages code_pages;    // table != NULL: k_codes is a paged pool
     long long kc_sb, kc_sh;
     const int32_t *seq_lens, *k_per_seq;
     int k_uniform, max_seq_len, k_max, Hq, Hkv;
@@ -80,6 +79,8 @@ struct FusedArgs {
     // crosses the bus once per CTA and never on the critical path of the attention phase.
     const uint16_t *v_new;
     uint32_t *status;   // stand-alone cluster gather: device status word (HA_DEV_BAD_INDEX)
+    CodePages code_pages;   // table != NULL: k_codes is a paged pool
+    int kv_shift;       // stand-alone cluster gather: unit head h reads K/V head h >> kv_shift (lists per query head)
 };
 
 __device__ __forceinline__ void st_dsmem_u32(uint32_t *local, uint32_t rank, uint32_t v) {
@@ -151,8 +152,9 @@ __device__ __forceinline__ void fused_attention(const FusedArgs &a, uint32_t ran
                                                 uint32_t (*s_mask)[kFusedMaxStages], bool &bad) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool paged = a.block_table != nullptr;   // rows are then addressed from the pool's base
-    const unsigned char *Kb = reinterpret_cast<const unsigned char *>(a.K.ptr + (paged ? 0LL : (long long)b * a.K.sb) + (long long)kvh * a.K.sh);
-    const unsigned char *Vb = reinterpret_cast<const unsigned char *>(a.V.ptr + (paged ? 0LL : (long long)b * a.V.sb) + (long long)kvh * a.V.sh);
+    const long long kv = kCheck ? (kvh >> a.kv_shift) : kvh;   // one list per query head: stand-alone calls only
+    const unsigned char *Kb = reinterpret_cast<const unsigned char *>(a.K.ptr + (paged ? 0LL : (long long)b * a.K.sb) + kv * a.K.sh);
+    const unsigned char *Vb = reinterpret_cast<const unsigned char *>(a.V.ptr + (paged ? 0LL : (long long)b * a.V.sb) + kv * a.V.sh);
     const int32_t *pages = paged ? a.block_table + (long long)b * a.bt_sb : nullptr;
     const long long k_row = a.K.sn * 2, v_row = a.V.sn * 2;
     unsigned char *my_ring = ring + warp * (S * kStageBytes);
@@ -711,8 +713,9 @@ static cudaError_t launch_gather_cluster_g(const FusedArgs &args, int B, cudaStr
 cudaError_t launch_gather_cluster(int B, int Hq, int Hkv, float sm_scale, const uint16_t *q, TensorView K, TensorView V,
                                   const int32_t *seq_lens, const int32_t *idx, long long idx_sb, long long idx_sh,
                                   const int32_t *count, int k_max, uint16_t *out, float *lse, uint32_t *status,
-                                  cudaStream_t st, const int32_t *block_table, long long bt_sb, int page_shift) {
+                                  cudaStream_t st, const int32_t *block_table, long long bt_sb, int page_shift, int kv_shift) {
     FusedArgs a{};
+    a.kv_shift = kv_shift;
     a.block_table = block_table; a.bt_sb = bt_sb; a.page_shift = page_shift;
     a.page_rows = (block_table && K.sn > 0) ? (int)(K.sb / K.sn) : 0;
     a.q = q; a.K = K; a.V = V; a.seq_lens = seq_lens; a.k_max = k_max; a.Hq = Hq; a.Hkv = Hkv;

@@ -93,13 +93,21 @@ __device__ __forceinline__ void sum_scores_of(const uint4 (&v)[LD], int base, in
     }
 }
 
-template <int LD, bool kEdge>
+// kEarly: before the programmatic-launch wait (through L1: the appended token is read again afterwards); later loads go past
+// L1, which may hold a line of such an early load.
+template <int LD, bool kEdge, bool kEarly>
 __device__ __forceinline__ void sum_load_tile(const uint32_t *row, int base, int lane, int hi, uint4 (&v)[LD]) {
 #pragma unroll
     for (int j = 0; j < LD; ++j) {
         const int t = base + j * 128 + 4 * lane;
-        if (kEdge) v[j] = (t < hi) ? load_codes4(row, t, hi) : make_uint4(0u, 0u, 0u, 0u);
-        else v[j] = __ldg(reinterpret_cast<const uint4 *>(row + t));
+        if (kEdge && t + 3 >= hi) {
+            v[j] = make_uint4(0u, 0u, 0u, 0u);
+            if (t + 0 < hi) v[j].x = __ldcg(row + t + 0);
+            if (t + 1 < hi) v[j].y = __ldcg(row + t + 1);
+            if (t + 2 < hi) v[j].z = __ldcg(row + t + 2);
+        } else {
+            v[j] = kEarly ? __ldg(reinterpret_cast<const uint4 *>(row + t)) : __ldcg(reinterpret_cast<const uint4 *>(row + t));
+        }
     }
 }
 
@@ -129,14 +137,6 @@ __global__ void __launch_bounds__(kSumThreads, LD <= 2 ? 5 : 3) score_sum_select
     const uint32_t *row = a.k_codes + (long long)b * a.kc_sb + (long long)(g >> a.row_shift) * a.kc_sh;
     int32_t *list = a.idx + (long long)b * a.idx_sb + (long long)g * a.idx_sh;
 
-    SumPlanes<G> pl;
-    {
-        uint32_t q[G];
-#pragma unroll
-        for (int j = 0; j < G; ++j) q[j] = __ldg(a.q_codes + (long long)b * a.Hq + (long long)g * G + j);
-        pl.build(q);
-    }
-
     // slice of this CTA: a multiple of four tokens, so that every 16-byte load stays inside it
     const int per = ((n + 3) / 4 + CS - 1) / CS * 4;
     const int lo = min(n, (int)rank * per), hi = min(n, lo + per);
@@ -145,18 +145,43 @@ __global__ void __launch_bounds__(kSumThreads, LD <= 2 ? 5 : 3) score_sum_select
     const int plain_end = min(wb.local_begin, hi);      // warp tiles inside [sink_end, plain_end) need no per-token checks
     auto is_edge = [&](int base) { return base < wb.sink_end || base + kWarpTokens > plain_end; };
 
+    // the first tile is requested before the launch wait; what a library kernel directly in front may still have been writing
+    // (slots n-1 and n-2) is read again after it
+    uint4 v[LD], nx[LD];
+    if (n_tiles > 0) {
+        const int base = lo + warp * kWarpTokens;
+        if (is_edge(base)) sum_load_tile<LD, true, true>(row, base, lane, hi, v);
+        else sum_load_tile<LD, false, true>(row, base, lane, hi, v);
+    }
     for (int i = tid; i < NB * 8; i += kSumThreads) reinterpret_cast<uint4 *>(&c_hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+    pdl_launch_dependents();
+    pdl_wait();
+    if (n_tiles > 0) {
+#pragma unroll
+        for (int j = 0; j < LD; ++j) {
+            const int t = lo + warp * kWarpTokens + j * 128 + 4 * lane;
+            if (t < hi) {
+                patch_token(v[j], t, n - 1, row);
+                patch_token(v[j], t, n - 2, row);
+            }
+        }
+    }
+    SumPlanes<G> pl;
+    {
+        uint32_t q[G];
+#pragma unroll
+        for (int j = 0; j < G; ++j) q[j] = __ldcg(a.q_codes + (long long)b * a.Hq + (long long)g * G + j);
+        pl.build(q);
+    }
     __syncthreads();
 
     // ---- pass 1: histogram of the slice
     int sc[4 * LD];
     {
-        uint4 v[LD], nx[LD];
         auto load = [&](int base, uint4 (&dst)[LD]) {
-            if (is_edge(base)) sum_load_tile<LD, true>(row, base, lane, hi, dst);
-            else sum_load_tile<LD, false>(row, base, lane, hi, dst);
+            if (is_edge(base)) sum_load_tile<LD, true, false>(row, base, lane, hi, dst);
+            else sum_load_tile<LD, false, false>(row, base, lane, hi, dst);
         };
-        if (n_tiles > 0) load(lo + warp * kWarpTokens, v);
         for (int it = 0; it < n_tiles; ++it) {
             const int base = lo + it * kTileTokens + warp * kWarpTokens;
             if (it + 1 < n_tiles) load(base + kTileTokens, nx);
@@ -265,9 +290,8 @@ __global__ void __launch_bounds__(kSumThreads, LD <= 2 ? 5 : 3) score_sum_select
             }
         } else {
             if (n_tiles != 1) {   // a slice of one tile still holds its scores in registers
-                uint4 v[LD];
-                if (edge) { sum_load_tile<LD, true>(row, base, lane, hi, v); sum_scores_of<G, LD, true>(v, base, lane, hi, wb, pl, sc); }
-                else { sum_load_tile<LD, false>(row, base, lane, hi, v); sum_scores_of<G, LD, false>(v, base, lane, hi, wb, pl, sc); }
+                if (edge) { sum_load_tile<LD, true, false>(row, base, lane, hi, v); sum_scores_of<G, LD, true>(v, base, lane, hi, wb, pl, sc); }
+                else { sum_load_tile<LD, false, false>(row, base, lane, hi, v); sum_scores_of<G, LD, false>(v, base, lane, hi, wb, pl, sc); }
             }
 #pragma unroll
             for (int i = 0; i < 4 * LD; ++i) {
@@ -382,13 +406,15 @@ static cudaError_t launch_sum_t(const SumArgs &a, int B, cudaStream_t st) {
     cfg.blockDim = dim3(kSumThreads);
     cfg.dynamicSmemBytes = kCacheBytes;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = CS;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     cudaError_t e = cudaLaunchKernelEx(&cfg, score_sum_select_kernel<G, CS, LD>, args);
     if (e != cudaSuccess) return e;
     count_launch();
