@@ -322,14 +322,14 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_kernel(const AttnArgs a)
             if (finalize) {
                 __threadfence();
                 // Merge of the parts: thread (dq, pg) owns dimensions 4dq..4dq+3 and the parts pg, pg+4, ...;
-                // a pass covers 16 (8 when G = 8) parts with every load issued before the first use (one L2 round trip),
+                // a pass covers 24 (12 when G = 8) parts with every load issued before the first use (one L2 round trip),
                 // then the four part groups are folded through shared memory.
                 const int dq = tid & 31, pg = tid >> 5;
                 float Mt[G], Lt[G];
                 float4 At[G];
 #pragma unroll
                 for (int j = 0; j < G; ++j) { Mt[j] = -CUDART_INF_F; Lt[j] = 0.0f; At[j] = make_float4(0.f, 0.f, 0.f, 0.f); }
-                constexpr int kEB = (G >= 8) ? 2 : 4;   // loads in flight per head and thread
+                constexpr int kEB = (G >= 8) ? 3 : 6;   // loads in flight per head and thread
                 for (int part0 = 0; part0 < n_parts; part0 += 4 * kEB) {
                     float4 av[G][kEB];
                     float mv[G][kEB], lv[G][kEB];
