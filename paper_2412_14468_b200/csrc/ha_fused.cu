@@ -100,15 +100,16 @@ __device__ __forceinline__ void st_dsmem_f32(float *local, uint32_t rank, float 
 // call; the barrier that publishes the input vectors also publishes them.  Signature v is written to
 // word v of `dst` in the shared memory of EVERY CTA of the cluster (lanes 0..CS-1 of the warp that holds it
 // store to CTAs 0..CS-1; the cluster barrier that follows makes the stores visible).
-template <int NV, int CS>
+// kRaw: thread o already holds component o of every vector in xr (fetched across the bus earlier).
+template <int NV, int CS, bool kRaw = false>
 __device__ __forceinline__ void fused_encode(const uint16_t *x0, long long x_stride, const uint16_t *sw1,
                                              const uint16_t *sw2, const uint16_t *sw3, float *actA, float *actB,
-                                             uint32_t *dst, float bias1, float bias2, float bias3) {
+                                             uint32_t *dst, float bias1, float bias2, float bias3, const uint16_t *xr = nullptr) {
     const int tid = threadIdx.x, o = tid & 127;
     const bool active = tid < 128;
     if (active) {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) actA[v * kD + o] = bf16_bits_to_float(__ldg(x0 + (long long)v * x_stride + o));
+        for (int v = 0; v < NV; ++v) actA[v * kD + o] = bf16_bits_to_float(kRaw ? xr[v] : __ldg(x0 + (long long)v * x_stride + o));
     }
     __syncthreads();
     float z[NV];
@@ -348,6 +349,28 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
             if (p < Lb && base < n) c[p] = codes_paged ? load_codes4_paged(a.code_pages, row, code_table, base, n) : load_codes4(row, base, n);
         }
     };
+    // Host-buffer step: everything that crosses the bus is requested first (a round trip of about 2 us), under the fetch and the
+    // transposition of the weights.  The stream is idle between such steps (each call waits for its result), so the launch wait
+    // in front of the requests costs nothing.
+    uint4 q_stage = make_uint4(0u, 0u, 0u, 0u);
+    uint2 kv_row = make_uint2(0u, 0u);
+    uint16_t x_raw[kQPer] = {};
+    if (kHost) {
+        pdl_wait();
+        if (tid < kD) {
+            if ((int)rank < kQCtas) {
+#pragma unroll
+                for (int v = 0; v < kQPer; ++v) x_raw[v] = __ldg(a.q + (head0 + kQPer * (int)rank + v) * kD + tid);
+            } else if ((int)rank == kQCtas && has_new_key) {
+                x_raw[0] = __ldg(a.k_new + ((long long)b * Hkv + kvh) * kD + tid);
+            }
+        }
+        // the unit's G query vectors (16 bytes per thread), parked in shared memory once the encoders are done with it
+        if (tid < G * 16) q_stage = __ldg(reinterpret_cast<const uint4 *>(a.q + head0 * kD) + tid);
+        // the appended rows: 32 threads x 8 bytes for K, 32 for V (contiguous cache only)
+        if ((int)rank == kQCtas && has_new_key && a.v_new && tid < 64)
+            kv_row = __ldg(reinterpret_cast<const uint2 *>(((tid < 32) ? a.k_new : a.v_new) + ((long long)b * Hkv + kvh) * kD) + (tid & 31));
+    }
     if (kPreload) load_signatures();
     // ENCODE roles: CTA r < kQCtas encodes kQPer query vectors (one per CTA while the cluster has room),
     // CTA kQCtas encodes the appended key; the other CTAs only scan
@@ -380,32 +403,25 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     }
     for (int i = tid; i < kBins * 32 / 4; i += kFusedThreads)
         reinterpret_cast<uint4 *>(&c_hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
-    pdl_wait();                  // q, k_new and everything older in the stream is final from here on
+    if (!kHost) pdl_wait();      // q, k_new and everything older in the stream is final from here on
     pdl_launch_dependents();
     cluster_wait();              // #0: all CTAs of the cluster are running (their shared memory may be written)
-    uint4 q_stage = make_uint4(0u, 0u, 0u, 0u);
     if (kHost) {
-        // the unit's G query vectors (16 bytes per thread) start their way across the bus now and are parked in
-        // shared memory once the encoders are done with it
-        if (tid < G * 16) q_stage = __ldg(reinterpret_cast<const uint4 *>(a.q + head0 * kD) + tid);
-        if (enc_k && a.v_new && tid < 64) {   // the appended rows: 32 threads x 8 bytes for K, 32 for V (contiguous cache only)
-            const int t = tid & 31;
-            const long long src = ((long long)b * Hkv + kvh) * kD;
+        if (enc_k && a.v_new && tid < 64) {
             const TensorView &X = (tid < 32) ? a.K : a.V;
-            const uint2 v = __ldg(reinterpret_cast<const uint2 *>(((tid < 32) ? a.k_new : a.v_new) + src) + t);
             // slot seq_len - 1 as the stand-alone append kernel takes it (n is the length clamped to max_seq_len)
             uint16_t *dst = const_cast<uint16_t *>(X.ptr) + (long long)b * X.sb + (long long)kvh * X.sh + (long long)(a.seq_lens[b] - 1) * X.sn;
-            reinterpret_cast<uint2 *>(dst)[t] = v;
+            reinterpret_cast<uint2 *>(dst)[tid & 31] = kv_row;
         }
     }
 
     // ---------------- P1: ENCODE in the first kQCtas CTAs (queries) and the next one (appended key)
     if (enc_q) {
-        fused_encode<kQPer, CS>(a.q + (head0 + kQPer * (int)rank) * kD, kD, sw1, sw2, sw3, actA, actB,
-                            s_codes + kQPer * (int)rank, bias1, bias2, bias3);
+        fused_encode<kQPer, CS, kHost>(a.q + (head0 + kQPer * (int)rank) * kD, kD, sw1, sw2, sw3, actA, actB,
+                                       s_codes + kQPer * (int)rank, bias1, bias2, bias3, x_raw);
     } else if (enc_k) {
-        fused_encode<1, CS>(a.k_new + ((long long)b * Hkv + kvh) * kD, kD, sw1, sw2, sw3, actA, actB, s_codes + G, bias1,
-                        bias2, bias3);
+        fused_encode<1, CS, kHost>(a.k_new + ((long long)b * Hkv + kvh) * kD, kD, sw1, sw2, sw3, actA, actB, s_codes + G, bias1,
+                                   bias2, bias3, x_raw);
     }
     cluster_sync_all();   // #1: every CTA holds all signatures (and its counters are zeroed)
     // the signatures also go to global memory (outputs of the step; nobody in this kernel reads them there):
