@@ -23,6 +23,15 @@ constexpr int kScanThreads = 256;
 constexpr int kPassTokens = kScanThreads * 16;   // four uint4 per thread
 constexpr int kClusterMaxSeq = 8 * 8 * 2048;     // longest sequence the cluster kernel takes (8 CTAs x 8 rows x 2048 tokens)
 
+// Clusters of 8 CTAs of 512 threads (two per SM, 36 clusters resident at once) instead of 256: with 24 to 36 units the hardware
+// stacks the small CTAs on half of the SMs.  Whole steps, groups of 4, us: 32 units of 70000 tokens 32.8 against 34.2, of 130000
+// 40.9 / 45.1, of 200000 53.2 / 56.5 (there against the two kernels); 24 units of 250000 50.6 / 53.1, but of 50000 22.4 / 22.1;
+// 16 units of 70000 25.3 / 24.5.  (Clusters of 16 of them for one sequence of 150000 or 250000 tokens win 5 us in back-to-back
+// calls and lose 1.2 us in a step, where the kernel in front holds their SMs.)
+inline bool large_clusters(long long units, int max_seq_len) {
+    return units >= 24 && units <= 36 && max_seq_len > 65536 && max_seq_len <= 8 * 8 * 4096;
+}
+
 // ------------------------------------------------------------------ long-sequence path (two kernels)
 
 // Kernel 1: one chunk per CTA.  Streams the chunk's signatures (four uint4 per thread in flight, the
@@ -295,18 +304,20 @@ constexpr int kClusterMaxRows = 8;   // rows of 8 tokens per lane: a lane's flag
 // kPaged: the signatures lie in a pool behind a block table.  Pages of 8 tokens or more hold a lane's 8 tokens in one piece, so
 // a row costs one table entry per lane (neighbouring lanes share it) and the same two 16-byte loads.  The table entries of the
 // next two rows are fetched while the current ones are scored; five CTAs per SM instead of six pay for the registers.
-template <int G, int CS, bool kPaged>
-__global__ void __launch_bounds__(kScanThreads, kPaged ? 5 : 6) score_select_cluster_kernel(
+// kThreads: 256, or 512 (large_clusters).
+template <int G, int CS, bool kPaged, int kThreads>
+__global__ void __launch_bounds__(kThreads, kThreads > 256 ? 2 : kPaged ? 5 : 6) score_select_cluster_kernel(
     const uint32_t *__restrict__ q_codes, const uint32_t *__restrict__ k_codes, long long kc_sb, long long kc_sh,
     const int32_t *__restrict__ seq_lens, int max_seq_len, const int32_t *__restrict__ k_per_seq, int k_uniform,
     int k_max, int Hq, int Hkv, int32_t *__restrict__ idx, long long idx_sb, long long idx_sh,
     int32_t *__restrict__ count, int32_t *__restrict__ hist_out, Windows win, const CodePages cp, int kv_shift) {
+    constexpr int kSlice = kThreads * 8;                       // tokens of one row of a CTA: eight per lane
     extern __shared__ __align__(16) unsigned char s_sc[];      // score + 1 of this CTA's tokens (0 = no token)
     __shared__ __align__(16) uint32_t c_hist[kBins][32];       // counters [level][lane]
     __shared__ int s_hist[kBins + 3];          // this CTA's histogram, read by the whole cluster
     __shared__ int s_tot[kBins], s_bef[kBins];
     __shared__ int sh_T, sh_r, sh_gt_before, sh_eq_before;
-    __shared__ int s_wcnt[kScanThreads / 32];
+    __shared__ int s_wcnt[kThreads / 32];
     const uint32_t rank = cluster_rank();
     const int g = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -321,11 +332,11 @@ __global__ void __launch_bounds__(kScanThreads, kPaged ? 5 : 6) score_select_clu
     const uint32_t *row = kPaged ? k_codes + (long long)kvh * cp.head_stride : k_codes + (long long)b * kc_sb + (long long)kvh * kc_sh;
     const int32_t *table_b = kPaged ? cp.table + (long long)b * cp.bt_sb : nullptr;
     // The sequence's own length is divided over the CS CTAs (ragged batches stay balanced): Rb rows per
-    // lane, a warp owns the 256*Rb tokens from wb on, a CTA 2048*Rb; row p of a lane is
+    // lane, a warp owns the 256*Rb tokens from wb on, a CTA kSlice*Rb; row p of a lane is
     // wb + 256 p + 8 lane .. + 7.
-    const int Rb = (n + CS * 2048 - 1) / (CS * 2048);
+    const int Rb = (n + CS * kSlice - 1) / (CS * kSlice);
     const int wl = warp * 256 * Rb;                    // the warp's first token inside the CTA's slice
-    const int wb = (int)rank * 2048 * Rb + wl;
+    const int wb = (int)rank * kSlice * Rb + wl;
 
     // paged: the pool words from which the lane's 8 tokens of row p are addressed by token number (pages of >= 8 tokens)
     auto row_ptr = [&](int p) -> const uint32_t * {
@@ -361,7 +372,7 @@ __global__ void __launch_bounds__(kScanThreads, kPaged ? 5 : 6) score_select_clu
         if ((lane & every) == 0 && t < n && !(kPaged && cp.shift < 3)) asm volatile("prefetch.global.L2 [%0];" ::"l"(row_ptr(p) + t));
     }
     if (kPaged) { r0 = row_ptr(2); r1 = row_ptr(3); }
-    for (int i = tid; i < kBins * 32 / 4; i += kScanThreads)
+    for (int i = tid; i < kBins * 32 / 4; i += kThreads)
         reinterpret_cast<uint4 *>(&c_hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < kBins + 3) s_hist[tid] = 0;
     pdl_launch_dependents();
@@ -439,7 +450,7 @@ __global__ void __launch_bounds__(kScanThreads, kPaged ? 5 : 6) score_select_clu
     }
     __syncthreads();
     // fold the counters: eight threads per level, four counters each
-    for (int i = tid; i < kBins * 8; i += kScanThreads) {
+    for (int i = tid; i < kBins * 8; i += kThreads) {
         const uint4 v = reinterpret_cast<const uint4 *>(&c_hist[i >> 3][0])[i & 7];
         const uint32_t ssum = (v.x + v.y) + (v.z + v.w);
         if (ssum) atomicAdd(&s_hist[i >> 3], (int)ssum);
@@ -477,7 +488,7 @@ __global__ void __launch_bounds__(kScanThreads, kPaged ? 5 : 6) score_select_clu
     int32_t *out = idx + (long long)b * idx_sb + (long long)g * idx_sh;
     if (rank == 0) {
         if (tid == 0) count[b * Hkv + g] = keep;
-        for (int i = keep + tid; i < k_max; i += kScanThreads) out[i] = -1;
+        for (int i = keep + tid; i < k_max; i += kThreads) out[i] = -1;
     }
     if (keep == 0) { cluster_wait(); return; }
 
@@ -509,23 +520,23 @@ __global__ void __launch_bounds__(kScanThreads, kPaged ? 5 : 6) score_select_clu
     if (lane == 31) s_wcnt[warp] = winc;
     __syncthreads();
     // tokens before this warp's range with S > T (always-kept tokens count as such) / S == T
-    int run_gt = sh_gt_before + forced_before(wbd, min((int)rank * 2048 * Rb, n)), run_eq = sh_eq_before;
+    int run_gt = sh_gt_before + forced_before(wbd, min((int)rank * kSlice * Rb, n)), run_eq = sh_eq_before;
 #pragma unroll
-    for (int w = 0; w < kScanThreads / 32; ++w) {
+    for (int w = 0; w < kThreads / 32; ++w) {
         if (w < warp) { run_gt += s_wcnt[w] & 0xffff; run_eq += (int)((unsigned)s_wcnt[w] >> 16); }
     }
     if (tot_packed != 0) {
         const int excl = winc - tot_packed;
         int g_run = run_gt + (excl & 0xffff);
         int q_run = run_eq + (int)((unsigned)excl >> 16);
-        const int first = (int)rank * 2048 * Rb + first_l;
+        const int first = (int)rank * kSlice * Rb + first_l;
         write_selected32(out, first, gt_lo, eq_lo, g_run, q_run, r);
         write_selected32(out, first + 32, gt_hi, eq_hi, g_run, q_run, r);
     }
     cluster_wait();
 }
 
-template <int G, int CS, bool kPaged>
+template <int G, int CS, bool kPaged, int kThreads = kScanThreads>
 static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint32_t *q_codes, const uint32_t *k_codes,
                                     long long kc_sb, long long kc_sh, const int32_t *seq_lens,
                                     const int32_t *k_per_seq, int k_uniform, int max_seq_len, int k_max, int32_t *idx,
@@ -536,15 +547,15 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
         int dev = 0;
         cudaGetDevice(&dev);
         if (dev >= 0 && dev < 64 && !opted[dev]) {
-            cudaError_t e = cudaFuncSetAttribute(score_select_cluster_kernel<G, CS, kPaged>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+            cudaError_t e = cudaFuncSetAttribute(score_select_cluster_kernel<G, CS, kPaged, kThreads>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
             if (e != cudaSuccess) return e;
             opted[dev] = true;
         }
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CS, Hkv, B);
-    cfg.blockDim = dim3(kScanThreads);
-    cfg.dynamicSmemBytes = (size_t)rows * 2048;   // one score byte per token of the CTA's slice (<= 16 KB)
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = (size_t)rows * kThreads * 8;   // one score byte per token of the CTA's slice (<= 16 KB, 32 KB with 512 threads)
     {
         // Launched behind another kernel, the CTAs land wherever room appears first, and an SM that takes six of them
         // while others hold two sets the kernel's time (the population-count unit is shared by the CTAs of an SM).
@@ -554,7 +565,7 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
         const int n_ctas = CS * Hkv * B, n_sm = sm_count();
         const int cap = (n_ctas + n_sm - 1) / n_sm;   // CTAs per SM
         const bool slack = CS == 2 || 2 * (cap * n_sm - n_ctas) >= n_sm;
-        if (n_ctas > n_sm && cap < (kPaged ? 5 : 6) && slack) {
+        if (kThreads == kScanThreads && n_ctas > n_sm && cap < (kPaged ? 5 : 6) && slack) {
             static size_t pad[64][6] = {};   // per device and cap: the least dynamic shared memory with which only `cap` CTAs fit
             int dev = 0;
             cudaGetDevice(&dev);
@@ -563,7 +574,7 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
                 size_t found = 0;
                 for (size_t kb = 8; kb <= 100 && !found; ++kb) {
                     int occ = 0;
-                    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, score_select_cluster_kernel<G, CS, kPaged>, kScanThreads, kb * 1024) != cudaSuccess) break;
+                    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, score_select_cluster_kernel<G, CS, kPaged, kThreads>, kThreads, kb * 1024) != cudaSuccess) break;
                     if (occ <= cap) found = kb * 1024;
                 }
                 pad[dev][cap] = found ? found : 1;
@@ -581,7 +592,7 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, score_select_cluster_kernel<G, CS, kPaged>, q_codes, k_codes, kc_sb, kc_sh,
+    cudaError_t e = cudaLaunchKernelEx(&cfg, score_select_cluster_kernel<G, CS, kPaged, kThreads>, q_codes, k_codes, kc_sb, kc_sh,
                                        seq_lens, max_seq_len, k_per_seq, k_uniform, k_max, Hq, Hkv, idx, idx_sb, idx_sh,
                                        count, hist_out, win, cp, kv_shift);
     if (e != cudaSuccess) return e;
@@ -595,6 +606,14 @@ static cudaError_t launch_g(int B, int Hq, int Hkv, const uint32_t *q_codes, con
                             int k_uniform, int max_seq_len, int k_max, int32_t *idx, long long idx_sb,
                             long long idx_sh, int32_t *count, int32_t *hist_out, int32_t *ws_hist,
                             unsigned char *ws_scores, cudaStream_t st, Windows win, CodePages cp, int row_shift) {
+    if (large_clusters((long long)B * Hkv, max_seq_len)) {
+        const int rows = (max_seq_len + 8 * 4096 - 1) / (8 * 4096), kv_shift = row_shift < 0 ? 0 : row_shift;
+#define HA_LARGE(PAGED) launch_cluster_t<G, 8, PAGED, 512>(rows, B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq,   \
+                                                           k_uniform, max_seq_len, k_max, idx, idx_sb, idx_sh, count, hist_out, st, \
+                                                           win, cp, kv_shift)
+        return cp.table ? HA_LARGE(true) : HA_LARGE(false);
+#undef HA_LARGE
+    }
     if (max_seq_len <= kClusterMaxSeq) {
         // Fused path: one cluster per unit.  Cluster size: the largest of 8, 4, 2 whose grid still fits
         // the GPU in one wave (about six 256-thread CTAs per SM), so that small batches get the most

@@ -82,3 +82,37 @@ def test_score_topk_paged_at_row_page_and_cluster_edges(page_size, lens):
 def test_whole_paged_step_in_one_launch_and_in_three(page_size, B):
     """Few units take the one-kernel step over the pools, 90 units ENCODE, SCORE + TOPK and GATHER-ATT one by one."""
     _whole_paged_step(page_size, B)
+
+
+@pytest.mark.parametrize("G", [1, 8])
+@pytest.mark.parametrize("lens", [(65537,) + (4095, 4096, 4097) + (0, 1) * 4, (262144,) + (70001,) * 11, (262145,) + (33000,) * 11,
+                                  (131072,) * 3 + tuple(range(60000, 60015))])
+@pytest.mark.parametrize("page_size", [0, 16])
+def test_score_topk_on_clusters_of_large_ctas(G, lens, page_size):
+    """24 to 36 units with sequences of 65537 to 262144 tokens: slices of 4096 tokens, one row and eight, sequences shorter than
+    a slice beside long ones, and the first length beyond the range."""
+    rng = np.random.default_rng(G + len(lens))
+    B, Hkv = len(lens), 2
+    Hq, n_cap, ks = Hkv * G, max(lens) // 64 * 64 + 64, [max(1, n // 9) for n in lens]
+    n_sink, n_local = 130, 7
+    k_max = max(ks) + n_sink + n_local
+    codes = rng.integers(0, 2**32, size=(B, Hkv, n_cap), dtype=np.uint64).astype(np.uint32)
+    codes[0, 0, :200] = codes[0, 0, 5]                              # ties decided by token index
+    qc = rng.integers(0, 2**32, size=(B, Hq), dtype=np.uint64).astype(np.uint32)
+    shape = ha.make_shape(B, Hq, Hkv, 1.0, n_sink=n_sink, n_local=n_local)
+    ws = ha.alloc_workspace(shape, n_cap, k_max)
+    idx = torch.full((B, Hkv, k_max), 5, dtype=torch.int32, device=DEV)
+    cnt = torch.full((B, Hkv), 5, dtype=torch.int32, device=DEV)
+    to = lambda a: torch.from_numpy(a.view(np.int32)).to(DEV)  # noqa: E731
+    lt, kt = torch.tensor(lens, dtype=torch.int32, device=DEV), torch.tensor(ks, dtype=torch.int32, device=DEV)
+    if page_size:
+        pool, table = _page_codes(codes, lens, page_size, rng)
+        ha.ha_score_topk_paged(shape, to(qc), to(pool), to(table), lt, kt, 0, max(lens), k_max, idx, cnt, ws)
+    else:
+        ha.ha_score_topk(shape, to(qc), to(codes), lt, kt, 0, max(lens), k_max, idx, cnt, ws)
+    got, n_got = idx.cpu().numpy(), cnt.cpu().numpy()
+    for b, n in enumerate(lens):
+        for g in range(Hkv):
+            s = oracle.score(qc[b, g * G:(g + 1) * G], codes[b, g, :n]) if n else np.zeros(0, np.int32)
+            ref = oracle.topk_windows(s, ks[b], n_sink, n_local)
+            assert n_got[b, g] == len(ref) and np.array_equal(got[b, g, :len(ref)], ref) and (got[b, g, len(ref):] == -1).all()
