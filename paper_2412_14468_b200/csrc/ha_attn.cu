@@ -24,9 +24,11 @@ namespace ha {
 
 constexpr int kAttnWarps = 4;
 constexpr int kAttnThreads = kAttnWarps * 32;
-constexpr int kStages = 3;                    // blocks of rows in flight per warp (ring in shared memory)
-constexpr int kWarpRingBytes = kStages * kStageBytes;
-constexpr int kAttnSmemBytes = kAttnWarps * kWarpRingBytes;
+// Blocks of rows per warp (ring in shared memory), kStages below: 3, or 2 for lists of up to 2048 entries.  Two stages ask less
+// of HBM at once and reach the same rate: 24 ragged lists of up to 2048 entries over pages 59.9 against 61.5 us per step, 64
+// lists of 1024 92.1 / 92.7; longer ragged lists keep the third (32 lists of up to 4096: 114.6 / 116 - 117).
+constexpr int kShortList = 2048;
+__host__ __device__ constexpr int attn_smem_bytes(int stages) { return kAttnWarps * stages * kStageBytes; }
 
 struct AttnArgs {
     const uint16_t *q;
@@ -51,8 +53,9 @@ struct AttnArgs {
     float *lse;
 };
 
-template <int G, bool kGather>
+template <int G, bool kGather, int kStages>
 __global__ void __launch_bounds__(kAttnThreads, 2) attn_kernel(const AttnArgs a) {
+    constexpr int kWarpRingBytes = kStages * kStageBytes, kAttnSmemBytes = attn_smem_bytes(kStages);
     extern __shared__ __align__(128) unsigned char ring[];   // kAttnWarps private rings, then the block prefix
     __shared__ float s_m[kAttnWarps][8], s_l[kAttnWarps][8];
     __shared__ uint32_t s_mask[kAttnWarps][kStages];
@@ -414,18 +417,18 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_kernel(const AttnArgs a)
     if (bad) atomicOr(a.status, HA_DEV_BAD_INDEX);
 }
 
-template <int G, bool kGather>
+template <int G, bool kGather, int kStages>
 static cudaError_t launch_attn_t(const AttnArgs &args, int grid, size_t smem, cudaStream_t st) {
     static bool done[64] = {};   // opt in to the ring's shared memory once per device
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(attn_kernel<G, kGather>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kAttnSmemBytes + (kMaxBalancedUnits + 1) * 4);
+        cudaError_t e = cudaFuncSetAttribute(attn_kernel<G, kGather, kStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             attn_smem_bytes(kStages) + (kMaxBalancedUnits + 1) * 4);
         if (e != cudaSuccess) return e;
         done[dev] = true;
     }
-    cudaError_t e = launch_pdl(attn_kernel<G, kGather>, dim3(grid), dim3(kAttnThreads), smem, st, args);
+    cudaError_t e = launch_pdl(attn_kernel<G, kGather, kStages>, dim3(grid), dim3(kAttnThreads), smem, st, args);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
@@ -437,7 +440,8 @@ static cudaError_t launch_attn_g(bool gather, const AttnArgs &args_in, cudaStrea
     const long long blocks_per_unit = (args.max_items + kBlockTokens - 1) / kBlockTokens;
     const long long t_max = blocks_per_unit * args.n_units;
     int grid;
-    size_t smem = kAttnSmemBytes;
+    const bool two_stages = gather && args.max_items <= kShortList;
+    size_t smem = attn_smem_bytes(two_stages ? 2 : 3);
     if (args.n_units <= kMaxBalancedUnits) {
         args.balanced = 1;
         long long want = (t_max + kAttnWarps - 1) / kAttnWarps;   // at least one block per warp
@@ -459,7 +463,8 @@ static cudaError_t launch_attn_g(bool gather, const AttnArgs &args_in, cudaStrea
         args.balanced = 0;
         grid = args.n_units;
     }
-    return gather ? launch_attn_t<G, true>(args, grid, smem, st) : launch_attn_t<G, false>(args, grid, smem, st);
+    if (two_stages) return launch_attn_t<G, true, 2>(args, grid, smem, st);
+    return gather ? launch_attn_t<G, true, 3>(args, grid, smem, st) : launch_attn_t<G, false, 3>(args, grid, smem, st);
 }
 
 cudaError_t launch_attention(bool gather, int B, int Hq, int Hkv, float sm_scale, const uint16_t *q,
