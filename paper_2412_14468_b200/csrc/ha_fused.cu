@@ -31,7 +31,10 @@ namespace ha {
 constexpr int kFusedMaxCS = 8;                               // CTAs per cluster (template parameter CS: 8 or 4; 2 is supported, unused)
 constexpr int kFusedWarps = 8;
 constexpr int kFusedThreads = kFusedWarps * 32;
-constexpr int kFusedMaxSeq = 32768;                          // 32 uint4 of signatures per thread position, shared by the cluster
+// Longest sequence, a template argument because a thread holds its share of the signatures in registers: 32768 in general;
+// 65536 (one-stage variant) and 131072 (two-stage variant) with clusters of 8, for the few units of one or two long sequences.
+constexpr int kFusedMaxSeq = 32768, kFusedMidSeq = 65536, kFusedLongSeq = 131072;
+constexpr int kFusedLongMaxK = 5120;                         // longest index list of the 131072-token variant
 constexpr int kFusedMaxStages = 2;                           // row blocks in flight per warp (template parameter S)
 constexpr int kFusedWeightBytes = (kD * kHid + kHid * kHid + kHid * kBits) * 2;
 constexpr int kFusedOneStageMaxK = 2048;                     // one-stage variant: longest index list
@@ -286,12 +289,12 @@ __device__ __forceinline__ void fused_attention(const FusedArgs &a, uint32_t ran
 // v_new in mapped host memory; the signatures in pages.
 constexpr int kModeDevice = 0, kModeHost = 1, kModePagedCodes = 2;
 
-template <int G, int S, int CS, int kMode>
+template <int G, int S, int CS, int kMode, int kMaxSeq>
 __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kernel(const FusedArgs a) {
     constexpr bool kHost = kMode == kModeHost, codes_paged = kMode == kModePagedCodes;
     constexpr int kFusedUnionBytes = fused_union_bytes(S);
     constexpr int kFusedActBytes = fused_act_bytes(G, CS);
-    constexpr int kL = kFusedMaxSeq / (CS * 4096) * 4;   // uint4 of signatures per thread: 4, 8 or 16
+    constexpr int kL = kMaxSeq / (CS * 4096) * 4;        // uint4 of signatures per thread: 4, 8 or 16
     constexpr int kFlagWords = (kL + 7) / 8;             // 32 tokens' flags per word
     constexpr int kQPer = fused_q_per_cta(G, CS);
     constexpr int kQCtas = G / kQPer;
@@ -765,14 +768,14 @@ static void fused_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2]
 
 // Opt in to the shared-memory carve-out (once per device) and return how many clusters of this variant the
 // device holds at once (0 on error).
-template <int G, int S, int CS, int kMode = kModeDevice>
+template <int G, int S, int CS, int kMode = kModeDevice, int kMaxSeq = kFusedMaxSeq>
 static int fused_prepare() {
     static int clusters[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
     if (!clusters[dev]) {
-        if (cudaFuncSetAttribute(fused_step_kernel<G, S, CS, kMode>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(fused_step_kernel<G, S, CS, kMode, kMaxSeq>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  fused_smem_bytes(G, S, CS)) != cudaSuccess)
             return 0;
         cudaLaunchConfig_t cfg;
@@ -780,26 +783,26 @@ static int fused_prepare() {
         fused_config<G, S, CS>(cfg, attr, 1, 64, nullptr);
         cfg.numAttrs = 1;   // the cluster shape is all the occupancy query looks at
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, fused_step_kernel<G, S, CS, kMode>, &cfg) != cudaSuccess || n <= 0) return 0;
+        if (cudaOccupancyMaxActiveClusters(&n, fused_step_kernel<G, S, CS, kMode, kMaxSeq>, &cfg) != cudaSuccess || n <= 0) return 0;
         clusters[dev] = n;
     }
     return clusters[dev];
 }
 
-template <int G, int S, int CS, int kMode = kModeDevice>
+template <int G, int S, int CS, int kMode = kModeDevice, int kMaxSeq = kFusedMaxSeq>
 static cudaError_t launch_fused_gsc(const FusedArgs &args, int B, cudaStream_t st) {
-    if (fused_prepare<G, S, CS, kMode>() <= 0) return cudaErrorInvalidConfiguration;
+    if (fused_prepare<G, S, CS, kMode, kMaxSeq>() <= 0) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     fused_config<G, S, CS>(cfg, attr, args.Hkv, B, st);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, fused_step_kernel<G, S, CS, kMode>, args);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fused_step_kernel<G, S, CS, kMode, kMaxSeq>, args);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
 }
 
 // Variant for a step of `units` (sequence, KV head) pairs with index lists of up to k_max entries: the number
-// of row stages per warp in *stages, the cluster size as the result, 0 if the step does not fit (a
+// of row stages per warp, the cluster size and the longest sequence; none if the step does not fit (a
 // cluster that had to wait for another one to finish would double the latency).
 //  * lists of up to 1024 entries (one block per warp with clusters of 8): the one-stage kernel, two CTAs per
 //    SM, with the larger cluster, 8 or 4 CTAs per unit, of which `units` are resident at once;
@@ -808,66 +811,68 @@ static cudaError_t launch_fused_gsc(const FusedArgs &args, int B, cudaStream_t s
 //    take their blocks one after the other).
 // Clusters of 2 work as well (the kernel is written for them) but lose to the three-kernel path at the batch
 // sizes they would serve (45.7 against 41.3 us at 128 units), so they are not offered.
+//  * sequences of more than 32768 tokens: clusters of 8, one-stage up to 65536 tokens and 2048 entries, else two-stage up to
+//    131072 tokens and kFusedLongMaxK entries, while `units` clusters are resident (33 and 15).  Against three launches, groups
+//    of 4, 8 units a sequence, lists of n / 32, us: one sequence of 65536 14.1 / 20.1, of 131072 21.9 / 26.5; four of 65536
+//    22.3 / 31.2.  With lists of n / 8 eight CTAs of two stages fetch too slowly: 60000 28.6 / 26.6, 100000 36.8 / 34.5.
+struct FusedVariant {
+    int cs, stages, max_seq;   // cs = 0: the step does not fit
+};
 template <int G>
-static int fused_variant(long long units, int k_max, int *stages) {
-    const bool one_block_per_warp = k_max <= kFusedMaxCS * kFusedWarps * kBlockTokens;
-    if (!one_block_per_warp && units <= fused_prepare<G, 2, 8>()) {
-        *stages = 2;
-        return 8;
+static FusedVariant fused_variant(long long units, int max_seq_len, int k_max) {
+    if (max_seq_len > kFusedMaxSeq) {
+        if (max_seq_len <= kFusedMidSeq && k_max <= kFusedOneStageMaxK && units <= fused_prepare<G, 1, 8, kModeDevice, kFusedMidSeq>())
+            return {8, 1, kFusedMidSeq};
+        if (max_seq_len <= kFusedLongSeq && k_max <= kFusedLongMaxK && units <= fused_prepare<G, 2, 8, kModeDevice, kFusedLongSeq>()) return {8, 2, kFusedLongSeq};
+        return {0, 0, 0};
     }
-    *stages = 1;
-    if (k_max > kFusedOneStageMaxK) return 0;
-    if (units <= fused_prepare<G, 1, 8>()) return 8;
-    if (units <= fused_prepare<G, 1, 4>()) return 4;
-    return 0;
+    const bool one_block_per_warp = k_max <= kFusedMaxCS * kFusedWarps * kBlockTokens;
+    if (!one_block_per_warp && units <= fused_prepare<G, 2, 8>()) return {8, 2, kFusedMaxSeq};
+    if (k_max > kFusedOneStageMaxK) return {0, 0, 0};
+    if (units <= fused_prepare<G, 1, 8>()) return {8, 1, kFusedMaxSeq};
+    if (units <= fused_prepare<G, 1, 4>()) return {4, 1, kFusedMaxSeq};
+    return {0, 0, 0};
+}
+
+static FusedVariant fused_variant_for(int B, int Hq, int Hkv, int max_seq_len, int k_max) {
+    if (Hkv <= 0) return {0, 0, 0};
+    const long long units = (long long)B * Hkv;
+    switch (Hq / Hkv) {
+        case 1: return fused_variant<1>(units, max_seq_len, k_max);
+        case 2: return fused_variant<2>(units, max_seq_len, k_max);
+        case 4: return fused_variant<4>(units, max_seq_len, k_max);
+        case 8: return fused_variant<8>(units, max_seq_len, k_max);
+        default: return {0, 0, 0};
+    }
 }
 
 bool fused_step_eligible(int B, int Hq, int Hkv, int max_seq_len, int k_max) {
-    if (max_seq_len > kFusedMaxSeq || Hkv <= 0) return false;
-    const long long units = (long long)B * Hkv;
-    int stages = 0;
-    switch (Hq / Hkv) {
-        case 1: return fused_variant<1>(units, k_max, &stages) > 0;
-        case 2: return fused_variant<2>(units, k_max, &stages) > 0;
-        case 4: return fused_variant<4>(units, k_max, &stages) > 0;
-        case 8: return fused_variant<8>(units, k_max, &stages) > 0;
-        default: return false;
-    }
+    return fused_variant_for(B, Hq, Hkv, max_seq_len, k_max).cs > 0;
 }
 
 bool fused_step_from_host_eligible(int B, int Hq, int Hkv, int max_seq_len, int k_max) {
-    if (max_seq_len > kFusedMaxSeq || Hkv <= 0) return false;
-    const long long units = (long long)B * Hkv;
-    int stages = 0, cs = 0;
-    switch (Hq / Hkv) {
-        case 1: cs = fused_variant<1>(units, k_max, &stages); break;
-        case 2: cs = fused_variant<2>(units, k_max, &stages); break;
-        case 4: cs = fused_variant<4>(units, k_max, &stages); break;
-        case 8: cs = fused_variant<8>(units, k_max, &stages); break;
-        default: return false;
+    const FusedVariant v = fused_variant_for(B, Hq, Hkv, max_seq_len, k_max);
+    return v.cs > 0 && v.stages == 1;
+}
+
+template <int G, int kMode>
+static cudaError_t launch_fused_m(const FusedVariant &v, const FusedArgs &args, int B, cudaStream_t st) {
+    if (v.stages == 1 && v.cs == 8 && v.max_seq == kFusedMidSeq) return launch_fused_gsc<G, 1, 8, kMode, kFusedMidSeq>(args, B, st);
+    if (v.stages == 1 && v.cs == 8) return launch_fused_gsc<G, 1, 8, kMode>(args, B, st);
+    if (v.stages == 1 && v.cs == 4) return launch_fused_gsc<G, 1, 4, kMode>(args, B, st);
+    if constexpr (kMode != kModeHost) {   // only the one-stage variants read their inputs across the bus
+        if (v.stages == 2 && v.max_seq == kFusedLongSeq) return launch_fused_gsc<G, 2, 8, kMode, kFusedLongSeq>(args, B, st);
+        if (v.stages == 2) return launch_fused_gsc<G, 2, 8, kMode>(args, B, st);
     }
-    return cs > 0 && stages == 1;
+    return cudaErrorInvalidConfiguration;
 }
 
 template <int G>
 static cudaError_t launch_fused_g(const FusedArgs &args, int B, cudaStream_t st) {
-    int stages = 0;
-    const int cs = fused_variant<G>((long long)B * args.Hkv, args.k_max, &stages);
-    if (args.v_new) {   // host-buffer entry: only the one-stage variants read their inputs across the bus
-        if (stages == 1 && cs == 8) return launch_fused_gsc<G, 1, 8, kModeHost>(args, B, st);
-        if (stages == 1 && cs == 4) return launch_fused_gsc<G, 1, 4, kModeHost>(args, B, st);
-        return cudaErrorInvalidConfiguration;
-    }
-    if (args.code_pages.table) {
-        if (stages == 2 && cs == 8) return launch_fused_gsc<G, 2, 8, kModePagedCodes>(args, B, st);
-        if (cs == 8) return launch_fused_gsc<G, 1, 8, kModePagedCodes>(args, B, st);
-        if (cs == 4) return launch_fused_gsc<G, 1, 4, kModePagedCodes>(args, B, st);
-        return cudaErrorInvalidConfiguration;
-    }
-    if (stages == 2 && cs == 8) return launch_fused_gsc<G, 2, 8>(args, B, st);
-    if (cs == 8) return launch_fused_gsc<G, 1, 8>(args, B, st);
-    if (cs == 4) return launch_fused_gsc<G, 1, 4>(args, B, st);
-    return cudaErrorInvalidConfiguration;
+    const FusedVariant v = fused_variant<G>((long long)B * args.Hkv, args.max_seq_len, args.k_max);
+    if (args.v_new) return launch_fused_m<G, kModeHost>(v, args, B, st);
+    if (args.code_pages.table) return launch_fused_m<G, kModePagedCodes>(v, args, B, st);
+    return launch_fused_m<G, kModeDevice>(v, args, B, st);
 }
 
 cudaError_t launch_fused_step(int B, int Hq, int Hkv, float sm_scale, const MapView &map_q, const MapView &map_k,

@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_2412_14468_b200 import binding as ha
 from paper_2412_14468_b200 import workloads as wl
-from tests._util import u16
+from tests._util import OUT_TOL, max_abs_diff_bf16, u16
 from tests.test_gpu_parity import _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
     test_whole_step_with_keys_values_and_signatures_all_paged as _whole_paged_step
 
@@ -116,3 +116,68 @@ def test_score_topk_on_clusters_of_large_ctas(G, lens, page_size):
             s = oracle.score(qc[b, g * G:(g + 1) * G], codes[b, g, :n]) if n else np.zeros(0, np.int32)
             ref = oracle.topk_windows(s, ks[b], n_sink, n_local)
             assert n_got[b, g] == len(ref) and np.array_equal(got[b, g, :len(ref)], ref) and (got[b, g, len(ref):] == -1).all()
+
+
+@pytest.mark.parametrize("G", [1, 4, 8])
+@pytest.mark.parametrize("lens,sparsity", [((32769, 1), 32), ((65536, 33000), 64), ((65535,), 16), ((65537, 4), 64), ((131072, 70001), 100)])
+def test_one_launch_step_of_long_sequences(G, lens, sparsity):
+    """Sequences beyond 32768 tokens in one launch (one row stage up to 65536 tokens and 2048 entries, two up to 131072): lists
+    and signatures equal to those of the entry points one by one, outputs to fp32 reordering; the same over pages, and from
+    host buffers."""
+    n_sink, n_local = 70, 40
+    cfg = wl.Config("long-fused", 71, len(lens), list(lens), None, 0.01, n_q_heads=2 * G, n_kv_heads=2, sparsity=sparsity)
+    w = wl.make_workload(cfg, DEV)
+    B, Hq, Hkv, n_cap = cfg.batch, 2 * G, 2, (w["n_cap"] + 63) // 64 * 64
+    k_max = w["k_max"] + n_sink + n_local
+    shape = ha.make_shape(B, Hq, Hkv, w["sm_scale"], n_sink=n_sink, n_local=n_local)
+    ws = ha.alloc_workspace(shape, n_cap, k_max)
+    mq, mk = ha.Mapping(w["map_q"]), ha.Mapping(w["map_k"])
+    clean = torch.zeros(B, Hkv, n_cap, dtype=torch.int32, device=DEV)
+    ha.ha_encode(mk, 1, w["K"], clean)
+    for b, n in enumerate(lens):                                   # slots past a sequence stay untouched by a step
+        clean[b, :, n:] = 0x11111111
+    last = w["seq_lens"].long() - 1
+    stale = clean.clone()
+    stale[torch.arange(B, device=DEV), :, last] = 0x0BADF00D
+    new = lambda *s, t=torch.int32: torch.zeros(*s, dtype=t, device=DEV)  # noqa: E731
+
+    qr, ir, cr, outr = new(B, Hq), new(B, Hkv, k_max), new(B, Hkv), new(B, Hq, 128, t=torch.bfloat16)
+    ha.ha_encode(mq, G, w["q"], qr.unsqueeze(2))
+    ha.ha_score_topk(shape, qr, clean, w["seq_lens"], w["k_per_seq"], 0, w["n_cap"], k_max, ir, cr, ws)
+    ha.ha_gather_attn(shape, w["q"], w["K"], w["V"], w["seq_lens"], ir, cr, k_max, outr, ws)
+
+    def check(idx, cnt, out, qc=None):
+        assert torch.equal(idx, ir) and torch.equal(cnt, cr) and (qc is None or torch.equal(qc, qr))
+        assert max_abs_diff_bf16(u16(out), u16(outr)) <= OUT_TOL
+        assert ha.ha_read_device_status(ws) == 0
+
+    def step(fn, *args):
+        qc, idx, cnt, out = new(B, Hq), new(B, Hkv, k_max), new(B, Hkv), new(B, Hq, 128, t=torch.bfloat16)
+        before = ha.ha_kernel_launches()
+        fn(shape, mq, mk, w["q"], w["k_new"], *args, w["seq_lens"], w["k_per_seq"], 0, w["n_cap"], k_max, qc, idx, cnt, out, ws)
+        assert ha.ha_kernel_launches() - before == 1
+        check(idx, cnt, out, qc)
+
+    codes = stale.clone()
+    step(ha.ha_sparse_decode, w["K"], w["V"], codes)
+    assert torch.equal(codes, clean)
+    page = 16
+    pps = n_cap // page
+    table = torch.randperm(B * pps, device=DEV, generator=torch.Generator(DEV).manual_seed(3)).view(B, pps)
+
+    def pool(x):
+        x = torch.nn.functional.pad(x, (0, 0) * (x.dim() - 3) + (0, n_cap - x.shape[2]))
+        p = torch.empty((B * pps, Hkv, page) + tuple(x.shape[3:]), dtype=x.dtype, device=DEV)
+        for b in range(B):
+            p[table[b]] = x[b].reshape((Hkv, pps, page) + tuple(x.shape[3:])).transpose(0, 1)
+        return p
+
+    pc = pool(stale)
+    step(ha.ha_sparse_decode_paged_codes, pool(w["K"]), pool(w["V"]), pc, table.to(torch.int32))
+    assert torch.equal(pc, pool(clean))
+    pin = lambda t: t.cpu().pin_memory()  # noqa: E731
+    codes, idx, cnt, out = stale.clone(), new(B, Hkv, k_max), new(B, Hkv), torch.zeros(B, Hq, 128, dtype=torch.bfloat16).pin_memory()
+    ha.ha_sparse_decode_host(shape, mq, mk, pin(w["q"]), pin(w["k_new"]), pin(w["v_new"]), w["K"].clone(), w["V"].clone(), codes,
+                             w["seq_lens"], w["k_per_seq"], 0, w["n_cap"], k_max, idx, cnt, out, ws)
+    check(idx, cnt, out)
+    assert torch.equal(codes, clean)
