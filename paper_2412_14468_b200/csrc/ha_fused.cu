@@ -37,7 +37,10 @@ constexpr int kFusedMaxSeq = 32768, kFusedMidSeq = 65536, kFusedLongSeq = 131072
 constexpr int kFusedLongMaxK = 5120;                         // longest index list of the 131072-token variant
 constexpr int kFusedMaxStages = 2;                           // row blocks in flight per warp (template parameter S)
 constexpr int kFusedWeightBytes = (kD * kHid + kHid * kHid + kHid * kBits) * 2;
-constexpr int kFusedOneStageMaxK = 2048;                     // one-stage variant: longest index list
+// Longest index list of the one-stage variant and of the stand-alone cluster gather: 32768 / 16 entries and the windows of the
+// paper's experiments fit.  Lists of 2304 entries, groups of 4, 8 units a sequence, against the kernels beyond the limit, us per
+// step: 4 sequences 22.1 / 29.2, 8 sequences 31.3 / 39.5 (one launch against three), 16 sequences 51.5 / 54.7 (GATHER-ATT).
+constexpr int kFusedOneStageMaxK = 2560;
 constexpr int kFusedListOffset = kFusedWarps * kStageBytes;  // one-stage variant: this CTA's part of the list sits behind the ring
 // query vectors per encoding CTA: the smallest divisor of G that leaves the cluster one CTA for the appended key
 __host__ __device__ constexpr int fused_q_per_cta(int G, int CS) {
@@ -54,7 +57,7 @@ __host__ __device__ constexpr int fused_part_bytes(int G, int CS) { return CS * 
 __host__ __device__ constexpr int fused_smem_bytes(int G, int S, int CS) {
     return fused_union_bytes(S) + fused_act_bytes(G, CS) + fused_part_bytes(G, CS);
 }
-static_assert(kFusedListOffset + kFusedOneStageMaxK / 2 * 4 <= kFusedWeightBytes, "the list part fits behind the one-stage ring");
+static_assert(kFusedOneStageMaxK % (4 * kBlockTokens) == 0 && kFusedListOffset + kFusedOneStageMaxK <= kFusedWeightBytes, "a quarter of the list (clusters of 4 or 8) fits behind the one-stage ring");
 
 struct FusedArgs {
     MapView map_q, map_k;
@@ -696,7 +699,7 @@ static int gather_cluster_size(long long units) {
     return 0;
 }
 
-// Lists of up to 2048 entries (a few blocks per warp) and as many units as clusters are resident at once.
+// Lists of up to kFusedOneStageMaxK entries (a few blocks per warp) and as many units as clusters are resident at once.
 bool gather_cluster_eligible(int B, int Hq, int Hkv, int k_max) {
     if (Hkv <= 0 || k_max > kFusedOneStageMaxK) return false;
     const long long units = (long long)B * Hkv;
@@ -811,7 +814,7 @@ static cudaError_t launch_fused_gsc(const FusedArgs &args, int B, cudaStream_t s
 //    take their blocks one after the other).
 // Clusters of 2 work as well (the kernel is written for them) but lose to the three-kernel path at the batch
 // sizes they would serve (45.7 against 41.3 us at 128 units), so they are not offered.
-//  * sequences of more than 32768 tokens: clusters of 8, one-stage up to 65536 tokens and 2048 entries, else two-stage up to
+//  * sequences of more than 32768 tokens: clusters of 8, one-stage up to 65536 tokens and 2560 entries, else two-stage up to
 //    131072 tokens and kFusedLongMaxK entries, while `units` clusters are resident (33 and 15).  Against three launches, groups
 //    of 4, 8 units a sequence, lists of n / 32, us: one sequence of 65536 14.1 / 20.1, of 131072 21.9 / 26.5; four of 65536
 //    22.3 / 31.2.  With lists of n / 8 eight CTAs of two stages fetch too slowly: 60000 28.6 / 26.6, 100000 36.8 / 34.5.

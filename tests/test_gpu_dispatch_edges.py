@@ -8,7 +8,7 @@ import oracle
 from paper_2412_14468_b200 import binding as ha
 from paper_2412_14468_b200 import workloads as wl
 from tests._util import OUT_TOL, max_abs_diff_bf16, u16
-from tests.test_gpu_parity import _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
+from tests.test_gpu_parity import _attn_inputs, _check_gather, _run_step, _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
     test_whole_step_with_keys_values_and_signatures_all_paged as _whole_paged_step
 
 pytestmark = pytest.mark.gpu
@@ -121,7 +121,7 @@ def test_score_topk_on_clusters_of_large_ctas(G, lens, page_size):
 @pytest.mark.parametrize("G", [1, 4, 8])
 @pytest.mark.parametrize("lens,sparsity", [((32769, 1), 32), ((65536, 33000), 64), ((65535,), 16), ((65537, 4), 64), ((131072, 70001), 100)])
 def test_one_launch_step_of_long_sequences(G, lens, sparsity):
-    """Sequences beyond 32768 tokens in one launch (one row stage up to 65536 tokens and 2048 entries, two up to 131072): lists
+    """Sequences beyond 32768 tokens in one launch (one row stage up to 65536 tokens and 2560 entries, two up to 131072): lists
     and signatures equal to those of the entry points one by one, outputs to fp32 reordering; the same over pages, and from
     host buffers."""
     n_sink, n_local = 70, 40
@@ -181,3 +181,25 @@ def test_one_launch_step_of_long_sequences(G, lens, sparsity):
                              w["seq_lens"], w["k_per_seq"], 0, w["n_cap"], k_max, idx, cnt, out, ws)
     check(idx, cnt, out)
     assert torch.equal(codes, clean)
+
+
+@pytest.mark.parametrize("B", [10, 30])
+@pytest.mark.parametrize("k,launches", [(2560, 1), (2561, 3)])
+def test_step_at_the_longest_list_of_one_launch(B, k, launches):
+    """20 and 60 units (clusters of 8 and of 4): the longest list that one launch takes and the first beyond it give the lists and
+    outputs of the entry points one by one; GATHER-ATT at these lengths against the oracle."""
+    cfg = wl.Config("longest-list", 72, B, [2 * k] * B, None, 0.02, n_q_heads=8, n_kv_heads=2, sparsity=2)
+    w = wl.make_workload(cfg, DEV)
+    _run_step(w)
+    before = ha.ha_kernel_launches()
+    r = _run_step(w)
+    assert ha.ha_kernel_launches() - before == launches + 1        # and the signature cache
+    shape = ha.make_shape(B, 8, 2, w["sm_scale"])
+    ws = ha.alloc_workspace(shape, 2 * k, k)
+    idx, cnt, out = torch.zeros_like(r["idx"]), torch.zeros_like(r["cnt"]), torch.zeros_like(r["out"])
+    ha.ha_score_topk(shape, r["qc"], r["kc"], w["seq_lens"], w["k_per_seq"], 0, 2 * k, k, idx, cnt, ws)
+    ha.ha_gather_attn(shape, w["q"], w["K"], w["V"], w["seq_lens"], idx, cnt, k, out, ws)
+    assert torch.equal(idx, r["idx"]) and torch.equal(cnt, r["cnt"]) and max_abs_diff_bf16(u16(out), u16(r["out"])) <= OUT_TOL
+    n = 3000
+    lists = np.random.default_rng(k).integers(0, n, size=(1, 2, k)).astype(np.int32)
+    _check_gather(*_attn_inputs(1, 8, 2, n, 5), [n], lists, np.full((1, 2), k, np.int32), 0.09)
