@@ -203,3 +203,13 @@ def test_step_at_the_longest_list_of_one_launch(B, k, launches):
     n = 3000
     lists = np.random.default_rng(k).integers(0, n, size=(1, 2, k)).astype(np.int32)
     _check_gather(*_attn_inputs(1, 8, 2, n, 5), [n], lists, np.full((1, 2), k, np.int32), 0.09)
+
+
+@pytest.mark.parametrize("k", [4095, 4096, 4097])
+def test_gather_attn_at_the_longest_list_of_clusters_of_four(k):
+    """44 units: up to 4096 entries on clusters of 4, more on the split-K kernel; full and ragged lists."""
+    B, Hkv, G, n = 22, 2, 2, 5000
+    rng = np.random.default_rng(k)
+    lists = rng.integers(0, n, size=(B, Hkv, k)).astype(np.int32)
+    cnt = np.where(np.arange(B * Hkv).reshape(B, Hkv) % 3 == 0, k, rng.integers(0, k, size=(B, Hkv))).astype(np.int32)
+    _check_gather(*_attn_inputs(B, Hkv * G, Hkv, n, 6), [n] * B, lists, cnt, 0.09)
