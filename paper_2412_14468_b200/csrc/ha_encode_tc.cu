@@ -359,6 +359,7 @@ __global__ void __launch_bounds__(kU_Threads, 1) encode_umma_kernel(const __grid
     __shared__ __align__(8) unsigned long long s_dbar[2];      // [group]: a hidden layer is summed
     __shared__ __align__(8) unsigned long long s_abar[2][2];   // [group][half]: 64 columns of it are converted (8 warps arrive)
     __shared__ __align__(8) unsigned long long s_obar[2];      // [group]: the 32 outputs are summed
+    __shared__ __align__(8) unsigned long long s_start;        // group 0's first hidden layer is converted; completes once
     __shared__ uint32_t s_tmem_base;
     __shared__ volatile int s_fail;
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -399,6 +400,7 @@ __global__ void __launch_bounds__(kU_Threads, 1) encode_umma_kernel(const __grid
         mbar_init(smem_u32(&s_dbar[1]), 1);
         mbar_init(smem_u32(&s_obar[0]), 1);
         mbar_init(smem_u32(&s_obar[1]), 1);
+        mbar_init(smem_u32(&s_start), kU_Convert / 32);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_fail = 0;
         if (kTma) {   // the first tiles are on their way while the weights are laid out
@@ -563,8 +565,9 @@ __global__ void __launch_bounds__(kU_Threads, 1) encode_umma_kernel(const __grid
             __syncwarp();
         };
         // the groups work half a tile apart, or both would multiply and both would convert at the same time: group 1 starts when
-        // group 0 has converted its first hidden layer
-        bool ok = g == 0 || n_tiles == 0 || wait(smem_u32(&s_abar[0][1]), 0u);
+        // group 0 has converted its first hidden layer.  The barrier has that one phase: group 0 does not wait for group 1, and a
+        // barrier that it completes a second time reads "not complete" again to a warp that looks late.
+        bool ok = g == 0 || n_tiles == 0 || wait(smem_u32(&s_start), 0u);
         int i = 0;
         for (; ok && i < n_tiles; ++i) {
             const uint32_t p = cols + (i & 1) * kU_Region, q = cols + ((i & 1) ^ 1) * kU_Region;
@@ -632,6 +635,7 @@ __global__ void __launch_bounds__(kU_Threads, 1) encode_umma_kernel(const __grid
             const bool copy = !kTma && i + 1 < tiles_of(g);
             if (copy) copy_x(g, w_lo + g + 2LL * (i + 1), (i + 1) & 1);
             if (!convert(g, region(g, i), 0u)) return false;
+            if (g == 0 && i == 0 && (tid & 31) == 0) mbar_arrive(smem_u32(&s_start));
             if (copy) copied_x(g, (i + 1) & 1);
             return true;
         };
