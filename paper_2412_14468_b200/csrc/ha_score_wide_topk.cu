@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kWideThreads) wide_write_kernel(const WideArgs
 // A cluster of up to eight CTAs owns a unit: every CTA leaves the scores of its slice in shared memory (16 bits per
 // token), the CTAs exchange their level counts through distributed shared memory between two cluster barriers, and each
 // compacts its own slice.  Against the three kernels for long sequences there is no memset, no histogram and no score
-// pass through global memory, and the signatures are requested before the programmatic-launch wait.
+// pass through global memory, and the first signatures are asked into L2 before the programmatic-launch wait.
 // Bound: the population-count unit (16 lanes per clock and SM; a token costs G popcounts per counted word), then HBM.
 // Carry-save adders on the logic unit fold the xor words of a token before they are counted: 3, 4 and 5 counted words
 // instead of 4, 8 and 16 for 128, 256 and 512 bits.
@@ -355,39 +355,40 @@ __global__ void __launch_bounds__(kWideThreads) wide_select_cluster_kernel(const
     const uint64_t *row = a.k_codes + (long long)b * a.kc_sb + (long long)g * a.kc_sh;
 
     // a pass: token base + (p kTok + i) 256 + tid for i < kTok, so that a warp reads consecutive signatures
-    auto load_token = [&](unsigned long long (&kw)[W], int t, bool early) {
+    auto load_token = [&](unsigned long long (&kw)[W], int t) {
         if (W == 1) {
-            kw[0] = early ? __ldg(reinterpret_cast<const unsigned long long *>(row + t)) : __ldcg(reinterpret_cast<const unsigned long long *>(row + t));
+            kw[0] = __ldcg(reinterpret_cast<const unsigned long long *>(row + t));
         } else {
 #pragma unroll
             for (int w = 0; w < W; w += 2) {
-                const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(row + (long long)t * W + w);
-                const ulonglong2 v = early ? __ldg(src) : __ldcg(src);
+                const ulonglong2 v = __ldcg(reinterpret_cast<const ulonglong2 *>(row + (long long)t * W + w));
                 kw[w] = v.x; kw[w + 1] = v.y;
             }
         }
     };
-    auto load_pass = [&](unsigned long long (&kw)[kTok][W], int p, bool early) {
+    auto load_pass = [&](unsigned long long (&kw)[kTok][W], int p) {
 #pragma unroll
         for (int i = 0; i < kTok; ++i) {
             const int l = (p * kTok + i) * kWideThreads + tid;
-            if (l < slice && base + l < n) load_token(kw[i], base + l, early);
+            if (l < slice && base + l < n) load_token(kw[i], base + l);
             else
 #pragma unroll
                 for (int w = 0; w < W; ++w) kw[i][w] = 0ull;
         }
     };
+    // The first pass is only asked into L2 before the launch wait (one request per 128-byte line) and loaded after it: the kernel
+    // in front may still be writing signatures, at any slot.
+#pragma unroll
+    for (int i = 0; i < kTok; ++i) {
+        const int l = i * kWideThreads + tid;
+        if (l % (16 / W) == 0 && l < slice && base + l < n)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(row + (long long)(base + l) * W));
+    }
     unsigned long long cur[kTok][W], nxt[kTok][W];
-    load_pass(cur, 0, true);
     for (int i = tid; i < levels * kCols; i += kWideThreads) c_hist[i] = 0u;
     pdl_launch_dependents();
     pdl_wait();
-    // the signatures that a library kernel directly in front may just have written (slots n-1 and n-2): read again
-#pragma unroll
-    for (int i = 0; i < kTok; ++i) {
-        const int l = i * kWideThreads + tid, t = base + l;
-        if (l < slice && t < n && t >= n - 2) load_token(cur[i], t, false);
-    }
+    load_pass(cur, 0);
     if (tid < a.G * W)
         s_q[tid / W][tid % W] = __ldcg(reinterpret_cast<const unsigned long long *>(a.q_codes) +
                                        ((long long)b * a.Hq + (long long)g * a.G + tid / W) * W + tid % W);
@@ -395,7 +396,7 @@ __global__ void __launch_bounds__(kWideThreads) wide_select_cluster_kernel(const
 
     const int n_pass = Rb * 8 / kTok;
     for (int p = 0; p < n_pass; ++p) {
-        if (p + 1 < n_pass) load_pass(nxt, p + 1, false);
+        if (p + 1 < n_pass) load_pass(nxt, p + 1);
         int best[kTok];
 #pragma unroll
         for (int i = 0; i < kTok; ++i) best[i] = a.n_bits;
