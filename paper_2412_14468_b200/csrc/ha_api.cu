@@ -372,7 +372,7 @@ static int sparse_decode_impl(const ha_shape *shape, const ha_mapping *map_q, co
     HA_CUDA(launch_score_topk(B, Hq, Hkv, q_codes, k_codes, kc_stride_b, kc_stride_h, seq_lens, k_per_seq, k_uniform,
                               max_seq_len, k_max, idx, idx_stride_b, idx_stride_h, count, nullptr,
                               ws_ptr<int32_t>(workspace, L.off_hist), ws_ptr<unsigned char>(workspace, L.off_scores), st,
-                              Windows{shape->n_sink, shape->n_local}, code_pages));
+                              Windows{shape->n_sink, shape->n_local}, code_pages, -1, /*in_step=*/true));
     if (gather_cluster_eligible(B, Hq, Hkv, k_max)) {
         // up to a cluster per unit resident at once and short lists: GATHER-ATT with the states merged in shared memory
         HA_CUDA(launch_gather_cluster(B, Hq, Hkv, shape->sm_scale, q, view(K), view(V), seq_lens, idx, idx_stride_b,

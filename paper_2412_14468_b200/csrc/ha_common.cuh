@@ -202,9 +202,10 @@ cudaError_t launch_score_topk(int B, int Hq, int Hkv, const uint32_t *q_codes, c
                               const int32_t *k_per_seq, int k_uniform, int max_seq_len, int k_max,
                               int32_t *idx, long long idx_sb, long long idx_sh, int32_t *count,
                               int32_t *hist_out, int32_t *ws_hist, unsigned char *ws_scores, cudaStream_t st, Windows win = Windows{0, 0},
-                              CodePages pages = CodePages{nullptr, 0, 0, 0, 0}, int row_shift = -1);
+                              CodePages pages = CodePages{nullptr, 0, 0, 0, 0}, int row_shift = -1, bool in_step = false);
 // pages.table != NULL: k_codes is a paged pool; row_shift >= 0: one unit per QUERY head
-// (Hq units per sequence, groups of one head), whose signature row is that of KV head h >> row_shift.
+// (Hq units per sequence, groups of one head), whose signature row is that of KV head h >> row_shift;
+// in_step: the kernel in front is the ENCODE of the same layer-step.
 
 // SCORE + TOPK with the group's per-head scores added instead of maximised (one cluster per unit, no scratch);
 // per_head: no reduction at all, one list per QUERY head (idx, count, hist_out then have n_q_heads rows per sequence).

@@ -7,7 +7,8 @@
 //
 //   P0  every CTA requests its slice of the signature cache; the encoding CTAs of the cluster fetch the
 //       query-side / key-side mapping weights and store them transposed in shared memory; all of it
-//       before the programmatic-launch wait, i.e. behind the preceding kernel.
+//       before the programmatic-launch wait, i.e. behind the preceding kernel (signatures in pages:
+//       behind the wait, since the block table may come from that kernel).
 //   P1  the first CTAs of the cluster encode the G query vectors (one per CTA when the cluster has room,
 //       else 2 or 4), the next CTA the appended key (fp32 fma chains, Eq. 2, one chain per thread); the
 //       signatures are stored into every CTA's shared memory (DSMEM); cluster barrier.
@@ -106,7 +107,7 @@ __device__ __forceinline__ void st_dsmem_f32(float *local, uint32_t rank, float 
 // call; the barrier that publishes the input vectors also publishes them.  Signature v is written to
 // word v of `dst` in the shared memory of EVERY CTA of the cluster (lanes 0..CS-1 of the warp that holds it
 // store to CTAs 0..CS-1; the cluster barrier that follows makes the stores visible).
-// kRaw: thread o already holds component o of every vector in xr (fetched across the bus earlier).
+// kRaw: thread o already holds component o of every vector in xr (fetched earlier).
 template <int NV, int CS, bool kRaw = false>
 __device__ __forceinline__ void fused_encode(const uint16_t *x0, long long x_stride, const uint16_t *sw1,
                                              const uint16_t *sw2, const uint16_t *sw3, float *actA, float *actB,
@@ -302,6 +303,9 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     constexpr int kQPer = fused_q_per_cta(G, CS);
     constexpr int kQCtas = G / kQPer;
     static_assert(kQCtas * kQPer == G && kQCtas < CS, "the cluster needs one more CTA for the appended key");
+    // the vectors to encode are fetched in front of whatever else crosses the bus, or of many loads through a block table
+    // (80847 tokens in pages of 16, 16 loads a thread: 27.4 against 29.1 us per step; four loads: 12.4 / 12.2 the other way)
+    constexpr bool kXFirst = kHost || (codes_paged && kL > 4);
     constexpr bool kPreload = (CS > 2);   // signatures requested before the launch wait (16 uint4 would not fit the registers)
     extern __shared__ __align__(128) unsigned char fsm[];
     // dynamic: [weights | row ring] union, activations, the cluster's states (used in CTA 0)
@@ -339,7 +343,7 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     const int32_t *code_table = a.code_pages.table + (codes_paged ? (long long)b * a.code_pages.bt_sb : 0);
     auto code_slot = [&](int t) -> uint32_t * {
         if (!codes_paged) return row + t;
-        return row + (long long)__ldg(code_table + (t >> a.code_pages.shift)) * a.code_pages.page_stride + (t & ((1 << a.code_pages.shift) - 1));
+        return row + (long long)__ldcg(code_table + (t >> a.code_pages.shift)) * a.code_pages.page_stride + (t & ((1 << a.code_pages.shift) - 1));
     };
     const bool has_new_key = (a.k_new != nullptr) && n > 0;
 
@@ -348,11 +352,25 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     const int wbase = ((int)rank * 1024 + warp * 128 + lane * 4) * Lb;
     uint4 c[kL];
     auto load_signatures = [&]() {
+        // a lane's tokens follow one another: one table entry per page that they reach, all requested before the first use
+        const int mask = (1 << a.code_pages.shift) - 1;
+        if (codes_paged && a.code_pages.shift >= 2) {
+#pragma unroll
+            for (int p = 0; p < kL; ++p) {
+                const int base = wbase + p * 4;
+                if (p < Lb && base < n && (p == 0 || (base & mask) == 0)) c[p].x = (uint32_t)__ldcg(code_table + (base >> a.code_pages.shift));
+            }
+        }
+        int page = 0;
 #pragma unroll
         for (int p = 0; p < kL; ++p) {
             const int base = wbase + p * 4;
+            if (codes_paged && (p == 0 || (base & mask) == 0)) page = (int)c[p].x;
             c[p] = make_uint4(0, 0, 0, 0);
-            if (p < Lb && base < n) c[p] = codes_paged ? load_codes4_paged(a.code_pages, row, code_table, base, n) : load_codes4(row, base, n);
+            if (p >= Lb || base >= n) continue;
+            if (!codes_paged) c[p] = load_codes4(row, base, n);
+            else if (a.code_pages.shift >= 2) c[p] = load_codes4(row + (long long)page * a.code_pages.page_stride + (base & mask) - base, base, n);
+            else c[p] = load_codes4_paged(a.code_pages, row, code_table, base, n);
         }
     };
     // Host-buffer step: everything that crosses the bus is requested first (a round trip of about 2 us), under the fetch and the
@@ -377,7 +395,7 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
         if ((int)rank == kQCtas && has_new_key && a.v_new && tid < 64)
             kv_row = __ldg(reinterpret_cast<const uint2 *>(((tid < 32) ? a.k_new : a.v_new) + ((long long)b * Hkv + kvh) * kD) + (tid & 31));
     }
-    if (kPreload) load_signatures();
+    if (kPreload && !codes_paged) load_signatures();
     // ENCODE roles: CTA r < kQCtas encodes kQPer query vectors (one per CTA while the cluster has room),
     // CTA kQCtas encodes the appended key; the other CTAs only scan
     const bool enc_q = (int)rank < kQCtas, enc_k = ((int)rank == kQCtas) && has_new_key;
@@ -411,6 +429,17 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
         reinterpret_cast<uint4 *>(&c_hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
     if (!kHost) pdl_wait();      // q, k_new and everything older in the stream is final from here on
     pdl_launch_dependents();
+    if (codes_paged) {           // the block table may come from the kernel in front
+        if (kXFirst && tid < kD) {
+            if (enc_q) {
+#pragma unroll
+                for (int v = 0; v < kQPer; ++v) x_raw[v] = __ldcg(a.q + (head0 + kQPer * (int)rank + v) * kD + tid);
+            } else if (enc_k) {
+                x_raw[0] = __ldcg(a.k_new + ((long long)b * Hkv + kvh) * kD + tid);
+            }
+        }
+        load_signatures();
+    }
     cluster_wait();              // #0: all CTAs of the cluster are running (their shared memory may be written)
     if (kHost) {
         if (enc_k && a.v_new && tid < 64) {
@@ -423,11 +452,11 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
 
     // ---------------- P1: ENCODE in the first kQCtas CTAs (queries) and the next one (appended key)
     if (enc_q) {
-        fused_encode<kQPer, CS, kHost>(a.q + (head0 + kQPer * (int)rank) * kD, kD, sw1, sw2, sw3, actA, actB,
-                                       s_codes + kQPer * (int)rank, bias1, bias2, bias3, x_raw);
+        fused_encode<kQPer, CS, kXFirst>(a.q + (head0 + kQPer * (int)rank) * kD, kD, sw1, sw2, sw3, actA, actB,
+                                         s_codes + kQPer * (int)rank, bias1, bias2, bias3, x_raw);
     } else if (enc_k) {
-        fused_encode<1, CS, kHost>(a.k_new + ((long long)b * Hkv + kvh) * kD, kD, sw1, sw2, sw3, actA, actB, s_codes + G, bias1,
-                                   bias2, bias3, x_raw);
+        fused_encode<1, CS, kXFirst>(a.k_new + ((long long)b * Hkv + kvh) * kD, kD, sw1, sw2, sw3, actA, actB, s_codes + G,
+                                   bias1, bias2, bias3, x_raw);
     }
     cluster_sync_all();   // #1: every CTA holds all signatures (and its counters are zeroed)
     // the signatures also go to global memory (outputs of the step; nobody in this kernel reads them there):
@@ -438,7 +467,7 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     uint32_t qc[G];
 #pragma unroll
     for (int j = 0; j < G; ++j) qc[j] = s_codes[j];
-    if (!kPreload) load_signatures();
+    if (!kPreload && !codes_paged) load_signatures();
     // Signatures that the early request may have seen in a stale state: slot n-1 (this step's appended token:
     // encoded above, or, when the step has no k_new, possibly written by an ha_encode call directly in front)
     // and slot n-2 (appended by a layer-step on the same cache directly in front, whose kernel lets this one
@@ -453,7 +482,7 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
         }
     };
     if (has_new_key) replace_slot(n - 1, s_codes[G]);
-    if (kPreload) {
+    if (kPreload && !codes_paged) {
         const int lo = wbase, hi = wbase + 4 * Lb;   // this lane's tokens (contiguous)
         if (!has_new_key && n - 1 >= lo && n - 1 < hi) replace_slot(n - 1, __ldcg(code_slot(n - 1)));
         if (n - 2 >= lo && n - 2 < hi) replace_slot(n - 2, __ldcg(code_slot(n - 2)));

@@ -5,13 +5,15 @@
 
 namespace ha {
 
+// Loaded from L2 (.cg): kernels overlap on an SM, and its L1 may hold a line that one of them fetched before a signature or a
+// table entry in it was written.
 __device__ __forceinline__ uint4 load_codes4(const uint32_t *row, int base, int n) {
     // tokens base..base+3 of a 16-byte aligned row; tokens >= n come back as don't-care zeros
-    if (base + 3 < n) return __ldg(reinterpret_cast<const uint4 *>(row + base));
+    if (base + 3 < n) return __ldcg(reinterpret_cast<const uint4 *>(row + base));
     uint4 v = make_uint4(0, 0, 0, 0);
-    if (base + 0 < n) v.x = __ldg(row + base + 0);
-    if (base + 1 < n) v.y = __ldg(row + base + 1);
-    if (base + 2 < n) v.z = __ldg(row + base + 2);
+    if (base + 0 < n) v.x = __ldcg(row + base + 0);
+    if (base + 1 < n) v.y = __ldcg(row + base + 1);
+    if (base + 2 < n) v.z = __ldcg(row + base + 2);
     return v;
 }
 
@@ -30,14 +32,14 @@ __device__ __forceinline__ void patch_token(uint4 &v, int base, int last, const 
 __device__ __forceinline__ uint4 load_codes4_paged(const CodePages &cp, const uint32_t *pool_head, const int32_t *table_b,
                                                    int base, int n) {
     if (cp.shift >= 2) {
-        const uint32_t *p = pool_head + (long long)__ldg(table_b + (base >> cp.shift)) * cp.page_stride + (base & ((1 << cp.shift) - 1));
+        const uint32_t *p = pool_head + (long long)__ldcg(table_b + (base >> cp.shift)) * cp.page_stride + (base & ((1 << cp.shift) - 1));
         return load_codes4(p - base, base, n);
     }
     uint32_t v[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int t = base + i;
-        if (t < n) v[i] = __ldg(pool_head + (long long)__ldg(table_b + (t >> cp.shift)) * cp.page_stride + (t & ((1 << cp.shift) - 1)));
+        if (t < n) v[i] = __ldcg(pool_head + (long long)__ldcg(table_b + (t >> cp.shift)) * cp.page_stride + (t & ((1 << cp.shift) - 1)));
     }
     return make_uint4(v[0], v[1], v[2], v[3]);
 }
@@ -45,7 +47,7 @@ __device__ __forceinline__ void patch_token_paged(uint4 &v, int base, int last, 
                                                   const int32_t *table_b) {
     const int e = last - base;
     if (e < 0 || e > 3) return;
-    const uint32_t c = __ldcg(pool_head + (long long)__ldg(table_b + (last >> cp.shift)) * cp.page_stride + (last & ((1 << cp.shift) - 1)));
+    const uint32_t c = __ldcg(pool_head + (long long)__ldcg(table_b + (last >> cp.shift)) * cp.page_stride + (last & ((1 << cp.shift) - 1)));
     if (e == 0) v.x = c; else if (e == 1) v.y = c; else if (e == 2) v.z = c; else v.w = c;
 }
 

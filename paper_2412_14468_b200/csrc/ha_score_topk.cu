@@ -13,8 +13,8 @@
 // No CTA ever spins on another: hand-offs are hardware cluster barriers or kernel boundaries.
 // The scanning kernels request their first signatures before the programmatic-launch wait, so that
 // the fetch overlaps the tail of the preceding kernel; the one signature that the preceding ENCODE
-// may still be writing (the appended token, slot n-1) is re-read after the wait.
-#include <cstdlib>
+// may still be writing (the appended token, slot n-1) is re-read after the wait.  A block table is
+// read before the wait only inside a layer-step (in_step), where ENCODE has waited for whatever wrote it.
 #include "ha_score_dev.cuh"
 
 namespace ha {
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_score_kernel(const uint32_t
                                                                  int chunk_tokens, long long score_row,
                                                                  unsigned char *__restrict__ ws_scores,
                                                                  int32_t *__restrict__ ws_hist, Windows win, CodePages cp,
-                                                                 int row_shift) {
+                                                                 int row_shift, bool in_step) {
     __shared__ __align__(16) uint32_t c_hist[kBins][32];
     __shared__ int s_hist[kBins + 3];
     __shared__ uint32_t s_qc[G];
@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_score_kernel(const uint32_t
     const int n = min(seq_lens[b], max_seq_len);
     const int start = chunk * chunk_tokens;
     if (start >= n) return;
+    if (paged && !in_step) pdl_wait();   // a block table may come from the kernel in front
     const int tid = threadIdx.x, lane = tid & 31;
     // contiguous cache: the unit's row; paged cache: the pool from this head's offset on
     const uint32_t *row = paged ? k_codes + (long long)kvh * cp.head_stride : k_codes + (long long)b * kc_sb + (long long)kvh * kc_sh;
@@ -310,7 +311,8 @@ __global__ void __launch_bounds__(kThreads, kThreads > 256 ? 2 : kPaged ? 5 : 6)
     const uint32_t *__restrict__ q_codes, const uint32_t *__restrict__ k_codes, long long kc_sb, long long kc_sh,
     const int32_t *__restrict__ seq_lens, int max_seq_len, const int32_t *__restrict__ k_per_seq, int k_uniform,
     int k_max, int Hq, int Hkv, int32_t *__restrict__ idx, long long idx_sb, long long idx_sh,
-    int32_t *__restrict__ count, int32_t *__restrict__ hist_out, Windows win, const CodePages cp, int kv_shift) {
+    int32_t *__restrict__ count, int32_t *__restrict__ hist_out, Windows win, const CodePages cp, int kv_shift,
+    bool in_step) {
     constexpr int kSlice = kThreads * 8;                       // tokens of one row of a CTA: eight per lane
     extern __shared__ __align__(16) unsigned char s_sc[];      // score + 1 of this CTA's tokens (0 = no token)
     __shared__ __align__(16) uint32_t c_hist[kBins][32];       // counters [level][lane]
@@ -352,13 +354,14 @@ __global__ void __launch_bounds__(kThreads, kThreads > 256 ? 2 : kPaged ? 5 : 6)
             hi = (p < Rb && t + 4 < n) ? load_codes4_paged(cp, row, table_b, t + 4, n) : make_uint4(0, 0, 0, 0);
         } else if (p < Rb && t + 8 <= n) {
             const uint4 *src = reinterpret_cast<const uint4 *>(src_row + t);
-            if (early) { lo = __ldg(src); hi = __ldg(src + 1); }
+            if (early) { lo = __ldg(src); hi = __ldg(src + 1); }   // L1 for the halves of a sector: 115.0 / 116.7 us, 32 sequences of 8192 - 131072
             else { lo = __ldcg(src); hi = __ldcg(src + 1); }
         } else {
             lo = (p < Rb && t < n) ? load_codes4(src_row, t, n) : make_uint4(0, 0, 0, 0);
             hi = (p < Rb && t + 4 < n) ? load_codes4(src_row, t + 4, n) : make_uint4(0, 0, 0, 0);
         }
     };
+    if (kPaged && !in_step) pdl_wait();   // a block table may come from the kernel in front
     uint4 c[4];   // two rows
     const uint32_t *r0 = row_ptr(0), *r1 = row_ptr(1);
     load_row(0, r0, c[0], c[1], true);
@@ -541,7 +544,7 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
                                     long long kc_sb, long long kc_sh, const int32_t *seq_lens,
                                     const int32_t *k_per_seq, int k_uniform, int max_seq_len, int k_max, int32_t *idx,
                                     long long idx_sb, long long idx_sh, int32_t *count, int32_t *hist_out,
-                                    cudaStream_t st, Windows win, CodePages cp, int kv_shift) {
+                                    cudaStream_t st, Windows win, CodePages cp, int kv_shift, bool in_step) {
     static bool opted[64] = {};   // opt in to the padded shared-memory sizes once per device
     {
         int dev = 0;
@@ -594,7 +597,7 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
     cfg.numAttrs = 2;
     cudaError_t e = cudaLaunchKernelEx(&cfg, score_select_cluster_kernel<G, CS, kPaged, kThreads>, q_codes, k_codes, kc_sb, kc_sh,
                                        seq_lens, max_seq_len, k_per_seq, k_uniform, k_max, Hq, Hkv, idx, idx_sb, idx_sh,
-                                       count, hist_out, win, cp, kv_shift);
+                                       count, hist_out, win, cp, kv_shift, in_step);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
@@ -605,12 +608,12 @@ static cudaError_t launch_g(int B, int Hq, int Hkv, const uint32_t *q_codes, con
                             long long kc_sb, long long kc_sh, const int32_t *seq_lens, const int32_t *k_per_seq,
                             int k_uniform, int max_seq_len, int k_max, int32_t *idx, long long idx_sb,
                             long long idx_sh, int32_t *count, int32_t *hist_out, int32_t *ws_hist,
-                            unsigned char *ws_scores, cudaStream_t st, Windows win, CodePages cp, int row_shift) {
+                            unsigned char *ws_scores, cudaStream_t st, Windows win, CodePages cp, int row_shift, bool in_step) {
     if (large_clusters((long long)B * Hkv, max_seq_len)) {
         const int rows = (max_seq_len + 8 * 4096 - 1) / (8 * 4096), kv_shift = row_shift < 0 ? 0 : row_shift;
 #define HA_LARGE(PAGED) launch_cluster_t<G, 8, PAGED, 512>(rows, B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq,   \
                                                            k_uniform, max_seq_len, k_max, idx, idx_sb, idx_sh, count, hist_out, st, \
-                                                           win, cp, kv_shift)
+                                                           win, cp, kv_shift, in_step)
         return cp.table ? HA_LARGE(true) : HA_LARGE(false);
 #undef HA_LARGE
     }
@@ -626,7 +629,7 @@ static cudaError_t launch_g(int B, int Hq, int Hkv, const uint32_t *q_codes, con
         const int rows = max(1, (max_seq_len + cs * 2048 - 1) / (cs * 2048));
         const int kv_shift = row_shift < 0 ? 0 : row_shift;
 #define HA_CL_ARGS rows, B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, idx, \
-                   idx_sb, idx_sh, count, hist_out, st, win, cp, kv_shift
+                   idx_sb, idx_sh, count, hist_out, st, win, cp, kv_shift, in_step
 #define HA_CL(CSZ) return cp.table ? launch_cluster_t<G, CSZ, true>(HA_CL_ARGS) : launch_cluster_t<G, CSZ, false>(HA_CL_ARGS)
         if (cs == 8) HA_CL(8);
         if (cs == 4) HA_CL(4);
@@ -639,7 +642,7 @@ static cudaError_t launch_g(int B, int Hq, int Hkv, const uint32_t *q_codes, con
     const long long score_row = (long long)score_row_bytes(max_seq_len);
     dim3 grid(n_chunks, Hkv, B);
     cudaError_t e = launch_pdl(scan_score_kernel<G>, grid, dim3(kScanThreads), 0, st, q_codes, k_codes, kc_sb, kc_sh,
-                               seq_lens, max_seq_len, Hq, Hkv, chunk_tokens, score_row, ws_scores, ws_hist, win, cp, row_shift);
+                               seq_lens, max_seq_len, Hq, Hkv, chunk_tokens, score_row, ws_scores, ws_hist, win, cp, row_shift, in_step);
     if (e != cudaSuccess) return e;
     e = launch_pdl(select_kernel, grid, dim3(kScanThreads), 0, st, seq_lens, max_seq_len, k_per_seq, k_uniform, k_max,
                    Hkv, chunk_tokens, score_row, (const unsigned char *)ws_scores, (const int32_t *)ws_hist, idx, idx_sb,
@@ -654,13 +657,13 @@ cudaError_t launch_score_topk(int B, int Hq, int Hkv, const uint32_t *q_codes, c
                               const int32_t *k_per_seq, int k_uniform, int max_seq_len, int k_max,
                               int32_t *idx, long long idx_sb, long long idx_sh, int32_t *count,
                               int32_t *hist_out, int32_t *ws_hist, unsigned char *ws_scores, cudaStream_t st, Windows win,
-                              CodePages cp, int row_shift) {
+                              CodePages cp, int row_shift, bool in_step) {
     if (row_shift >= 0) {   // one unit per query head: groups of one head over Hq unit heads
         return launch_g<1>(B, Hq, Hq, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, idx, idx_sb,
-                           idx_sh, count, hist_out, ws_hist, ws_scores, st, win, cp, row_shift);
+                           idx_sh, count, hist_out, ws_hist, ws_scores, st, win, cp, row_shift, in_step);
     }
 #define HA_ARGS B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, idx, \
-                idx_sb, idx_sh, count, hist_out, ws_hist, ws_scores, st, win, cp, -1
+                idx_sb, idx_sh, count, hist_out, ws_hist, ws_scores, st, win, cp, -1, in_step
     switch (Hq / Hkv) {
         case 1: return launch_g<1>(HA_ARGS);
         case 2: return launch_g<2>(HA_ARGS);

@@ -121,3 +121,32 @@ def _run(c, append, scan):
 @pytest.mark.parametrize("bits", [64, 256])
 def test_a_wide_signature_written_directly_in_front_of_its_selection(B, n, bits):
     _run(_Calls(B, 4, n, bits=bits), "encode", "wide")
+
+
+# the kernel in front: lets the kernels behind it start at once and writes its buffer some 20 us later
+LATE_COPY = """
+extern "C" __global__ void late_copy(const int *src, int *dst, int n) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    for (int i = 0; i < 20; ++i) __nanosleep(1000);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) dst[i] = src[i];
+}"""
+
+
+@pytest.mark.parametrize("B,n", [(2, 20000), (20, 3001), (1, 100003), (1, 262147)])
+@pytest.mark.parametrize("scan", ["topk", "step"])
+def test_a_block_table_is_read_behind_whatever_writes_it(B, n, scan):
+    """The table names other pages of the same pool until the kernel in front has written it."""
+    c = _Calls(B, 4, n, paged=True)
+    late_copy = torch.cuda._compile_kernel(LATE_COPY, "late_copy")
+    table = c.table
+    slot = torch.full((B,), n // 2, dtype=torch.int32, device=DEV)
+    c.reset(slot)
+    c.append("encode", slot)
+    c.table = torch.empty_like(table)
+    for _ in range(3):
+        c.table.copy_(table.roll(1, 1))
+        torch.cuda.synchronize()
+        late_copy(grid=(1, 1, 1), block=(1024, 1, 1), args=[table, c.table, table.numel()])
+        c.scan(scan)
+        c.check(slot)
+    assert ha.ha_read_device_status(c.ws) == 0
