@@ -20,15 +20,15 @@
  *     256-byte aligned, prepared once with ha_workspace_init.  Calls that share a workspace must
  *     be ordered on one stream.
  *   - Kernels are launched with programmatic stream serialization: a kernel may start while its
- *     predecessor in the stream is finishing, and reads seq_lens, k_per_seq and the key signatures
- *     before it waits for that predecessor.  This is safe behind ordinary kernels and copies (they
- *     complete before anything of this library starts) and between calls of this library: the only
- *     signatures a library kernel directly in front may still be writing are those of the appended
- *     tokens, i.e. slot seq_len-1 (ha_encode with slot[b] = seq_len[b]-1, or this step's own k_new)
- *     and slot seq_len-2 (a layer-step on the same cache for a sequence one token shorter), and every
- *     scanning kernel reads these again after its wait.  A caller whose own preceding kernel both
- *     writes those arrays AND releases its dependents early (griddepcontrol.launch_dependents) must
- *     release them only after the writes.
+ *     predecessor in the stream is finishing, and before it waits for that predecessor it reads the
+ *     mapping networks, seq_lens, k_per_seq and key signatures that lie in a contiguous 32-bit cache
+ *     (not block tables, paged or wide signatures, query signatures, q, K, V or index lists, except
+ *     behind a kernel of the same call that has waited).  This is safe behind ordinary kernels and
+ *     copies (they complete before anything of this library starts) and between calls of this
+ *     library, at any slots and lengths: a kernel that writes signatures lets the kernels behind it
+ *     start when they are written, or the kernels that read them early read those again.  A caller
+ *     whose own preceding kernel both writes those arrays AND releases its dependents early
+ *     (griddepcontrol.launch_dependents) must release them only after the writes.
  *   - seq_lens[b] <= max_seq_len (where a call takes max_seq_len) and seq_lens[b] <= the number of
  *     token slots of K, V and k_codes are the caller's promise.  SCORE + TOPK clamps a longer
  *     sequence to max_seq_len; the append of the host-buffer entries and GATHER-ATT do not clamp.

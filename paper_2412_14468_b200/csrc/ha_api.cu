@@ -345,6 +345,7 @@ static int sparse_decode_impl(const ha_shape *shape, const ha_mapping *map_q, co
     jq.n_heads = Hq; jq.heads_per_kv = Hq / Hkv; jq.n_cta = B * Hkv;
     jq.n_out = kBits;
     jq.map = view(map_q);
+    jq.release_early = 1;
     EncodeJob jk{};
     if (k_new) {
         jk.x = k_new; jk.x_sb = (long long)Hkv * kD; jk.x_sh = kD;
@@ -354,6 +355,7 @@ static int sparse_decode_impl(const ha_shape *shape, const ha_mapping *map_q, co
         jk.n_out = kBits;
         jk.map = view(map_k);
         jk.pages = code_pages;
+        jk.release_early = 1;
     }
     HA_CUDA(launch_encode_vectors(jq, jk, st));
     if (pipelined) {
@@ -377,7 +379,7 @@ static int sparse_decode_impl(const ha_shape *shape, const ha_mapping *map_q, co
         // up to a cluster per unit resident at once and short lists: GATHER-ATT with the states merged in shared memory
         HA_CUDA(launch_gather_cluster(B, Hq, Hkv, shape->sm_scale, q, view(K), view(V), seq_lens, idx, idx_stride_b,
                                       idx_stride_h, count, k_max, out, lse, ws_ptr<uint32_t>(workspace, 0), st, block_table,
-                                      bt_stride_b, page_shift));
+                                      bt_stride_b, page_shift, 0, /*in_step=*/true));
         return HA_OK;
     }
     HA_CUDA(launch_attention(true, B, Hq, Hkv, shape->sm_scale, q, view(K), view(V), seq_lens, idx, idx_stride_b,
@@ -693,6 +695,7 @@ int ha_encode_wide(const ha_mapping *map, int32_t heads_per_kv, const ha_tensor 
         a.n_heads = n_heads; a.heads_per_kv = heads_per_kv; a.n_cta = batch * (n_heads / heads_per_kv);
         a.n_out = map->n_bits;
         a.map = view(map);
+        a.release_early = 1;   // the wide selection reads no signature before its launch wait
         EncodeJob none{};
         HA_CUDA(launch_encode_vectors(a, none, (cudaStream_t)stream));
         return HA_OK;

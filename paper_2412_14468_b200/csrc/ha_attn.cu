@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_kernel(const AttnArgs a)
     // programmatic-launch wait.  Inside a whole layer-step the list LENGTHS are min(k, n) by
     // construction, so the work distribution is computed before the wait, from inputs that no kernel
     // of the step writes; a stand-alone call reads the caller's count array instead, after the wait.
-    pdl_launch_dependents();
+    if (!a.count_from_k) pdl_launch_dependents();
     const bool early = kGather ? (a.count_from_k != 0) : true;
     if (!early) pdl_wait();
 
@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_kernel(const AttnArgs a)
         x_end = (unit_count(u) + kBlockTokens - 1) / kBlockTokens;
     }
     if (early) pdl_wait();   // nothing is written, and nothing of the preceding kernels read, before this point
+    if (a.count_from_k) pdl_launch_dependents();   // a step's ENCODE, which released its SCORE early, has ended by now
     if (a.balanced) {
         for (int v = cta; v < a.n_units; v += P)
             if (s_pref[v + 1] == s_pref[v]) write_empty(v);

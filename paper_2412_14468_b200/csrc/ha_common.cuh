@@ -79,7 +79,13 @@ inline int chunk_tokens_for(int n_units, int max_seq_len, int n_sm) {
 
 // ---- programmatic dependent launch: a kernel launched with launch_pdl may start while its
 // predecessor in the stream is still running; everything it reads from, or writes over, earlier
-// work must come after pdl_wait().
+// work must come after pdl_wait().  Three rules make the exceptions sound:
+//  * before the wait only mapping networks, sequence lengths, budgets and contiguous 32-bit signatures are read (inside a
+//    layer-step, behind its ENCODE, paged ones and the block table too);
+//  * a kernel that writes signatures releases its dependents when they are written.  The ENCODE of a layer-step releases
+//    early: its SCORE reads the appended token again, and GATHER-ATT releases the next call behind its own wait.
+//    ha_encode_wide does too: the wide selection reads no signature before its wait;
+//  * at least one CTA of every grid waits, so that a wait reaches back through everything older in the stream.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -163,6 +169,7 @@ struct EncodeJob {
     int n_out, out_blocks;   // outputs of the last layer (bits of a signature) and, set by the launcher, the CTAs that share them
     MapView map;
     CodePages pages;         // pages.table != NULL: `codes` is a paged pool and the slot a token of the sequence
+    int release_early;       // 1: the kernels behind start before the signatures are written
 };
 #ifdef __CUDACC__
 // where the signature of (sequence b, head h, token slot) is stored
@@ -253,7 +260,7 @@ cudaError_t launch_gather_cluster(int B, int Hq, int Hkv, float sm_scale, const 
                                   const int32_t *seq_lens, const int32_t *idx, long long idx_sb, long long idx_sh,
                                   const int32_t *count, int k_max, uint16_t *out, float *lse, uint32_t *status,
                                   cudaStream_t st, const int32_t *block_table = nullptr, long long bt_sb = 0,
-                                  int page_shift = 0, int kv_shift = 0);   // kv_shift as in launch_attention
+                                  int page_shift = 0, int kv_shift = 0, bool in_step = false);   // kv_shift as in launch_attention
 
 // Signatures of 64 .. 512 bits through ENCODE and SCORE + TOPK (packed 64-bit words; strides in words).
 cudaError_t launch_encode_wide(const MapView &map, int n_bits, int heads_per_kv, TensorView x, int B, int H, int T,

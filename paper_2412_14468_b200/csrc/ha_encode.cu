@@ -81,9 +81,12 @@ __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, E
     const float bias3 = J.map.b3 ? __ldg(J.map.b3 + net * ld3 + blk * kOut + (tid & (kOut - 1))) : 0.0f;
     // The weights do not depend on earlier kernels of the stream; the vectors to encode may.  The
     // kernels behind this one are released only after the wait: whatever they read before their own
-    // wait (sequence lengths, budgets, signatures) is then final, whoever wrote it earlier in the stream.
+    // wait (sequence lengths, budgets, signatures) is then final, whoever wrote it earlier in the stream.  Of this kernel's own
+    // signatures that holds inside a layer-step (q_codes are read after the wait and slot n-1 again after it) and for wide ones;
+    // any other call may write any slot, and its dependents start when the CTAs have ended.  (Lists per query head, 2 sequences
+    // of 32768: 26.8 us per step against 27.1 with an early release, whose parked CTAs share the SMs of ENCODE.)
     pdl_wait();
-    pdl_launch_dependents();
+    if (J.release_early) pdl_launch_dependents();
 
     // wait for one weight matrix; if the bulk copy never reports completion, load it the ordinary way
     // (the decision is taken by the whole CTA together, so that the barrier below is never divergent)
@@ -252,7 +255,7 @@ __global__ void __launch_bounds__(64 * NG) encode_tile_kernel(EncodeJob ja, Enco
         b2[e] = J.map.b2 ? __ldg(J.map.b2 + net * kHid + 2 * op + e) : 0.0f;
     }
     pdl_wait();                 // the vectors may come from the kernel in front; the weights do not
-    pdl_launch_dependents();
+    if (J.release_early) pdl_launch_dependents();
 
     // the tile's vectors -> fp32 rows (slots past the batch are zero rows; their signatures are dropped)
     for (int e = tid; e < TV * (kD / 8); e += kTileThreads) {

@@ -87,7 +87,8 @@ struct FusedArgs {
     const uint16_t *v_new;
     uint32_t *status;   // stand-alone cluster gather: device status word (HA_DEV_BAD_INDEX)
     CodePages code_pages;   // table != NULL: k_codes is a paged pool
-    int kv_shift;       // stand-alone cluster gather: unit head h reads K/V head h >> kv_shift (lists per query head)
+    int kv_shift;       // cluster gather: unit head h reads K/V head h >> kv_shift (lists per query head)
+    int in_step;        // cluster gather: the third kernel of a layer-step
 };
 
 __device__ __forceinline__ void st_dsmem_u32(uint32_t *local, uint32_t rank, uint32_t v) {
@@ -107,11 +108,11 @@ __device__ __forceinline__ void st_dsmem_f32(float *local, uint32_t rank, float 
 // call; the barrier that publishes the input vectors also publishes them.  Signature v is written to
 // word v of `dst` in the shared memory of EVERY CTA of the cluster (lanes 0..CS-1 of the warp that holds it
 // store to CTAs 0..CS-1; the cluster barrier that follows makes the stores visible).
-// kRaw: thread o already holds component o of every vector in xr (fetched earlier).
+// kRaw: thread o already holds component o of every vector in xr (fetched earlier).  Returns signature v in warp v.
 template <int NV, int CS, bool kRaw = false>
-__device__ __forceinline__ void fused_encode(const uint16_t *x0, long long x_stride, const uint16_t *sw1,
-                                             const uint16_t *sw2, const uint16_t *sw3, float *actA, float *actB,
-                                             uint32_t *dst, float bias1, float bias2, float bias3, const uint16_t *xr = nullptr) {
+__device__ __forceinline__ uint32_t fused_encode(const uint16_t *x0, long long x_stride, const uint16_t *sw1,
+                                                 const uint16_t *sw2, const uint16_t *sw3, float *actA, float *actB,
+                                                 uint32_t *dst, float bias1, float bias2, float bias3, const uint16_t *xr = nullptr) {
     const int tid = threadIdx.x, o = tid & 127;
     const bool active = tid < 128;
     if (active) {
@@ -143,8 +144,10 @@ __device__ __forceinline__ void fused_encode(const uint16_t *x0, long long x_str
             vec_layer_t<1>(actA + v * kD, sw3, lane, z3);
             const uint32_t code = __ballot_sync(0xffffffffu, z3[0] > 0.0f);
             if (lane < CS) st_dsmem_u32(dst + v, (uint32_t)lane, code);
+            return code;
         }
     }
+    return 0u;
 }
 
 // GATHER-ATT over this CTA's share of a unit's index list, blocks [blk_lo, blk_hi) of 16 entries, and the merge
@@ -428,7 +431,7 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     for (int i = tid; i < kBins * 32 / 4; i += kFusedThreads)
         reinterpret_cast<uint4 *>(&c_hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
     if (!kHost) pdl_wait();      // q, k_new and everything older in the stream is final from here on
-    pdl_launch_dependents();
+    if (!enc_k) pdl_launch_dependents();   // the CTA of the appended key: further down, when its signature is written
     if (codes_paged) {           // the block table may come from the kernel in front
         if (kXFirst && tid < kD) {
             if (enc_q) {
@@ -451,27 +454,27 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
     }
 
     // ---------------- P1: ENCODE in the first kQCtas CTAs (queries) and the next one (appended key)
+    uint32_t new_code = 0u;   // warp 0 of the CTA of the appended key
     if (enc_q) {
         fused_encode<kQPer, CS, kXFirst>(a.q + (head0 + kQPer * (int)rank) * kD, kD, sw1, sw2, sw3, actA, actB,
                                          s_codes + kQPer * (int)rank, bias1, bias2, bias3, x_raw);
     } else if (enc_k) {
-        fused_encode<1, CS, kXFirst>(a.k_new + ((long long)b * Hkv + kvh) * kD, kD, sw1, sw2, sw3, actA, actB, s_codes + G,
+        new_code = fused_encode<1, CS, kXFirst>(a.k_new + ((long long)b * Hkv + kvh) * kD, kD, sw1, sw2, sw3, actA, actB, s_codes + G,
                                    bias1, bias2, bias3, x_raw);
     }
-    cluster_sync_all();   // #1: every CTA holds all signatures (and its counters are zeroed)
-    // the signatures also go to global memory (outputs of the step; nobody in this kernel reads them there):
-    // stored after the barrier, so that its release had nothing but shared-memory stores to wait for
+    cluster_arrive();     // #1: every CTA holds all signatures (and its counters are zeroed)
+    // the signatures also go to global memory (outputs of the step; nobody in this kernel reads them there), behind the release
+    // of the barrier, which then had nothing but shared-memory stores to wait for
+    if (enc_k && tid == 0) *code_slot(n - 1) = new_code;
+    __syncwarp();
+    cluster_wait();
     if (enc_q && tid < kQPer) a.q_codes[head0 + kQPer * (int)rank + tid] = s_codes[kQPer * (int)rank + tid];
-    if (enc_k && tid == 0) *code_slot(n - 1) = s_codes[G];
     if (kHost && tid < G * 16) reinterpret_cast<uint4 *>(actA)[tid] = q_stage;   // the activations are dead
     uint32_t qc[G];
 #pragma unroll
     for (int j = 0; j < G; ++j) qc[j] = s_codes[j];
     if (!kPreload && !codes_paged) load_signatures();
-    // Signatures that the early request may have seen in a stale state: slot n-1 (this step's appended token:
-    // encoded above, or, when the step has no k_new, possibly written by an ha_encode call directly in front)
-    // and slot n-2 (appended by a layer-step on the same cache directly in front, whose kernel lets this one
-    // start before it has stored its signature).  Everything older was complete before this kernel started.
+    // slot n-1 is this step's appended token, encoded above
     auto replace_slot = [&](int t, uint32_t kc) {
 #pragma unroll
         for (int p = 0; p < kL; ++p) {
@@ -482,11 +485,6 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
         }
     };
     if (has_new_key) replace_slot(n - 1, s_codes[G]);
-    if (kPreload && !codes_paged) {
-        const int lo = wbase, hi = wbase + 4 * Lb;   // this lane's tokens (contiguous)
-        if (!has_new_key && n - 1 >= lo && n - 1 < hi) replace_slot(n - 1, __ldcg(code_slot(n - 1)));
-        if (n - 2 >= lo && n - 2 < hi) replace_slot(n - 2, __ldcg(code_slot(n - 2)));
-    }
 
     // ---------------- P2: SCORE, histogram, threshold, compaction
     uint32_t sc[kL];
@@ -541,7 +539,16 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
         st_dsmem_u32(reinterpret_cast<uint32_t *>(&s_all[rank][lane]), (uint32_t)warp, s_hist[lane]);
         if (lane == 0) st_dsmem_u32(reinterpret_cast<uint32_t *>(&s_all[rank][32]), (uint32_t)warp, s_hist[32]);
     }
-    cluster_sync_all();   // #2: every CTA holds all histograms of the cluster
+    cluster_arrive();     // #2: every CTA holds all histograms of the cluster
+    // Kernels behind this one may read signatures before their own launch wait: the CTA that appended one releases them here,
+    // where its store has long arrived and the fence fits under the barrier (one sequence of 32768 tokens 11.03 us per step;
+    // right behind the store 11.35, in front of barrier #3 11.04 but five ragged sequences 18.6 against 18.3).
+    if (enc_k && tid == 0) {
+        __threadfence();
+        pdl_launch_dependents();
+    }
+    __syncwarp();
+    cluster_wait();
     // every warp derives the threshold for itself (lane l owns level l, level 32 is read by every lane)
     int T, r, gt_before, eq_before;
     {
@@ -663,8 +670,9 @@ __global__ void __launch_bounds__(kFusedThreads, 2) gather_cluster_kernel(const 
     const uint32_t rank = cluster_rank();
     const int kvh = blockIdx.y, b = blockIdx.z;
     const long long head0 = (long long)b * a.Hq + (long long)kvh * G;
-    pdl_launch_dependents();
+    if (!a.in_step) pdl_launch_dependents();
     pdl_wait();   // the list, its length and the rows may come from the kernels in front
+    if (a.in_step) pdl_launch_dependents();   // the step's ENCODE, which released its SCORE early, has ended by now
     cluster_wait();
     const int n = a.seq_lens[b];
     const int keep = max(0, min(a.count[b * a.Hkv + kvh], a.k_max));
@@ -773,9 +781,9 @@ static cudaError_t launch_gather_cluster_g(const FusedArgs &args, int B, cudaStr
 cudaError_t launch_gather_cluster(int B, int Hq, int Hkv, float sm_scale, const uint16_t *q, TensorView K, TensorView V,
                                   const int32_t *seq_lens, const int32_t *idx, long long idx_sb, long long idx_sh,
                                   const int32_t *count, int k_max, uint16_t *out, float *lse, uint32_t *status,
-                                  cudaStream_t st, const int32_t *block_table, long long bt_sb, int page_shift, int kv_shift) {
+                                  cudaStream_t st, const int32_t *block_table, long long bt_sb, int page_shift, int kv_shift, bool in_step) {
     FusedArgs a{};
-    a.kv_shift = kv_shift;
+    a.kv_shift = kv_shift; a.in_step = in_step ? 1 : 0;
     a.block_table = block_table; a.bt_sb = bt_sb; a.page_shift = page_shift;
     a.page_rows = (block_table && K.sn > 0) ? (int)(K.sb / K.sn) : 0;
     a.q = q; a.K = K; a.V = V; a.seq_lens = seq_lens; a.k_max = k_max; a.Hq = Hq; a.Hkv = Hkv;

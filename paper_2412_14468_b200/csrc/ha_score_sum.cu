@@ -93,8 +93,7 @@ __device__ __forceinline__ void sum_scores_of(const uint4 (&v)[LD], int base, in
     }
 }
 
-// kEarly: before the programmatic-launch wait (through L1: the appended token is read again afterwards); later loads go past
-// L1, which may hold a line of such an early load.
+// kEarly: before the programmatic-launch wait, through L1; later loads go to L2, where the kernels in front left the signatures.
 template <int LD, bool kEdge, bool kEarly>
 __device__ __forceinline__ void sum_load_tile(const uint32_t *row, int base, int lane, int hi, uint4 (&v)[LD]) {
 #pragma unroll
@@ -145,8 +144,7 @@ __global__ void __launch_bounds__(kSumThreads, LD <= 2 ? 5 : 3) score_sum_select
     const int plain_end = min(wb.local_begin, hi);      // warp tiles inside [sink_end, plain_end) need no per-token checks
     auto is_edge = [&](int base) { return base < wb.sink_end || base + kWarpTokens > plain_end; };
 
-    // the first tile is requested before the launch wait; what a library kernel directly in front may still have been writing
-    // (slots n-1 and n-2) is read again after it
+    // the first tile is requested before the launch wait: every kernel that writes signatures lets this one start behind them
     uint4 v[LD], nx[LD];
     if (n_tiles > 0) {
         const int base = lo + warp * kWarpTokens;
@@ -156,16 +154,6 @@ __global__ void __launch_bounds__(kSumThreads, LD <= 2 ? 5 : 3) score_sum_select
     for (int i = tid; i < NB * 8; i += kSumThreads) reinterpret_cast<uint4 *>(&c_hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
     pdl_launch_dependents();
     pdl_wait();
-    if (n_tiles > 0) {
-#pragma unroll
-        for (int j = 0; j < LD; ++j) {
-            const int t = lo + warp * kWarpTokens + j * 128 + 4 * lane;
-            if (t < hi) {
-                patch_token(v[j], t, n - 1, row);
-                patch_token(v[j], t, n - 2, row);
-            }
-        }
-    }
     SumPlanes<G> pl;
     {
         uint32_t q[G];

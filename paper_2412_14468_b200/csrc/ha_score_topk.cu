@@ -12,9 +12,10 @@
 //    one score byte per token passed through the workspace (scan_score_kernel, select_kernel).
 // No CTA ever spins on another: hand-offs are hardware cluster barriers or kernel boundaries.
 // The scanning kernels request their first signatures before the programmatic-launch wait, so that
-// the fetch overlaps the tail of the preceding kernel; the one signature that the preceding ENCODE
-// may still be writing (the appended token, slot n-1) is re-read after the wait.  A block table is
-// read before the wait only inside a layer-step (in_step), where ENCODE has waited for whatever wrote it.
+// the fetch overlaps the tail of the preceding kernel.  Every kernel that writes signatures lets its
+// dependents start behind them, except the ENCODE of a layer-step (in_step): its one signature (the
+// appended token, slot n-1) is re-read after the wait.  A block table is read before the wait only
+// inside a layer-step, where ENCODE has waited for whatever wrote it.
 #include "ha_score_dev.cuh"
 
 namespace ha {
@@ -58,7 +59,10 @@ __global__ void __launch_bounds__(kScanThreads) scan_score_kernel(const uint32_t
     const int32_t *table_b = paged ? cp.table + (long long)b * cp.bt_sb : nullptr;
     const int n = min(seq_lens[b], max_seq_len);
     const int start = chunk * chunk_tokens;
-    if (start >= n) return;
+    if (start >= n) {
+        if (chunk == 0) pdl_wait();   // at least one CTA of a grid waits, also when every sequence is empty
+        return;
+    }
     if (paged && !in_step) pdl_wait();   // a block table may come from the kernel in front
     const int tid = threadIdx.x, lane = tid & 31;
     // contiguous cache: the unit's row; paged cache: the pool from this head's offset on
@@ -106,13 +110,8 @@ __global__ void __launch_bounds__(kScanThreads) scan_score_kernel(const uint32_t
         for (int j = 0; j < 4; ++j) {
             const int base = pass + j * 1024 + tid * 4;
             if (base < end) {
-                if (paged) {
-                    patch_token_paged(cur[j], base, n - 1, cp, row, table_b);
-                    patch_token_paged(cur[j], base, n - 2, cp, row, table_b);
-                } else {
-                    patch_token(cur[j], base, n - 1, row);   // the appended token may just have been written,
-                    patch_token(cur[j], base, n - 2, row);   // and the one before it by a layer-step directly in front
-                }
+                if (paged) patch_token_paged(cur[j], base, n - 1, cp, row, table_b);   // the step's ENCODE may just have written it
+                else patch_token(cur[j], base, n - 1, row);
                 const int h0 = hamming(cur[j].x), h1 = hamming(cur[j].y), h2 = hamming(cur[j].z), h3 = hamming(cur[j].w);
                 // bytes 33 - h = score + 1 (0 = no token); no byte borrows because h <= 32
                 uint32_t s4 = 0x21212121u - ((uint32_t)h0 | ((uint32_t)h1 << 8) | ((uint32_t)h2 << 16) | ((uint32_t)h3 << 24));
@@ -380,21 +379,19 @@ __global__ void __launch_bounds__(kThreads, kThreads > 256 ? 2 : kPaged ? 5 : 6)
     if (tid < kBins + 3) s_hist[tid] = 0;
     pdl_launch_dependents();
     pdl_wait();
-    // the signatures that a library kernel directly in front may just have written (slot n-1 by ENCODE, slot n-2
-    // by a layer-step for the sequence one token shorter): re-read by the one lane that holds them
-#pragma unroll
-    for (int back = 1; back <= 2; ++back) {
-        const int e_last = (n - back) - wb;
+    // the signature that the ENCODE of a layer-step may just have written (slot n-1): re-read by the one lane that holds it
+    {
+        const int e_last = (n - 1) - wb;
         if (e_last >= 0 && e_last < 512 && e_last < 256 * Rb && ((e_last & 255) >> 3) == lane) {
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
                 const int t = wb + j * 256 + lane * 8;
                 if (kPaged) {
-                    patch_token_paged(c[2 * j], t, n - back, cp, row, table_b);
-                    patch_token_paged(c[2 * j + 1], t + 4, n - back, cp, row, table_b);
+                    patch_token_paged(c[2 * j], t, n - 1, cp, row, table_b);
+                    patch_token_paged(c[2 * j + 1], t + 4, n - 1, cp, row, table_b);
                 } else {
-                    patch_token(c[2 * j], t, n - back, row);
-                    patch_token(c[2 * j + 1], t + 4, n - back, row);
+                    patch_token(c[2 * j], t, n - 1, row);
+                    patch_token(c[2 * j + 1], t + 4, n - 1, row);
                 }
             }
         }

@@ -117,6 +117,21 @@ def _run(c, append, scan):
     assert ha.ha_read_device_status(c.ws) == 0
 
 
+# few units (one-launch step, large clusters), many units (three launches), a sequence beyond the cluster kernels
+@pytest.mark.parametrize("B,n", [(2, 20000), (20, 3001), (1, 262147)])
+@pytest.mark.parametrize("scan", ["topk", "sum", "per_head", "step"])
+@pytest.mark.parametrize("append", ["encode", "step"])
+def test_a_signature_written_directly_in_front_of_a_scan(B, n, scan, append):
+    _run(_Calls(B, 4, n), append, scan)
+
+
+@pytest.mark.parametrize("B,n", [(2, 20000), (20, 3001), (1, 262147)])
+@pytest.mark.parametrize("scan", ["topk", "step"])
+@pytest.mark.parametrize("append", ["encode", "step"])
+def test_a_signature_written_into_a_page_directly_in_front_of_a_scan(B, n, scan, append):
+    _run(_Calls(B, 4, n, paged=True), append, scan)
+
+
 @pytest.mark.parametrize("B,n", [(2, 20000), (20, 3001), (1, 140001)])
 @pytest.mark.parametrize("bits", [64, 256])
 def test_a_wide_signature_written_directly_in_front_of_its_selection(B, n, bits):
@@ -150,3 +165,20 @@ def test_a_block_table_is_read_behind_whatever_writes_it(B, n, scan):
         c.scan(scan)
         c.check(slot)
     assert ha.ha_read_device_status(c.ws) == 0
+
+
+@pytest.mark.parametrize("n", [20000, 262147])
+def test_a_call_of_empty_sequences_between_the_two(n):
+    """A grid in which no CTA has work still waits for the kernels in front of it."""
+    c = _Calls(2, 4, n)
+    empty = torch.zeros_like(c.lens)
+    idx, cnt = torch.zeros_like(c.idx), torch.zeros_like(c.cnt)
+    for r in range(REPEATS):
+        slot = torch.full((2,), 977 * r, dtype=torch.int32, device=DEV)
+        c.reset(slot)
+        torch.cuda.synchronize()
+        c.append("step", slot)
+        ha.ha_score_topk(c.shape, c.q_codes, c.codes, empty, None, K, n, K, idx, cnt, c.ws)
+        c.scan("topk")
+        c.check(slot)
+    assert (cnt == 0).all()
