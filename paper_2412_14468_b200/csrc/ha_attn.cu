@@ -53,7 +53,13 @@ struct AttnArgs {
     float *lse;
 };
 
-template <int G, bool kGather, int kStages>
+// kManyParts: 24 parts per pass of the merge instead of 16; 238 registers instead of 185 with groups of 4 (250 / 214 with 8).
+// At 185 the next step's ENCODE finds room beside two CTAs while this kernel runs; at 238 it does not.  Parts pass through the
+// merge only where a unit is cut over CTAs, so 24 is for grids of more than 16 CTAs per unit (one sequence of 524288 tokens, 37
+// parts: 42.6 against 43.0 us per step) and, for the registers alone, for grids that take whole units and cut none (64
+// sequences of 32768: 92.0 / 92.8).  The others cut units into a few parts and gain by the early ENCODE (32 ragged sequences of
+// up to 131072 tokens 114.2 / 114.5, 24 in pages 59.6 / 60.1).
+template <int G, bool kGather, int kStages, bool kManyParts>
 __global__ void __launch_bounds__(kAttnThreads, 2) attn_kernel(const AttnArgs a) {
     constexpr int kWarpRingBytes = kStages * kStageBytes, kAttnSmemBytes = attn_smem_bytes(kStages);
     extern __shared__ __align__(128) unsigned char ring[];   // kAttnWarps private rings, then the block prefix
@@ -326,14 +332,15 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_kernel(const AttnArgs a)
             if (finalize) {
                 __threadfence();
                 // Merge of the parts: thread (dq, pg) owns dimensions 4dq..4dq+3 and the parts pg, pg+4, ...;
-                // a pass covers 24 (12 when G = 8) parts with every load issued before the first use (one L2 round trip),
+                // a pass covers 16 parts, 24 with kManyParts (G = 8: 8, 12), with every load issued before the first use (one
+                // L2 round trip),
                 // then the four part groups are folded through shared memory.
                 const int dq = tid & 31, pg = tid >> 5;
                 float Mt[G], Lt[G];
                 float4 At[G];
 #pragma unroll
                 for (int j = 0; j < G; ++j) { Mt[j] = -CUDART_INF_F; Lt[j] = 0.0f; At[j] = make_float4(0.f, 0.f, 0.f, 0.f); }
-                constexpr int kEB = (G >= 8) ? 3 : 6;   // loads in flight per head and thread
+                constexpr int kEB = kManyParts ? ((G >= 8) ? 3 : 6) : ((G >= 8) ? 2 : 4);   // loads in flight per head and thread
                 for (int part0 = 0; part0 < n_parts; part0 += 4 * kEB) {
                     float4 av[G][kEB];
                     float mv[G][kEB], lv[G][kEB];
@@ -418,18 +425,18 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_kernel(const AttnArgs a)
     if (bad) atomicOr(a.status, HA_DEV_BAD_INDEX);
 }
 
-template <int G, bool kGather, int kStages>
+template <int G, bool kGather, int kStages, bool kManyParts>
 static cudaError_t launch_attn_t(const AttnArgs &args, int grid, size_t smem, cudaStream_t st) {
     static bool done[64] = {};   // opt in to the ring's shared memory once per device
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev >= 0 && dev < 64 && !done[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(attn_kernel<G, kGather, kStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaError_t e = cudaFuncSetAttribute(attn_kernel<G, kGather, kStages, kManyParts>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              attn_smem_bytes(kStages) + (kMaxBalancedUnits + 1) * 4);
         if (e != cudaSuccess) return e;
         done[dev] = true;
     }
-    cudaError_t e = launch_pdl(attn_kernel<G, kGather, kStages>, dim3(grid), dim3(kAttnThreads), smem, st, args);
+    cudaError_t e = launch_pdl(attn_kernel<G, kGather, kStages, kManyParts>, dim3(grid), dim3(kAttnThreads), smem, st, args);
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
@@ -441,6 +448,7 @@ static cudaError_t launch_attn_g(bool gather, const AttnArgs &args_in, cudaStrea
     const long long blocks_per_unit = (args.max_items + kBlockTokens - 1) / kBlockTokens;
     const long long t_max = blocks_per_unit * args.n_units;
     int grid;
+    bool many_parts = true;
     const bool two_stages = gather && args.max_items <= kShortList;
     size_t smem = attn_smem_bytes(two_stages ? 2 : 3);
     if (args.n_units <= kMaxBalancedUnits) {
@@ -459,13 +467,16 @@ static cudaError_t launch_attn_g(bool gather, const AttnArgs &args_in, cudaStrea
             const int m = (args.n_units + grid - 1) / grid;
             if (args.n_units % m == 0 && (long long)(args.n_units / m) * 5 >= (long long)grid * 4) grid = args.n_units / m;
         }
+        many_parts = grid > 16 * args.n_units || args.n_units % grid == 0;
         smem += (size_t)(args.n_units + 1) * 4;
     } else {
         args.balanced = 0;
         grid = args.n_units;
     }
-    if (two_stages) return launch_attn_t<G, true, 2>(args, grid, smem, st);
-    return gather ? launch_attn_t<G, true, 3>(args, grid, smem, st) : launch_attn_t<G, false, 3>(args, grid, smem, st);
+#define HA_ATTN(GATHER, STAGES) (many_parts ? launch_attn_t<G, GATHER, STAGES, true>(args, grid, smem, st) : launch_attn_t<G, GATHER, STAGES, false>(args, grid, smem, st))
+    if (two_stages) return HA_ATTN(true, 2);
+    return gather ? HA_ATTN(true, 3) : HA_ATTN(false, 3);
+#undef HA_ATTN
 }
 
 cudaError_t launch_attention(bool gather, int B, int Hq, int Hkv, float sm_scale, const uint16_t *q,

@@ -213,3 +213,14 @@ def test_gather_attn_at_the_longest_list_of_clusters_of_four(k):
     lists = rng.integers(0, n, size=(B, Hkv, k)).astype(np.int32)
     cnt = np.where(np.arange(B * Hkv).reshape(B, Hkv) % 3 == 0, k, rng.integers(0, k, size=(B, Hkv))).astype(np.int32)
     _check_gather(*_attn_inputs(B, Hkv * G, Hkv, n, 6), [n] * B, lists, cnt, 0.09)
+
+
+@pytest.mark.parametrize("B,G", [(1, 8), (17, 4), (18, 4), (17, 8), (18, 8), (17, 1), (300, 1), (592, 2)])
+def test_gather_attn_split_k_merges_of_many_and_of_few_parts(B, G):
+    """One unit cut over every CTA, 17 CTAs per unit (the first grid whose merge takes the wide pass) and 16, units that are cut
+    in two, and whole units per CTA; lists in any order."""
+    n, k = 300, 4200
+    lists = np.random.default_rng(B).integers(0, n, size=(B, 1, k)).astype(np.int32)
+    cnt = np.full((B, 1), k, np.int32)
+    cnt[::3] -= 1001
+    _check_gather(*_attn_inputs(B, G, 1, n, 6), [n] * B, lists, cnt, 0.09)
