@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kVecThreads) encode_vec_kernel(EncodeJob ja, E
     // wait for one weight matrix; if the bulk copy never reports completion, load it the ordinary way
     // (the decision is taken by the whole CTA together, so that the barrier below is never divergent)
     auto weights_ready = [&](int which, uint16_t *dst, const uint16_t *src, int width, int ld) {
-        const bool ok = mbar_wait_bounded(bar0 + 8 * which);
+        const bool ok = mbar_wait_bounded<0>(bar0 + 8 * which);
         if (__syncthreads_or(!ok)) {
             const int per_row = width / 8;
             for (int c = tid; c < kHid * per_row; c += kVecThreads)

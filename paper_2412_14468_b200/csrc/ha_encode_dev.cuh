@@ -25,10 +25,13 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait for one phase of an mbarrier; false if it has not completed after the limit (never seen).  test_wait first:
 // try_wait takes some 300 cycles even when the phase is complete (measured; test_wait 40), so it only parks a warp whose
-// barrier is far from ready.
+// barrier is far from ready.  kTests = 0 parks at once: the weights of encode_vec_kernel, whose CTAs share their SMs with a
+// kernel that is still at work (lists per query head 26.2 -> 25.9 us per step, one sequence of 524288 tokens 42.6 -> 42.5;
+// encode_tile_kernel keeps the tests: 64 sequences of 32768 91.9 against 92.1 without).
+template <int kTests = 32>
 __device__ __forceinline__ bool mbar_wait_parity(uint32_t bar, uint32_t parity) {
 #pragma unroll 1
-    for (int it = 0; it < 32; ++it)
+    for (int it = 0; it < kTests; ++it)
         if (mbar_test(bar, parity)) return true;
 #pragma unroll 1
     for (int it = 0; it < (1 << 18); ++it) {
@@ -40,7 +43,8 @@ __device__ __forceinline__ bool mbar_wait_parity(uint32_t bar, uint32_t parity) 
     return false;
 }
 // Phase 0: the arrival of a bulk copy.  A caller that gets false fetches the data with ordinary loads instead.
-__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar) { return mbar_wait_parity(bar, 0u); }
+template <int kTests = 32>
+__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar) { return mbar_wait_parity<kTests>(bar, 0u); }
 
 // z[v] += sum_k hin[v][k] * w[k][o], ascending k, one fmaf per term; the VT chains are independent
 // (vector v starts at hin + v * vstride).
