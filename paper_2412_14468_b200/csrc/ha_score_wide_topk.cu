@@ -511,22 +511,12 @@ __global__ void __launch_bounds__(kWideThreads) wide_select_cluster_kernel(const
 }
 
 template <int W>
-static cudaError_t launch_wide_cluster(const WideArgs &a, int B, int cs, int rows, cudaStream_t st) {
-    const size_t smem = (size_t)rows * kWideSlice * 2 + (size_t)(a.n_bits + 1) * WideShape<W>::kCols * 4;
-    static std::atomic<bool> opted[64];   // opt in to more than 48 KB of shared memory once per device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64 || !opted[dev].load(std::memory_order_acquire)) {
-        cudaError_t e = cudaFuncSetAttribute(wide_select_cluster_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-        if (e != cudaSuccess) return e;
-        if (dev >= 0 && dev < 64) opted[dev].store(true, std::memory_order_release);
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(cs, a.Hkv, B);
+static void wide_cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute (&attr)[2], int Hkv, int B, int cs, int rows, cudaStream_t st) {
+    cfg = cudaLaunchConfig_t{};
+    cfg.gridDim = dim3(cs, Hkv, B);
     cfg.blockDim = dim3(kWideThreads);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = (size_t)rows * kWideSlice * 2 + (size_t)(W * 64 + 1) * WideShape<W>::kCols * 4;
     cfg.stream = st;
-    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cs;
     attr[0].val.clusterDim.y = 1;
@@ -535,7 +525,51 @@ static cudaError_t launch_wide_cluster(const WideArgs &a, int B, int cs, int row
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, wide_select_cluster_kernel<W>, a, rows);
+}
+
+// How many clusters of cs CTAs with `rows` rows of tokens each the device holds at once (0 on error); the answers are kept per
+// device.  Registers set it up to four rows (64, 63, 121, 113 at 64, 128, 256, 512 bits: four CTAs of 256 threads per SM or two),
+// shared memory beyond.
+template <int W>
+static int wide_resident_clusters(int cs, int rows) {
+    static std::atomic<int> known[64][3][kWideMaxRows + 1];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return 0;
+    std::atomic<int> &k = known[dev][cs == 8 ? 2 : cs == 4 ? 1 : 0][rows];
+    int n = k.load(std::memory_order_acquire);
+    if (n > 0) return n;
+    if (cudaFuncSetAttribute(wide_select_cluster_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024) != cudaSuccess) return 0;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    wide_cluster_config<W>(cfg, attr, 1, 64, cs, rows, nullptr);
+    cfg.numAttrs = 1;   // the cluster shape is all the occupancy query looks at
+    if (cudaOccupancyMaxActiveClusters(&n, wide_select_cluster_kernel<W>, &cfg) != cudaSuccess || n <= 0) return 0;
+    k.store(n, std::memory_order_release);
+    return n;
+}
+
+// One cluster per unit: the largest of 8, 4, 2 CTAs of which all units' are resident at once, or two thirds of them where a
+// second wave costs less than smaller clusters (512 bits, bound by its loads; the step from 4 to 2; CTAs of more than six rows,
+// few and long); at least as many as the rows of a CTA hold.  Whole steps of 32768 tokens a sequence, 8 units each, groups of 4, us, with the chosen size and the other:
+//    64, 128 bits   64 units on 8: 36.5 and 42.5, on 4: 42.7 and 53.6;  112 on 4, 128 bits: 60.9, on 2: 85.4;
+//                   152 units on 4 (148 resident): 72.4 and 90.1, on 2: 77.1 and 98.4
+//    256 bits       40 units on 4: 51.8, on 8 (36 resident): 54.9;  80 on 4 (74 resident): 81.3, on 2: 82.6, but 104 88.6 / 83.8
+//    512 bits       40 units on 8: 91.4, on 4: 98.0;  48: 101.5 / 98.1, ragged 87.4 / 96.4;  80 on 4: 163, on 2: 174
+// Sequences of 65536 (eight rows with 4): 128 bits, 80 units on 8: 87.3, on 4: 93.0, ragged 68.8 / 77.4; 256 bits, 40 units 81.7 /
+// 80.4, ragged 66.9 / 76.4; of 40000 (five rows) the other way: 69.3 / 66.9 and 67.4 / 59.7.
+template <int W>
+static cudaError_t launch_wide_cluster(const WideArgs &a, int B, cudaStream_t st) {
+    auto rows_of = [&](int cs) { return max(1, (a.max_seq_len + cs * kWideSlice - 1) / (cs * kWideSlice)); };
+    int cs = 8;
+    while (cs > 2 && rows_of(cs / 2) <= kWideMaxRows &&
+           2LL * B * a.Hkv > (W == 8 || cs == 4 || rows_of(cs / 2) > 6 ? 3LL : 2LL) * wide_resident_clusters<W>(cs, rows_of(cs)))
+        cs >>= 1;
+    if (wide_resident_clusters<W>(cs, rows_of(cs)) <= 0) return cudaErrorInvalidConfiguration;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr[2];
+    wide_cluster_config<W>(cfg, attr, a.Hkv, B, cs, rows_of(cs), st);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, wide_select_cluster_kernel<W>, a, rows_of(cs));
     if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
@@ -573,17 +607,11 @@ cudaError_t launch_score_topk_wide(int B, int Hq, int Hkv, int n_bits, const uin
     a.scores = reinterpret_cast<uint16_t *>(ws + L.off_scores);
     a.score_row = (long long)L.score_row;
     if (max_seq_len <= kWideClusterMaxSeq) {
-        // One cluster per unit: the largest of 8, 4, 2 CTAs whose grid is resident at once (three CTAs per SM), so that few
-        // units get the most CTAs each; at least as many as the rows of a CTA hold.
-        int cs = 8;
-        while (cs > 2 && (long long)B * Hkv * cs > 3LL * sm_count()) cs >>= 1;
-        while (max_seq_len > cs * kWideMaxRows * kWideSlice) cs <<= 1;
-        const int rows = max(1, (max_seq_len + cs * kWideSlice - 1) / (cs * kWideSlice));
         switch (n_bits / 64) {
-            case 1: return launch_wide_cluster<1>(a, B, cs, rows, st);
-            case 2: return launch_wide_cluster<2>(a, B, cs, rows, st);
-            case 4: return launch_wide_cluster<4>(a, B, cs, rows, st);
-            case 8: return launch_wide_cluster<8>(a, B, cs, rows, st);
+            case 1: return launch_wide_cluster<1>(a, B, st);
+            case 2: return launch_wide_cluster<2>(a, B, st);
+            case 4: return launch_wide_cluster<4>(a, B, st);
+            case 8: return launch_wide_cluster<8>(a, B, st);
             default: return cudaErrorInvalidValue;
         }
     }

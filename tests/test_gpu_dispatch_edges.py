@@ -224,3 +224,15 @@ def test_gather_attn_split_k_merges_of_many_and_of_few_parts(B, G):
     cnt = np.full((B, 1), k, np.int32)
     cnt[::3] -= 1001
     _check_gather(*_attn_inputs(B, G, 1, n, 6), [n] * B, lists, cnt, 0.09)
+
+
+@pytest.mark.parametrize("n_bits,B,n", [(64, 37, 2049), (64, 38, 2100), (128, 112, 300), (256, 18, 9000), (256, 19, 9000),
+                                        (512, 27, 4097), (512, 28, 4097), (512, 60, 300), (64, 30, 66000), (512, 2, 131072)])
+def test_score_topk_wide_where_the_cluster_size_changes(n_bits, B, n):
+    """Two units a sequence: as many clusters of 8 or 4 as are resident at once and one more, at few and at eight rows per CTA."""
+    rng = np.random.default_rng(B)
+    W, Hkv = n_bits // 64, 2
+    lens = [n - 7 * (b % 5) for b in range(B)]
+    kc = _wide_codes(rng, B * Hkv * n, W).reshape(B, Hkv, n, W)
+    qc = _wide_codes(rng, B * Hkv, W).reshape(B, Hkv, W)
+    _check_score_topk_wide(n_bits, qc, kc, lens, [max(1, m // 9) for m in lens], Hkv, Hkv, 2, 3)
