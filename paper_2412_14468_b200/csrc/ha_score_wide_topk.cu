@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(kWideThreads) wide_write_kernel(const WideArgs
 // A cluster of up to eight CTAs owns a unit: every CTA leaves the scores of its slice in shared memory (16 bits per
 // token), the CTAs exchange their level counts through distributed shared memory between two cluster barriers, and each
 // compacts its own slice.  Against the three kernels for long sequences there is no memset, no histogram and no score
-// pass through global memory, and the first signatures are asked into L2 before the programmatic-launch wait.
+// pass through global memory, and the signatures are asked into L2 before the programmatic-launch wait.
 // Bound: the population-count unit (16 lanes per clock and SM; a token costs G popcounts per counted word), then HBM.
 // Carry-save adders on the logic unit fold the xor words of a token before they are counted: 3, 4 and 5 counted words
 // instead of 4, 8 and 16 for 128, 256 and 512 bits.
@@ -376,14 +376,12 @@ __global__ void __launch_bounds__(kWideThreads) wide_select_cluster_kernel(const
                 for (int w = 0; w < W; ++w) kw[i][w] = 0ull;
         }
     };
-    // The first pass is only asked into L2 before the launch wait (one request per 128-byte line) and loaded after it: the kernel
-    // in front may still be writing signatures, at any slot.
-#pragma unroll
-    for (int i = 0; i < kTok; ++i) {
-        const int l = i * kWideThreads + tid;
-        if (l % (16 / W) == 0 && l < slice && base + l < n)
-            asm volatile("prefetch.global.L2 [%0];" ::"l"(row + (long long)(base + l) * W));
-    }
+    // The signatures are only asked into L2 before the launch wait (one request per 128-byte line) and loaded behind it: the
+    // kernel in front may still be writing one, at any slot.  The whole slice, since HBM is idle under ENCODE: 5 ragged sequences
+    // of up to 65536 tokens at 256 bits 61.8 us per step, with the first four passes 65.3, with the first alone 66.9; 6 ragged ones
+    // of 32768 at 512 bits 81.3 / 83.2 / 87.5.
+    for (int l = tid * (16 / W); l < min(slice, n - base); l += kWideThreads * (16 / W))
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(row + (long long)(base + l) * W));
     unsigned long long cur[kTok][W], nxt[kTok][W];
     for (int i = tid; i < levels * kCols; i += kWideThreads) c_hist[i] = 0u;
     pdl_launch_dependents();
