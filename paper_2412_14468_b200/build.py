@@ -2,7 +2,8 @@
 marshalling of the binding into paper_2412_14468_b200/_hostcall.so, which links against it.
 
 Every .cu file becomes an object under csrc/build/ (compiled in parallel, recompiled only when it or a header
-changed), then the objects are linked into the shared library."""
+changed), then the objects are linked into the shared library.  The marshalling is recompiled as well when torch or Python is
+another one than it was compiled against."""
 from __future__ import annotations
 
 import glob
@@ -19,6 +20,7 @@ OBJ = os.path.join(CSRC, "build")
 LIB = os.path.join(HERE, "libhashattn.so")
 HOST_SRC = os.path.join(CSRC, "host", "ha_hostcall.cpp")
 HOST_LIB = os.path.join(HERE, "_hostcall.so")
+HOST_STAMP = os.path.join(OBJ, "_hostcall.key")     # what HOST_LIB was compiled against
 
 NVCC_FLAGS = [
     "-std=c++17", "-O3", "-lineinfo",
@@ -47,6 +49,20 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _hostcall_key() -> str:
+    """The headers and the interpreter that the extension module is bound to: it fits no other torch and no other Python."""
+    import torch
+    return "\n".join([torch.__version__, os.path.dirname(torch.__file__), str(torch._C._GLIBCXX_USE_CXX11_ABI), sys.version,
+                      sysconfig.get_paths()["include"]])
+
+
+def _hostcall_stale() -> bool:
+    if _stale(HOST_LIB, [HOST_SRC, os.path.join(ROOT, "include", "hashattn.h")]) or not os.path.exists(HOST_STAMP):
+        return True
+    with open(HOST_STAMP) as f:
+        return f.read() != _hostcall_key()
+
+
 def _build_hostcall() -> None:
     """The extension module over torch's own C++ headers; g++ is enough, it has no device code."""
     import torch
@@ -60,6 +76,8 @@ def _build_hostcall() -> None:
     cmd += ["-L", HERE, "-l:" + os.path.basename(LIB), "-L", os.path.join(root, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu",
             "-ltorch_python", "-Wl,-rpath,$ORIGIN"]
     subprocess.run(cmd, check=True)
+    with open(HOST_STAMP, "w") as f:
+        f.write(_hostcall_key())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -80,7 +98,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         os.remove(stale)
     if todo or force or _stale(LIB, objs):
         subprocess.run([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", LIB] + objs, check=True)
-    if force or _stale(HOST_LIB, [HOST_SRC, os.path.join(ROOT, "include", "hashattn.h")]):
+    if force or _hostcall_stale():
         _build_hostcall()
     return LIB
 

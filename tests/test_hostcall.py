@@ -35,3 +35,15 @@ def test_host_step_wants_contiguous_host_buffers():
     t = torch.zeros(2, 2)
     with pytest.raises(TypeError):
         ha.SparseDecodeHostStep(ha.make_shape(1, 32, 8, 0.1), None, None, t.t(), t, t, t, t, t, t, None, 1, 1, 1, t, t, t, t, stream=0)
+
+
+@pytest.mark.parametrize("change", [None, "torch", "python"])
+def test_the_extension_is_rebuilt_for_another_torch_or_python(monkeypatch, change):
+    built_again = []
+    monkeypatch.setattr(ha_build, "_build_hostcall", lambda: built_again.append(True))
+    if change == "torch":
+        monkeypatch.setattr(torch, "__version__", torch.__version__ + ".other")
+    elif change == "python":
+        monkeypatch.setattr(ha_build.sys, "version", "3.99")
+    ha_build.build()
+    assert bool(built_again) == (change is not None)
