@@ -24,10 +24,15 @@ namespace ha {
 
 constexpr int kAttnWarps = 4;
 constexpr int kAttnThreads = kAttnWarps * 32;
-// Blocks of rows per warp (ring in shared memory), kStages below: 3, or 2 for lists of up to 2048 entries.  Two stages ask less
-// of HBM at once and reach the same rate: 24 ragged lists of up to 2048 entries over pages 59.9 against 61.5 us per step, 64
-// lists of 1024 92.1 / 92.7; longer ragged lists keep the third (32 lists of up to 4096: 114.6 / 116 - 117).
-constexpr int kShortList = 2048;
+// Blocks of rows per warp (ring in shared memory), kStages below: 2 or 3.  Two stages ask less of HBM at once and leave shared
+// memory to the next step's ENCODE, a third helps the CTAs that work on alone when ragged lists end.  us per step with 2 / 3:
+//   one budget for all sequences (lists of equal length)   24 x 1024 48.0 / 48.7, x 2048 64.3 / 65.1, x 3072 83.6 / 84.6,
+//     x 4096 97.0 / 97.8;  64 x 3072 192.5 / 193.1;  4 x 8192 50.2 / 51.4;  1 x 16384 41.9 / 42.6
+//   ragged (longest)   64 x 512 68.8 / 70.0, 40 x 1250 65.4 / 66.3, 48 x 1536 76.5 / 75.2, 24 x 2048 63.4 / 63.3,
+//     24 x 3072 71.4 / 71.4, 48 x 3072 108.9 / 106.1, 16 x 8192 105.9 / 104.7
+//   in pages of 16     24 x 1024 56.3 / 57.7, 40 x 2048 93.5 / 96.4, 24 ragged x 2560 74.4 / 75.4, x 3072 77.0 / 78.8;
+//     24 x 4096 124.8 / 131.6, ragged 86.9 / 88.5, ragged x 5120 95.6 / 94.9;  8 x 8192 93.3 / 91.5, ragged 69.1 / 68.1
+constexpr int kShortList = 2048, kShortPagedList = 4096;
 __host__ __device__ constexpr int attn_smem_bytes(int stages) { return kAttnWarps * stages * kStageBytes; }
 
 struct AttnArgs {
@@ -449,7 +454,8 @@ static cudaError_t launch_attn_g(bool gather, const AttnArgs &args_in, cudaStrea
     const long long t_max = blocks_per_unit * args.n_units;
     int grid;
     bool many_parts = true;
-    const bool two_stages = gather && args.max_items <= kShortList;
+    const bool one_budget = args.count_from_k && !args.k_per_seq && !args.block_table;
+    const bool two_stages = gather && (one_budget || args.max_items <= (args.block_table ? kShortPagedList : kShortList));
     size_t smem = attn_smem_bytes(two_stages ? 2 : 3);
     if (args.n_units <= kMaxBalancedUnits) {
         args.balanced = 1;

@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_2412_14468_b200 import binding as ha
 from paper_2412_14468_b200 import workloads as wl
-from tests._util import OUT_TOL, max_abs_diff_bf16, u16
+from tests._util import OUT_TOL, assert_out_close, max_abs_diff_bf16, u16
 from tests.test_gpu_parity import _attn_inputs, _check_gather, _run_step, _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
     test_whole_step_with_keys_values_and_signatures_all_paged as _whole_paged_step
 
@@ -236,3 +236,34 @@ def test_score_topk_wide_where_the_cluster_size_changes(n_bits, B, n):
     kc = _wide_codes(rng, B * Hkv * n, W).reshape(B, Hkv, n, W)
     qc = _wide_codes(rng, B * Hkv, W).reshape(B, Hkv, W)
     _check_score_topk_wide(n_bits, qc, kc, lens, [max(1, m // 9) for m in lens], Hkv, Hkv, 2, 3)
+
+
+@pytest.mark.parametrize("uniform,k", [(True, 2048), (True, 2049), (True, 4100), (False, 2048), (False, 2049), (False, 4100)])
+def test_step_on_the_split_k_kernel_with_two_and_with_three_row_stages(uniform, k):
+    """160 units: one budget for all sequences takes two row stages at any length, a budget per sequence up to 2048 entries.  All
+    signatures, lists and outputs against the oracle."""
+    B, Hq, Hkv = 80, 4, 2
+    n = 4200 if k > 3000 else 2100
+    cfg = wl.Config("row-stages", 73, B, [n] * B, k, 0.02, n_q_heads=Hq, n_kv_heads=Hkv)
+    w = wl.make_workload(cfg, DEV)
+    lens = [n - (0 if uniform else 3 * (b % 7)) for b in range(B)]
+    ks = [k - (0 if uniform else 5 * (b % 11)) for b in range(B)]
+    shape = ha.make_shape(B, Hq, Hkv, w["sm_scale"])
+    ws = ha.alloc_workspace(shape, n, k)
+    mq, mk = ha.Mapping(w["map_q"]), ha.Mapping(w["map_k"])
+    kc = torch.zeros(B, Hkv, -(-n // 4) * 4, dtype=torch.int32, device=DEV)
+    ha.ha_encode(mk, 1, w["K"], kc)
+    new = lambda *s, t=torch.int32: torch.zeros(*s, dtype=t, device=DEV)  # noqa: E731
+    qc, idx, cnt, out = new(B, Hq), new(B, Hkv, k), new(B, Hkv), new(B, Hq, 128, t=torch.bfloat16)
+    i32 = lambda v: torch.tensor(v, dtype=torch.int32, device=DEV)  # noqa: E731
+    Kc = kc.cpu().numpy().view(np.uint32)[:, :, :n].copy()
+    ha.ha_sparse_decode(shape, mq, None, w["q"], None, w["K"], w["V"], kc, i32(lens), None if uniform else i32(ks), k if uniform else 0, n, k,
+                        qc, idx, cnt, out, ws)
+    ref = oracle.decode_step(u16(w["q"]), None, u16(w["K"]), u16(w["V"]), Kc, wl.mapping_numpy(w["map_q"]), wl.mapping_numpy(w["map_k"]),
+                             lens, ks, sm_scale=w["sm_scale"], n_threads=4)
+    got, n_got = idx.cpu().numpy(), cnt.cpu().numpy()
+    assert np.array_equal(n_got, ref["count"])
+    for b in range(B):
+        assert np.array_equal(got[b, :, :ks[b]], ref["idx"][b, :, :ks[b]]) and (got[b, :, ks[b]:] == -1).all()
+    assert_out_close(u16(out), ref["out"])
+    assert ha.ha_read_device_status(ws) == 0
