@@ -221,13 +221,13 @@ cudaError_t launch_encode_tc(const MapView &map, int heads_per_kv, TensorView x,
 // ------------------------------------------------------------------ tcgen05 version
 //
 // The same chain of three GEMMs on the fifth-generation tensor cores.  A tile of 128 tokens is
-// M = 128 rows = the 128 lanes of tensor memory; threads r and r + 128 of a group own row r.
+// M = 128 rows = the 128 lanes of tensor memory; threads r, r + 128, r + 256 and r + 384 convert row r.
 //   layer 1  D[128 x 128] = X W1 + b1   A = token tile in shared memory (K-major core matrices),
 //                                       B = W1 in shared memory (N-major core matrices), 8 x K16;
 //                                       the bias is one more K16 step: A = a constant tile whose
 //                                       rows are (1, 1, 0, ...), B = two rows holding b1 as a bf16
 //                                       pair hi + lo
-//   epilogue threads read their row of D (tcgen05.ld), apply ReLU, split into a bf16 pair hi + lo
+//   epilogue threads read their quarter of a row of D (tcgen05.ld), apply ReLU, split into a bf16 pair hi + lo
 //            (cvt.rn.bf16x2) and write both to tensor memory as the next A operand (tcgen05.st)
 //   layer 2  D = A_hi W2 + A_lo W2 + b2  A from tensor memory, 16 x K16 + the bias step
 //   layer 3  D[128 x 32] likewise; the epilogue packs the 32 sign bits of a row into its code.
@@ -345,8 +345,8 @@ __device__ __forceinline__ void tma_load_tile(uint32_t dst, const CUtensorMap *t
                  ::"r"(dst), "l"(tmap), "r"(0), "r"(t0), "r"(0), "r"(h), "r"(b), "r"(bar) : "memory");
 }
 
-// kTma: token tiles arrive through TMA (one thread per group issues one box copy and the tile's mbarrier
-// counts the bytes); otherwise every thread copies 16-byte pieces with cp.async.
+// kTma: token tiles arrive through TMA (a group's issuing warp issues one box copy and the tile's mbarrier
+// counts the bytes); otherwise the converting threads copy 16-byte pieces with cp.async.
 template <bool kTma>
 __global__ void __launch_bounds__(kU_Threads, 1) encode_umma_kernel(const __grid_constant__ CUtensorMap tmap, MapView map,
                                                                    int heads_per_kv, TensorView x, int B, int H, int T,

@@ -1,7 +1,8 @@
 // The whole layer-step in ONE launch, for small batches (as many (sequence, KV head) units as clusters
-// are resident at once: on a 148-SM device 33 clusters of 8 CTAs or 71 of 4 with index lists of up to 1024
-// entries, 15 clusters of 8 with longer lists) and sequences of up to 32768 tokens: ENCODE -> SCORE -> TOPK
-// -> GATHER-ATT (Section 4 recipe, Section 4.1 "Implementation") with one thread-block cluster of CS
+// are resident at once: on a 148-SM device 33 clusters of 8 CTAs or 71 of 4 with index lists of up to 2560
+// entries, 15 clusters of 8 with longer lists) and sequences of up to 32768 tokens, 65536 for up to 33 units and
+// 131072 for up to 15 (fused_variant has the rule): ENCODE -> SCORE -> TOPK -> GATHER-ATT (Section 4
+// recipe, Section 4.1 "Implementation") with one thread-block cluster of CS
 // CTAs per unit, so that a small-batch decode step has no kernel boundary or global-memory hand-off on
 // its critical path:
 //
@@ -20,6 +21,7 @@
 //       shared-memory stages, QK^T and PV on the tensor cores, online softmax; the CTA states
 //       are written into CTA 0's shared memory (DSMEM stores), cluster barrier, CTA 0 merges,
 //       normalises and rounds once to bf16.
+// A kernel behind this one starts when the appended signatures are written (barrier #2).
 // Every cross-CTA hand-off is a push followed by a hardware cluster barrier (no flag, no spin, no remote
 // read).  Results are bit-identical to the multi-kernel path for signatures, counts and index lists;
 // attention outputs agree within the usual fp32 reordering.
@@ -33,7 +35,7 @@ constexpr int kFusedMaxCS = 8;                               // CTAs per cluster
 constexpr int kFusedWarps = 8;
 constexpr int kFusedThreads = kFusedWarps * 32;
 // Longest sequence, a template argument because a thread holds its share of the signatures in registers: 32768 in general;
-// 65536 (one-stage variant) and 131072 (two-stage variant) with clusters of 8, for the few units of one or two long sequences.
+// 65536 (one-stage variant, 33 units) and 131072 (two-stage variant, 15 units) with clusters of 8.
 constexpr int kFusedMaxSeq = 32768, kFusedMidSeq = 65536, kFusedLongSeq = 131072;
 constexpr int kFusedLongMaxK = 5120;                         // longest index list of the 131072-token variant
 constexpr int kFusedMaxStages = 2;                           // row blocks in flight per warp (template parameter S)
