@@ -69,7 +69,12 @@ __device__ __forceinline__ int ld_dsmem(const int *local, uint32_t rank) {
     asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(ra) : "memory");
     return v;
 }
-
+// write an int of CTA `rank`'s shared memory at the address that `local` has in this CTA
+__device__ __forceinline__ void st_dsmem(int *local, uint32_t rank, int v) {
+    uint32_t a = (uint32_t)__cvta_generic_to_shared(local), ra;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));
+    asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(ra), "r"(v) : "memory");
+}
 
 // Score byte of a token that is always in context (Windows): above every real score + 1 (<= 33), so the
 // flag arithmetic below sees "score > T" for every threshold, and small enough that no byte sum reaches 256.

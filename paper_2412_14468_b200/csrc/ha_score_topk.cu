@@ -4,11 +4,13 @@
 // score T and how many tokens r of score exactly T are still needed; the selection is every token
 // above T plus the first r tokens at T in index order, written in ascending token order.
 //
-// Two implementations share the arithmetic:
+// Three implementations share the arithmetic:
 //  * sequences of up to 131072 tokens: ONE kernel, a thread-block cluster per (sequence, KV head)
 //    (score_select_cluster_kernel, second half of this file), over contiguous or paged signatures (24 sequences of 2000 -
 //    65536 tokens in pages of 16, whole step: 61.4 us against 84.1 us with the two kernels below);
-//  * longer sequences: two kernels over chunks of the sequence, with the per-chunk histograms and
+//  * many units of unequal length, and long sequences from 24 units on: ONE kernel whose clusters take several units each
+//    (score_select_batch_kernel; batch_cluster_size has the rule);
+//  * other longer sequences: two kernels over chunks of the sequence, with the per-chunk histograms and
 //    one score byte per token passed through the workspace (scan_score_kernel, select_kernel).
 // No CTA ever spins on another: hand-offs are hardware cluster barriers or kernel boundaries.
 // The scanning kernels request their first signatures before the programmatic-launch wait, so that
@@ -600,12 +602,519 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
     return cudaGetLastError();
 }
 
+// ------------------------------------------------------------------ several units per cluster
+//
+// As many clusters of CS = 1, 2, 4 or 8 CTAs (512 threads, two per SM) as are resident at once share the units out among them: by
+// falling length, forth and back, so that ragged batches end together.  A cluster takes up to eight units at a time through every
+// phase: scores of all of them, one exchange of histograms, thresholds, lists.  The fixed part (launch, first rows, barriers,
+// thresholds: 7 us) is thus paid once, not in every wave of one-unit clusters, no SM is left with more CTAs than another, and the
+// bytes of any sequence fit (96 KB of counters and score bytes per CTA), so the long ones need no second kernel.
+//
+// Bound: the population count (groups of 4 and 8: 14.4 us for 512 units of 32768 tokens and 4 heads, 18 - 23 us measured for the
+// scoring), HBM for groups of 1.  Alone, against the one-unit clusters (us): 32 sequences of 8192 - 131072 tokens 41.6 -> 35.3, 24 of
+// 2000 - 65536 18.0 -> 15.1, 64 of 2000 - 32768 24.3 -> 19.3, 48 of 8000 - 65536 in groups of 2 29.0 -> 22.0.
+//  * Reading: the signatures are asked into L2 before the launch wait and read behind it, two rows of 128 tokens per warp ahead of
+//    the scoring.
+//  * Score bytes: 32 consecutive tokens are 8 words, and byte e of word j belongs to token 8 e + j.  Stored byte by byte in that order
+//    (no packing; the 32 bytes of an instruction lie in 8 banks), eight words give the 32 flags "above / at the threshold" of their
+//    tokens, in token order, with an add, a shift and one three-input operation per word.
+//  * Writing: a lane takes whole groups of 32 tokens, works out which of them are selected and visits only those.
+// Tried: equal shares of all rows whatever the unit boundaries (a cooperative launch, units settled by counters): balanced to the
+// row, but such a launch waits for the kernel in front to drain and pays 15 us of fixed parts (16 units of 32768: 19.8 against 11.9);
+// the 32 x 32 bits of products on the tensor cores (kind::mxf4, signatures spread over tensor memory): 28 us against 20 us for the
+// same tokens counted with popc, the stores into tensor memory alone take 10.
+
+// The scores (bytes of s_sc) and flags of 32 consecutive tokens, in token order: bit i = token i of the group.  gt: score above T.
+__device__ __forceinline__ void group_flags(const unsigned char *group, uint32_t c_gt, uint32_t c_ge, uint32_t &gt, uint32_t &ge) {
+    const uint4 lo = reinterpret_cast<const uint4 *>(group)[0], hi = reinterpret_cast<const uint4 *>(group)[1];
+    const uint32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    gt = 0u;
+    ge = 0u;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        gt = (gt >> 1) | ((w[j] + c_gt) & 0x80808080u);
+        ge = (ge >> 1) | ((w[j] + c_ge) & 0x80808080u);
+    }
+}
+
+// One unit of a batch, as every CTA of the cluster sees it.
+struct BatchUnit {
+    int b, g, n, keep, keep_rest;   // sequence, head of the unit, tokens; list length, and the heavy tokens among it
+    int row0, rows;                 // this CTA's rows of 128 tokens
+    int off, tab;                   // its score bytes and, pages of 16 tokens or more, its entries of the block table in the pool
+    WindowBounds win;
+    int T, r, gt_before, eq_before;
+};
+
+constexpr int kSelThreads = 512, kSelWarps = kSelThreads / 32;
+constexpr int kSelUnits = 8;                          // units of a batch
+constexpr int kSelHist = kBins * 32 * 4;              // bytes of a unit's counters [level][lane]
+constexpr int kSelSort = 512;                         // sequences that are dealt out by length
+constexpr int kSelPool = 96 * 1024;                   // counters, score bytes and table entries of a batch: two CTAs per SM
+
+// Bytes of a slice's entries of the block table (one more where the slice begins inside a page).
+__host__ __device__ constexpr int batch_table_bytes(int rows, int shift) { return ((rows * 128 >> shift) + 5) / 4 * 16; }
+
+// kPaged: the signatures lie in a pool behind a block table.  Pages of 4 tokens or more hold a lane's 4 tokens in one piece, so
+// a row costs one table entry per lane (neighbouring lanes share it) and the same 16-byte load.
+template <int G, int CS, bool kPaged>
+__global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
+    const uint32_t *__restrict__ q_codes, const uint32_t *__restrict__ k_codes, long long kc_sb, long long kc_sh,
+    const int32_t *__restrict__ seq_lens, int max_seq_len, const int32_t *__restrict__ k_per_seq, int k_uniform,
+    int k_max, int B, int Hq, int Hkv, int32_t *__restrict__ idx, long long idx_sb, long long idx_sh,
+    int32_t *__restrict__ count, int32_t *__restrict__ hist_out, Windows win, const CodePages cp, int kv_shift,
+    bool in_step, bool staged) {
+    extern __shared__ __align__(128) unsigned char pool[];     // counters of the batch's units, then their score bytes
+    __shared__ int s_all[CS][kSelUnits][kBins + 3];            // histograms of the cluster's CTAs
+    __shared__ BatchUnit s_u[kSelUnits];
+    __shared__ uint32_t s_nq[kSelUnits][G];
+    __shared__ uint32_t s_wcnt[kSelWarps];
+    __shared__ int s_len[kSelSort], s_k[kSelSort];
+    __shared__ uint16_t s_perm[kSelSort];
+    __shared__ int s_units;
+    const int rank = CS > 1 ? (int)cluster_rank() : 0;
+    if (CS > 1) cluster_arrive();                              // its wait stands in front of the first remote store
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int C = gridDim.x / CS, cl = blockIdx.x / CS, n_units = B * Hkv;
+    auto len_of = [&](int b) -> int { return max(min(seq_lens[b], max_seq_len), 0); };
+    auto budget_of = [&](int b) -> int { return k_per_seq ? k_per_seq[b] : k_uniform; };
+
+    // ---- the cluster's units: all units by falling length, dealt out to the clusters forth and back
+    const bool sorted = B <= kSelSort;
+    if (B <= 64) {   // by the warp that needs them
+        if (warp == 0) {
+            const int l0 = lane < B ? len_of(lane) : -1, l1 = lane + 32 < B ? len_of(lane + 32) : -1;
+            const int k0 = lane < B ? budget_of(lane) : 0, k1 = lane + 32 < B ? budget_of(lane + 32) : 0;
+            int r0 = 0, r1 = 0;
+#pragma unroll 8
+            for (int j = 0; j < min(B, 32); ++j) {
+                const int v = __shfl_sync(0xffffffffu, l0, j);
+                r0 += (v > l0 || (v == l0 && j < lane)) ? 1 : 0;
+                r1 += v >= l1 ? 1 : 0;
+            }
+#pragma unroll 8
+            for (int j = 0; j < B - 32; ++j) {
+                const int v = __shfl_sync(0xffffffffu, l1, j);
+                r0 += v > l0 ? 1 : 0;
+                r1 += (v > l1 || (v == l1 && j < lane)) ? 1 : 0;
+            }
+            if (lane < B) { s_perm[r0] = (uint16_t)lane; s_len[lane] = l0; s_k[lane] = k0; }
+            if (lane + 32 < B) { s_perm[r1] = (uint16_t)(lane + 32); s_len[lane + 32] = l1; s_k[lane + 32] = k1; }
+            __syncwarp();
+        }
+    } else if (sorted) {
+        for (int i = tid; i < B; i += kSelThreads) { s_len[i] = len_of(i); s_k[i] = budget_of(i); }
+        __syncthreads();
+        for (int i = tid; i < B; i += kSelThreads) {
+            const int mine = s_len[i];
+            int at = 0;
+            for (int j = 0; j < B; ++j) at += (s_len[j] > mine || (s_len[j] == mine && j < i)) ? 1 : 0;
+            s_perm[at] = (uint16_t)i;
+        }
+        __syncthreads();
+    }
+    auto unit_of = [&](int j) -> int { return j * C + ((j & 1) ? C - 1 - cl : cl); };   // the cluster's j-th unit
+
+    bool first_batch = true;
+    for (int j0 = 0;;) {
+        // ---- the batch: as many of the next units as fit the pool
+        if (warp == 0) {
+            BatchUnit u = {};
+            const int at = lane < kSelUnits ? unit_of(j0 + lane) : n_units;
+            int need = 1 << 28;
+            if (at < n_units) {
+                const int sb = at / Hkv;
+                u.b = sorted ? s_perm[sb] : sb;
+                u.g = at - sb * Hkv;
+                u.n = sorted ? s_len[u.b] : len_of(u.b);
+                u.win = window_bounds(win, u.n);
+                const int forced = forced_before(u.win, u.n), k = sorted ? s_k[u.b] : budget_of(u.b);
+                u.keep_rest = max(0, min(min(k, k_max - forced), u.n - forced));
+                u.keep = forced + u.keep_rest;
+                const int rows = (u.n + 127) >> 7;
+                u.row0 = rows * rank / CS;
+                u.rows = rows * (rank + 1) / CS - u.row0;
+                need = kSelHist + (rows + CS - 1) / CS * 128;
+                if (kPaged && staged) need += batch_table_bytes((rows + CS - 1) / CS, cp.shift);
+                u.tab = kSelHist + (rows + CS - 1) / CS * 128;
+            }
+            int inc = need;
+#pragma unroll
+            for (int dd = 1; dd < kSelUnits; dd <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, inc, dd);
+                if (lane >= dd) inc = min(inc + v, 1 << 28);
+            }
+            const int U = __popc(__ballot_sync(0xffffffffu, at < n_units && inc <= kSelPool));
+            u.off = inc - need - lane * kSelHist + U * kSelHist;
+            u.tab += u.off - kSelHist;
+            if (lane < U) s_u[lane] = u;
+            if (lane == 0) s_units = U;
+        }
+        __syncthreads();
+        const int U = s_units;
+        if (U == 0) break;   // cluster-uniform
+        j0 += U;
+
+        // ---- the batch's signatures start their way from HBM to L2 (one request per 128-byte line), its part of the block table
+        // into shared memory
+        auto in_page = [&](const uint32_t *row, int page, int t) -> const uint32_t * {   // (the launcher sees to it that the stride fits)
+            return row + (long long)page * (int)cp.page_stride + (t & ((1 << cp.shift) - 1));
+        };
+        auto row_of = [&](const BatchUnit &u) -> const uint32_t * {
+            const int kvh = u.g >> kv_shift;   // the KV head whose signatures this unit scans
+            return kPaged ? k_codes + (long long)kvh * cp.head_stride : k_codes + (long long)u.b * kc_sb + (long long)kvh * kc_sh;
+        };
+        if (kPaged && !in_step && first_batch) pdl_wait();   // a block table may come from the kernel in front
+        for (int i = 0; i < U; ++i) {
+            const BatchUnit &u = s_u[i];
+            const uint32_t *row = row_of(u);
+            const int first = u.row0 * 128, end = min(u.n, (u.row0 + u.rows) * 128);
+            if (kPaged) {
+                if (cp.shift < 2) continue;
+                const int32_t *table = cp.table + (long long)u.b * cp.bt_sb;
+                const int e0 = first >> cp.shift, e1 = (end + (1 << cp.shift) - 1) >> cp.shift;
+                int32_t *tab = reinterpret_cast<int32_t *>(pool + u.tab);
+                for (int e = e0 + tid; e < e1 && first < end; e += kSelThreads) {   // a page of one head is one run of bytes
+                    const int page = __ldg(table + e), t0 = max(e << cp.shift, first), t1 = min((e + 1) << cp.shift, end);
+                    if (kPaged && staged) tab[e - e0] = page;
+                    for (int t = t0; t < t1; t += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(in_page(row, page, t)));
+                }
+            } else {
+                for (int t = first + tid * 32; t < end; t += kSelThreads * 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + t));
+            }
+        }
+        for (int i = tid; i < U * (kSelHist / 16); i += kSelThreads) reinterpret_cast<uint4 *>(pool)[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (first_batch) {
+            pdl_launch_dependents();
+            pdl_wait();
+        }
+        if (tid < U * G) {   // popc(code ^ ~q) = 32 - Hamming distance
+            const BatchUnit &u = s_u[tid / G];
+            s_nq[tid / G][tid % G] = ~__ldcg(q_codes + (long long)u.b * Hq + u.g * G + tid % G);
+        }
+        __syncthreads();
+
+        // ---- scores and this CTA's histograms.  A warp walks its rows of all the units, two at a time; the next two (of the next
+        // unit if need be) are on their way while it scores
+        {
+            struct Rows { const uint32_t *row; const int32_t *table; int i, p, p_end, tok, n, e0; } at;   // tok: the lane's token of row 0
+            at.i = -1;
+            at.p = at.p_end = at.tok = at.n = at.e0 = 0;
+            at.row = nullptr;
+            at.table = nullptr;
+            auto settle = [&]() {   // on to the next unit in which this warp has rows
+                while (at.p >= at.p_end && ++at.i < U) {
+                    const BatchUnit &u = s_u[at.i];
+                    at.p = u.rows * warp / kSelWarps;
+                    at.p_end = u.rows * (warp + 1) / kSelWarps;
+                    at.tok = u.row0 * 128 + lane * 4;
+                    at.n = u.n;
+                    at.row = row_of(u);
+                    if (kPaged) {
+                        at.table = staged ? reinterpret_cast<const int32_t *>(pool + u.tab) : cp.table + (long long)u.b * cp.bt_sb;
+                        at.e0 = staged ? u.row0 * 128 >> cp.shift : 0;
+                    }
+                }
+            };
+            auto load = [&](uint4 (&c)[2]) {
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int t = at.tok + (at.p + j) * 128;
+                    c[j] = make_uint4(0u, 0u, 0u, 0u);
+                    if (at.p + j < at.p_end && t < at.n) {
+                        if (kPaged && cp.shift < 2) c[j] = load_codes4_paged(cp, at.row, at.table, t, at.n);
+                        else if (kPaged) c[j] = load_codes4(in_page(at.row, at.table[(t >> cp.shift) - at.e0], t) - t, t, at.n);
+                        else c[j] = load_codes4(at.row, t, at.n);
+                    }
+                }
+            };
+            uint4 c[2], nxt[2];
+            settle();
+            if (at.i < U) load(c);
+            int cur = -1, n = 0, sink_end = 0, local_begin = 0;
+            uint32_t base0 = 0u, nq[G];
+            unsigned char *sc_lane = pool;
+#pragma unroll
+            for (int j = 0; j < G; ++j) nq[j] = 0u;
+            auto bump = [&](int s) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(base0 + (uint32_t)s * 128u) : "memory"); };
+            auto score = [&](uint32_t code) {
+                int s = __popc(code ^ nq[0]);
+#pragma unroll
+                for (int j = 1; j < G; ++j) s = max(s, __popc(code ^ nq[j]));
+                return s;
+            };
+            while (at.i < U) {   // warp-uniform
+                const int i = at.i, p0 = at.p, p_end = at.p_end, tok = at.tok;
+                at.p += 2;
+                settle();
+                if (at.i < U) load(nxt);
+                if (i != cur) {
+                    const BatchUnit &u = s_u[i];
+                    cur = i;
+                    n = u.n;
+                    sink_end = u.win.sink_end;
+                    local_begin = u.win.local_begin;
+                    base0 = (uint32_t)__cvta_generic_to_shared(pool + i * kSelHist + lane * 4);
+                    // token e of the lane's four is token 8 x + y of its group of 32 with x = (lane & 7) >> 1, y = 4 (lane & 1) + e
+                    sc_lane = pool + u.off + (lane >> 3) * 32 + (lane & 1) * 16 + ((lane & 7) >> 1);
+#pragma unroll
+                    for (int j = 0; j < G; ++j) nq[j] = s_nq[i][j];
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int p = p0 + j, t = tok + p * 128;
+                    if (p < p_end) {
+                        const int s[4] = {score(c[j].x), score(c[j].y), score(c[j].z), score(c[j].w)};
+                        unsigned char *dst = sc_lane + p * 128;
+                        if (t + 4 <= n && t >= sink_end && t + 4 <= local_begin) {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) { bump(s[e]); dst[e * 4] = (unsigned char)s[e]; }
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const bool forced = t + e < sink_end || t + e >= local_begin;
+                                if (t + e < n) {   // bytes of tokens past the end are never looked at
+                                    if (!forced) bump(s[e]);
+                                    dst[e * 4] = (unsigned char)(forced ? (int)kForcedByte : s[e]);
+                                }
+                            }
+                        }
+                    }
+                }
+                c[0] = nxt[0];
+                c[1] = nxt[1];
+            }
+        }
+        __syncthreads();
+        // ---- fold the counters: one level per warp at a time; lane r < CS hands the sum to CTA r
+        if (CS > 1) cluster_wait();   // every CTA of the cluster runs, and is done with the last batch's histograms
+        for (int l = warp; l < U * kBins; l += kSelWarps) {
+            const int sum = (int)__reduce_add_sync(0xffffffffu, reinterpret_cast<const uint32_t *>(pool)[l * 32 + lane]);
+            const int i = l / kBins;
+            if (CS == 1) { if (lane == 0) s_all[0][i][l - i * kBins] = sum; }
+            else if (lane < CS) st_dsmem(&s_all[rank][i][l - i * kBins], (uint32_t)lane, sum);
+        }
+        if (CS > 1) cluster_sync_all();   // every CTA's histograms have arrived
+        else __syncthreads();
+        if (warp < U) {
+            BatchUnit &u = s_u[warp];
+            int tot = 0, bef = 0, tot32 = 0, bef32 = 0;
+#pragma unroll
+            for (int q = 0; q < CS; ++q) {
+                const int v = s_all[q][warp][lane], v32 = s_all[q][warp][32];
+                tot += v;
+                tot32 += v32;
+                if (q < rank) { bef += v; bef32 += v32; }
+            }
+            int T, r, gt_before, eq_before;
+            find_threshold(tot, bef, tot32, bef32, u.keep_rest, lane, T, r, gt_before, eq_before);
+            const int unit = u.b * Hkv + u.g;
+            if (lane == 0) {
+                u.T = T;
+                u.r = r;
+                u.gt_before = gt_before + forced_before(u.win, min(u.row0 * 128, u.n));   // always-kept tokens count as above
+                u.eq_before = eq_before;
+                if (rank == 0) count[unit] = u.keep;
+            }
+            if (rank == 0 && hist_out) {
+                hist_out[(long long)unit * kBins + lane] = tot;
+                if (lane == 0) hist_out[(long long)unit * kBins + 32] = tot32;
+            }
+        }
+        __syncthreads();
+        first_batch = false;
+        const bool more = unit_of(j0) < n_units;   // cluster-uniform
+        if (CS > 1 && more) cluster_arrive();      // done with the histograms
+
+        // ---- list entries.  W warps per unit, each takes a contiguous share of the CTA's groups of 32 tokens.
+        // Flags "S > T" / "S >= T", kept where the group's scores were: a byte s + 127 - T has bit 7 set iff s > T, s + 128 - T
+        // iff s >= T (T <= 33, and no byte of a token before the end carries into the next).
+        const int W = U > 4 ? kSelWarps / 8 : U > 2 ? kSelWarps / 4 : kSelWarps / U, i = warp / W;
+        const bool busy = i < U;
+        const BatchUnit &u = s_u[busy ? i : 0];
+        const int part = warp - i * W, first_tok = u.row0 * 128, n = u.n, keep = u.keep, r = u.r;
+        const int n_groups = busy ? max(0, min(4 * u.rows, (n - first_tok + 31) >> 5)) : 0;
+        const int q_lo = n_groups * part / W, q_n = n_groups * (part + 1) / W - q_lo;   // the warp's groups
+        unsigned char *sc = pool + u.off + q_lo * 32;
+        uint2 *flags = reinterpret_cast<uint2 *>(sc);   // of the groups so far, where the scores of the first quarter of them were
+        int32_t *out = idx + (long long)u.b * idx_sb + (long long)u.g * idx_sh;
+        if (busy) {
+            const uint32_t c_gt = 0x7f7f7f7fu - (uint32_t)u.T * 0x01010101u, c_ge = 0x80808080u - (uint32_t)u.T * 0x01010101u;
+            uint32_t cnt = 0u;   // flags of this lane's groups: S > T in the low half, S == T in the high half
+            for (int q0 = 0; q0 < q_n; q0 += 32) {   // warp-uniform
+                const int q = q0 + lane;
+                uint32_t gt = 0u, ge = 0u;
+                if (q < q_n) {
+                    group_flags(sc + q * 32, c_gt, c_ge, gt, ge);
+                    const int left = n - (first_tok + (q_lo + q) * 32);
+                    if (left < 32) { const uint32_t live = (1u << left) - 1u; gt &= live; ge &= live; }
+                }
+                __syncwarp();   // the scores are read before flags overwrite them
+                if (q < q_n) flags[q] = make_uint2(gt, ge ^ gt);   // score > T implies score >= T
+                cnt += (uint32_t)__popc(gt) + ((uint32_t)__popc(ge ^ gt) << 16);
+            }
+            cnt = __reduce_add_sync(0xffffffffu, cnt);
+            if (lane == 0) s_wcnt[warp] = cnt;
+            for (int q = keep + (rank * W + part) * 32 + lane; q < k_max; q += CS * W * 32) out[q] = -1;
+        }
+        __syncthreads();
+        if (busy && keep > 0) {
+            // a lane takes `per` consecutive groups: one scan over the lanes for all of the warp's groups
+            const int per = (q_n + 31) >> 5, q_first = min(lane * per, q_n), q_last = min(q_first + per, q_n);
+            int n_gt = 0, n_eq = 0;
+            for (int q = q_first; q < q_last; ++q) { const uint2 f = flags[q]; n_gt += __popc(f.x); n_eq += __popc(f.y); }
+            int inc = n_gt | (n_eq << 16);
+#pragma unroll
+            for (int dd = 1; dd < 32; dd <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, inc, dd);
+                if (lane >= dd) inc += v;
+            }
+            // tokens before this lane's groups with S > T / S == T
+            int run_gt = u.gt_before + (inc & 0xffff) - n_gt, run_eq = u.eq_before + (int)((unsigned)inc >> 16) - n_eq;
+            for (int w = i * W; w < warp; ++w) { run_gt += (int)(s_wcnt[w] & 0xffffu); run_eq += (int)(s_wcnt[w] >> 16); }
+            int32_t *dst = out + run_gt + min(run_eq, r);
+            int room = r - run_eq;   // tokens at the threshold that are still wanted
+            for (int q = q_first; q < q_last; ++q) {
+                const uint2 f = flags[q];
+                const int here = __popc(f.y), first = first_tok + (q_lo + q) * 32;
+                uint32_t sel = f.x;
+                if (room >= here) sel |= f.y;
+                else for (uint32_t m = f.y; room > 0; --room) { sel |= m & (0u - m); m &= m - 1u; }   // the group in which the last one lies
+                room -= here;
+                for (; sel; sel &= sel - 1u) *dst++ = first + __ffs((int)sel) - 1;
+            }
+        }
+        if (!more) break;
+        __syncthreads();   // the pool and the descriptors are reused
+    }
+    if (first_batch) pdl_wait();   // a cluster without units (never launched): at least one CTA of a grid waits
+}
+
+// The most clusters of a variant that are resident at once on the current device (0: the query failed).
+template <int G, int CS, bool kPaged>
+static int resident_batch_clusters() {
+    static int cached[64] = {};   // 0: not asked yet
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return 0;
+    if (!cached[dev]) {
+        auto kernel = score_select_batch_kernel<G, CS, kPaged>;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelPool) != cudaSuccess) return 0;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(CS);
+        cfg.blockDim = dim3(kSelThreads);
+        cfg.dynamicSmemBytes = kSelPool;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = CS;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n <= 0) return 0;
+        cached[dev] = n;
+    }
+    return cached[dev];
+}
+
+template <int G, int CS, bool kPaged>
+static cudaError_t launch_batch_t(int B, int Hq, int Hkv, const uint32_t *q_codes, const uint32_t *k_codes,
+                                    long long kc_sb, long long kc_sh, const int32_t *seq_lens,
+                                    const int32_t *k_per_seq, int k_uniform, int max_seq_len, int k_max, int32_t *idx,
+                                    long long idx_sb, long long idx_sh, int32_t *count, int32_t *hist_out,
+                                    cudaStream_t st, Windows win, CodePages cp, int kv_shift, bool in_step) {
+    const int rows = ((max_seq_len + 127) / 128 + CS - 1) / CS;   // of the longest slice
+    const bool staged = kPaged && cp.shift >= 4 && kSelHist + rows * 128 + batch_table_bytes(rows, cp.shift) <= kSelPool;
+    const int most = resident_batch_clusters<G, CS, kPaged>();
+    if (most <= 0) return cudaErrorInvalidConfiguration;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(CS * min((long long)most, (long long)B * Hkv)));
+    cfg.blockDim = dim3(kSelThreads);
+    cfg.dynamicSmemBytes = kSelPool;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = CS;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = CS > 1 ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, score_select_batch_kernel<G, CS, kPaged>, q_codes, k_codes, kc_sb, kc_sh,
+                                       seq_lens, max_seq_len, k_per_seq, k_uniform, k_max, B, Hq, Hkv, idx, idx_sb, idx_sh,
+                                       count, hist_out, win, cp, kv_shift, in_step, staged);
+    if (e != cudaSuccess) return e;
+    count_launch();
+    return cudaGetLastError();
+}
+
+// CTAs per cluster of the batch kernel, 0: one of the other kernels.  What decides is how the units fill the clusters that are
+// resident at once (296 CTAs, 148 clusters of 2, 71 of 4, 33 of 8 on 148 SMs): the other kernels give every unit a cluster of its
+// own and pay its fixed part of 7 us in every wave, and beyond 131072 tokens two kernels and the way of the scores through global
+// memory.  Whole steps, 8 units a sequence, groups of 4, us with the kernels there were / with this one:
+//   ragged, clusters of 1   30 sequences of 10000 - 20000 tokens 40.7 / 39.3 (of 2: 40.4), 50 of 2000 - 30000 64.0 / 58.3 (60.4), 64 of
+//                           300 - 4000 48.8 / 46.5 (51.4); 28 of 2000 - 33000 44.3 / 44.1 (41.3), hence the line at 32768 tokens
+//   ragged, clusters of 2   13 of 2000 - 30000 30.8 / 28.9, 22 of 1000 - 20000 33.9 / 33.9, 26 of 4000 - 65000 64.8 / 60.5, 32 of 8192 -
+//                           131072 105.6 / 96.5, but 10 of 4000 - 60000 35.3 / 37.7
+//   ... in pages of 16      24 of 20000 - 40000 55.9 / 53.7, 18 of 60000 - 130000 100.5 / 93.4; 16 of 2000 - 30000 29.6 / 30.1, 19 of 20000 -
+//                           40000 46.5 / 48.6; pages of 1 lose (10 of 10000 - 110000 75.8 / 98.0), so smaller pages stay out
+//   ragged, clusters of 4   9 of 20000 - 130000 46.1 / 44.1, 6 of 20000 - 140000 49.1 / 44.3; 10 in pages 49.2 / 50.9
+//   one length              64 of 1200 31.6 / 29.2, of 9000 46.7 / 44.4, but of 16000 59.8 / 60.1 and of 32768 92.2 / 95.2; 50 of 4000 32.8 / 33.7
+//   beyond 131072 tokens    4 of 300000 69.2 / 61.5, 8 of 150000 71.2 / 63.4, 10 of 160000 88.6 / 83.4, 23 of 10000 - 170000 147.6 / 92.0;
+//                           1 of 300000 30.7 / 32.1
+template <int G>
+static int batch_cluster_size(long long units, int max_seq_len, bool ragged, const CodePages &cp) {
+    const bool paged = cp.table != nullptr;
+    if (paged && (cp.shift < 4 || cp.page_stride != (int)cp.page_stride)) return 0;
+    auto fits = [&](int cs) { return kSelHist + ((max_seq_len + 127LL) / 128 + cs - 1) / cs * 128 <= kSelPool; };
+    if (max_seq_len > kClusterMaxSeq) {
+        if (units < 24 || units > 65536 || large_clusters(units, max_seq_len)) return 0;
+        const long long resident[4] = {0, paged ? resident_batch_clusters<G, 2, true>() : resident_batch_clusters<G, 2, false>(),
+                                       paged ? resident_batch_clusters<G, 4, true>() : resident_batch_clusters<G, 4, false>(),
+                                       paged ? resident_batch_clusters<G, 8, true>() : resident_batch_clusters<G, 8, false>()};
+        int best = 0;
+        long long best_cost = 0;
+        for (int e = 1; e < 4; ++e) {   // units of the fullest cluster, per CTA
+            if (!fits(1 << e) || resident[e] <= 0) continue;
+            const long long cost = (units + resident[e] - 1) / resident[e] * (8 >> e);
+            if (!best || cost < best_cost) { best = 1 << e; best_cost = cost; }
+        }
+        return best;
+    }
+    int cs = 0;
+    if (ragged) {
+        if (units >= 232 && max_seq_len <= 32768) cs = 1;
+        else if (units >= 184 || (units >= 104 && (!paged || max_seq_len > 49152))) cs = 2;
+        else if (units >= 40 && units < 72 && max_seq_len > 98304) cs = 4;
+    } else if (units >= 464 && max_seq_len <= 12288) {
+        cs = 1;
+    }
+    return cs && fits(cs) ? cs : 0;
+}
+
 template <int G>
 static cudaError_t launch_g(int B, int Hq, int Hkv, const uint32_t *q_codes, const uint32_t *k_codes,
                             long long kc_sb, long long kc_sh, const int32_t *seq_lens, const int32_t *k_per_seq,
                             int k_uniform, int max_seq_len, int k_max, int32_t *idx, long long idx_sb,
                             long long idx_sh, int32_t *count, int32_t *hist_out, int32_t *ws_hist,
                             unsigned char *ws_scores, cudaStream_t st, Windows win, CodePages cp, int row_shift, bool in_step) {
+    {
+        const int kv_shift = row_shift < 0 ? 0 : row_shift;
+#define HA_BATCH(CSZ) case CSZ: return cp.table ? launch_batch_t<G, CSZ, true>(HA_BATCH_ARGS) : launch_batch_t<G, CSZ, false>(HA_BATCH_ARGS)
+#define HA_BATCH_ARGS B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, idx, \
+                      idx_sb, idx_sh, count, hist_out, st, win, cp, kv_shift, in_step
+        switch (batch_cluster_size<G>((long long)B * Hkv, max_seq_len, k_per_seq != nullptr, cp)) {
+            HA_BATCH(1);
+            HA_BATCH(2);
+            HA_BATCH(4);
+            HA_BATCH(8);
+            default: break;
+        }
+#undef HA_BATCH
+#undef HA_BATCH_ARGS
+    }
     if (large_clusters((long long)B * Hkv, max_seq_len)) {
         const int rows = (max_seq_len + 8 * 4096 - 1) / (8 * 4096), kv_shift = row_shift < 0 ? 0 : row_shift;
 #define HA_LARGE(PAGED) launch_cluster_t<G, 8, PAGED, 512>(rows, B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq,   \

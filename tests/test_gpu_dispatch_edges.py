@@ -8,7 +8,7 @@ import oracle
 from paper_2412_14468_b200 import binding as ha
 from paper_2412_14468_b200 import workloads as wl
 from tests._util import OUT_TOL, assert_out_close, max_abs_diff_bf16, u16
-from tests.test_gpu_parity import _attn_inputs, _check_gather, _run_step, _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
+from tests.test_gpu_parity import _attn_inputs, _check_gather, _run_step, _check_score_topk, _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
     test_whole_step_with_keys_values_and_signatures_all_paged as _whole_paged_step
 
 pytestmark = pytest.mark.gpu
@@ -116,6 +116,72 @@ def test_score_topk_on_clusters_of_large_ctas(G, lens, page_size):
             s = oracle.score(qc[b, g * G:(g + 1) * G], codes[b, g, :n]) if n else np.zeros(0, np.int32)
             ref = oracle.topk_windows(s, ks[b], n_sink, n_local)
             assert n_got[b, g] == len(ref) and np.array_equal(got[b, g, :len(ref)], ref) and (got[b, g, len(ref):] == -1).all()
+
+
+def _batch_lens(n_seqs, longest):
+    """Unequal lengths with the edges of a row of 128 tokens and of a group of 32 among them, not in order."""
+    edges = [0, 1, 31, 32, 33, 127, 128, 129, 255, 257]
+    step = max(1, longest // n_seqs)
+    lens = [max(1, longest - 3 - i * step) for i in range(n_seqs - len(edges) - 1)]
+    return edges[::2] + lens[::2] + [longest] + edges[1::2] + lens[1::2]
+
+
+@pytest.mark.parametrize("G,Hkv,lens", [
+    (4, 4, _batch_lens(58, 2600)),       # 232 units: one CTA a cluster, lengths sorted by one warp
+    (1, 2, _batch_lens(130, 900)),       # 260 units, lengths sorted by the CTA
+    (2, 1, _batch_lens(700, 700)),       # more sequences than are sorted, more than eight units a cluster
+    (8, 4, _batch_lens(26, 5001)),       # 104 units: clusters of 2
+    (4, 8, _batch_lens(23, 7000)),       # 184 units: clusters of 2, also in pages
+    (4, 8, _batch_lens(13, 49153)),      # 104 units of more than 49152 tokens: clusters of 2, also in pages
+    (2, 2, _batch_lens(20, 98305)),      # 40 units of more than 98304 tokens: clusters of 4
+    (4, 4, _batch_lens(12, 131073)),     # beyond the one-unit clusters: 48 units, clusters of 4
+    (1, 2, _batch_lens(12, 262145)),     # 24 units beyond the large CTAs: clusters of 8
+    (1, 2, _batch_lens(12, 393000)),     # slices that leave no room for the block table
+])
+@pytest.mark.parametrize("page_size", [0, 16, 128])
+def test_score_topk_with_several_units_per_cluster(G, Hkv, lens, page_size):
+    """Every cluster size of the batch kernel at the edges of its rule: ragged lengths dealt out by length, several batches per
+    cluster, windows, ties at the threshold, budgets of nothing and of everything, contiguous and in pages."""
+    rng = np.random.default_rng(len(lens) + page_size)
+    B, Hq, n_cap = len(lens), Hkv * G, max(lens) // 128 * 128 + 128
+    ks = [(0, n, max(1, n // 11), max(1, n // 40))[i % 4] if n < 3000 else n // 40 for i, n in enumerate(lens)]
+    n_sink, n_local = (130, 7) if page_size == 16 else (0, 0)
+    k_max = max(max(ks) + n_sink + n_local, 1)
+    codes = rng.integers(0, 2**32, size=(B, Hkv, n_cap), dtype=np.uint64).astype(np.uint32)
+    codes[:, :, 100:400] = codes[:, :, 100:101]                     # ties decided by token index
+    qc = rng.integers(0, 2**32, size=(B, Hq), dtype=np.uint64).astype(np.uint32)
+    qc[:, 0] = codes[:, 0, 100]                                     # ... at the highest score for the first unit
+    shape = ha.make_shape(B, Hq, Hkv, 1.0, n_sink=n_sink, n_local=n_local)
+    ws = ha.alloc_workspace(shape, n_cap, k_max)
+    idx = torch.full((B, Hkv, k_max), 5, dtype=torch.int32, device=DEV)
+    cnt = torch.full((B, Hkv), 5, dtype=torch.int32, device=DEV)
+    hist = torch.full((B, Hkv, 33), 5, dtype=torch.int32, device=DEV)
+    to = lambda a: torch.from_numpy(a.view(np.int32)).to(DEV)  # noqa: E731
+    lt, kt = torch.tensor(lens, dtype=torch.int32, device=DEV), torch.tensor(ks, dtype=torch.int32, device=DEV)
+    if page_size:
+        pool, table = _page_codes(codes, lens, page_size, rng)
+        ha.ha_score_topk_paged(shape, to(qc), to(pool), to(table), lt, kt, 0, max(lens), k_max, idx, cnt, ws, hist_out=hist)
+    else:
+        ha.ha_score_topk(shape, to(qc), to(codes), lt, kt, 0, max(lens), k_max, idx, cnt, ws, hist_out=hist)
+    got, n_got, h_got = idx.cpu().numpy(), cnt.cpu().numpy(), hist.cpu().numpy()
+    for b, n in enumerate(lens):
+        free = np.ones(n, bool)
+        free[:n_sink] = False
+        free[max(n - n_local, 0):] = False
+        for g in range(Hkv):
+            s = oracle.score(qc[b, g * G:(g + 1) * G], codes[b, g, :n]) if n else np.zeros(0, np.int32)
+            ref = oracle.topk_windows(s, ks[b], n_sink, n_local)
+            assert n_got[b, g] == len(ref) and np.array_equal(got[b, g, :len(ref)], ref) and (got[b, g, len(ref):] == -1).all()
+            assert np.array_equal(h_got[b, g], np.bincount(s[free], minlength=33))
+
+
+def test_score_topk_of_many_short_sequences_of_one_length():
+    """464 units of at most 12288 tokens, one budget: one CTA a cluster, two batches."""
+    rng = np.random.default_rng(9)
+    B, Hkv, G, n = 58, 8, 4, 1111
+    codes = rng.integers(0, 2**32, size=(B, Hkv, 1112), dtype=np.uint64).astype(np.uint32)
+    qc = rng.integers(0, 2**32, size=(B, Hkv * G), dtype=np.uint64).astype(np.uint32)
+    _check_score_topk(qc, codes, [n] * B, [40] * B, Hkv * G, Hkv, k_uniform=40)
 
 
 @pytest.mark.parametrize("G", [1, 4, 8])
