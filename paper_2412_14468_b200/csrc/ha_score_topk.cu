@@ -1055,9 +1055,10 @@ static cudaError_t launch_batch_t(int B, int Hq, int Hkv, const uint32_t *q_code
 // own and pay its fixed part of 7 us in every wave, and beyond 131072 tokens two kernels and the way of the scores through global
 // memory.  Whole steps, 8 units a sequence, groups of 4, us with the kernels there were / with this one:
 //   ragged, clusters of 1   30 sequences of 10000 - 20000 tokens 40.7 / 39.3 (of 2: 40.4), 50 of 2000 - 30000 64.0 / 58.3 (60.4), 64 of
-//                           300 - 4000 48.8 / 46.5 (51.4); 28 of 2000 - 33000 44.3 / 44.1 (41.3), hence the line at 32768 tokens
+//                           300 - 4000 48.8 / 46.5 (51.4); 28 of 2000 - 33000 44.3 / 44.1 (41.3), hence the line at 32768 tokens; 31 of
+//                           600 - 4500 28.9 / 29.6, 40 of 900 - 7000 34.1 / 33.6
 //   ragged, clusters of 2   13 of 2000 - 30000 30.8 / 28.9, 22 of 1000 - 20000 33.9 / 33.9, 26 of 4000 - 65000 64.8 / 60.5, 32 of 8192 -
-//                           131072 105.6 / 96.5, but 10 of 4000 - 60000 35.3 / 37.7
+//                           131072 105.6 / 96.5, but 10 of 4000 - 60000 35.3 / 37.7 and 20 of 900 - 7000 27.1 / 29.8
 //   ... in pages of 16      24 of 20000 - 40000 55.9 / 53.7, 18 of 60000 - 130000 100.5 / 93.4; 16 of 2000 - 30000 29.6 / 30.1, 19 of 20000 -
 //                           40000 46.5 / 48.6; pages of 1 lose (10 of 10000 - 110000 75.8 / 98.0), so smaller pages stay out
 //   ragged, clusters of 4   9 of 20000 - 130000 46.1 / 44.1, 6 of 20000 - 140000 49.1 / 44.3; 10 in pages 49.2 / 50.9
@@ -1085,8 +1086,8 @@ static int batch_cluster_size(long long units, int max_seq_len, bool ragged, con
     }
     int cs = 0;
     if (ragged) {
-        if (units >= 232 && max_seq_len <= 32768) cs = 1;
-        else if (units >= 184 || (units >= 104 && (!paged || max_seq_len > 49152))) cs = 2;
+        if (units >= 232 && max_seq_len <= 32768) cs = (max_seq_len > 8192 || units >= 464) ? 1 : 0;
+        else if (max_seq_len > 16384 && (units >= 184 || (units >= 104 && (!paged || max_seq_len > 49152)))) cs = 2;
         else if (units >= 40 && units < 72 && max_seq_len > 98304) cs = 4;
     } else if (units >= 464 && max_seq_len <= 12288) {
         cs = 1;

@@ -127,11 +127,11 @@ def _batch_lens(n_seqs, longest):
 
 
 @pytest.mark.parametrize("G,Hkv,lens", [
-    (4, 4, _batch_lens(58, 2600)),       # 232 units: one CTA a cluster, lengths sorted by one warp
-    (1, 2, _batch_lens(130, 900)),       # 260 units, lengths sorted by the CTA
+    (4, 4, _batch_lens(58, 8193)),       # 232 units: one CTA a cluster, lengths sorted by one warp
+    (1, 2, _batch_lens(240, 900)),       # 480 short units, lengths sorted by the CTA
     (2, 1, _batch_lens(700, 700)),       # more sequences than are sorted, more than eight units a cluster
-    (8, 4, _batch_lens(26, 5001)),       # 104 units: clusters of 2
-    (4, 8, _batch_lens(23, 7000)),       # 184 units: clusters of 2, also in pages
+    (8, 4, _batch_lens(26, 16385)),      # 104 units: clusters of 2
+    (4, 8, _batch_lens(23, 16400)),      # 184 units: clusters of 2, also in pages
     (4, 8, _batch_lens(13, 49153)),      # 104 units of more than 49152 tokens: clusters of 2, also in pages
     (2, 2, _batch_lens(20, 98305)),      # 40 units of more than 98304 tokens: clusters of 4
     (4, 4, _batch_lens(12, 131073)),     # beyond the one-unit clusters: 48 units, clusters of 4
