@@ -241,7 +241,7 @@ cudaError_t launch_encode_tc(const MapView &map, int heads_per_kv, TensorView x,
 //    columns by 32 columns: layer 1 fills P, layer 2 reads P and fills Q, layer 3 reads Q and puts its 32 columns into P, the
 //    next tile starts in Q.  A tile never waits for the sign bits of the one before;
 //  * layers 2 and 3 are issued in halves of 64 inputs: they start when half of the inputs are converted.
-// Measured, 8 heads x 32768 keys: 36.9 us (523 TFLOP/s of algorithmic work) against 50.5 us with the MMAs issued by a thread of
+// Measured, 8 heads x 32768 keys: 36.9 us under ncu (523 TFLOP/s of algorithmic work) against 50.5 us with the MMAs issued by a thread of
 // the converting warps and eight warps per tile.  What is left is the chain of hand-offs of two tiles in flight (6600 cycles per
 // pair of tiles, 4000 of them with the tensor pipe busy); a third tile does not fit tensor memory.  The operands' swizzle made
 // no difference by itself: an MMA of 128 x 128 x 16 takes 65 cycles either way when nothing else runs.
@@ -403,16 +403,8 @@ __global__ void __launch_bounds__(kU_Threads, 1) encode_umma_kernel(const __grid
         mbar_init(smem_u32(&s_start), kU_Convert / 32);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_fail = 0;
-        if (kTma) {   // the first tiles are on their way while the weights are laid out
-            tma_x(0, w_lo, 0);
-            if (tiles_of(1) > 0) tma_x(1, w_lo + 1, 0);
-        }
     }
     __syncwarp();
-    if (warp == 0) {   // one warp allocates the tensor memory and passes the allocation right on
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(kU_TmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
     // ---- weights, the bias rows k = 128 (hi) and 129 (lo) behind them, and the constant tile of ones
     {
         const unsigned char *g1 = reinterpret_cast<const unsigned char *>(map.w1 + (size_t)net * kD * kHid);
@@ -430,6 +422,19 @@ __global__ void __launch_bounds__(kU_Threads, 1) encode_umma_kernel(const __grid
             cp_async16(smem_u32(sW3) + (k >> 3) * 512 + nb * 128 + (k & 7) * 16, g3 + (size_t)e * 16, 16u);
         }
         cp_async_commit();
+        // Nothing of the kernel in front is read, and nothing written, before this point: its end overlaps the launch, the barriers
+        // and the fetch of the weights (us per call, back to back, 8 heads of 32768 keys 34.8 -> 31.9, of 8192 16.5 -> 13.9, of 256 10.4 -> 9.2).  The kernels behind start when this one has ended, as they read signatures before their
+        // own wait.  The tensor memory is allocated behind the wait: a kernel in front may still want it for itself.
+        pdl_wait();
+        if (warp == 0) {   // one warp allocates the tensor memory and passes the allocation right on
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(kU_TmemCols) : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        }
+        if (kTma && tid == 0) {   // the first tiles are on their way while the biases are laid out
+            tma_x(0, w_lo, 0);
+            if (tiles_of(1) > 0) tma_x(1, w_lo + 1, 0);
+        }
+        __syncwarp();
         // rows 128 .. 143 (W3: k-groups 16 and 17): zero, then the bias pair in the first two
         for (int i = tid; i < 2048 / 16; i += kU_Threads) {
 #pragma unroll
@@ -702,12 +707,10 @@ cudaError_t launch_encode_umma(const MapView &map, int heads_per_kv, TensorView 
     cudaError_t e = tma ? cudaFuncSetAttribute(encode_umma_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kU_Smem)
                         : cudaFuncSetAttribute(encode_umma_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kU_Smem);
     if (e != cudaSuccess) return e;
-    if (tma)
-        encode_umma_kernel<true><<<(int)(n_nets * per), kU_Threads, kU_Smem, st>>>(tm, map, heads_per_kv, x, B, H, T, (int)per,
-                                                                                  codes, c_sb, c_sh, status);
-    else
-        encode_umma_kernel<false><<<(int)(n_nets * per), kU_Threads, kU_Smem, st>>>(tm, map, heads_per_kv, x, B, H, T, (int)per,
-                                                                                   codes, c_sb, c_sh, status);
+    const dim3 grid((unsigned)(n_nets * per));
+    e = tma ? launch_pdl(encode_umma_kernel<true>, grid, dim3(kU_Threads), kU_Smem, st, tm, map, heads_per_kv, x, B, H, T, (int)per, codes, c_sb, c_sh, status)
+            : launch_pdl(encode_umma_kernel<false>, grid, dim3(kU_Threads), kU_Smem, st, tm, map, heads_per_kv, x, B, H, T, (int)per, codes, c_sb, c_sh, status);
+    if (e != cudaSuccess) return e;
     count_launch();
     return cudaGetLastError();
 }
