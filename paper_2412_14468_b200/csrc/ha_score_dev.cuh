@@ -112,6 +112,16 @@ __device__ __forceinline__ void write_selected32(int32_t *list, int first, uint3
     visit_selected32(first, gt, eq, g_run, q_run, r, [&](int pos, int t) { list[pos] = t; });
 }
 
+// The same with the selected ones worked out first, so that only they are visited: `room` tokens of score T are still wanted when the
+// 32 begin (<= 0: none), dst is where the first selected one goes.  Returns dst behind the last.
+__device__ __forceinline__ int32_t *write_exact32(int32_t *dst, int first, uint32_t gt, uint32_t eq, int room) {
+    uint32_t sel = gt;
+    if (room >= __popc(eq)) sel |= eq;
+    else for (uint32_t m = eq; room > 0; --room) { sel |= m & (0u - m); m &= m - 1u; }   // the 32 in which the last one lies
+    for (; sel; sel &= sel - 1u) *dst++ = first + __ffs((int)sel) - 1;
+    return dst;
+}
+
 // Warp-wide threshold search over the 33 score levels.  Lane l passes the count of level l (tot) and
 // the part of it that lies before the caller's own slice (bef); level 32 comes in tot32 / bef32.
 // Returns T = largest level with #{S >= T} >= keep, r = keep - #{S > T}, and the numbers of tokens

@@ -146,8 +146,11 @@ __global__ void __launch_bounds__(kScanThreads) scan_score_kernel(const uint32_t
 }
 
 // Kernel 2: one chunk per CTA.  Sums the chunk histograms (total, and the part before its own
-// chunk), derives T, r and its output offset, then walks its chunk's score bytes (16 consecutive
-// tokens per thread and pass) and writes the selected token indices in ascending order.
+// chunk), derives T, r and its output offset, then walks its chunk's score bytes and writes the
+// selected token indices in ascending order, visiting only those.  A thread takes 16 kQuads consecutive tokens per pass: 32, so that
+// a chunk of 8192 tokens is one pass (one sequence of 524288 tokens 37.3 -> 36.7 us per step, of 300000 at 8x 53.9 -> 51.8), 16 for
+// the shortest chunks, where half of the threads would have nothing (200000 tokens in pages 27.9 / 28.6).
+template <int kQuads>
 __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__restrict__ seq_lens, int max_seq_len,
                                                              const int32_t *__restrict__ k_per_seq, int k_uniform,
                                                              int k_max, int Hkv, int chunk_tokens, long long score_row,
@@ -158,6 +161,7 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
                                                              int32_t *__restrict__ hist_out, Windows win) {
     __shared__ int s_wtot[kScanThreads / 32][kBins + 3], s_wbef[kScanThreads / 32][kBins + 3];
     __shared__ int warp_tot[kScanThreads / 32];
+    constexpr int kPer = 16 * kQuads, kPass = kScanThreads * kPer;   // tokens of a thread and of the CTA per pass
     const int chunk = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = max(min(seq_lens[b], max_seq_len), 0);
@@ -174,8 +178,12 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
     const uint4 *srow = reinterpret_cast<const uint4 *>(ws_scores + ((long long)b * Hkv + g) * score_row);
     const int start = chunk * chunk_tokens, end = min(n, start + chunk_tokens);
     // first pass of score bytes: requested now, used after the threshold is known
-    uint4 sv_next = make_uint4(0u, 0u, 0u, 0u);
-    if (chunk < n_chunks && start + tid * 16 < end) sv_next = __ldcg(srow + ((start + tid * 16) >> 4));
+    uint4 sv_next[kQuads];
+#pragma unroll
+    for (int h = 0; h < kQuads; ++h) {
+        const int base = start + tid * kPer + h * 16;
+        sv_next[h] = (chunk < n_chunks && base < end) ? __ldcg(srow + (base >> 4)) : make_uint4(0u, 0u, 0u, 0u);
+    }
 
     // totals per score level, and the part contributed by the chunks before this one.  Lane l of warp w sums
     // level l over the chunks w, w + 8, ... (coalesced rows of the counter table, every load issued before
@@ -236,23 +244,26 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
     const uint32_t c_gt = 0x7f7f7f7fu - T4, c_ge = 0x80808080u - T4;
     // tokens before this pass with S > T (always-kept tokens count as such) / S == T
     int run_gt = gt_before + forced_before(wbd, start), run_eq = eq_before;
-    for (int pass = start; pass < end; pass += kPassTokens) {
-        const int base = pass + tid * 16;
-        const uint4 sv = sv_next;
-        sv_next = make_uint4(0u, 0u, 0u, 0u);
-        if (base + kPassTokens < end) sv_next = __ldcg(srow + ((base + kPassTokens) >> 4));   // next pass, in flight
-        const uint32_t sw[4] = {sv.x, sv.y, sv.z, sv.w};
-        uint32_t gt16 = 0u, ge16 = 0u;   // bit i = token base + i
+    for (int pass = start; pass < end; pass += kPass) {
+        const int base = pass + tid * kPer;
+        uint32_t gt32 = 0u, ge32 = 0u;   // bit i = token base + i
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            // words past the chunk were never written: drop them (end is a multiple of 4 or the sequence end)
-            const uint32_t w = (base + 4 * j < end) ? sw[j] : 0u;
-            gt16 |= high_bits_to_nibble(w + c_gt) << (4 * j);
-            ge16 |= high_bits_to_nibble(w + c_ge) << (4 * j);
+        for (int h = 0; h < kQuads; ++h) {
+            const uint4 sv = sv_next[h];
+            const int next = base + kPass + h * 16;
+            sv_next[h] = next < end ? __ldcg(srow + (next >> 4)) : make_uint4(0u, 0u, 0u, 0u);   // next pass, in flight
+            const uint32_t sw[4] = {sv.x, sv.y, sv.z, sv.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                // words past the chunk were never written: drop them (end is a multiple of 4 or the sequence end)
+                const uint32_t w = (base + 16 * h + 4 * j < end) ? sw[j] : 0u;
+                gt32 |= high_bits_to_nibble(w + c_gt) << (16 * h + 4 * j);
+                ge32 |= high_bits_to_nibble(w + c_ge) << (16 * h + 4 * j);
+            }
         }
-        const uint32_t eq16 = ge16 ^ gt16;   // score > T implies score >= T
-        const int packed = __popc(gt16) | (__popc(eq16) << 16);
-        // block-wide exclusive prefix of the packed (gt, eq) counts (a pass has 4096 tokens: 16-bit halves suffice)
+        const uint32_t eq32 = ge32 ^ gt32;   // score > T implies score >= T
+        const int packed = __popc(gt32) | (__popc(eq32) << 16);
+        // block-wide exclusive prefix of the packed (gt, eq) counts (a pass has at most 8192 tokens: 16-bit halves suffice)
         int inc = packed;
 #pragma unroll
         for (int dd = 1; dd < 32; dd <<= 1) {
@@ -268,12 +279,8 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
             if (w < warp) wpre += v;
             all += v;
         }
-        if (packed != 0) {
-            const int excl = wpre + inc - packed;
-            int g_run = run_gt + (excl & 0xffff);
-            int q_run = run_eq + (int)((unsigned)excl >> 16);
-            write_selected32(out, base, gt16, eq16, g_run, q_run, r);
-        }
+        const int excl = wpre + inc - packed, q_run = run_eq + (int)((unsigned)excl >> 16);
+        write_exact32(out + run_gt + (excl & 0xffff) + min(q_run, r), base, gt32, eq32, r - q_run);
         run_gt += all & 0xffff;
         run_eq += (int)((unsigned)all >> 16);
         __syncthreads();   // warp_tot is rewritten by the next pass
@@ -977,11 +984,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
             for (int q = q_first; q < q_last; ++q) {
                 const uint2 f = flags[q];
                 const int here = __popc(f.y), first = first_tok + (q_lo + q) * 32;
-                uint32_t sel = f.x;
-                if (room >= here) sel |= f.y;
-                else for (uint32_t m = f.y; room > 0; --room) { sel |= m & (0u - m); m &= m - 1u; }   // the group in which the last one lies
+                dst = write_exact32(dst, first, f.x, f.y, room);
                 room -= here;
-                for (; sel; sel &= sel - 1u) *dst++ = first + __ffs((int)sel) - 1;
             }
         }
         if (!more) break;
@@ -1151,7 +1155,7 @@ static cudaError_t launch_g(int B, int Hq, int Hkv, const uint32_t *q_codes, con
     cudaError_t e = launch_pdl(scan_score_kernel<G>, grid, dim3(kScanThreads), 0, st, q_codes, k_codes, kc_sb, kc_sh,
                                seq_lens, max_seq_len, Hq, Hkv, chunk_tokens, score_row, ws_scores, ws_hist, win, cp, row_shift, in_step);
     if (e != cudaSuccess) return e;
-    e = launch_pdl(select_kernel, grid, dim3(kScanThreads), 0, st, seq_lens, max_seq_len, k_per_seq, k_uniform, k_max,
+    e = launch_pdl(chunk_tokens > kPassTokens ? select_kernel<2> : select_kernel<1>, grid, dim3(kScanThreads), 0, st, seq_lens, max_seq_len, k_per_seq, k_uniform, k_max,
                    Hkv, chunk_tokens, score_row, (const unsigned char *)ws_scores, (const int32_t *)ws_hist, idx, idx_sb,
                    idx_sh, count, hist_out, win);
     if (e != cudaSuccess) return e;
