@@ -536,11 +536,10 @@ __global__ void __launch_bounds__(kThreads, kThreads > 256 ? 2 : kPaged ? 5 : 6)
     }
     if (tot_packed != 0) {
         const int excl = winc - tot_packed;
-        int g_run = run_gt + (excl & 0xffff);
-        int q_run = run_eq + (int)((unsigned)excl >> 16);
-        const int first = (int)rank * kSlice * Rb + first_l;
-        write_selected32(out, first, gt_lo, eq_lo, g_run, q_run, r);
-        write_selected32(out, first + 32, gt_hi, eq_hi, g_run, q_run, r);
+        const int q_run = run_eq + (int)((unsigned)excl >> 16), first = (int)rank * kSlice * Rb + first_l;
+        int32_t *dst = out + run_gt + (excl & 0xffff) + min(q_run, r);
+        dst = write_exact32(dst, first, gt_lo, eq_lo, r - q_run);
+        write_exact32(dst, first + 32, gt_hi, eq_hi, r - q_run - __popc(eq_lo));
     }
     cluster_wait();
 }
