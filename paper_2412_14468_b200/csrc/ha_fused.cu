@@ -618,21 +618,30 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
             all_eq += wq;
         }
         const int excl = winc - tot_packed;
-        int g_run = run_gt + (excl & 0xffff), q_run = run_eq + (int)((unsigned)excl >> 16);
+        const int g_run = run_gt + (excl & 0xffff), q_run = run_eq + (int)((unsigned)excl >> 16);
+        const int pos = g_run + min(q_run, r);   // of this lane's first selected token
+        int room = r - q_run;                    // tokens at the threshold that are still wanted
         if (kLocalList) {
             const int pos0 = cta_gt + min(cta_eq, r), cnt = all_gt + min(all_eq, r) - pos0;   // this CTA's run of positions
+            int32_t *dst = s_sel + (pos - pos0);
 #pragma unroll
-            for (int w = 0; w < kFlagWords; ++w)
-                visit_selected32(wbase + 32 * w, gtw[w], eqw[w], g_run, q_run, r, [&](int pos, int t) { s_sel[pos - pos0] = t; });
+            for (int w = 0; w < kFlagWords; ++w) {
+                dst = write_exact32(dst, wbase + 32 * w, gtw[w], eqw[w], room);
+                room -= __popc(eqw[w]);
+            }
             __syncthreads();
             const int per_cta = bpc * kBlockTokens;
             for (int i = tid; i < cnt; i += kFusedThreads) {
-                const int pos = pos0 + i, owner = pos / per_cta;
-                st_dsmem_u32(reinterpret_cast<uint32_t *>(&s_list[pos - owner * per_cta]), (uint32_t)owner, (uint32_t)s_sel[i]);
+                const int at = pos0 + i, owner = at / per_cta;
+                st_dsmem_u32(reinterpret_cast<uint32_t *>(&s_list[at - owner * per_cta]), (uint32_t)owner, (uint32_t)s_sel[i]);
             }
         } else {
+            int32_t *dst = list + pos;
 #pragma unroll
-            for (int w = 0; w < kFlagWords; ++w) write_selected32(list, wbase + 32 * w, gtw[w], eqw[w], g_run, q_run, r);
+            for (int w = 0; w < kFlagWords; ++w) {
+                dst = write_exact32(dst, wbase + 32 * w, gtw[w], eqw[w], room);
+                room -= __popc(eqw[w]);
+            }
         }
     }
     cluster_sync_all();   // #3: the index list is complete and visible to the whole cluster
