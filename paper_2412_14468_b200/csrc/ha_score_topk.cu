@@ -1056,16 +1056,17 @@ static cudaError_t launch_batch_t(int B, int Hq, int Hkv, const uint32_t *q_code
 // CTAs per cluster of the batch kernel, 0: one of the other kernels.  What decides is how the units fill the clusters that are
 // resident at once (296 CTAs, 148 clusters of 2, 71 of 4, 33 of 8 on 148 SMs): the other kernels give every unit a cluster of its
 // own and pay its fixed part of 7 us in every wave, and beyond 131072 tokens two kernels and the way of the scores through global
-// memory.  Whole steps, 8 units a sequence, groups of 4, us with the kernels there were / with this one:
-//   ragged, clusters of 1   30 sequences of 10000 - 20000 tokens 40.7 / 39.3 (of 2: 40.4), 50 of 2000 - 30000 64.0 / 58.3 (60.4), 64 of
-//                           300 - 4000 48.8 / 46.5 (51.4); 28 of 2000 - 33000 44.3 / 44.1 (41.3), hence the line at 32768 tokens; 31 of
-//                           600 - 4500 28.9 / 29.6, 40 of 900 - 7000 34.1 / 33.6
-//   ragged, clusters of 2   13 of 2000 - 30000 30.8 / 28.9, 22 of 1000 - 20000 33.9 / 33.9, 26 of 4000 - 65000 64.8 / 60.5, 32 of 8192 -
-//                           131072 105.6 / 96.5, but 10 of 4000 - 60000 35.3 / 37.7 and 20 of 900 - 7000 27.1 / 29.8
-//   ... in pages of 16      24 of 20000 - 40000 55.9 / 53.7, 18 of 60000 - 130000 100.5 / 93.4; 16 of 2000 - 30000 29.6 / 30.1, 19 of 20000 -
-//                           40000 46.5 / 48.6; pages of 1 lose (10 of 10000 - 110000 75.8 / 98.0), so smaller pages stay out
-//   ragged, clusters of 4   9 of 20000 - 130000 46.1 / 44.1, 6 of 20000 - 140000 49.1 / 44.3; 10 in pages 49.2 / 50.9
-//   one length              64 of 1200 31.6 / 29.2, of 9000 46.7 / 44.4, but of 16000 59.8 / 60.1 and of 32768 92.2 / 95.2; 50 of 4000 32.8 / 33.7
+// memory.  Whole steps, 8 units a sequence, groups of 4, us with the other kernels / with this one:
+//   ragged, clusters of 1   38 sequences of 800 - 12000 tokens 45.5 / 44.8, 30 of 10000 - 20000 40.0 / 39.4 (of 2: 40.6), 50 of 2000 -
+//                           30000 62.4 / 58.4 (60.4), 64 of 300 - 4000 48.6 / 46.5 (51.4); 28 of 2000 - 33000 43.4 / 44.3 (41.5), hence
+//                           the line at 32768 tokens; 31 of 600 - 4500 28.9 / 29.6, 40 of 900 - 7000 34.1 / 33.6
+//   ... in pages of 16      50 of 2000 - 30000 68.4 / 64.0, 64 of 700 - 12000 64.2 / 60.0, but 40 of 6000 - 12000 39.8 / 40.7
+//   ragged, clusters of 2   24 of 2000 - 65536 63.6 / 60.8, 26 of 4000 - 65000 63.1 / 60.9, 32 of 8192 - 131072 102.2 / 96.1, but 22 of 1000 -
+//                           20000 33.5 / 34.1, 19 of 3000 - 90000 55.7 / 56.9
+//   ... in pages of 16      26 of 4000 - 65000 72.3 / 67.4, 16 of 50000 - 100000 74.1 / 71.9, 19 of 3000 - 90000 63.0 / 62.1; 16 of 2000 - 30000
+//                           29.1 / 29.8; pages of 1 lose (10 of 10000 - 110000 75.8 / 98.0), so smaller pages stay out
+//   ragged, clusters of 4   9 of 20000 - 130000 44.4 / 43.9, 6 of 20000 - 125000 45.4 / 42.2
+//   one length              64 of 1200 31.4 / 29.2, of 4000 34.9 / 33.4, of 9000 45.9 / 44.5, of 12000 51.3 / 51.4; 50 of 4000 32.8 / 33.7
 //   beyond 131072 tokens    4 of 300000 69.2 / 61.5, 8 of 150000 71.2 / 63.4, 10 of 160000 88.6 / 83.4, 23 of 10000 - 170000 147.6 / 92.0;
 //                           1 of 300000 30.7 / 32.1
 template <int G>
@@ -1089,10 +1090,10 @@ static int batch_cluster_size(long long units, int max_seq_len, bool ragged, con
     }
     int cs = 0;
     if (ragged) {
-        if (units >= 232 && max_seq_len <= 32768) cs = (max_seq_len > 8192 || units >= 464) ? 1 : 0;
-        else if (max_seq_len > 16384 && (units >= 184 || (units >= 104 && (!paged || max_seq_len > 49152)))) cs = 2;
+        if (units >= 232 && max_seq_len <= 32768) cs = (units >= 464 || (max_seq_len > 8192 && units >= (paged ? 384 : 232))) ? 1 : 0;
+        else if ((units >= 184 && max_seq_len > 16384) || (paged && units >= 104 && max_seq_len > 49152)) cs = 2;
         else if (units >= 40 && units < 72 && max_seq_len > 98304) cs = 4;
-    } else if (units >= 464 && max_seq_len <= 12288) {
+    } else if (units >= 464 && max_seq_len <= 10240) {
         cs = 1;
     }
     return cs && fits(cs) ? cs : 0;

@@ -130,9 +130,9 @@ def _batch_lens(n_seqs, longest):
     (4, 4, _batch_lens(58, 8193)),       # 232 units: one CTA a cluster, lengths sorted by one warp
     (1, 2, _batch_lens(240, 900)),       # 480 short units, lengths sorted by the CTA
     (2, 1, _batch_lens(700, 700)),       # more sequences than are sorted, more than eight units a cluster
-    (8, 4, _batch_lens(26, 16385)),      # 104 units: clusters of 2
-    (4, 8, _batch_lens(23, 16400)),      # 184 units: clusters of 2, also in pages
-    (4, 8, _batch_lens(13, 49153)),      # 104 units of more than 49152 tokens: clusters of 2, also in pages
+    (8, 8, _batch_lens(24, 16385)),      # 192 units: clusters of 2
+    (4, 8, _batch_lens(48, 8193)),       # 384 units: one CTA a cluster, also in pages
+    (4, 8, _batch_lens(13, 49153)),      # 104 units of more than 49152 tokens: clusters of 2 in pages
     (2, 2, _batch_lens(20, 98305)),      # 40 units of more than 98304 tokens: clusters of 4
     (4, 4, _batch_lens(12, 131073)),     # beyond the one-unit clusters: 48 units, clusters of 4
     (1, 2, _batch_lens(12, 262145)),     # 24 units beyond the large CTAs: clusters of 8
@@ -176,7 +176,7 @@ def test_score_topk_with_several_units_per_cluster(G, Hkv, lens, page_size):
 
 
 def test_score_topk_of_many_short_sequences_of_one_length():
-    """464 units of at most 12288 tokens, one budget: one CTA a cluster, two batches."""
+    """464 units of at most 10240 tokens, one budget: one CTA a cluster."""
     rng = np.random.default_rng(9)
     B, Hkv, G, n = 58, 8, 4, 1111
     codes = rng.integers(0, 2**32, size=(B, Hkv, 1112), dtype=np.uint64).astype(np.uint32)
