@@ -626,7 +626,7 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
             int32_t *dst = s_sel + (pos - pos0);
 #pragma unroll
             for (int w = 0; w < kFlagWords; ++w) {
-                dst = write_exact32(dst, wbase + 32 * w, gtw[w], eqw[w], room);
+                dst = write_selected32(dst, wbase + 32 * w, gtw[w], eqw[w], room);
                 room -= __popc(eqw[w]);
             }
             __syncthreads();
@@ -639,7 +639,7 @@ __global__ void __launch_bounds__(kFusedThreads, S == 1 ? 2 : 1) fused_step_kern
             int32_t *dst = list + pos;
 #pragma unroll
             for (int w = 0; w < kFlagWords; ++w) {
-                dst = write_exact32(dst, wbase + 32 * w, gtw[w], eqw[w], room);
+                dst = write_selected32(dst, wbase + 32 * w, gtw[w], eqw[w], room);
                 room -= __popc(eqw[w]);
             }
         }

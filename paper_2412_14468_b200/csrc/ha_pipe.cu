@@ -364,8 +364,8 @@ struct ScoreRole {
                 const int all = __shfl_sync(0xffffffffu, inc, 31);
                 if (packed != 0) {
                     const int excl = inc - packed;
-                    int g_run = run_gt + (excl & 0xffff), q_run = run_eq + (int)((unsigned)excl >> 16);
-                    write_selected32(list, first, gt, eq, g_run, q_run, r);
+                    const int g_run = run_gt + (excl & 0xffff), q_run = run_eq + (int)((unsigned)excl >> 16);
+                    write_selected32(list + g_run + min(q_run, r), first, gt, eq, r - q_run);
                 }
                 run_gt += all & 0xffff;
                 run_eq += (int)((unsigned)all >> 16);

@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
             all += v;
         }
         const int excl = wpre + inc - packed, q_run = run_eq + (int)((unsigned)excl >> 16);
-        write_exact32(out + run_gt + (excl & 0xffff) + min(q_run, r), base, gt32, eq32, r - q_run);
+        write_selected32(out + run_gt + (excl & 0xffff) + min(q_run, r), base, gt32, eq32, r - q_run);
         run_gt += all & 0xffff;
         run_eq += (int)((unsigned)all >> 16);
         __syncthreads();   // warp_tot is rewritten by the next pass
@@ -304,9 +304,8 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
 // shared-memory reductions: a lane only meets its own column, so an instruction never conflicts
 // with itself, and nothing waits for a result.
 // Writing: lane l owns the 8*Rb consecutive tokens l*8*Rb .. of its warp's range, so the prefix sums
-// need one warp-shuffle scan plus one exchange of eight warp totals; only flagged tokens are
-// visited, with plain integer arithmetic (the selection never queues behind the scoring for the
-// population-count unit).
+// need one warp-shuffle scan plus one exchange of eight warp totals; only selected tokens are
+// visited.
 
 constexpr int kClusterMaxRows = 8;   // rows of 8 tokens per lane: a lane's flags fit one 64-bit word each
 
@@ -538,8 +537,8 @@ __global__ void __launch_bounds__(kThreads, kThreads > 256 ? 2 : kPaged ? 5 : 6)
         const int excl = winc - tot_packed;
         const int q_run = run_eq + (int)((unsigned)excl >> 16), first = (int)rank * kSlice * Rb + first_l;
         int32_t *dst = out + run_gt + (excl & 0xffff) + min(q_run, r);
-        dst = write_exact32(dst, first, gt_lo, eq_lo, r - q_run);
-        write_exact32(dst, first + 32, gt_hi, eq_hi, r - q_run - __popc(eq_lo));
+        dst = write_selected32(dst, first, gt_lo, eq_lo, r - q_run);
+        write_selected32(dst, first + 32, gt_hi, eq_hi, r - q_run - __popc(eq_lo));
     }
     cluster_wait();
 }
@@ -983,7 +982,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
             for (int q = q_first; q < q_last; ++q) {
                 const uint2 f = flags[q];
                 const int here = __popc(f.y), first = first_tok + (q_lo + q) * 32;
-                dst = write_exact32(dst, first, f.x, f.y, room);
+                dst = write_selected32(dst, first, f.x, f.y, room);
                 room -= here;
             }
         }

@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kWideThreads) wide_write_kernel(const WideArgs
         if (packed != 0) {
             const int excl = wpre + inc - packed;
             const int g_run = run_gt + (excl & 0xffff), q_run = run_eq + (int)((unsigned)excl >> 16);
-            write_exact32(list + g_run + min(q_run, r), first, gt, eq, r - q_run);
+            write_selected32(list + g_run + min(q_run, r), first, gt, eq, r - q_run);
         }
         run_gt += all & 0xffff;
         run_eq += (int)((unsigned)all >> 16);
@@ -503,8 +503,8 @@ __global__ void __launch_bounds__(kWideThreads) wide_select_cluster_kernel(const
         g_run += excl & 0xffff;
         q_run += (int)((unsigned)excl >> 16);
         int32_t *dst = list + g_run + min(q_run, r);
-        dst = write_exact32(dst, base + first_l, gt_lo, eq_lo, r - q_run);
-        write_exact32(dst, base + first_l + 32, gt_hi, eq_hi, r - q_run - __popc(eq_lo));
+        dst = write_selected32(dst, base + first_l, gt_lo, eq_lo, r - q_run);
+        write_selected32(dst, base + first_l + 32, gt_hi, eq_hi, r - q_run - __popc(eq_lo));
     }
     cluster_wait();
 }
