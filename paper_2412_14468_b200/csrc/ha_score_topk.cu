@@ -1073,16 +1073,20 @@ static int batch_cluster_size(long long units, int max_seq_len, bool ragged, con
     const bool paged = cp.table != nullptr;
     if (paged && (cp.shift < 4 || cp.page_stride != (int)cp.page_stride)) return 0;
     auto fits = [&](int cs) { return kSelHist + ((max_seq_len + 127LL) / 128 + cs - 1) / cs * 128 <= kSelPool; };
+    auto resident = [&](int cs) -> long long {   // 0: the query failed, and one of the other kernels takes the call
+        if (cs == 1) return paged ? resident_batch_clusters<G, 1, true>() : resident_batch_clusters<G, 1, false>();
+        if (cs == 2) return paged ? resident_batch_clusters<G, 2, true>() : resident_batch_clusters<G, 2, false>();
+        if (cs == 4) return paged ? resident_batch_clusters<G, 4, true>() : resident_batch_clusters<G, 4, false>();
+        return paged ? resident_batch_clusters<G, 8, true>() : resident_batch_clusters<G, 8, false>();
+    };
     if (max_seq_len > kClusterMaxSeq) {
         if (units < 24 || units > 65536 || large_clusters(units, max_seq_len)) return 0;
-        const long long resident[4] = {0, paged ? resident_batch_clusters<G, 2, true>() : resident_batch_clusters<G, 2, false>(),
-                                       paged ? resident_batch_clusters<G, 4, true>() : resident_batch_clusters<G, 4, false>(),
-                                       paged ? resident_batch_clusters<G, 8, true>() : resident_batch_clusters<G, 8, false>()};
         int best = 0;
         long long best_cost = 0;
         for (int e = 1; e < 4; ++e) {   // units of the fullest cluster, per CTA
-            if (!fits(1 << e) || resident[e] <= 0) continue;
-            const long long cost = (units + resident[e] - 1) / resident[e] * (8 >> e);
+            const long long n = fits(1 << e) ? resident(1 << e) : 0;
+            if (n <= 0) continue;
+            const long long cost = (units + n - 1) / n * (8 >> e);
             if (!best || cost < best_cost) { best = 1 << e; best_cost = cost; }
         }
         return best;
@@ -1095,7 +1099,7 @@ static int batch_cluster_size(long long units, int max_seq_len, bool ragged, con
     } else if (units >= 464 && max_seq_len <= 10240) {
         cs = 1;
     }
-    return cs && fits(cs) ? cs : 0;
+    return cs && fits(cs) && resident(cs) > 0 ? cs : 0;
 }
 
 template <int G>
