@@ -105,6 +105,20 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
+
+// Opts a kernel in to `smem` bytes of dynamic shared memory and returns how many clusters of cfg's shape the current device holds
+// at once; 0: no answer.  A failure leaves no error behind, because another kernel then takes the call and its launcher ends in
+// cudaGetLastError().
+template <typename... KArgs>
+inline int ask_resident_clusters(void (*kernel)(KArgs...), const cudaLaunchConfig_t &cfg, int smem) {
+    int n = 0;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return n > 0 ? n : 0;
+}
 #endif
 
 void count_launch(int n = 1);

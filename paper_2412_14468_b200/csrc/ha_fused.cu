@@ -722,16 +722,11 @@ static int gather_cluster_prepare() {
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
     if (!clusters[dev]) {
-        if (cudaFuncSetAttribute(gather_cluster_kernel<G, CS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 gather_cluster_smem_bytes(G, CS)) != cudaSuccess)
-            return 0;
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[2];
         gather_cluster_config<G, CS>(cfg, attr, 1, 64, nullptr);
         cfg.numAttrs = 1;   // the cluster shape is all the occupancy query looks at
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, gather_cluster_kernel<G, CS>, &cfg) != cudaSuccess || n <= 0) return 0;
-        clusters[dev] = n;
+        clusters[dev] = ask_resident_clusters(gather_cluster_kernel<G, CS>, cfg, gather_cluster_smem_bytes(G, CS));
     }
     return clusters[dev];
 }
@@ -835,16 +830,11 @@ static int fused_prepare() {
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
     if (!clusters[dev]) {
-        if (cudaFuncSetAttribute(fused_step_kernel<G, S, CS, kMode, kMaxSeq>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 fused_smem_bytes(G, S, CS)) != cudaSuccess)
-            return 0;
         cudaLaunchConfig_t cfg;
         cudaLaunchAttribute attr[2];
         fused_config<G, S, CS>(cfg, attr, 1, 64, nullptr);
         cfg.numAttrs = 1;   // the cluster shape is all the occupancy query looks at
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, fused_step_kernel<G, S, CS, kMode, kMaxSeq>, &cfg) != cudaSuccess || n <= 0) return 0;
-        clusters[dev] = n;
+        clusters[dev] = ask_resident_clusters(fused_step_kernel<G, S, CS, kMode, kMaxSeq>, cfg, fused_smem_bytes(G, S, CS));
     }
     return clusters[dev];
 }

@@ -581,7 +581,10 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
                 size_t found = 0;
                 for (size_t kb = 8; kb <= 100 && !found; ++kb) {
                     int occ = 0;
-                    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, score_select_cluster_kernel<G, CS, kPaged, kThreads>, kThreads, kb * 1024) != cudaSuccess) break;
+                    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, score_select_cluster_kernel<G, CS, kPaged, kThreads>, kThreads, kb * 1024) != cudaSuccess) {
+                        cudaGetLastError();   // no cap, and no error of this query behind the launch
+                        break;
+                    }
                     if (occ <= cap) found = kb * 1024;
                 }
                 pad[dev][cap] = found ? found : 1;
@@ -1000,8 +1003,6 @@ static int resident_batch_clusters() {
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return 0;
     if (!cached[dev]) {
-        auto kernel = score_select_batch_kernel<G, CS, kPaged>;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSelPool) != cudaSuccess) return 0;
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(CS);
         cfg.blockDim = dim3(kSelThreads);
@@ -1013,9 +1014,7 @@ static int resident_batch_clusters() {
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n <= 0) return 0;
-        cached[dev] = n;
+        cached[dev] = ask_resident_clusters(score_select_batch_kernel<G, CS, kPaged>, cfg, kSelPool);
     }
     return cached[dev];
 }

@@ -538,12 +538,11 @@ static int wide_resident_clusters(int cs, int rows) {
     std::atomic<int> &k = known[dev][cs == 8 ? 2 : cs == 4 ? 1 : 0][rows];
     int n = k.load(std::memory_order_acquire);
     if (n > 0) return n;
-    if (cudaFuncSetAttribute(wide_select_cluster_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024) != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[2];
     wide_cluster_config<W>(cfg, attr, 1, 64, cs, rows, nullptr);
     cfg.numAttrs = 1;   // the cluster shape is all the occupancy query looks at
-    if (cudaOccupancyMaxActiveClusters(&n, wide_select_cluster_kernel<W>, &cfg) != cudaSuccess || n <= 0) return 0;
+    n = ask_resident_clusters(wide_select_cluster_kernel<W>, cfg, 64 * 1024);
     k.store(n, std::memory_order_release);
     return n;
 }
