@@ -5,8 +5,9 @@
 
 namespace ha {
 
-// Loaded from L2 (.cg): kernels overlap on an SM, and its L1 may hold a line that one of them fetched before a signature or a
-// table entry in it was written.
+// Loaded from L2 (.cg): a CTA may be resident while a kernel in front of it still writes signatures or table entries, and loads
+// through L1 as read-only data (ld.global.nc, __ldg) are only defined for memory that nobody writes as long as the kernel lives.
+// (On a B200 no such load behind griddepcontrol.wait returned an old value in 1.8 million, its line read before the wait or not.)
 __device__ __forceinline__ uint4 load_codes4(const uint32_t *row, int base, int n) {
     // tokens base..base+3 of a 16-byte aligned row; tokens >= n come back as don't-care zeros
     if (base + 3 < n) return __ldcg(reinterpret_cast<const uint4 *>(row + base));

@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(kThreads, kThreads > 256 ? 2 : kPaged ? 5 : 6)
         if (!kPaged) return row;
         const int t = wb + p * 256 + lane * 8;
         if (cp.shift < 3 || p >= Rb || t >= n) return row;
-        return row + (long long)__ldg(table_b + (t >> cp.shift)) * cp.page_stride - (t & ~((1 << cp.shift) - 1));
+        return row + (long long)__ldcg(table_b + (t >> cp.shift)) * cp.page_stride - (t & ~((1 << cp.shift) - 1));
     };
     auto load_row = [&](int p, const uint32_t *src_row, uint4 &lo, uint4 &hi, bool early) {
         const int t = wb + p * 256 + lane * 8;
@@ -783,7 +783,7 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
                 const int e0 = first >> cp.shift, e1 = (end + (1 << cp.shift) - 1) >> cp.shift;
                 int32_t *tab = reinterpret_cast<int32_t *>(pool + u.tab);
                 for (int e = e0 + tid; e < e1 && first < end; e += kSelThreads) {   // a page of one head is one run of bytes
-                    const int page = __ldg(table + e), t0 = max(e << cp.shift, first), t1 = min((e + 1) << cp.shift, end);
+                    const int page = __ldcg(table + e), t0 = max(e << cp.shift, first), t1 = min((e + 1) << cp.shift, end);
                     if (kPaged && staged) tab[e - e0] = page;
                     for (int t = t0; t < t1; t += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(in_page(row, page, t)));
                 }
@@ -831,7 +831,10 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
                     c[j] = make_uint4(0u, 0u, 0u, 0u);
                     if (at.p + j < at.p_end && t < at.n) {
                         if (kPaged && cp.shift < 2) c[j] = load_codes4_paged(cp, at.row, at.table, t, at.n);
-                        else if (kPaged) c[j] = load_codes4(in_page(at.row, at.table[(t >> cp.shift) - at.e0], t) - t, t, at.n);
+                        else if (kPaged) {
+                            const int32_t *entry = at.table + ((t >> cp.shift) - at.e0);   // in shared memory if staged
+                            c[j] = load_codes4(in_page(at.row, staged ? *entry : __ldcg(entry), t) - t, t, at.n);
+                        }
                         else c[j] = load_codes4(at.row, t, at.n);
                     }
                 }

@@ -15,6 +15,9 @@ RESIDENT = {1: 296, 2: 148, 4: 71, 8: 33}          # clusters of 512-thread CTAs
 PTR = 1 << 20                                       # an address that nothing looks behind
 BATCH = "score_select_batch_kernel"
 
+# (sequences, KV heads of one query head, tokens, CTAs per cluster): with one budget per sequence these take clusters of several units
+SEVERAL_UNITS_PER_CLUSTER = [(120, 4, 3001, 1), (62, 4, 33000, 2), (12, 4, 140001, 4), (6, 4, 270001, 8)]
+
 
 class Fake:
     def __init__(self, directory, name="fake"):

@@ -9,6 +9,7 @@ import torch
 import oracle
 from paper_2412_14468_b200 import binding as ha
 from paper_2412_14468_b200 import workloads as wl
+from tests._fake import SEVERAL_UNITS_PER_CLUSTER
 from tests._util import u16
 from tests.test_gpu_parity import _wide_mapping
 
@@ -20,7 +21,7 @@ K, REPEATS, PAGE = 16, 12, 16
 class _Calls:
     """One cache with heads of one query each, and the calls that append to it and scan it."""
 
-    def __init__(self, B, H, n, paged=False, bits=32):
+    def __init__(self, B, H, n, paged=False, bits=32, budgets=False):
         g = torch.Generator(DEV).manual_seed(B + n)
         rng = np.random.default_rng(n)
         self.B, self.H, self.n, self.W, self.bits, self.paged = B, H, n, bits // 64, bits, paged
@@ -28,6 +29,7 @@ class _Calls:
         self.q = torch.randn(B, H, 128, device=DEV, generator=g).to(torch.bfloat16)
         self.K = torch.randn(B, H, room, 128, device=DEV, generator=g).to(torch.bfloat16)
         self.lens = torch.full((B,), n, dtype=torch.int32, device=DEV)
+        self.budget = (torch.full((B,), K, dtype=torch.int32, device=DEV), 0) if budgets else (None, K)   # one per sequence, or one for all
         self.shape = ha.make_shape(B, H, H, 0.09)
         self.ws, self.ws_wide = ha.alloc_workspace(self.shape, n, K), ha.alloc_workspace_wide(self.shape, n)
         new = lambda *s, t=torch.int32: torch.zeros(*s, dtype=t, device=DEV)  # noqa: E731
@@ -78,14 +80,14 @@ class _Calls:
             self.step(slot + 1, self.q)
 
     def step(self, lens, k_new):
-        common = (lens, None, K, self.n, K, torch.zeros_like(self.q_codes), self.idx, self.cnt, self.out, self.ws)
+        common = (lens, *self.budget, self.n, K, torch.zeros_like(self.q_codes), self.idx, self.cnt, self.out, self.ws)
         if self.paged:
             ha.ha_sparse_decode_paged_codes(self.shape, self.map, self.map, self.q, k_new, self.K, self.K, self.codes, self.table, *common)
         else:
             ha.ha_sparse_decode(self.shape, self.map, self.map, self.q, k_new, self.K, self.K, self.codes, *common)
 
     def scan(self, how):
-        args = (self.lens, None, K)
+        args = (self.lens, *self.budget)
         if how == "step":
             self.step(self.lens, None)
         elif how == "wide":
@@ -132,6 +134,13 @@ def test_a_signature_written_into_a_page_directly_in_front_of_a_scan(B, n, scan,
     _run(_Calls(B, 4, n, paged=True), append, scan)
 
 
+@pytest.mark.parametrize("B,H,n,_cs", SEVERAL_UNITS_PER_CLUSTER)
+@pytest.mark.parametrize("paged,scan,append", [(False, "topk", "encode"), (False, "step", "step"), (False, "topk", "step"),
+                                               (True, "topk", "encode"), (True, "step", "step")])
+def test_a_signature_written_directly_in_front_of_clusters_of_several_units(B, H, n, _cs, paged, scan, append):
+    _run(_Calls(B, H, n, paged=paged, budgets=True), append, scan)
+
+
 @pytest.mark.parametrize("B,n", [(2, 20000), (20, 3001), (1, 140001)])
 @pytest.mark.parametrize("bits", [64, 256])
 def test_a_wide_signature_written_directly_in_front_of_its_selection(B, n, bits):
@@ -147,11 +156,12 @@ extern "C" __global__ void late_copy(const int *src, int *dst, int n) {
 }"""
 
 
-@pytest.mark.parametrize("B,n", [(2, 20000), (20, 3001), (1, 100003), (1, 262147)])
+@pytest.mark.parametrize("B,H,n,budgets", [(2, 4, 20000, False), (20, 4, 3001, False), (1, 4, 100003, False), (1, 4, 262147, False)] +
+                         [(B, H, n, True) for B, H, n, _ in SEVERAL_UNITS_PER_CLUSTER])
 @pytest.mark.parametrize("scan", ["topk", "step"])
-def test_a_block_table_is_read_behind_whatever_writes_it(B, n, scan):
+def test_a_block_table_is_read_behind_whatever_writes_it(B, H, n, budgets, scan):
     """The table names other pages of the same pool until the kernel in front has written it."""
-    c = _Calls(B, 4, n, paged=True)
+    c = _Calls(B, H, n, paged=True, budgets=budgets)
     late_copy = torch.cuda._compile_kernel(LATE_COPY, "late_copy")
     table = c.table
     slot = torch.full((B,), n // 2, dtype=torch.int32, device=DEV)
