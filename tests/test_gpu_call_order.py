@@ -192,3 +192,36 @@ def test_a_call_of_empty_sequences_between_the_two(n):
         c.scan("topk")
         c.check(slot)
     assert (cnt == 0).all()
+
+
+@pytest.mark.parametrize("B,n", [(2, 20000), (20, 3001), (1, 262147)])
+def test_a_prompt_is_encoded_over_signatures_that_the_call_in_front_still_scans(B, n):
+    """ha_encode_prefill starts while the selection in front of it runs, and overwrites the cache that it reads."""
+    c = _Calls(B, 4, n)
+    for r in range(REPEATS):
+        slot = torch.full((B,), 977 * r % n, dtype=torch.int32, device=DEV)
+        c.reset(slot)
+        c.append("encode", slot)
+        torch.cuda.synchronize()
+        c.scan("topk")
+        ha.ha_encode_prefill(c.map, 1, c.K, c.codes, workspace=c.ws)
+        c.check(slot)
+    assert ha.ha_read_device_status(c.ws) == 0
+
+
+@pytest.mark.parametrize("B,n", [(2, 20000), (1, 130), (3, 8192)])
+def test_a_prompt_is_encoded_behind_whatever_writes_its_tokens(B, n):
+    """The tokens are other ones until the kernel in front, which lets its dependents start at once, has written them."""
+    c = _Calls(B, 4, n)
+    late_copy = torch.cuda._compile_kernel(LATE_COPY, "late_copy")
+    want, x = torch.zeros_like(c.codes), torch.empty_like(c.K)
+    ha.ha_encode_prefill(c.map, 1, c.K, want, workspace=c.ws)
+    words, to = c.K.view(torch.int32), x.view(torch.int32)
+    for _ in range(3):
+        x.copy_(c.K.roll(1, 2))
+        c.codes.zero_()
+        torch.cuda.synchronize()
+        late_copy(grid=(1, 1, 1), block=(1024, 1, 1), args=[words, to, words.numel()])
+        ha.ha_encode_prefill(c.map, 1, x, c.codes, workspace=c.ws)
+        assert torch.equal(c.codes, want)
+    assert ha.ha_read_device_status(c.ws) == 0
