@@ -657,7 +657,9 @@ struct BatchUnit {
 constexpr int kSelThreads = 512, kSelWarps = kSelThreads / 32;
 constexpr int kSelUnits = 8;                          // units of a batch
 constexpr int kSelHist = kBins * 32 * 4;              // bytes of a unit's counters [level][lane]
-constexpr int kSelSort = 512;                         // sequences that are dealt out by length
+constexpr int kSelSort = 512;                         // sequences that are dealt out by length: at most one per thread
+constexpr int kSelStepBits = 6;                       // more than 64 sequences: by this many top bits of the longest length
+static_assert(kSelSort <= kSelThreads && (1 << kSelStepBits) * kSelWarps == 2 * kSelThreads, "a sequence and two counts per thread");
 constexpr int kSelPool = 96 * 1024;                   // counters, score bytes and table entries of a batch: two CTAs per SM
 
 // Bytes of a slice's entries of the block table (one more where the slice begins inside a page).
@@ -711,14 +713,39 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
             __syncwarp();
         }
     } else if (sorted) {
-        for (int i = tid; i < B; i += kSelThreads) { s_len[i] = len_of(i); s_k[i] = budget_of(i); }
+        // More of them: counting sort by the top bits of the length, one sequence per thread.  The counts [step][warp] lie in the
+        // pool, which nothing else uses yet.  Every CTA sorts all lengths for itself, and ranks by
+        // comparing every pair cost up to 15 us (whole steps, 2 heads, 1500 tokens: 256 sequences 32.9 us, now 29.2; 512 62.8, 48.1).
+        int *at = reinterpret_cast<int *>(pool);
+        const int mine = tid < B ? len_of(tid) : -1;
+        if (tid < B) { s_len[tid] = mine; s_k[tid] = budget_of(tid); }
+        reinterpret_cast<int2 *>(at)[tid] = make_int2(0, 0);
+        const int longest_here = __reduce_max_sync(0xffffffffu, mine);
+        if (lane == 0) s_wcnt[warp] = (uint32_t)max(longest_here, 0);
         __syncthreads();
-        for (int i = tid; i < B; i += kSelThreads) {
-            const int mine = s_len[i];
-            int at = 0;
-            for (int j = 0; j < B; ++j) at += (s_len[j] > mine || (s_len[j] == mine && j < i)) ? 1 : 0;
-            s_perm[at] = (uint16_t)i;
+        uint32_t longest = 0u;
+#pragma unroll
+        for (int w = 0; w < kSelWarps; ++w) longest = max(longest, s_wcnt[w]);
+        const int shift = max(0, 32 - kSelStepBits - __clz((int)longest));   // longest >> shift is the largest of 64 steps, or less
+        const int step = tid < B ? (1 << kSelStepBits) - 1 - (mine >> shift) : 1 << kSelStepBits;   // the longest first
+        const uint32_t same = __match_any_sync(0xffffffffu, step);
+        const int before = __popc(same & ((1u << lane) - 1u));
+        if (tid < B && before == 0) at[step * kSelWarps + warp] = __popc(same);
+        __syncthreads();
+        const int2 c = reinterpret_cast<const int2 *>(at)[tid];
+        int sum = c.x + c.y;
+#pragma unroll
+        for (int dd = 1; dd < 32; dd <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, sum, dd);
+            if (lane >= dd) sum += v;
         }
+        if (lane == 31) s_wcnt[warp] = (uint32_t)sum;
+        __syncthreads();
+        sum -= c.x + c.y;
+        for (int w = 0; w < warp; ++w) sum += (int)s_wcnt[w];
+        reinterpret_cast<int2 *>(at)[tid] = make_int2(sum, sum + c.x);
+        __syncthreads();
+        if (tid < B) s_perm[at[step * kSelWarps + warp] + before] = (uint16_t)tid;
         __syncthreads();
     }
     auto unit_of = [&](int j) -> int { return j * C + ((j & 1) ? C - 1 - cl : cl); };   // the cluster's j-th unit

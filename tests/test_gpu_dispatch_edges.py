@@ -129,7 +129,10 @@ def _batch_lens(n_seqs, longest):
 @pytest.mark.parametrize("G,Hkv,lens", [
     (4, 4, _batch_lens(58, 8193)),       # 232 units: one CTA a cluster, lengths sorted by one warp
     (1, 2, _batch_lens(240, 900)),       # 480 short units, lengths sorted by the CTA
-    (2, 1, _batch_lens(700, 700)),       # more sequences than are sorted, more than eight units a cluster
+    (1, 8, _batch_lens(65, 300)),        # 65 sequences: one more than one warp sorts
+    (1, 1, _batch_lens(512, 300)),       # 512: as many as are sorted
+    (1, 1, [0] * 511 + [1]),             # ... and hardly any step between their lengths
+    (2, 1, _batch_lens(700, 700)),       # more sequences than are sorted
     (8, 8, _batch_lens(24, 16385)),      # 192 units: clusters of 2
     (4, 8, _batch_lens(48, 8193)),       # 384 units: one CTA a cluster, also in pages
     (4, 8, _batch_lens(13, 49153)),      # 104 units of more than 49152 tokens: clusters of 2 in pages
