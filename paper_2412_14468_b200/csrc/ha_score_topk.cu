@@ -806,13 +806,16 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
             const int first = u.row0 * 128, end = min(u.n, (u.row0 + u.rows) * 128);
             if (kPaged) {
                 if (cp.shift < 2) continue;
+                // a page of one head is one run of bytes: a request per page of up to 32 tokens, or per 32 tokens of a larger one
+                // (a thread per page, whatever its size, left few threads with all requests of a slice: 24 sequences of 8192 - 65536 in
+                // pages of 65536, whole step 66.8 us, now 60.6, 48 of 4096 - 32768 in pages of 16384 67.9, now 63.9)
                 const int32_t *table = cp.table + (long long)u.b * cp.bt_sb;
-                const int e0 = first >> cp.shift, e1 = (end + (1 << cp.shift) - 1) >> cp.shift;
+                const int every = min(cp.shift, 5), e0 = first >> cp.shift;
                 int32_t *tab = reinterpret_cast<int32_t *>(pool + u.tab);
-                for (int e = e0 + tid; e < e1 && first < end; e += kSelThreads) {   // a page of one head is one run of bytes
-                    const int page = __ldcg(table + e), t0 = max(e << cp.shift, first), t1 = min((e + 1) << cp.shift, end);
-                    if (kPaged && staged) tab[e - e0] = page;
-                    for (int t = t0; t < t1; t += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(in_page(row, page, t)));
+                for (int t = first + (tid << every); t < end; t += kSelThreads << every) {   // first: a multiple of 128
+                    const int e = t >> cp.shift, page = __ldcg(table + e);
+                    if (staged && (t == first || t == e << cp.shift)) tab[e - e0] = page;
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(in_page(row, page, t)));
                 }
             } else {
                 for (int t = first + tid * 32; t < end; t += kSelThreads * 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + t));

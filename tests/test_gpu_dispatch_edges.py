@@ -141,7 +141,7 @@ def _batch_lens(n_seqs, longest):
     (1, 2, _batch_lens(12, 262145)),     # 24 units beyond the large CTAs: clusters of 8
     (1, 2, _batch_lens(12, 393000)),     # slices that leave no room for the block table
 ])
-@pytest.mark.parametrize("page_size", [0, 16, 128])
+@pytest.mark.parametrize("page_size", [0, 16, 128, 4096])
 def test_score_topk_with_several_units_per_cluster(G, Hkv, lens, page_size):
     """Every cluster size of the batch kernel at the edges of its rule: ragged lengths dealt out by length, several batches per
     cluster, windows, ties at the threshold, budgets of nothing and of everything, contiguous and in pages."""
