@@ -1084,54 +1084,71 @@ static cudaError_t launch_batch_t(int B, int Hq, int Hkv, const uint32_t *q_code
     return cudaGetLastError();
 }
 
-// CTAs per cluster of the batch kernel, 0: one of the other kernels.  What decides is how the units fill the clusters that are
-// resident at once (296 CTAs, 148 clusters of 2, 71 of 4, 33 of 8 on 148 SMs): the other kernels give every unit a cluster of its
-// own and pay its fixed part of 7 us in every wave, and beyond 131072 tokens two kernels and the way of the scores through global
-// memory.  Whole steps, 8 units a sequence, groups of 4, us with the other kernels / with this one:
-//   ragged, clusters of 1   38 sequences of 800 - 12000 tokens 45.5 / 44.8, 30 of 10000 - 20000 40.0 / 39.4 (of 2: 40.6), 50 of 2000 -
-//                           30000 62.4 / 58.4 (60.4), 64 of 300 - 4000 48.6 / 46.5 (51.4); 28 of 2000 - 33000 43.4 / 44.3 (41.5), hence
-//                           the line at 32768 tokens; 31 of 600 - 4500 28.9 / 29.6, 40 of 900 - 7000 34.1 / 33.6
-//   ... in pages of 16      50 of 2000 - 30000 68.4 / 64.0, 64 of 700 - 12000 64.2 / 60.0, but 40 of 6000 - 12000 39.8 / 40.7
-//   ragged, clusters of 2   24 of 2000 - 65536 63.6 / 60.8, 26 of 4000 - 65000 63.1 / 60.9, 32 of 8192 - 131072 102.2 / 96.1, but 22 of 1000 -
-//                           20000 33.5 / 34.1, 19 of 3000 - 90000 55.7 / 56.9
-//   ... in pages of 16      26 of 4000 - 65000 72.3 / 67.4, 16 of 50000 - 100000 74.1 / 71.9, 19 of 3000 - 90000 63.0 / 62.1; 16 of 2000 - 30000
-//                           29.1 / 29.8; pages of 1 lose (10 of 10000 - 110000 75.8 / 98.0), so smaller pages stay out
-//   ragged, clusters of 4   9 of 20000 - 130000 44.4 / 43.9, 6 of 20000 - 125000 45.4 / 42.2
-//   one length              64 of 1200 31.4 / 29.2, of 4000 34.9 / 33.4, of 9000 45.9 / 44.5, of 12000 51.3 / 51.4; 50 of 4000 32.8 / 33.7
-//   beyond 131072 tokens    4 of 300000 69.2 / 61.5, 8 of 150000 71.2 / 63.4, 10 of 160000 88.6 / 83.4, 23 of 10000 - 170000 147.6 / 92.0;
-//                           1 of 300000 30.7 / 32.1
+// CTAs per cluster of the batch kernel, 0: one of the other kernels.  Those give every unit a cluster of its own, pay its fixed part
+// of 7 us in every wave and size the cluster for max_seq_len, and beyond 131072 tokens they are two kernels with the scores in
+// global memory between them; but their CTAs leave one by one and make room for GATHER-ATT, and equal units fill them evenly.  So
+// this kernel wins where lengths differ, where max_seq_len is a capacity and where sequences are short; the lengths themselves are on
+// the device.  Lines by the clusters that are resident (296 of 1, 148 of 2, 71 of 4, 33 of 8 on 148 SMs).  Whole steps, gain of this
+// kernel over the others in percent, lengths from n / s to n with s = 1, 1.2, 2 and 16; 8 heads in groups of 4 where nothing else is said:
+//  * up to 10240 tokens, one CTA, whatever the lengths (s = 1, 1.2, 4, 16): 480 units of 1000 +5 +6 +5 +5, of 5000 +5 +3 +2 +3;
+//    1024 of 5000 +8 +7 +5 +5; 2048 of 1000 +11 +13 +14 +15.  Longer or in larger groups only if the CTAs are filled evenly: 512 of 8000
+//    +1 0 +2 +3, 592 of 10240 +1 +2 +5 +4, 1024 of 10240 +1 +4 +4 +4, but 464 of 8000 -2 0 +2 +1, 640 of 8192 -2 0 +4 +5; groups of 8: 512 of
+//    4000 0 +3 (s = 1, 4), of 8192 -3 +2; fewer units: 384 of 3000 -5 -5 -3 -3
+//  * up to 32768, where clusters of 2 hold a unit: 512 of 32768 -6 -5 -1 +3, 592 of 32768 -3 -2 0 +4, 384 of 16000 -4 -3 -1 +3, so never; except
+//    lists per query head (append, queries, lists, attention: 464 of 16000 +2 +3 +4 +4, 512 of 32768 0 +3 +2 +5; 1024 of 24000 -6 -2 0 +4)
+//  * beyond, clusters of 2, and only with one budget per sequence, the one sign of unequal lengths that the host has.  Up to 65536
+//    contiguous: 256 of 50000 +2 -1 0 +3, 296 of 65536 -1 -2 0 +2, but 192 of 50000 -5 -4 0 +3, 384 of 65536 -8 -6 -2 +2; in pages of 16: 192 of 50000
+//    +1 0 +2 +5, 296 of 65536 0 +1 +2 +3, 384 of 50000 -5 -3 +1 +4.  Up to 131072: 192 of 100000 -8 -3 +1 +4, 256 of 100000 -4 -3 +3 +8, 296 of 100000 0 0
+//    +4 +9; long equal units are given away here (256 of 131072 tokens are 17 GB of K and V in a layer) for wide ranges and for
+//    capacities: max_seq_len 131072, lengths of 500 - 2000 and 4000 - 16000: 192 units +12 +9, 256 +21 +18, 512 +31 +21.  In pages of 16,
+//    128 of 100000 +4 +4 +3 -2; 104 of 131072 -1 0 -2 -9, 160 of 100000 -14 -12 +2 +4.  Clusters of 4: 68 of 131072 in groups of 1, 4, 8
+//    +11 +8 +16 (s = 1) and +1 +3 +6 (16), 64 of 100000 +1 +1 -3 +1, but 40 of 131072 -9 -9 -7 -8, 56 -3 -2 -3 -3
+//  * beyond 131072 (s = 1, 1.3, 8): from 104 units on the smallest cluster that holds a unit, since sequences are short of such a capacity
+//    (120 of 140000 +9 +13 +16, 192 of 140000 +13 +18 +31, 136 of 300000 +11 +15 +28; lengths of 500 - 2000 in 200000 with clusters of 4
+//    -21 with 128 units, -34 with 512, hence the end at 3 units a cluster).  Fewer units: the size whose fullest cluster has the least
+//    to do, unless that is twice the even share (36 of 300000 -5 -3 +4; 32 +2 +5 +11, 40 +1 +3 +10, 56 +8 +10 +11), in groups of 8 1.6 times
+//    (40 of 300000 -6 -3 -1).
 template <int G>
-static int batch_cluster_size(long long units, int max_seq_len, bool ragged, const CodePages &cp) {
+static int batch_cluster_size(long long units, int max_seq_len, bool budgets, bool per_head, const CodePages &cp) {
     const bool paged = cp.table != nullptr;
-    if (paged && (cp.shift < 4 || cp.page_stride != (int)cp.page_stride)) return 0;
-    auto fits = [&](int cs) { return kSelHist + ((max_seq_len + 127LL) / 128 + cs - 1) / cs * 128 <= kSelPool; };
+    if (units < 24 || units > 65536 || (paged && (cp.shift < 4 || cp.page_stride != (int)cp.page_stride))) return 0;
+    const long long n = max_seq_len;
     auto resident = [&](int cs) -> long long {   // 0: the query failed, and one of the other kernels takes the call
         if (cs == 1) return paged ? resident_batch_clusters<G, 1, true>() : resident_batch_clusters<G, 1, false>();
         if (cs == 2) return paged ? resident_batch_clusters<G, 2, true>() : resident_batch_clusters<G, 2, false>();
         if (cs == 4) return paged ? resident_batch_clusters<G, 4, true>() : resident_batch_clusters<G, 4, false>();
         return paged ? resident_batch_clusters<G, 8, true>() : resident_batch_clusters<G, 8, false>();
     };
-    if (max_seq_len > kClusterMaxSeq) {
-        if (units < 24 || units > 65536 || large_clusters(units, max_seq_len)) return 0;
-        int best = 0;
-        long long best_cost = 0;
-        for (int e = 1; e < 4; ++e) {   // units of the fullest cluster, per CTA
-            const long long n = fits(1 << e) ? resident(1 << e) : 0;
-            if (n <= 0) continue;
-            const long long cost = (units + n - 1) / n * (8 >> e);
-            if (!best || cost < best_cost) { best = 1 << e; best_cost = cost; }
-        }
-        return best;
+    const long long c1 = resident(1), c2 = resident(2), c4 = resident(4);
+    if (c1 <= 0 || c2 <= 0 || c4 <= 0) return 0;
+    const bool many = 9 * units >= 14 * c1;   // for one CTA a unit
+    if (n <= 10240) {
+        const long long fullest = (units + c1 - 1) / c1;
+        const bool even = 6 * units >= 5 * fullest * c1;
+        return many && (n * G <= 20480 || (even && n * G <= 40960)) ? 1 : 0;
     }
-    int cs = 0;
-    if (ragged) {
-        if (units >= 232 && max_seq_len <= 32768) cs = (units >= 464 || (max_seq_len > 8192 && units >= (paged ? 384 : 232))) ? 1 : 0;
-        else if ((units >= 184 && max_seq_len > 16384) || (paged && units >= 104 && max_seq_len > 49152)) cs = 2;
-        else if (units >= 40 && units < 72 && max_seq_len > 98304) cs = 4;
-    } else if (units >= 464 && max_seq_len <= 10240) {
-        cs = 1;
+    if (n <= kClusterMaxSeq) {
+        if (!budgets) return 0;
+        if (n <= 32768) return per_head && many && units <= 2 * c1 ? 1 : 0;
+        if (n <= 65536) return (paged ? 5 * units >= 6 * c2 : 3 * units >= 5 * c2 && units <= 2 * c2) ? 2 : 0;
+        if (5 * units >= 6 * c2 || (paged && 6 * units >= 5 * c2 && units <= c2)) return 2;
+        return n > 98304 && 10 * units >= 9 * c4 && units <= c4 ? 4 : 0;
     }
-    return cs && fits(cs) && resident(cs) > 0 ? cs : 0;
+    if (large_clusters(units, max_seq_len)) return 0;
+    auto fits = [&](int cs) { return kSelHist + ((n + 127) / 128 + cs - 1) / cs * 128 <= kSelPool; };
+    if (10 * units >= 7 * c2) {
+        if (fits(2)) return 2;
+        return units > 3 * c4 ? 0 : fits(4) ? 4 : fits(8) && resident(8) > 0 ? 8 : 0;
+    }
+    int best = 0;
+    long long best_cost = 0;   // units of the fullest cluster, in eighths per CTA
+    for (int cs = 2; cs <= 8; cs *= 2) {
+        const long long c = fits(cs) ? resident(cs) : 0;
+        if (c <= 0) continue;
+        const long long cost = (units + c - 1) / c * (8 / cs);
+        if (!best || cost < best_cost) { best = cs; best_cost = cost; }
+    }
+    return 5 * best_cost * c1 <= (G == 8 ? 64 : 80) * units ? best : 0;
 }
 
 template <int G>
@@ -1145,7 +1162,7 @@ static cudaError_t launch_g(int B, int Hq, int Hkv, const uint32_t *q_codes, con
 #define HA_BATCH(CSZ) case CSZ: return cp.table ? launch_batch_t<G, CSZ, true>(HA_BATCH_ARGS) : launch_batch_t<G, CSZ, false>(HA_BATCH_ARGS)
 #define HA_BATCH_ARGS B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, idx, \
                       idx_sb, idx_sh, count, hist_out, st, win, cp, kv_shift, in_step
-        switch (batch_cluster_size<G>((long long)B * Hkv, max_seq_len, k_per_seq != nullptr, cp)) {
+        switch (batch_cluster_size<G>((long long)B * Hkv, max_seq_len, k_per_seq != nullptr, row_shift >= 0, cp)) {
             HA_BATCH(1);
             HA_BATCH(2);
             HA_BATCH(4);

@@ -1,23 +1,19 @@
 // A CUDA runtime that launches nothing: the library's objects are linked against it, so that the host side (which kernel takes a
 // call, with which grid, and what a failing query leaves behind) runs without a GPU.  Launches are recorded in order.
-#include <cstdint>
-#include <cstring>
 #include <map>
 #include <string>
 #include <vector>
 
 #include <cuda_runtime_api.h>
 
-struct Launch { std::string name; int grid[3], block, cluster; size_t smem; void **args; unsigned char last[32]; };
+struct Launch { std::string name; int ctas, cluster, smem, last; };
 static std::map<const void *, std::string> &names() { static std::map<const void *, std::string> n; return n; }
 static std::vector<Launch> launches;
 static cudaError_t last_error = cudaSuccess;
 static int cluster_answer[17], fail_queries = 0;
 
-static void record(const void *func, dim3 grid, dim3 block, int cluster, size_t smem, void **args, int n_args) {
-    Launch l{names()[func], {(int)grid.x, (int)grid.y, (int)grid.z}, (int)block.x, cluster, smem, args, {}};
-    if (args && n_args > 0) memcpy(l.last, args[n_args - 1], 1);
-    launches.push_back(l);
+static void record(const void *func, dim3 grid, int cluster, size_t smem, int last) {
+    launches.push_back(Launch{names()[func], (int)(grid.x * grid.y * grid.z), cluster, (int)smem, last});
 }
 
 extern "C" {
@@ -29,13 +25,13 @@ void __cudaRegisterVar(void **, char *, char *, const char *, int, size_t, int, 
 static dim3 c_grid, c_block; static size_t c_smem; static void *c_stream;
 unsigned __cudaPushCallConfiguration(dim3 g, dim3 b, size_t s, void *st) { c_grid = g; c_block = b; c_smem = s; c_stream = st; return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3 *g, dim3 *b, size_t *s, void *st) { *g = c_grid; *b = c_block; *s = c_smem; *(void **)st = c_stream; return cudaSuccess; }
-cudaError_t cudaLaunchKernel(const void *f, dim3 g, dim3 b, void **, size_t s, cudaStream_t) { record(f, g, b, 1, s, nullptr, 0); return cudaSuccess; }
+cudaError_t cudaLaunchKernel(const void *f, dim3 g, dim3, void **, size_t s, cudaStream_t) { record(f, g, 1, s, 0); return cudaSuccess; }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args) {
     int cluster = 1;
     for (unsigned i = 0; i < c->numAttrs; ++i)
         if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) cluster = c->attrs[i].val.clusterDim.x;
     const bool batch = names()[f].find("score_select_batch_kernel") != std::string::npos;
-    record(f, c->gridDim, c->blockDim, cluster, c->dynamicSmemBytes, args, batch ? 22 : 0);   // its last argument: table staged
+    record(f, c->gridDim, cluster, c->dynamicSmemBytes, batch ? *(const bool *)args[21] : 0);   // its last argument: table staged
     return cudaSuccess;
 }
 cudaError_t cudaGetLastError(void) { const cudaError_t e = last_error; last_error = cudaSuccess; return e; }
@@ -63,9 +59,9 @@ void fake_answers(int of1, int of2, int of4, int of8) { cluster_answer[1] = of1;
 void fake_fail_queries(int fail) { fail_queries = fail; }
 void fake_clear(void) { launches.clear(); last_error = cudaSuccess; }
 int fake_launches(void) { return (int)launches.size(); }
-const char *fake_launch(int i, int *grid, int *block, int *cluster, int *last_arg) {
+const char *fake_launch(int i, int *ctas, int *cluster, int *smem, int *last) {
     const Launch &l = launches[i];
-    *grid = l.grid[0] * l.grid[1] * l.grid[2]; *block = l.block; *cluster = l.cluster; *last_arg = l.last[0];
+    *ctas = l.ctas; *cluster = l.cluster; *smem = l.smem; *last = l.last;
     return l.name.c_str();
 }
 }

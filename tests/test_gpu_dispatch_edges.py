@@ -7,6 +7,7 @@ import torch
 import oracle
 from paper_2412_14468_b200 import binding as ha
 from paper_2412_14468_b200 import workloads as wl
+from tests._fake import BATCH_CASES, NEXT_TO_BATCH_CASES
 from tests._util import OUT_TOL, assert_out_close, max_abs_diff_bf16, u16
 from tests.test_gpu_parity import _attn_inputs, _check_gather, _run_step, _check_score_topk, _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
     test_whole_step_with_keys_values_and_signatures_all_paged as _whole_paged_step
@@ -118,33 +119,12 @@ def test_score_topk_on_clusters_of_large_ctas(G, lens, page_size):
             assert n_got[b, g] == len(ref) and np.array_equal(got[b, g, :len(ref)], ref) and (got[b, g, len(ref):] == -1).all()
 
 
-def _batch_lens(n_seqs, longest):
-    """Unequal lengths with the edges of a row of 128 tokens and of a group of 32 among them, not in order."""
-    edges = [0, 1, 31, 32, 33, 127, 128, 129, 255, 257]
-    step = max(1, longest // n_seqs)
-    lens = [max(1, longest - 3 - i * step) for i in range(n_seqs - len(edges) - 1)]
-    return edges[::2] + lens[::2] + [longest] + edges[1::2] + lens[1::2]
-
-
-@pytest.mark.parametrize("G,Hkv,lens", [
-    (4, 4, _batch_lens(58, 8193)),       # 232 units: one CTA a cluster, lengths sorted by one warp
-    (1, 2, _batch_lens(240, 900)),       # 480 short units, lengths sorted by the CTA
-    (1, 8, _batch_lens(65, 300)),        # 65 sequences: one more than one warp sorts
-    (1, 1, _batch_lens(512, 300)),       # 512: as many as are sorted
-    (1, 1, [0] * 511 + [1]),             # ... and hardly any step between their lengths
-    (2, 1, _batch_lens(700, 700)),       # more sequences than are sorted
-    (8, 8, _batch_lens(24, 16385)),      # 192 units: clusters of 2
-    (4, 8, _batch_lens(48, 8193)),       # 384 units: one CTA a cluster, also in pages
-    (4, 8, _batch_lens(13, 49153)),      # 104 units of more than 49152 tokens: clusters of 2 in pages
-    (2, 2, _batch_lens(20, 98305)),      # 40 units of more than 98304 tokens: clusters of 4
-    (4, 4, _batch_lens(12, 131073)),     # beyond the one-unit clusters: 48 units, clusters of 4
-    (1, 2, _batch_lens(12, 262145)),     # 24 units beyond the large CTAs: clusters of 8
-    (1, 2, _batch_lens(12, 393000)),     # slices that leave no room for the block table
-])
-@pytest.mark.parametrize("page_size", [0, 16, 128, 4096])
+@pytest.mark.parametrize("G,Hkv,lens,page_size", [(c[0], c[1], c[2], page) for c in BATCH_CASES + NEXT_TO_BATCH_CASES for page in c[3]],
+                         ids=lambda v: f"{len(v)}x{max(v)}" if isinstance(v, list) else None)
 def test_score_topk_with_several_units_per_cluster(G, Hkv, lens, page_size):
-    """Every cluster size of the batch kernel at the edges of its rule: ragged lengths dealt out by length, several batches per
-    cluster, windows, ties at the threshold, budgets of nothing and of everything, contiguous and in pages."""
+    """Every cluster size of the batch kernel at the edges of its rule, and the other kernels beside them: lengths dealt out,
+    several batches per cluster, windows, ties at the threshold, budgets of nothing and of everything, contiguous and in pages.
+    (test_dispatch.py holds the cases to their kernels, batches and staged tables.)"""
     rng = np.random.default_rng(len(lens) + page_size)
     B, Hq, n_cap = len(lens), Hkv * G, max(lens) // 128 * 128 + 128
     ks = [(0, n, max(1, n // 11), max(1, n // 40))[i % 4] if n < 3000 else n // 40 for i, n in enumerate(lens)]

@@ -213,10 +213,11 @@ def test_score_topk_long_sequences(lens, n_cap):
         _check_score_topk(qc, kc, lens, ks, Hq, Hkv)
 
 
-@pytest.mark.parametrize("B,Hkv,G,n_hi", [(16, 8, 4, 2100), (30, 8, 2, 9000), (40, 4, 4, 2100), (14, 8, 1, 30000)])
+@pytest.mark.parametrize("B,Hkv,G,n_hi", [(16, 8, 4, 2100), (30, 8, 2, 9000), (40, 4, 4, 2100), (14, 8, 1, 30000),
+                                          (10, 8, 1, 30000)])
 def test_score_topk_grids_that_are_launched_with_a_cap_on_ctas_per_sm(B, Hkv, G, n_hi):
     """Batches whose cluster grid needs fewer than six CTAs per SM are launched with padded shared memory (at most
-    ceil(CTAs / SMs) CTAs per SM): clusters of 4, 2, 4 and 8 here, ragged lengths, same lists as the oracle."""
+    ceil(CTAs / SMs) CTAs per SM): clusters of 4, 2, 4, 4 and 8 here, ragged lengths, same lists as the oracle."""
     rng = np.random.default_rng(500 + B)
     Hq = Hkv * G
     lens = [int(v) for v in rng.integers(1, n_hi, size=B)]
