@@ -649,7 +649,7 @@ __device__ __forceinline__ void group_flags(const unsigned char *group, uint32_t
 struct BatchUnit {
     int b, g, n, keep, keep_rest;   // sequence, head of the unit, tokens; list length, and the heavy tokens among it
     int row0, rows;                 // this CTA's rows of 128 tokens
-    int off, tab;                   // its score bytes and, pages of 16 tokens or more, its entries of the block table in the pool
+    int off, tab;                   // its score bytes and, where staged, its entries of the block table in the pool
     WindowBounds win;
     int T, r, gt_before, eq_before;
 };
@@ -665,8 +665,10 @@ constexpr int kSelPool = 96 * 1024;                   // counters, score bytes a
 // Bytes of a slice's entries of the block table (one more where the slice begins inside a page).
 __host__ __device__ constexpr int batch_table_bytes(int rows, int shift) { return ((rows * 128 >> shift) + 5) / 4 * 16; }
 
-// kPaged: the signatures lie in a pool behind a block table.  Pages of 4 tokens or more hold a lane's 4 tokens in one piece, so
-// a row costs one table entry per lane (neighbouring lanes share it) and the same 16-byte load.
+// Every cluster of the grid has a unit (launch_batch_t).
+// kPaged: the signatures lie in a pool behind a block table, in pages of 16 tokens or more (smaller ones lose, batch_cluster_size).
+// They hold a lane's 4 tokens in one piece, so a row costs one table entry per lane (neighbouring lanes share it) and the same
+// 16-byte load.
 template <int G, int CS, bool kPaged>
 __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
     const uint32_t *__restrict__ q_codes, const uint32_t *__restrict__ k_codes, long long kc_sb, long long kc_sh,
@@ -714,8 +716,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
         }
     } else if (sorted) {
         // More of them: counting sort by the top bits of the length, one sequence per thread.  The counts [step][warp] lie in the
-        // pool, which nothing else uses yet.  Every CTA sorts all lengths for itself, and ranks by
-        // comparing every pair cost up to 15 us (whole steps, 2 heads, 1500 tokens: 256 sequences 32.9 us, now 29.2; 512 62.8, 48.1).
+        // pool, which nothing else uses yet.  Every CTA sorts all lengths for itself, and ranks by comparing every pair cost up to
+        // 15 us (whole steps, 2 heads, 1500 tokens: 256 sequences 32.9 us, now 29.2; 512 62.8, 48.1).
         int *at = reinterpret_cast<int *>(pool);
         const int mine = tid < B ? len_of(tid) : -1;
         if (tid < B) { s_len[tid] = mine; s_k[tid] = budget_of(tid); }
@@ -805,7 +807,6 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
             const uint32_t *row = row_of(u);
             const int first = u.row0 * 128, end = min(u.n, (u.row0 + u.rows) * 128);
             if (kPaged) {
-                if (cp.shift < 2) continue;
                 // a page of one head is one run of bytes: a request per page of up to 32 tokens, or per 32 tokens of a larger one
                 // (a thread per page, whatever its size, left few threads with all requests of a slice: 24 sequences of 8192 - 65536 in
                 // pages of 65536, whole step 66.8 us, now 60.6, 48 of 4096 - 32768 in pages of 16384 67.9, now 63.9)
@@ -860,12 +861,12 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
                     const int t = at.tok + (at.p + j) * 128;
                     c[j] = make_uint4(0u, 0u, 0u, 0u);
                     if (at.p + j < at.p_end && t < at.n) {
-                        if (kPaged && cp.shift < 2) c[j] = load_codes4_paged(cp, at.row, at.table, t, at.n);
-                        else if (kPaged) {
+                        if (kPaged) {
                             const int32_t *entry = at.table + ((t >> cp.shift) - at.e0);   // in shared memory if staged
                             c[j] = load_codes4(in_page(at.row, staged ? *entry : __ldcg(entry), t) - t, t, at.n);
+                        } else {
+                            c[j] = load_codes4(at.row, t, at.n);
                         }
-                        else c[j] = load_codes4(at.row, t, at.n);
                     }
                 }
             };
@@ -1025,7 +1026,6 @@ __global__ void __launch_bounds__(kSelThreads, 2) score_select_batch_kernel(
         if (!more) break;
         __syncthreads();   // the pool and the descriptors are reused
     }
-    if (first_batch) pdl_wait();   // a cluster without units (never launched): at least one CTA of a grid waits
 }
 
 // The most clusters of a variant that are resident at once on the current device (0: the query failed).
@@ -1059,7 +1059,7 @@ static cudaError_t launch_batch_t(int B, int Hq, int Hkv, const uint32_t *q_code
                                     long long idx_sb, long long idx_sh, int32_t *count, int32_t *hist_out,
                                     cudaStream_t st, Windows win, CodePages cp, int kv_shift, bool in_step) {
     const int rows = ((max_seq_len + 127) / 128 + CS - 1) / CS;   // of the longest slice
-    const bool staged = kPaged && cp.shift >= 4 && kSelHist + rows * 128 + batch_table_bytes(rows, cp.shift) <= kSelPool;
+    const bool staged = kPaged && kSelHist + rows * 128 + batch_table_bytes(rows, cp.shift) <= kSelPool;
     const int most = resident_batch_clusters<G, CS, kPaged>();
     if (most <= 0) return cudaErrorInvalidConfiguration;
     cudaLaunchConfig_t cfg = {};
@@ -1087,27 +1087,31 @@ static cudaError_t launch_batch_t(int B, int Hq, int Hkv, const uint32_t *q_code
 // CTAs per cluster of the batch kernel, 0: one of the other kernels.  Those give every unit a cluster of its own, pay its fixed part
 // of 7 us in every wave and size the cluster for max_seq_len, and beyond 131072 tokens they are two kernels with the scores in
 // global memory between them; but their CTAs leave one by one and make room for GATHER-ATT, and equal units fill them evenly.  So
-// this kernel wins where lengths differ, where max_seq_len is a capacity and where sequences are short; the lengths themselves are on
-// the device.  Lines by the clusters that are resident (296 of 1, 148 of 2, 71 of 4, 33 of 8 on 148 SMs).  Whole steps, gain of this
-// kernel over the others in percent, lengths from n / s to n with s = 1, 1.2, 2 and 16; 8 heads in groups of 4 where nothing else is said:
-//  * up to 10240 tokens, one CTA, whatever the lengths (s = 1, 1.2, 4, 16): 480 units of 1000 +5 +6 +5 +5, of 5000 +5 +3 +2 +3;
-//    1024 of 5000 +8 +7 +5 +5; 2048 of 1000 +11 +13 +14 +15.  Longer or in larger groups only if the CTAs are filled evenly: 512 of 8000
-//    +1 0 +2 +3, 592 of 10240 +1 +2 +5 +4, 1024 of 10240 +1 +4 +4 +4, but 464 of 8000 -2 0 +2 +1, 640 of 8192 -2 0 +4 +5; groups of 8: 512 of
-//    4000 0 +3 (s = 1, 4), of 8192 -3 +2; fewer units: 384 of 3000 -5 -5 -3 -3
-//  * up to 32768, where clusters of 2 hold a unit: 512 of 32768 -6 -5 -1 +3, 592 of 32768 -3 -2 0 +4, 384 of 16000 -4 -3 -1 +3, so never; except
-//    lists per query head (append, queries, lists, attention: 464 of 16000 +2 +3 +4 +4, 512 of 32768 0 +3 +2 +5; 1024 of 24000 -6 -2 0 +4)
-//  * beyond, clusters of 2, and only with one budget per sequence, the one sign of unequal lengths that the host has.  Up to 65536
-//    contiguous: 256 of 50000 +2 -1 0 +3, 296 of 65536 -1 -2 0 +2, but 192 of 50000 -5 -4 0 +3, 384 of 65536 -8 -6 -2 +2; in pages of 16: 192 of 50000
-//    +1 0 +2 +5, 296 of 65536 0 +1 +2 +3, 384 of 50000 -5 -3 +1 +4.  Up to 131072: 192 of 100000 -8 -3 +1 +4, 256 of 100000 -4 -3 +3 +8, 296 of 100000 0 0
-//    +4 +9; long equal units are given away here (256 of 131072 tokens are 17 GB of K and V in a layer) for wide ranges and for
-//    capacities: max_seq_len 131072, lengths of 500 - 2000 and 4000 - 16000: 192 units +12 +9, 256 +21 +18, 512 +31 +21.  In pages of 16,
-//    128 of 100000 +4 +4 +3 -2; 104 of 131072 -1 0 -2 -9, 160 of 100000 -14 -12 +2 +4.  Clusters of 4: 68 of 131072 in groups of 1, 4, 8
-//    +11 +8 +16 (s = 1) and +1 +3 +6 (16), 64 of 100000 +1 +1 -3 +1, but 40 of 131072 -9 -9 -7 -8, 56 -3 -2 -3 -3
-//  * beyond 131072 (s = 1, 1.3, 8): from 104 units on the smallest cluster that holds a unit, since sequences are short of such a capacity
-//    (120 of 140000 +9 +13 +16, 192 of 140000 +13 +18 +31, 136 of 300000 +11 +15 +28; lengths of 500 - 2000 in 200000 with clusters of 4
-//    -21 with 128 units, -34 with 512, hence the end at 3 units a cluster).  Fewer units: the size whose fullest cluster has the least
-//    to do, unless that is twice the even share (36 of 300000 -5 -3 +4; 32 +2 +5 +11, 40 +1 +3 +10, 56 +8 +10 +11), in groups of 8 1.6 times
-//    (40 of 300000 -6 -3 -1).
+// this kernel wins where lengths differ, where max_seq_len is a capacity and where sequences are short.  The lengths themselves are
+// on the device.  The lines are in clusters resident at once: 296 of 1, 148 of 2, 71 of 4, 33 of 8 on 148 SMs.
+// Gain of this kernel over the others in a whole step in percent, with lengths from n / s to n, for four spreads s: 1, 1.1 - 1.3,
+// 2 - 4, 8 - 16; 8 heads in groups of 4 where nothing else is said, "480 of 1000" = 480 units with n = 1000:
+//  * up to 10240 tokens, one CTA, whatever the lengths: 480 of 1000 +5 +6 +5 +5, of 5000 +5 +3 +2 +3; 1024 of 5000 +8 +7 +5 +5;
+//    2048 of 1000 +11 +13 +14 +15; but 384 of 3000 -5 -5 -5 -3.  Longer, or in larger groups, only where the CTAs are filled
+//    evenly: 512 of 8000 +1 0 +2 +3, 560 of 10240 +1 +2 +5 +4, 1024 of 10240 +1 +4 +4 +4, but 464 of 8000 -2 0 +2 +1, 640 of 8192 -2 0 +4 +5;
+//    in groups of 8, 512 of 4000 0 and +3 (s = 1, 4), of 8192 -3 and +2
+//  * up to 32768, where clusters of 2 hold a unit, never: 512 of 32768 -6 -5 -1 +3, 592 of 32768 -3 -2 0 +4, 384 of 16000 -4 -3 -1 +3.
+//    Except lists per query head (append, queries, lists, attention): 464 of 16000 +2 +3 +4 +4, 512 of 32768 0 +3 +2 +5, but
+//    1024 of 24000 -6 -2 0 +4
+//  * beyond, clusters of 2, and only with one budget per sequence, the one sign of unequal lengths that the host has.  Up to 65536,
+//    contiguous: 256 of 50000 +2 -1 0 +3, 296 of 65536 -1 -2 0 +2, but 192 of 50000 -5 -4 0 +3, 384 of 65536 -8 -6 -2 +2; in pages of
+//    16: 192 of 50000 +1 0 +2 +5, 296 of 65536 0 +1 +2 +3, 384 of 50000 -5 -3 +1 +4.  Up to 131072: 192 of 100000 -8 -3 +1 +4, 256 of
+//    100000 -4 -3 +3 +8, 296 of 100000 0 0 +4 +9.  Long units of one length are given away here (256 of 131072 tokens are 17 GB of K
+//    and V in a layer) for wide ranges and for capacities: n = 131072, but lengths of 500 - 2000 and of 4000 - 16000: 192 units +12
+//    and +9, 256 +21 and +18, 512 +31 and +21.  In pages of 16, 128 of 100000 +4 +4 +3 -2, but 104 of 131072 -1 0 -2 -9, 160 of 100000
+//    -14 -12 +2 +4.  Clusters of 4: 68 of 131072 in groups of 1, 4 and 8 +11, +8, +16 (s = 1) and +1, +3, +6 (s = 16), 64 of 100000
+//    +1 +1 -3 +1, but 40 of 131072 -9 -9 -7 -8, 56 -3 -2 -3 -3
+//  * beyond 131072, three spreads, 1, 1.3 and 8.  From 104 units on the smallest cluster that holds a unit, as sequences are short of
+//    such a capacity: 120 of 140000 +9 +13 +16, 192 of 140000 +13 +18 +31, 136 of 300000 +11 +15 +28; lengths of 500 - 2000 in 200000
+//    with clusters of 4 -21 with 128 units, -34 with 512, hence the end at 3 units a cluster.  Fewer units: the size whose fullest
+//    cluster has the least to do, unless that is twice the even share (36 of 300000 -5 -3 +4; 32 +2 +5 +11, 40 +1 +3 +10, 56 +8 +10
+//    +11), or 1.6 times in groups of 8 (40 of 300000 -6 -3 -1)
+//  * pages of fewer than 16 tokens never: 10 sequences of 10000 - 110000 in pages of 1 75.8 us per step, 98.0 here.
 template <int G>
 static int batch_cluster_size(long long units, int max_seq_len, bool budgets, bool per_head, const CodePages &cp) {
     const bool paged = cp.table != nullptr;
