@@ -76,6 +76,9 @@ NEXT_TO_BATCH_CASES = [
     (1, 8, [200] * 26 + [200000], (0, 16)),          # 216 short units in a capacity that takes clusters of 4
 ]
 
+# lists per query head over pages: (sequences, KV heads, group size, longest, CTAs per cluster)
+PER_HEAD_BATCH_CASES = [(58, 2, 4, 900, 1), (15, 8, 4, 12000, 1), (37, 8, 2, 32768, 1), (23, 2, 4, 40000, 2), (13, 4, 2, 140000, 2)]
+
 
 def batches(Hkv, lens, cs, clusters, page=0, staged=False, most=8, pool=96 * 1024):
     """Batches of the busiest cluster: units by falling length, dealt out forth and back, as many at a time as fit the pool."""

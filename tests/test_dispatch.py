@@ -2,7 +2,7 @@
 import pytest
 
 from paper_2412_14468_b200 import binding as ha
-from tests._fake import BATCH, BATCH_CASES, NEXT_TO_BATCH_CASES, RESIDENT, SEVERAL_UNITS_PER_CLUSTER, Fake, batches
+from tests._fake import BATCH, BATCH_CASES, NEXT_TO_BATCH_CASES, PER_HEAD_BATCH_CASES, RESIDENT, SEVERAL_UNITS_PER_CLUSTER, Fake, batches
 
 
 def test_a_failing_occupancy_query_leaves_no_error_behind(tmp_path):
@@ -50,6 +50,13 @@ def test_cases_beside_clusters_of_several_units(fake, case):
     for page in pages:
         assert fake.score_topk(len(lens), G, Hkv, max(lens), page=page) == ha.HA_OK
         assert BATCH not in [k for k, *_ in fake.launches()], page
+
+
+@pytest.mark.parametrize("B,Hkv,G,longest,cs", PER_HEAD_BATCH_CASES)
+def test_cases_of_lists_per_query_head_on_clusters_of_several_units(fake, B, Hkv, G, longest, cs):
+    assert fake.score_topk(B, G, Hkv, longest, page=16, per_head=True) == ha.HA_OK
+    (kernel, args, ctas, cluster, *_), = fake.launches()
+    assert kernel == BATCH and args == [1, cs, 1] and cluster == cs and ctas == cs * min(RESIDENT[cs], B * Hkv * G)
 
 
 @pytest.mark.parametrize("page", [0, 16, 64])

@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_2412_14468_b200 import binding as ha
 from paper_2412_14468_b200 import workloads as wl
-from tests._fake import BATCH_CASES, NEXT_TO_BATCH_CASES
+from tests._fake import BATCH_CASES, NEXT_TO_BATCH_CASES, PER_HEAD_BATCH_CASES, ragged
 from tests._util import OUT_TOL, assert_out_close, max_abs_diff_bf16, u16
 from tests.test_gpu_parity import _attn_inputs, _check_gather, _run_step, _check_score_topk, _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
     test_whole_step_with_keys_values_and_signatures_all_paged as _whole_paged_step
@@ -156,6 +156,32 @@ def test_score_topk_with_several_units_per_cluster(G, Hkv, lens, page_size):
             ref = oracle.topk_windows(s, ks[b], n_sink, n_local)
             assert n_got[b, g] == len(ref) and np.array_equal(got[b, g, :len(ref)], ref) and (got[b, g, len(ref):] == -1).all()
             assert np.array_equal(h_got[b, g], np.bincount(s[free], minlength=33))
+
+
+@pytest.mark.parametrize("B,Hkv,G,longest,_cs", PER_HEAD_BATCH_CASES)
+@pytest.mark.parametrize("page_size", [16, 64])
+def test_score_topk_per_head_with_several_units_per_cluster(B, Hkv, G, longest, _cs, page_size):
+    """Lists per query head over pages: G units share the signatures of a KV head."""
+    rng = np.random.default_rng(B + page_size)
+    lens = ragged(B, longest)
+    ks = [max(1, n // 30) for n in lens]
+    k_max, Hq = max(ks), Hkv * G
+    codes = rng.integers(0, 2**32, size=(B, Hkv, longest), dtype=np.uint64).astype(np.uint32)
+    codes[:, :, 100:400] = codes[:, :, 100:101]                     # ties decided by token index
+    qc = rng.integers(0, 2**32, size=(B, Hq), dtype=np.uint64).astype(np.uint32)
+    pool, table = _page_codes(codes, lens, page_size, rng)
+    shape = ha.make_shape(B, Hq, Hkv, 1.0)
+    ws = ha.alloc_workspace(ha.make_shape(B, Hq, Hq, 1.0), longest, k_max)
+    idx = torch.full((B, Hq, k_max), 5, dtype=torch.int32, device=DEV)
+    cnt = torch.full((B, Hq), 5, dtype=torch.int32, device=DEV)
+    to = lambda a: torch.from_numpy(a.view(np.int32)).to(DEV)  # noqa: E731
+    ha.ha_score_topk_per_head_paged(shape, to(qc), to(pool), to(table), torch.tensor(lens, dtype=torch.int32, device=DEV),
+                                    torch.tensor(ks, dtype=torch.int32, device=DEV), 0, longest, k_max, idx, cnt, ws)
+    got, n_got = idx.cpu().numpy(), cnt.cpu().numpy()
+    for b, n in enumerate(lens):
+        for h in range(Hq):
+            ref = oracle.topk(oracle.score(qc[b, h:h + 1], codes[b, h // G, :n]) if n else np.zeros(0, np.int32), ks[b])
+            assert n_got[b, h] == len(ref) and np.array_equal(got[b, h, :len(ref)], ref) and (got[b, h, len(ref):] == -1).all()
 
 
 def test_score_topk_of_many_short_sequences_of_one_length():
