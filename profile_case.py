@@ -53,16 +53,23 @@ def score_only(args):
     cfg = wl.CONFIGS[args.config]
     B = args.batch if args.batch is not None else cfg.batch
     n, k = cfg.n, cfg.k
-    assert n is not None, "score-only runs need a config with one fixed length"
     dev = "cuda:0"
     torch.cuda.set_device(0)
+    if args.lengths:     # ragged: one length and one budget per sequence
+        lo, n = args.lengths
+        lens = torch.randint(lo, n + 1, (B,), generator=torch.Generator("cpu").manual_seed(wl.BASE_SEED)).tolist()
+        k = max(1, n // cfg.sparsity)
+        budgets = torch.tensor([max(1, v // cfg.sparsity) for v in lens], dtype=torch.int32, device=dev)
+    else:
+        assert n is not None, "score-only runs need a config with one fixed length, or --lengths"
+        lens, budgets = [n] * B, None
     Hq, Hkv = cfg.n_q_heads, cfg.n_kv_heads
     g = torch.Generator(dev).manual_seed(wl.BASE_SEED + 77)
-    kc = torch.randint(-2**31, 2**31 - 1, (B, Hkv, n), dtype=torch.int32, device=dev, generator=g)
+    kc = torch.randint(-2**31, 2**31 - 1, (B, Hkv, -(-n // 4) * 4), dtype=torch.int32, device=dev, generator=g)
     qc = torch.randint(-2**31, 2**31 - 1, (B, Hq), dtype=torch.int32, device=dev, generator=g)
     shape = ha.make_shape(B, Hq, Hkv, 1.0)
     ws = ha.alloc_workspace(shape, n, k, device=dev)
-    lens = torch.full((B,), n, dtype=torch.int32, device=dev)
+    tokens, lens = sum(lens), torch.tensor(lens, dtype=torch.int32, device=dev)
     idx = torch.zeros(B, Hkv, k, dtype=torch.int32, device=dev)
     cnt = torch.zeros(B, Hkv, dtype=torch.int32, device=dev)
     flush = torch.zeros(256 << 20, dtype=torch.uint8, device=dev)
@@ -72,7 +79,7 @@ def score_only(args):
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         torch.cuda._sleep(200000)   # the GPU is busy while the host enqueues: the events bracket the kernels only
         e0.record()
-        ha.ha_score_topk(shape, qc, kc, lens, None, k, n, k, idx, cnt, ws)
+        ha.ha_score_topk(shape, qc, kc, lens, budgets, k, n, k, idx, cnt, ws)
         e1.record()
         torch.cuda.synchronize()
         print(f"step {s}: {e0.elapsed_time(e1) * 1e3:.1f} us (plain launch, L2 flushed)")
@@ -81,11 +88,11 @@ def score_only(args):
             e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             torch.cuda._sleep(200000)
             e0.record()
-            ha.ha_score_topk_sum(shape, qc, kc, lens, None, k, k, idx, cnt)
+            ha.ha_score_topk_sum(shape, qc, kc, lens, budgets, k, k, idx, cnt)
             e1.record()
             torch.cuda.synchronize()
             print(f"step {s} summed group scores: {e0.elapsed_time(e1) * 1e3:.1f} us (plain launch, L2 flushed)")
-    print("signature bytes per step:", B * Hkv * n * 4)
+    print("signature bytes per step:", tokens * Hkv * 4)
 
 
 def score_wide(args):
@@ -194,6 +201,8 @@ def main():
                          "its split-K kernel also where few units with short rows would get the cluster kernel")
     ap.add_argument("--score-only", action="store_true",
                     help="SCORE + TOPK alone on random signatures (no K/V allocated: large batches stay small)")
+    ap.add_argument("--lengths", type=int, nargs=2, metavar=("LO", "HI"), default=None,
+                    help="with --score-only: sequences of LO to HI tokens, each with a budget of its own")
     ap.add_argument("--group-sum", action="store_true",
                     help="with --score-only: also run ha_score_topk_sum (per-head scores added instead of maximised)")
     ap.add_argument("--score-wide", action="store_true",
