@@ -148,8 +148,10 @@ __global__ void __launch_bounds__(kScanThreads) scan_score_kernel(const uint32_t
 // Kernel 2: one chunk per CTA.  Sums the chunk histograms (total, and the part before its own
 // chunk), derives T, r and its output offset, then walks its chunk's score bytes and writes the
 // selected token indices in ascending order, visiting only those.  A thread takes 16 kQuads consecutive tokens per pass: 32, so that
-// a chunk of 8192 tokens is one pass (one sequence of 524288 tokens 37.3 -> 36.7 us per step, of 300000 at 8x 53.9 -> 51.8), 16 for
-// the shortest chunks, where half of the threads would have nothing (200000 tokens in pages 27.9 / 28.6).
+// a chunk of 8192 tokens is one pass (one sequence of 524288 tokens 39.7 -> 38.3 us per step, of 300000 at 8x 53.2 -> 50.7), but 16
+// of what is one pass of those anyway, where half of the threads would have nothing: the rest of a long sequence, all of a short one
+// (256 units of 500 - 2000 tokens in a max_seq_len of 200000 30.1 us with 32, 29.3), and the shortest chunks, for which the kernel is
+// compiled without the second half (one sequence of 200000 25.3 with it, 24.9).
 template <int kQuads>
 __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__restrict__ seq_lens, int max_seq_len,
                                                              const int32_t *__restrict__ k_per_seq, int k_uniform,
@@ -161,7 +163,6 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
                                                              int32_t *__restrict__ hist_out, Windows win) {
     __shared__ int s_wtot[kScanThreads / 32][kBins + 3], s_wbef[kScanThreads / 32][kBins + 3];
     __shared__ int warp_tot[kScanThreads / 32];
-    constexpr int kPer = 16 * kQuads, kPass = kScanThreads * kPer;   // tokens of a thread and of the CTA per pass
     const int chunk = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int n = max(min(seq_lens[b], max_seq_len), 0);
@@ -177,12 +178,14 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
 
     const uint4 *srow = reinterpret_cast<const uint4 *>(ws_scores + ((long long)b * Hkv + g) * score_row);
     const int start = chunk * chunk_tokens, end = min(n, start + chunk_tokens);
+    const int quads = end - start > kPassTokens ? kQuads : 1;              // CTA-uniform
+    const int per = 16 * quads, pass_tokens = kScanThreads * per;          // tokens of a thread and of the CTA per pass
     // first pass of score bytes: requested now, used after the threshold is known
     uint4 sv_next[kQuads];
 #pragma unroll
     for (int h = 0; h < kQuads; ++h) {
-        const int base = start + tid * kPer + h * 16;
-        sv_next[h] = (chunk < n_chunks && base < end) ? __ldcg(srow + (base >> 4)) : make_uint4(0u, 0u, 0u, 0u);
+        const int base = start + tid * per + h * 16;
+        sv_next[h] = (chunk < n_chunks && base < end && h < quads) ? __ldcg(srow + (base >> 4)) : make_uint4(0u, 0u, 0u, 0u);
     }
 
     // totals per score level, and the part contributed by the chunks before this one.  Lane l of warp w sums
@@ -244,14 +247,14 @@ __global__ void __launch_bounds__(kScanThreads) select_kernel(const int32_t *__r
     const uint32_t c_gt = 0x7f7f7f7fu - T4, c_ge = 0x80808080u - T4;
     // tokens before this pass with S > T (always-kept tokens count as such) / S == T
     int run_gt = gt_before + forced_before(wbd, start), run_eq = eq_before;
-    for (int pass = start; pass < end; pass += kPass) {
-        const int base = pass + tid * kPer;
+    for (int pass = start; pass < end; pass += pass_tokens) {
+        const int base = pass + tid * per;
         uint32_t gt32 = 0u, ge32 = 0u;   // bit i = token base + i
 #pragma unroll
         for (int h = 0; h < kQuads; ++h) {
             const uint4 sv = sv_next[h];
-            const int next = base + kPass + h * 16;
-            sv_next[h] = next < end ? __ldcg(srow + (next >> 4)) : make_uint4(0u, 0u, 0u, 0u);   // next pass, in flight
+            const int next = base + pass_tokens + h * 16;
+            sv_next[h] = (next < end && h < quads) ? __ldcg(srow + (next >> 4)) : make_uint4(0u, 0u, 0u, 0u);   // next pass, in flight
             const uint32_t sw[4] = {sv.x, sv.y, sv.z, sv.w};
 #pragma unroll
             for (int j = 0; j < 4; ++j) {

@@ -73,7 +73,7 @@ NEXT_TO_BATCH_CASES = [
     (4, 4, ragged(17, 98304), (0,)),
     (1, 3, ragged(12, 262145), (0, 16)),             # 36 units beyond 131072 tokens: two rounds of few clusters
     (8, 4, [140000] * 9 + [1], (0,)),                # 40 units in groups of 8
-    (1, 8, [200] * 26 + [200000], (0, 16)),          # 216 short units in a capacity that takes clusters of 4
+    (1, 8, [200, 4095, 4096, 4097, 0] * 5 + [8193, 200000], (0, 16)),   # 216 short units in a capacity that takes clusters of 4
 ]
 
 # lists per query head over pages: (sequences, KV heads, group size, longest, CTAs per cluster)
