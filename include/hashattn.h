@@ -154,7 +154,9 @@ int ha_encode_prefill(const ha_mapping *map, int32_t heads_per_kv, const ha_tens
  *   q_codes    u32 [batch][n_q_heads]
  *   k_codes    u32 [batch][n_kv_heads][>= seq_len], token-contiguous, rows 16-byte aligned
  *   seq_lens   i32 [batch]
- *   k_per_seq  i32 [batch] or NULL (then k_uniform is used for every sequence)
+ *   k_per_seq  i32 [batch] or NULL (then k_uniform is used for every sequence).  Beyond 32768 tokens many
+ *              units take a kernel for unequal lengths if budgets are given one by one: sequences of one length
+ *              and one budget are better given NULL and k_uniform
  *   idx        out i32 [batch][n_kv_heads][k_max] (strides given), ascending token index,
  *              entries count..k_max-1 set to -1; k_max = max budget = the k passed to
  *              ha_workspace_bytes or less

@@ -423,8 +423,10 @@ __global__ void __launch_bounds__(kU_Threads, 1) encode_umma_kernel(const __grid
         }
         cp_async_commit();
         // Nothing of the kernel in front is read, and nothing written, before this point: its end overlaps the launch, the barriers
-        // and the fetch of the weights (us per call, back to back, 8 heads of 32768 keys 34.8 -> 31.9, of 8192 16.5 -> 13.9, of 256 10.4 -> 9.2).  The kernels behind start when this one has ended, as they read signatures before their
-        // own wait.  The tensor memory is allocated behind the wait: a kernel in front may still want it for itself.
+        // and the fetch of the weights (us per call, 40 calls back to back over four inputs, 8 heads of 32768 keys 34.9 -> 33.2, of
+        // 8192 16.5 -> 13.9, of 256 10.3 -> 9.1; the kernel by itself takes what it took).  The kernels behind start when this one has
+        // ended, as they read signatures before their own wait.  The tensor memory is allocated behind the wait: a kernel in front may
+        // still want it for itself.
         pdl_wait();
         if (warp == 0) {   // one warp allocates the tensor memory and passes the allocation right on
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem_base)), "r"(kU_TmemCols) : "memory");

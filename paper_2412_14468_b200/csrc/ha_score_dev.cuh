@@ -90,7 +90,7 @@ __device__ __forceinline__ uint32_t high_bits_to_nibble(uint32_t x) {
 // Writes the selected ones of 32 consecutive tokens from `first` on in ascending order: those with S > T (gt) and the first `room` of
 // those with S == T (eq; room <= 0: none).  dst is where the first of them goes; returns dst behind the last.  The selected ones are
 // worked out before any is visited: of the tokens at the threshold, often many times the wanted ones, a lane would visit all while
-// the rest of its warp waits (64 sequences of 32768 tokens 92.0 -> 89.6 us per step, 5 ragged ones in one launch 18.6 -> 17.2).
+// the rest of its warp waits (64 sequences of 32768 tokens 92.0 -> 89.6 us per step, 5 ragged ones in one launch 18.3 -> 17.2).
 __device__ __forceinline__ int32_t *write_selected32(int32_t *dst, int first, uint32_t gt, uint32_t eq, int room) {
     uint32_t sel = gt;
     if (room >= __popc(eq)) sel |= eq;

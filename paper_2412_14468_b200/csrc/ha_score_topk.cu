@@ -8,8 +8,8 @@
 //  * sequences of up to 131072 tokens: ONE kernel, a thread-block cluster per (sequence, KV head)
 //    (score_select_cluster_kernel, second half of this file), over contiguous or paged signatures (24 sequences of 2000 -
 //    65536 tokens in pages of 16, whole step: 61.4 us against 84.1 us with the two kernels below);
-//  * many units of unequal length, and long sequences from 24 units on: ONE kernel whose clusters take several units each
-//    (score_select_batch_kernel; batch_cluster_size has the rule);
+//  * many short units, many units of more than 32768 tokens with a budget each, and more than 131072 tokens from 24 units on: ONE
+//    kernel whose clusters take several units each (score_select_batch_kernel; batch_cluster_size has the rule);
 //  * other longer sequences: two kernels over chunks of the sequence, with the per-chunk histograms and
 //    one score byte per token passed through the workspace (scan_score_kernel, select_kernel).
 // No CTA ever spins on another: hand-offs are hardware cluster barriers or kernel boundaries.
@@ -619,7 +619,7 @@ static cudaError_t launch_cluster_t(int rows, int B, int Hq, int Hkv, const uint
 // falling length, forth and back, so that ragged batches end together.  A cluster takes up to eight units at a time through every
 // phase: scores of all of them, one exchange of histograms, thresholds, lists.  The fixed part (launch, first rows, barriers,
 // thresholds: 7 us) is thus paid once, not in every wave of one-unit clusters, no SM is left with more CTAs than another, and the
-// bytes of any sequence fit (96 KB of counters and score bytes per CTA), so the long ones need no second kernel.
+// bytes of a sequence of up to 750000 tokens fit (96 KB of counters and score bytes per CTA), so the long ones need no second kernel.
 //
 // Bound: the population count (groups of 4 and 8: 14.4 us for 512 units of 32768 tokens and 4 heads, 18 - 23 us measured for the
 // scoring), HBM for groups of 1.  Alone, against the one-unit clusters (us): 32 sequences of 8192 - 131072 tokens 41.6 -> 35.3, 24 of
