@@ -1097,10 +1097,12 @@ static cudaError_t launch_batch_t(int B, int Hq, int Hkv, const uint32_t *q_code
 //  * up to 10240 tokens, one CTA, whatever the lengths: 480 of 1000 +5 +6 +5 +5, of 5000 +5 +3 +2 +3; 1024 of 5000 +8 +7 +5 +5;
 //    2048 of 1000 +11 +13 +14 +15; but 384 of 3000 -5 -5 -5 -3.  Longer, or in larger groups, only where the CTAs are filled
 //    evenly: 512 of 8000 +1 0 +2 +3, 560 of 10240 +1 +2 +5 +4, 1024 of 10240 +1 +4 +4 +4, but 464 of 8000 -2 0 +2 +1, 640 of 8192 -2 0 +4 +5;
-//    in groups of 8, 512 of 4000 0 and +3 (s = 1, 4), of 8192 -3 and +2
+//    in groups of 8, 512 of 4000 0 and +3 (s = 1, 4), of 8192 -3 and +2.  Lists of up to 768 entries: longer ones take GATHER-ATT
+//    long enough for its early CTAs to count (n / k = 2, 4, 8, 16, 32, s = 1: 512 of 8192 -2 -1 0 0 +1, in pages of 16 -3 -6 -5 -2 0, of 1500
+//    +1 +5 +8 +9 +10; 1024 of 8192 in pages -2 -5 -3 +1 +3)
 //  * up to 32768, where clusters of 2 hold a unit, never: 512 of 32768 -6 -5 -1 +3, 592 of 32768 -3 -2 0 +4, 384 of 16000 -4 -3 -1 +3.
-//    Except lists per query head (append, queries, lists, attention): 464 of 16000 +2 +3 +4 +4, 512 of 32768 0 +3 +2 +5, but
-//    1024 of 24000 -6 -2 0 +4
+//    Except lists per query head of up to 1024 entries (append, queries, lists, attention): 464 of 16000 +2 +3 +4 +4, 512 of 32768
+//    0 +3 +2 +5, but 1024 of 24000 -6 -2 0 +4, and with 2048 entries 512 of 32768 -4 and +3 (s = 1, 4)
 //  * beyond, clusters of 2, and only with one budget per sequence, the one sign of unequal lengths that the host has.  Up to 65536,
 //    contiguous: 256 of 50000 +2 -1 0 +3, 296 of 65536 -1 -2 0 +2, but 192 of 50000 -5 -4 0 +3, 384 of 65536 -8 -6 -2 +2; in pages of
 //    16: 192 of 50000 +1 0 +2 +5, 296 of 65536 0 +1 +2 +3, 384 of 50000 -5 -3 +1 +4.  Up to 131072: 192 of 100000 -8 -3 +1 +4, 256 of
@@ -1116,7 +1118,7 @@ static cudaError_t launch_batch_t(int B, int Hq, int Hkv, const uint32_t *q_code
 //    +11), or 1.6 times in groups of 8 (40 of 300000 -6 -3 -1)
 //  * pages of fewer than 16 tokens never: 10 sequences of 10000 - 110000 in pages of 1 75.8 us per step, 98.0 here.
 template <int G>
-static int batch_cluster_size(long long units, int max_seq_len, bool budgets, bool per_head, const CodePages &cp) {
+static int batch_cluster_size(long long units, int max_seq_len, int k_max, bool budgets, bool per_head, const CodePages &cp) {
     const bool paged = cp.table != nullptr;
     if (units < 24 || units > 65536 || (paged && (cp.shift < 4 || cp.page_stride != (int)cp.page_stride))) return 0;
     const long long n = max_seq_len;
@@ -1132,11 +1134,11 @@ static int batch_cluster_size(long long units, int max_seq_len, bool budgets, bo
     if (n <= 10240) {
         const long long fullest = (units + c1 - 1) / c1;
         const bool even = 6 * units >= 5 * fullest * c1;
-        return many && (n * G <= 20480 || (even && n * G <= 40960)) ? 1 : 0;
+        return many && k_max <= 768 && (n * G <= 20480 || (even && n * G <= 40960)) ? 1 : 0;
     }
     if (n <= kClusterMaxSeq) {
         if (!budgets) return 0;
-        if (n <= 32768) return per_head && many && units <= 2 * c1 ? 1 : 0;
+        if (n <= 32768) return per_head && many && units <= 2 * c1 && k_max <= 1024 ? 1 : 0;
         if (n <= 65536) return (paged ? 5 * units >= 6 * c2 : 3 * units >= 5 * c2 && units <= 2 * c2) ? 2 : 0;
         if (5 * units >= 6 * c2 || (paged && 6 * units >= 5 * c2 && units <= c2)) return 2;
         return n > 98304 && 10 * units >= 9 * c4 && units <= c4 ? 4 : 0;
@@ -1169,7 +1171,7 @@ static cudaError_t launch_g(int B, int Hq, int Hkv, const uint32_t *q_codes, con
 #define HA_BATCH(CSZ) case CSZ: return cp.table ? launch_batch_t<G, CSZ, true>(HA_BATCH_ARGS) : launch_batch_t<G, CSZ, false>(HA_BATCH_ARGS)
 #define HA_BATCH_ARGS B, Hq, Hkv, q_codes, k_codes, kc_sb, kc_sh, seq_lens, k_per_seq, k_uniform, max_seq_len, k_max, idx, \
                       idx_sb, idx_sh, count, hist_out, st, win, cp, kv_shift, in_step
-        switch (batch_cluster_size<G>((long long)B * Hkv, max_seq_len, k_per_seq != nullptr, row_shift >= 0, cp)) {
+        switch (batch_cluster_size<G>((long long)B * Hkv, max_seq_len, k_max, k_per_seq != nullptr, row_shift >= 0, cp)) {
             HA_BATCH(1);
             HA_BATCH(2);
             HA_BATCH(4);

@@ -80,6 +80,11 @@ NEXT_TO_BATCH_CASES = [
 PER_HEAD_BATCH_CASES = [(58, 2, 4, 900, 1), (15, 8, 4, 12000, 1), (37, 8, 2, 32768, 1), (23, 2, 4, 40000, 2), (13, 4, 2, 140000, 2)]
 
 
+def budgets(lens):
+    """A budget per sequence: among short ones nothing and everything."""
+    return [(0, n, max(1, n // 11), max(1, n // 40))[i % 4] if n < 600 else n // 40 for i, n in enumerate(lens)]
+
+
 def batches(Hkv, lens, cs, clusters, page=0, staged=False, most=8, pool=96 * 1024):
     """Batches of the busiest cluster: units by falling length, dealt out forth and back, as many at a time as fit the pool."""
     order = sorted(range(len(lens)), key=lambda b: -lens[b]) if len(lens) <= 512 else range(len(lens))

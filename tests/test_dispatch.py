@@ -2,7 +2,7 @@
 import pytest
 
 from paper_2412_14468_b200 import binding as ha
-from tests._fake import BATCH, BATCH_CASES, NEXT_TO_BATCH_CASES, PER_HEAD_BATCH_CASES, RESIDENT, SEVERAL_UNITS_PER_CLUSTER, Fake, batches
+from tests._fake import BATCH, BATCH_CASES, NEXT_TO_BATCH_CASES, PER_HEAD_BATCH_CASES, RESIDENT, SEVERAL_UNITS_PER_CLUSTER, Fake, batches, budgets, ragged
 
 
 def test_a_failing_occupancy_query_leaves_no_error_behind(tmp_path):
@@ -36,7 +36,7 @@ def test_cases_of_clusters_of_several_units(fake, case):
     """The GPU test of these calls reaches the cluster size, the number of batches and the staging that it is there for."""
     G, Hkv, lens, pages, cs, n_batches, staged = case
     for page in pages:
-        assert fake.score_topk(len(lens), G, Hkv, max(lens), page=page) == ha.HA_OK
+        assert fake.score_topk(len(lens), G, Hkv, max(lens), page=page, k_max=max(max(budgets(lens)) + 137, 1)) == ha.HA_OK
         (kernel, args, ctas, cluster, _, is_staged), = fake.launches()
         assert kernel == BATCH and args == [G, cs, int(page > 0)] and cluster == cs
         assert ctas == cs * min(RESIDENT[cs], len(lens) * Hkv)
@@ -54,9 +54,16 @@ def test_cases_beside_clusters_of_several_units(fake, case):
 
 @pytest.mark.parametrize("B,Hkv,G,longest,cs", PER_HEAD_BATCH_CASES)
 def test_cases_of_lists_per_query_head_on_clusters_of_several_units(fake, B, Hkv, G, longest, cs):
-    assert fake.score_topk(B, G, Hkv, longest, page=16, per_head=True) == ha.HA_OK
+    assert fake.score_topk(B, G, Hkv, longest, page=16, per_head=True, k_max=max(budgets(ragged(B, longest)))) == ha.HA_OK
     (kernel, args, ctas, cluster, *_), = fake.launches()
     assert kernel == BATCH and args == [1, cs, 1] and cluster == cs and ctas == cs * min(RESIDENT[cs], B * Hkv * G)
+
+
+@pytest.mark.parametrize("B,Hkv,n,per_head,longest_list", [(64, 8, 8192, False, 768), (64, 8, 8192, True, 768), (15, 8, 16000, True, 1024)])
+def test_long_lists_stay_with_clusters_of_one_unit(fake, B, Hkv, n, per_head, longest_list):
+    for k_max in (longest_list, longest_list + 1):
+        assert fake.score_topk(B, 4, Hkv, n, page=16, per_head=per_head, k_max=k_max) == ha.HA_OK
+    assert [k for k, *_ in fake.launches()] == [BATCH, "score_select_cluster_kernel"]
 
 
 @pytest.mark.parametrize("page", [0, 16, 64])

@@ -7,7 +7,7 @@ import torch
 import oracle
 from paper_2412_14468_b200 import binding as ha
 from paper_2412_14468_b200 import workloads as wl
-from tests._fake import BATCH_CASES, NEXT_TO_BATCH_CASES, PER_HEAD_BATCH_CASES, ragged
+from tests._fake import BATCH_CASES, NEXT_TO_BATCH_CASES, PER_HEAD_BATCH_CASES, budgets, ragged
 from tests._util import OUT_TOL, assert_out_close, max_abs_diff_bf16, u16
 from tests.test_gpu_parity import _attn_inputs, _check_gather, _run_step, _check_score_topk, _check_score_topk_wide, _page_codes, _wide_codes, _wide_mapping, \
     test_whole_step_with_keys_values_and_signatures_all_paged as _whole_paged_step
@@ -127,7 +127,7 @@ def test_score_topk_with_several_units_per_cluster(G, Hkv, lens, page_size):
     (test_dispatch.py holds the cases to their kernels, batches and staged tables.)"""
     rng = np.random.default_rng(len(lens) + page_size)
     B, Hq, n_cap = len(lens), Hkv * G, max(lens) // 128 * 128 + 128
-    ks = [(0, n, max(1, n // 11), max(1, n // 40))[i % 4] if n < 3000 else n // 40 for i, n in enumerate(lens)]
+    ks = budgets(lens)
     n_sink, n_local = (130, 7) if page_size == 16 else (0, 0)
     k_max = max(max(ks) + n_sink + n_local, 1)
     codes = rng.integers(0, 2**32, size=(B, Hkv, n_cap), dtype=np.uint64).astype(np.uint32)
@@ -164,7 +164,7 @@ def test_score_topk_per_head_with_several_units_per_cluster(B, Hkv, G, longest, 
     """Lists per query head over pages: G units share the signatures of a KV head."""
     rng = np.random.default_rng(B + page_size)
     lens = ragged(B, longest)
-    ks = [max(1, n // 30) for n in lens]
+    ks = budgets(lens)
     k_max, Hq = max(ks), Hkv * G
     codes = rng.integers(0, 2**32, size=(B, Hkv, longest), dtype=np.uint64).astype(np.uint32)
     codes[:, :, 100:400] = codes[:, :, 100:101]                     # ties decided by token index
